@@ -36,12 +36,15 @@ Workspace plan_workspace(const lif_layer_desc& d, int ffn_grid_max) {
   w.n_tmp = take(64);
   w.z_partial = take(z_ctas * S * d.rank * 4);
   w.mask_words = take(n_mask * 4);
-  w.new_mask_words = take((size_t)new_mask_entries(d) * 8);
+  w.new_mask_words = take((size_t)new_mask_entries(d) * 2 * 8);
   w.keep_tok = take(d.spec_keep > 0 ? F : 0);
   w.h_rows = take(d.n_streams > 1 ? (size_t)kBatchedMaxKSplit * F * 8 * 4 *
                                         (d.gate_mode == LIF_GATE_BUNDLED ? 2 : 1)
                                   : 0);
   w.gate_val = take(d.gate_mode == LIF_GATE_RESIDENT ? S * F * 4 : 0);
+  w.hit_rows = take(F * 4);
+  w.step_sync = take(step_sync_bytes());
+  w.step_tagged = take(step_tagged_bytes(d));
   size_t partial_rows = (size_t)ffn_grid_max;
   if (ffn_batched_supported(d) && (size_t)kBatchedMaxPartitions * S > partial_rows)
     partial_rows = (size_t)kBatchedMaxPartitions * S;
@@ -56,7 +59,7 @@ static lif_status check_shape(const lif_layer_desc* d) {
   if (!d) return LIF_ERR_INVALID_ARG;
   if (d->d_model < 8 || d->d_model % 8 || d->d_model > 8192) return LIF_ERR_INVALID_ARG;
   if (d->d_ff < 8 || d->d_ff % 8 || d->d_ff >= (1 << 21)) return LIF_ERR_INVALID_ARG;
-  if (d->rank < 8 || d->rank % 8 || d->rank > 2048) return LIF_ERR_INVALID_ARG;
+  if (d->rank < 8 || d->rank % 8 || d->rank > kMaxRank) return LIF_ERR_INVALID_ARG;
   if (d->window_k < 1) return LIF_ERR_INVALID_ARG;
   if (d->capacity < 1 || d->capacity > d->d_ff) return LIF_ERR_INVALID_ARG;
   if (d->n_streams < 1 || d->n_streams > kMaxStreams) return LIF_ERR_INVALID_ARG;
@@ -156,6 +159,9 @@ lif_status lif_create_layer(const lif_layer_desc* desc, lif_layer** out) {
   L->z_partial = (float*)(b + ws.z_partial);
   L->mask_words = (uint32_t*)(b + ws.mask_words);
   L->new_mask_words = (unsigned long long*)(b + ws.new_mask_words);
+  L->hit_rows = (uint32_t*)(b + ws.hit_rows);
+  L->step_sync = (uint32_t*)(b + ws.step_sync);
+  L->step_tagged = (uint32_t*)(b + ws.step_tagged);
   L->keep_tok = desc->spec_keep > 0 ? (int8_t*)(b + ws.keep_tok) : nullptr;
   L->y_partial = (float*)(b + ws.y_partial);
   L->h_rows = (float*)(b + ws.h_rows);
@@ -178,7 +184,8 @@ lif_status lif_create_layer(const lif_layer_desc* desc, lif_layer** out) {
     L->split_ffn = 1;
     L->fused_plan = window_plan_supported(*desc) ? 1 : 0;
     L->fused_fetch = 1;
-    ok = cudaEventCreateWithFlags(&L->ev_plan, cudaEventDisableTiming) == cudaSuccess;
+    ok = step_configure(L) == cudaSuccess && predict_configure(L) == cudaSuccess;
+    ok = ok && cudaEventCreateWithFlags(&L->ev_plan, cudaEventDisableTiming) == cudaSuccess;
     if (ok && cudaEventCreateWithFlags(&L->ev_fetch, cudaEventDisableTiming) != cudaSuccess) {
       cudaEventDestroy(L->ev_plan);
       ok = false;
@@ -315,6 +322,17 @@ lif_status lif_decode_step(lif_layer* L, const void* dev_x, float* dev_y, void* 
     ev = L->tm_events + (size_t)(L->tm_cursor++) * kTimingEvents;
   if (ev) tm_record(ev[0], sc);
   bool ok;
+  // One input stream: predictor, then everything else in one launch, unless the caller times the
+  // phases or has set a knob of the separate kernels.
+  if (L->step_ok && !ev && L->fused_plan && L->split_ffn && L->fused_fetch &&
+      L->fetch_grid == L->n_sm && L->ffn_grid == L->n_sm && L->ffn_stages == L->ffn_stages_max) {
+    L->single_step = 1;
+    ok = launch_predict(L, x, nullptr, L->active_idx, L->n_tmp, sc, nullptr, 0) == cudaSuccess;
+    L->single_step = 0;
+    ok = ok && launch_step(L, x, dev_y, sc) == cudaSuccess;
+    if (!ok) cudaGetLastError();
+    return ok ? LIF_OK : LIF_ERR_CUDA;
+  }
   // With append_first the row moves and the bundle writes touch different rows, so given a
   // second stream the moves leave the critical chain (they only precede the cached rows' FFN).
   const bool moves_aside = L->desc.append_first && sf != sc;
@@ -353,12 +371,14 @@ lif_status lif_decode_step(lif_layer* L, const void* dev_x, float* dev_y, void* 
     ok = ok && launch_fetch_early(L, sc, kEarlyWatch) == cudaSuccess;
     if (ev) tm_record(ev[6], sc);
     if (moves_aside) ok = ok && cudaStreamWaitEvent(sc, L->ev_fetch, 0) == cudaSuccess;
+    L->ends_step = 1;
     if (L->desc.ffn_mode == 0)
       ok = ok && launch_ffn(L, x, L->active_slots, L->counts + LIF_CNT_N_ACTIVE, nullptr, dev_y,
                             false, sc, ev) == cudaSuccess;
     else
       ok = ok && launch_ffn(L, x, nullptr, L->counts + LIF_CNT_NUM_USED, nullptr, dev_y, false,
                             sc, ev) == cudaSuccess;
+    L->ends_step = 0;
     if (!ok) cudaGetLastError();
     return ok ? LIF_OK : LIF_ERR_CUDA;
   }
@@ -374,12 +394,14 @@ lif_status lif_decode_step(lif_layer* L, const void* dev_x, float* dev_y, void* 
     ok = ok && cudaEventRecord(L->ev_fetch, sf) == cudaSuccess;
     ok = ok && cudaStreamWaitEvent(sc, L->ev_fetch, 0) == cudaSuccess;
   }
+  L->ends_step = 1;
   if (L->desc.ffn_mode == 0)
     ok = ok && launch_ffn(L, x, L->active_slots, L->counts + LIF_CNT_N_ACTIVE, nullptr, dev_y,
                           false, sc, ev) == cudaSuccess;
   else
     ok = ok && launch_ffn(L, x, nullptr, L->counts + LIF_CNT_NUM_USED, nullptr, dev_y, false,
                           sc, ev) == cudaSuccess;
+  L->ends_step = 0;
   if (!ok) cudaGetLastError();
   return ok ? LIF_OK : LIF_ERR_CUDA;
 }
@@ -670,7 +692,9 @@ lif_status lif_restore(lif_layer* L, const void* host_buf, size_t bytes) {
     }
     in += p[i].bytes;
   }
-  if (launch_refill(L, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+  // entries of predictor runs after the snapshot must not be taken for those of the next run
+  if (cudaMemset(L->new_mask_words, 0, (size_t)new_mask_entries(L->desc) * 2 * 8) != cudaSuccess ||
+      launch_refill(L, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
     cudaGetLastError();
     return LIF_ERR_CUDA;
   }

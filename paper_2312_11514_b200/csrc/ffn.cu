@@ -237,12 +237,14 @@ ffn_reduce_kernel(const float* __restrict__ p0, const int32_t* __restrict__ n0,
       t = make_float4(lo.x, lo.y, hi.x, hi.y);
     }
   }
+  // (settled before the score kernel of this step started)
+  const int run = next_run_after_wait && blockIdx.x == 0 && tid == 0 ? __ldcg(next_run_after_wait) : 0;
   pdl_wait();
   pdl_trigger();
   // every earlier kernel of the step is complete: the next predictor run gets its number here,
-  // long before it starts (a predictor without a first stage of its own relies on this)
+  // long before it starts
   if (next_run_after_wait && blockIdx.x == 0 && tid == 0)
-    *next_run_after_wait = (int)((unsigned)*next_run_after_wait + 1u);   // wraps
+    advance_run(next_run_after_wait, run);
   // counts as the kernels that wrote the partials clamp them: [0, n_cap]
   const int v0 = min(G, max(0, min(*n0, n_cap))), v1 = p1 ? min(G, max(0, min(*n1, n_cap))) : 0;
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -368,7 +370,8 @@ cudaError_t launch_ffn(lif_layer* L, const __half* x, const int32_t* slots, cons
     e = launch_k(ffn_reduce_kernel, dim3((d / 4 + kSumCols - 1) / kSumCols), dim3(kSumThreads), 0, st, L->use_pdl,
                  (const float*)L->y_partial, n, (const float*)nullptr, (const int32_t*)nullptr,
                  L->ffn_grid, (const __half*)D.dev_bias_down, d, y + (size_t)s * d, d,
-                 accumulate ? 1 : 0, D.capacity, (int*)nullptr);
+                 accumulate ? 1 : 0, D.capacity,
+                 L->ends_step && s == D.n_streams - 1 ? (int*)(L->counts + CNT_PREDICTOR_RUN) : (int*)nullptr);
     if (e != cudaSuccess) return e;
   }
   if (ev) tm_record(ev[9], st);
@@ -414,7 +417,8 @@ cudaError_t launch_partial_sum(lif_layer* L, const float* partial, const int32_t
   return launch_k(ffn_reduce_kernel, dim3((width / 4 + kSumCols - 1) / kSumCols),
                   dim3(kSumThreads), 0, st, L->use_pdl, partial, n, (const float*)nullptr,
                   (const int32_t*)nullptr, partitions, (const __half*)L->desc.dev_bias_down,
-                  L->desc.d_model, y, width, 0, L->desc.capacity, (int*)nullptr);
+                  L->desc.d_model, y, width, 0, L->desc.capacity,
+                  L->ends_step ? (int*)(L->counts + CNT_PREDICTOR_RUN) : (int*)nullptr);
 }
 
 // Fetch + FFN of a single-stream decode step.  The critical chain stays on `st` with dependent

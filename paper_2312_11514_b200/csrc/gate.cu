@@ -32,7 +32,7 @@ gate_scores_kernel(const __half* __restrict__ x, const __half* __restrict__ gate
                    uint32_t* mask_words, int* ticket, int* __restrict__ active_idx,
                    int* __restrict__ n_active, int compact, int nwords,
                    const int32_t* __restrict__ slot_of, unsigned long long* new_mask_words,
-                   const int* predictor_run) {
+                   int* predictor_run) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint4* xs = reinterpret_cast<uint4*>(smem_raw);          // [S][d / 8]
   __shared__ int act_flag[kGateTile];     // bit 0: active, bit 1: active and not cached yet
@@ -138,15 +138,22 @@ gate_scores_kernel(const __half* __restrict__ x, const __half* __restrict__ gate
       const unsigned long long e = (unsigned long long)mn | ((unsigned long long)(unsigned)run << 32);
       asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(new_mask_words + blockIdx.x), "l"(e)
                    : "memory");
+      // likewise the active neurons themselves
+      const unsigned long long ea = (unsigned long long)m | ((unsigned long long)(unsigned)run << 32);
+      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(new_mask_words + gridDim.x + blockIdx.x),
+                   "l"(ea) : "memory");
     }
   }
   if (!compact) return;     // the consumer reads the bit mask itself
   compact_mask_last_cta(mask_words, nwords, ticket, active_idx, n_active, warp_sums, &is_last);
+  // every CTA has read this run's number: the next run gets one of its own (in a decode step
+  // the kernel that ends the step does this)
+  if (is_last && tid == 0) advance_run(predictor_run, run);
 }
 
 template <int S>
 cudaError_t launch_gate_s(lif_layer* L, const __half* x, float* logits, int32_t* active_idx,
-                          int32_t* n_active, cudaStream_t st, int compact) {
+                          int32_t* n_active, cudaStream_t st, int compact, int* run) {
   const lif_layer_desc& D = L->desc;
   const int grid = (D.d_ff + kGateTile - 1) / kGateTile;
   const size_t smem = (size_t)S * D.d_model * 2;
@@ -161,7 +168,7 @@ cudaError_t launch_gate_s(lif_layer* L, const __half* x, float* logits, int32_t*
                   D.d_ff, L->gate_val, logits, L->mask_words,
                   (int*)(L->counts + CNT_TICKET_PREDICT), (int*)active_idx, (int*)n_active, compact,
                   (D.d_ff + 31) / 32, (const int32_t*)L->slot_of, L->new_mask_words,
-                  (int*)(L->counts + CNT_PREDICTOR_RUN));
+                  run);
 }
 
 }  // namespace
@@ -169,18 +176,20 @@ cudaError_t launch_gate_s(lif_layer* L, const __half* x, float* logits, int32_t*
 int gate_predict_tile() { return kGateTile; }
 
 cudaError_t launch_gate_predict(lif_layer* L, const __half* x, float* logits, int32_t* active_idx,
-                                int32_t* n_active, cudaStream_t st, cudaEvent_t* ev, int compact) {
+                                int32_t* n_active, cudaStream_t st, cudaEvent_t* ev, int compact,
+                                bool consumed) {
+  int* run = (int*)(L->counts + (consumed ? CNT_PREDICTOR_RUN : CNT_NO_RUN));
   if (ev) tm_record(ev[1], st);     // no first stage in this mode
   cudaError_t e = cudaErrorInvalidValue;
   switch (L->desc.n_streams) {
-    case 1: e = launch_gate_s<1>(L, x, logits, active_idx, n_active, st, compact); break;
-    case 2: e = launch_gate_s<2>(L, x, logits, active_idx, n_active, st, compact); break;
-    case 3: e = launch_gate_s<3>(L, x, logits, active_idx, n_active, st, compact); break;
-    case 4: e = launch_gate_s<4>(L, x, logits, active_idx, n_active, st, compact); break;
-    case 5: e = launch_gate_s<5>(L, x, logits, active_idx, n_active, st, compact); break;
-    case 6: e = launch_gate_s<6>(L, x, logits, active_idx, n_active, st, compact); break;
-    case 7: e = launch_gate_s<7>(L, x, logits, active_idx, n_active, st, compact); break;
-    case 8: e = launch_gate_s<8>(L, x, logits, active_idx, n_active, st, compact); break;
+    case 1: e = launch_gate_s<1>(L, x, logits, active_idx, n_active, st, compact, run); break;
+    case 2: e = launch_gate_s<2>(L, x, logits, active_idx, n_active, st, compact, run); break;
+    case 3: e = launch_gate_s<3>(L, x, logits, active_idx, n_active, st, compact, run); break;
+    case 4: e = launch_gate_s<4>(L, x, logits, active_idx, n_active, st, compact, run); break;
+    case 5: e = launch_gate_s<5>(L, x, logits, active_idx, n_active, st, compact, run); break;
+    case 6: e = launch_gate_s<6>(L, x, logits, active_idx, n_active, st, compact, run); break;
+    case 7: e = launch_gate_s<7>(L, x, logits, active_idx, n_active, st, compact, run); break;
+    case 8: e = launch_gate_s<8>(L, x, logits, active_idx, n_active, st, compact, run); break;
   }
   if (ev) tm_record(ev[2], st);
   return e;

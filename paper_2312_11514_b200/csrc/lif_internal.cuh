@@ -13,7 +13,9 @@ namespace lif {
 // Private entries of the counts block (public ones: LIF_CNT_* in lif.h).
 enum {
   CNT_TICKET_PREDICT = 16,  // "last block done" counter of the score kernel
-  CNT_PREDICTOR_RUN = 17,   // number of the predictor run whose masks are (being) written
+  CNT_PREDICTOR_RUN = 17,   // number of the predictor run whose masks are (being) written; advanced
+                            // by the kernel that ends a decode step, or by the run that compacts
+  CNT_NO_RUN = 18,          // always 0: runs that no step consumes are tagged with it
   CNT_TOTALS = 32           // four uint64: bytes_fetched, rows_moved, rows_active, rows_cached
 };
 
@@ -31,13 +33,14 @@ inline int z_cta_count(int d_model) {
 }
 constexpr int kLogitTile = 128;     // neurons per CTA in the second predictor stage
 constexpr int kMaxStreams = 8;
+constexpr int kMaxRank = 2048;
 constexpr int kTimingEvents = 10;   // z0 z1 s1 w1 m1 | f0 f1 | g0 g1 r1
 
 struct Workspace {
   // offsets in bytes from the workspace base; every block 256-byte aligned
   size_t counts, pointers, slot_of, last_active, bias, active_idx, evict_ids, evict_slots,
       move_src, move_dst, load_ids, load_slots, active_slots, hit_slots, n_tmp, z_partial,
-      mask_words, new_mask_words, keep_tok, h_rows, gate_val, y_partial, total;
+      mask_words, new_mask_words, keep_tok, h_rows, gate_val, hit_rows, step_sync, step_tagged, y_partial, total;
 };
 
 // fp16 elements per bundle / cache row: up | down, preceded by the gate row when it is bundled
@@ -63,6 +66,7 @@ struct lif_layer {
   // Neurons predicted active that have no cache row yet, as 64-bit entries {bits, run}: the low
   // half holds the bits of 32 consecutive neurons (of one predictor CTA's neurons, where those
   // are fewer), the high half the number of the predictor run that stored it (one store).
+  // A second block of as many entries holds the active neurons themselves in the same form.
   unsigned long long* new_mask_words;
   int8_t* keep_tok;   // [d_ff] last kept token per neuron (speculative mode)
   float* y_partial;
@@ -73,6 +77,12 @@ struct lif_layer {
   int fb_ok, fb_up_stages, fb_parts, fb_cols, fb_partitions;
   int fb_ksplit, fb_kps, fb_up_partitions, fb_parts_min, fb_up_group, fb_up_two_ctas;
   size_t fb_up_smem, fb_down_smem;
+  // single-launch decode step (step.cu); step_ok = 0: it does not apply to this layer
+  int step_ok, step_cache_ctas, step_group, step_cache_stages, step_fetch_stages;
+  size_t step_smem;
+  uint32_t* hit_rows;         // plan of the step: rows (before the moves) and neurons of the hits
+  uint32_t* step_sync;        // its counters
+  uint32_t* step_tagged;      // its tagged partial sums (no tag of a step to come)
   int n_sm;
   int z_ctas;         // CTAs of the first predictor stage
   int ffn_grid;       // CTAs of the sparse-FFN kernel
@@ -83,6 +93,8 @@ struct lif_layer {
   int move_grid;
   unsigned wait_polls; // poll limit of the first wait on each bulk copy in the FFN kernels
   int early_fetch;    // knob: the plain fetch of lif_decode_step starts early behind the window kernel
+  int ends_step;      // set by lif_decode_step: the FFN's last kernel advances the run number
+  int single_step;    // set by lif_decode_step: the single-launch step follows the predictor
   int watch_chain;    // set by lif_decode_step while it launches a step whose fetch kernel watches
                       // the predictor: window and row-move kernels release their dependents at entry
   int use_pdl;        // programmatic dependent launch along the compute stream
@@ -122,7 +134,8 @@ cudaError_t launch_predict(lif_layer* L, const __half* x, float* logits, int32_t
                            int compact = 1);   // compact = 0: leave only the bit mask
 // Resident gate projection as the predictor: scores, threshold, bit mask, optional compaction.
 cudaError_t launch_gate_predict(lif_layer* L, const __half* x, float* logits, int32_t* active_idx,
-                                int32_t* n_active, cudaStream_t st, cudaEvent_t* ev, int compact);
+                                int32_t* n_active, cudaStream_t st, cudaEvent_t* ev, int compact,
+                                bool consumed = true);
 bool window_plan_supported(const lif_layer_desc& D);
 // with_moves = false: the caller launches the row moves itself (launch_moves)
 cudaError_t launch_window_plan(lif_layer* L, cudaStream_t st, cudaEvent_t* ev = nullptr,
@@ -158,6 +171,12 @@ inline int new_mask_entries(const lif_layer_desc& D) {
 enum { kEarlyNone = 0, kEarlyLists = 1, kEarlyMask = 2, kEarlyWatch = 3 };
 cudaError_t launch_fetch_ffn(lif_layer* L, const __half* x, float* partial, cudaStream_t st,
                              int early);
+// Everything of a single-stream decode step behind the predictor, in one launch (step.cu).
+size_t step_sync_bytes();
+size_t step_tagged_bytes(const lif_layer_desc& D);
+cudaError_t predict_configure(const lif_layer* L);
+cudaError_t step_configure(lif_layer* L);
+cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st);
 cudaError_t launch_refill(lif_layer* L, cudaStream_t st);
 cudaError_t launch_probe(const void* dev_src_alias, void* dev_dst, size_t bytes, size_t chunk,
                          int grid, cudaStream_t st);
@@ -195,23 +214,44 @@ size_t ffn_smem_for(const lif_layer* L, int stages);
 // a cross-stream event wait included (measured: a kernel that read another stream's output
 // ahead of its wait raced in graph replay only).  So what a kernel reads before pdl_wait() must
 // be weights, or data that was final before each kernel ahead of it passed its own wait.
+// full_smem: the launch prefers the full shared-memory carve-out.  An SM changes its carve-out only
+// when it is empty, so a kernel that needs much shared memory cannot become resident beside one
+// launched with another preference.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                     cudaStream_t st, int pdl, Args... args) {
+cudaError_t launch_k2(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                      cudaStream_t st, int pdl, int full_smem, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (pdl) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (full_smem) {
+    at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[n++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+  }
   cfg.attrs = at;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                     cudaStream_t st, int pdl, Args... args) {
+  return launch_k2(kernel, grid, block, smem, st, pdl, 0, args...);
 }
 
 #ifdef __CUDACC__
+// The next predictor run gets a number of its own (0 stays 0: see CNT_NO_RUN).
+// `now`: the number of the run that ends, read when it began (reading it here would put a memory
+// round trip at the end of the kernel).
+__device__ __forceinline__ void advance_run(int* run, int now) {
+  if (now) *run = now == -1 ? 1 : (int)((unsigned)now + 1u);
+}
 // Block until every earlier kernel of the stream has completed and its writes are visible
 // (no-op for a kernel launched without the attribute).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -242,6 +282,14 @@ __device__ __forceinline__ uint4 ld_stream16(const void* p) {
                : "memory");
   return v;
 }
+
+// 16-byte asynchronous copy into shared memory (no register holds the data while it travels);
+// own_copies_wait(): the thread's copies have landed and it may read them
+__device__ __forceinline__ void copy_async16(void* smem, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(smem)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void own_copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // eight fp16 values -> fp32
 __device__ __forceinline__ void unpack8(const uint4& v, float* f) {

@@ -17,7 +17,8 @@ namespace {
 template <int S>
 __global__ void __launch_bounds__(kThreads)
 predict_z_kernel(const __half* __restrict__ x, const __half* __restrict__ A, int d, int r,
-                 int rows_per_cta, float* __restrict__ z_partial, int* predictor_run) {
+                 int rows_per_cta, int staged, float* __restrict__ z_partial) {
+  extern __shared__ __align__(16) uint4 staged_rows[];   // [staged][kThreads]
   __shared__ float red[2048];
   const int ncg = r >> 3;            // 8-column groups (16 bytes each)
   const int nrl = kThreads / ncg;    // row lanes
@@ -32,19 +33,22 @@ predict_z_kernel(const __half* __restrict__ x, const __half* __restrict__ A, int
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[s][e] = 0.f;
 
-  // A is a weight: its first 8 rows per thread are put in flight before the dependency wait,
-  // x (possibly written by the previous kernel) only after it.
+  // A is a weight: the thread's first 8 rows go into registers and the next `staged` into its own
+  // slots of shared memory before the dependency wait, x (possibly written by the previous kernel)
+  // comes only after it.  The kernel is resident long before its input is complete, so behind the
+  // wait nothing of A is left to load (rows that were cost 2 us per launch at 4544 x 128).
   uint4 aq[8];
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const int m = m0 + rl + u * nrl;
     aq[u] = (rl < nrl && m < m1) ? ld_stream16(A + (size_t)m * r + cg * 8) : make_uint4(0, 0, 0, 0);
   }
+  for (int u = 0; u < staged; ++u) {
+    const int m = m0 + rl + (8 + u) * nrl;
+    if (rl < nrl && m < m1) copy_async16(staged_rows + u * kThreads + tid, A + (size_t)m * r + cg * 8);
+  }
   pdl_wait();
   pdl_trigger();
-  // every earlier kernel is complete: a new predictor run begins, and its number is settled
-  // before the score kernel, which tags its mask words with it, passes its own wait
-  if (blockIdx.x == 0 && tid == 0) *predictor_run = (int)((unsigned)*predictor_run + 1u);   // wraps
   if (rl < nrl) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
@@ -60,8 +64,23 @@ predict_z_kernel(const __half* __restrict__ x, const __half* __restrict__ A, int
         }
       }
     }
+    own_copies_wait();
 #pragma unroll 4
-    for (int m = m0 + rl + 8 * nrl; m < m1; m += nrl) {
+    for (int u = 0; u < staged; ++u) {
+      const int m = m0 + rl + (8 + u) * nrl;
+      if (m < m1) {
+        float af[8];
+        unpack8(staged_rows[u * kThreads + tid], af);
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          const float xs = __half2float(x[(size_t)s * d + m]);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) acc[s][e] = fmaf(xs, af[e], acc[s][e]);
+        }
+      }
+    }
+#pragma unroll 4
+    for (int m = m0 + rl + (8 + staged) * nrl; m < m1; m += nrl) {
       float af[8];
       unpack8(ld_stream16(A + (size_t)m * r + cg * 8), af);
 #pragma unroll
@@ -98,8 +117,8 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
                       float* __restrict__ logits, uint32_t* mask_words, int* ticket,
                       int* __restrict__ active_idx, int* __restrict__ n_active, int compact,
                       int8_t* __restrict__ keep_tok, int keep, const int32_t* __restrict__ slot_of,
-                      unsigned long long* new_mask_words, const int* predictor_run) {
-  extern __shared__ float zs[];                 // [S][r]
+                      unsigned long long* new_mask_words, int* predictor_run, int staged) {
+  extern __shared__ __align__(16) float zs[];   // [S][r], then the rows of B beyond the first 128
   __shared__ float red[16][kLogitTile];
   __shared__ int warp_sums[kThreads / 32];
   __shared__ int is_last;
@@ -115,14 +134,23 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
     const int j = rs + 16 * u;
     bq[u] = (col < F && j < r) ? ld_stream16(B + (size_t)j * F + col) : make_uint4(0, 0, 0, 0);
   }
+  // the next rows go into the thread's own slots of shared memory (see predict_z_kernel)
+  uint4* staged_rows = reinterpret_cast<uint4*>(zs + S * r) + tid;
+  for (int u = 0; u < staged; ++u) {
+    const int j = rs + 16 * (8 + u);
+    if (col < F && j < r) copy_async16(staged_rows + u * kThreads, B + (size_t)j * F + col);
+  }
   const int my_col = blockIdx.x * kLogitTile + tid;   // used by threads < kLogitTile
   const float my_c = (tid < kLogitTile && my_col < F) ? c[my_col] : 0.f;
   // The window state was last written by this layer's previous step, complete long before this
   // kernel could start: whether the neuron already has a cache row is read here, so the mask of
   // neurons to bring in (active and not cached) costs no round trip of its own.
   const int my_row = (tid < kLogitTile && my_col < F) ? slot_of[my_col] : 0;
-  pdl_wait();
+  // Released before this kernel's own wait: what follows (the window kernel or the single-launch
+  // step) reads ahead of its wait only the window state, complete before stage 1 passed its own
+  // wait and released this kernel, and entries that carry this run's number.
   pdl_trigger();
+  pdl_wait();
   const int run = (tid < kLogitTile && (tid & 31) == 0) ? __ldcg(predictor_run) : 0;
   if (S == 1) {
     // one stream: every partial of a sum is requested before the first is used (one memory
@@ -165,10 +193,13 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
     for (int e = 0; e < 8; ++e) acc[s][e] = 0.f;
   for (int j0 = 0; j0 < r; j0 += 128) {
     if (j0 > 0) {
+      if (j0 == 128) own_copies_wait();
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int j = j0 + rs + 16 * u;
-        bq[u] = (col < F && j < r) ? ld_stream16(B + (size_t)j * F + col) : make_uint4(0, 0, 0, 0);
+        const int j = j0 + rs + 16 * u, at = (j0 >> 4) - 8 + u;
+        bq[u] = make_uint4(0, 0, 0, 0);
+        if (col < F && j < r)
+          bq[u] = at < staged ? staged_rows[at * kThreads] : ld_stream16(B + (size_t)j * F + col);
       }
     }
 #pragma unroll
@@ -216,46 +247,87 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
       const unsigned long long e = (unsigned long long)mn | ((unsigned long long)(unsigned)run << 32);
       asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(
                        new_mask_words + blockIdx.x * (kLogitTile / 32) + (tid >> 5)), "l"(e) : "memory");
+      const unsigned long long ea = (unsigned long long)m | ((unsigned long long)(unsigned)run << 32);
+      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(
+                       new_mask_words + (gridDim.x + blockIdx.x) * (kLogitTile / 32) + (tid >> 5)),
+                   "l"(ea) : "memory");
     }
   }
 
   if (!compact) return;     // the consumer reads the bit mask itself
   compact_mask_last_cta(mask_words, gridDim.x * (kLogitTile / 32), ticket, active_idx, n_active,
                         warp_sums, &is_last);
+  // every CTA has read this run's number: the next run gets one of its own (in a decode step
+  // that reads the mask itself, the kernel that ends the step does this)
+  if (is_last && tid == 0) advance_run(predictor_run, run);
+}
+
+// Rows per thread that are staged in shared memory, at most 48 KB of them per CTA.
+constexpr int kMaxStaged = 12;
+int z_staged_rows(const lif_layer_desc& D) {
+  const int lanes = kThreads / (D.rank / 8) > 0 ? kThreads / (D.rank / 8) : 1;
+  const int rows = (z_rows_per_cta(D.d_model) + lanes - 1) / lanes - 8;
+  return rows < 0 ? 0 : (rows > kMaxStaged ? kMaxStaged : rows);
+}
+int logit_staged_rows(const lif_layer_desc& D) {
+  const int rows = (D.rank + 15) / 16 - 8;
+  return rows < 0 ? 0 : (rows > kMaxStaged ? kMaxStaged : rows);
 }
 
 template <int S>
 cudaError_t launch_predict_s(lif_layer* L, const __half* x, float* logits, int32_t* active_idx,
                              int32_t* n_active, cudaStream_t st, cudaEvent_t* ev, int compact) {
   const lif_layer_desc& D = L->desc;
-  cudaError_t e = launch_k(predict_z_kernel<S>, dim3(L->z_ctas), dim3(kThreads), 0, st, L->use_pdl,
+  const int z_staged = z_staged_rows(D);
+  cudaError_t e = launch_k2(predict_z_kernel<S>, dim3(L->z_ctas), dim3(kThreads),
+                           (size_t)z_staged * kThreads * 16, st, L->use_pdl, L->single_step,
                            x, (const __half*)D.dev_pred_A, D.d_model, D.rank,
-                           z_rows_per_cta(D.d_model), L->z_partial,
-                           (int*)(L->counts + CNT_PREDICTOR_RUN));
+                           z_rows_per_cta(D.d_model), z_staged, L->z_partial);
   if (e != cudaSuccess) return e;
   if (ev) tm_record(ev[1], st);
   const int grid = (D.d_ff + kLogitTile - 1) / kLogitTile;
-  const size_t smem = (size_t)S * D.rank * sizeof(float);
-  if (smem > 32 * 1024) {
-    e = cudaFuncSetAttribute(predict_logits_kernel<S, false>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(predict_logits_kernel<S, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const int staged = logit_staged_rows(D);
+  const size_t smem = (size_t)S * D.rank * sizeof(float) + (size_t)staged * kThreads * 16;
   auto kernel = L->keep_tok ? predict_logits_kernel<S, true> : predict_logits_kernel<S, false>;
-  e = launch_k(kernel, dim3(grid), dim3(kThreads), smem, st, L->use_pdl,
+  e = launch_k2(kernel, dim3(grid), dim3(kThreads), smem, st, L->use_pdl, L->single_step,
                (const float*)L->z_partial, L->z_ctas, (const __half*)D.dev_pred_B, D.dev_pred_c,
                D.threshold_logit, D.rank, D.d_ff, logits, L->mask_words,
                (int*)(L->counts + CNT_TICKET_PREDICT), (int*)active_idx, (int*)n_active, compact,
                L->keep_tok, D.spec_keep, (const int32_t*)L->slot_of, L->new_mask_words,
-               (int*)(L->counts + CNT_PREDICTOR_RUN));
+               (int*)(L->counts + CNT_PREDICTOR_RUN), staged);
   if (ev) tm_record(ev[2], st);
   return e;
 }
 
+// Opt-ins of the kernels for S streams (once per layer).
+template <int S>
+cudaError_t predict_configure_s() {
+  const void* kernels[3] = {(const void*)predict_z_kernel<S>, (const void*)predict_logits_kernel<S, false>,
+                            (const void*)predict_logits_kernel<S, true>};
+  for (const void* k : kernels) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kMaxStaged * kThreads * 16 +
+                                             (k == kernels[0] ? 0 : S * kMaxRank * (int)sizeof(float)));
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 }  // namespace
+
+cudaError_t predict_configure(const lif_layer* L) {
+  switch (L->desc.n_streams) {
+    case 1: return predict_configure_s<1>();
+    case 2: return predict_configure_s<2>();
+    case 3: return predict_configure_s<3>();
+    case 4: return predict_configure_s<4>();
+    case 5: return predict_configure_s<5>();
+    case 6: return predict_configure_s<6>();
+    case 7: return predict_configure_s<7>();
+    case 8: return predict_configure_s<8>();
+  }
+  return cudaErrorInvalidValue;
+}
 
 cudaError_t launch_predict_one(lif_layer* L, int kernel, const __half* x, cudaStream_t st) {
   const lif_layer_desc& D = L->desc;
@@ -263,21 +335,22 @@ cudaError_t launch_predict_one(lif_layer* L, int kernel, const __half* x, cudaSt
   if (D.gate_mode == LIF_GATE_RESIDENT)
     return kernel == LIF_KERNEL_PREDICT_SCORES
                ? launch_gate_predict(L, x, nullptr, L->active_idx, L->n_tmp, st, nullptr,
-                                     L->fused_plan ? 0 : 1)
+                                     L->fused_plan ? 0 : 1, false)
                : cudaErrorInvalidValue;
   if (kernel == LIF_KERNEL_PREDICT_Z)
-    return launch_k(predict_z_kernel<1>, dim3(L->z_ctas), dim3(kThreads), 0, st, L->use_pdl, x,
+    return launch_k(predict_z_kernel<1>, dim3(L->z_ctas), dim3(kThreads),
+                    (size_t)z_staged_rows(D) * kThreads * 16, st, L->use_pdl, x,
                     (const __half*)D.dev_pred_A, D.d_model, D.rank, z_rows_per_cta(D.d_model),
-                    L->z_partial, (int*)(L->counts + CNT_PREDICTOR_RUN));
+                    z_staged_rows(D), L->z_partial);
   const int grid = (D.d_ff + kLogitTile - 1) / kLogitTile;
   return launch_k(L->keep_tok ? predict_logits_kernel<1, true> : predict_logits_kernel<1, false>,
                   dim3(grid), dim3(kThreads),
-                  (size_t)D.rank * sizeof(float), st, L->use_pdl, (const float*)L->z_partial,
+                  (size_t)D.rank * sizeof(float) + (size_t)logit_staged_rows(D) * kThreads * 16, st, L->use_pdl, (const float*)L->z_partial,
                   L->z_ctas, (const __half*)D.dev_pred_B, D.dev_pred_c, D.threshold_logit, D.rank,
                   D.d_ff, (float*)nullptr, L->mask_words, (int*)(L->counts + CNT_TICKET_PREDICT),
                   (int*)L->active_idx, (int*)L->n_tmp, L->fused_plan ? 0 : 1, L->keep_tok,
                   D.spec_keep, (const int32_t*)L->slot_of, L->new_mask_words,
-                  (int*)(L->counts + CNT_PREDICTOR_RUN));
+                  (int*)(L->counts + CNT_NO_RUN), logit_staged_rows(D));
 }
 
 cudaError_t launch_predict(lif_layer* L, const __half* x, float* logits, int32_t* active_idx,

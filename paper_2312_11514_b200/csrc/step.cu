@@ -1,0 +1,951 @@
+// One launch for everything of a single-stream decode step behind the predictor: window update,
+// row moves, fetch of the new bundles, sparse FFN over cached and new rows, and the sum.
+//
+// The CTAs of the grid (one per SM) take parts of the step, in the order in which they start:
+//   window CTA   (first)   the plan of Section 3.3: lists, counters and state, from the
+//                          predictor's entries; publishes the plan with one flag
+//   cache CTAs   (middle)  wait for the plan; row moves, then the FFN terms of the rows that were
+//                          already cached (bulk copies into shared memory, a warp per row)
+//   fetch CTAs   (last)    find the new neurons themselves in the predictor's entries, bring their
+//                          bundles over the host link through a ring of bulk copies, add their FFN
+//                          terms from shared memory, copy them to their cache rows, and in the end
+//                          add up all partial sums
+// A CTA waits only for CTAs that took their parts before it (the fetch CTAs also for one
+// another, at the very end, when nothing else is left to run), every wait is bounded, and every CTA
+// makes its arrivals on all paths, so the counters are complete whatever happened.
+//
+// Why one launch: the parts run side by side without an event or a stream of their own (five
+// launches and two event pairs less per layer-step), and the fetch does not wait for the window
+// plan: it needs the plan only for the place of a bundle that has already arrived.
+// Why few fetch CTAs: about 200 KB of host reads in flight fill the link (8 CTAs with two 16 KB
+// copies each reach the same 49.8 GB/s as 148 CTAs).  More in flight does not read faster, it only
+// queues up in front of everything else: with host loads in flight on all SMs a dependent load
+// beside them takes 1800 cycles instead of 290, and an HBM stream of the whole chip falls from 3.6
+// to 0.9 TB/s (2.3 TB/s with 16 CTAs and two copies each).
+#include "lif_internal.cuh"
+#include "mask_compact.cuh"
+#include "window.cuh"
+
+namespace lif {
+namespace {
+
+constexpr int kStepThreads = 512;
+constexpr int kStepWarps = kStepThreads / 32;
+constexpr int kStepChunks = 8192 / 8 / kStepThreads;   // 16-byte chunks per thread and vector
+constexpr int kEntriesPerThread = 2;                   // <= 1024 entries: d_ff <= 32768
+constexpr int kStepWatchPolls = 64;                    // about 30 us
+constexpr unsigned kStepSpinLimit = 1u << 20;          // polls of a counter: about a second
+constexpr int kSumDepth = 4;                           // partial sums per thread in flight
+constexpr int kFetchCtas = 16;
+constexpr unsigned short kNoSlot = 0xffff;
+
+// Counters of the layer's steps.  They only grow: the ticket tells the step as well as the part, and
+// what a CTA waits for is a counter's value after that many steps (modulo 2^32), so nothing has
+// to be put back at the end.
+struct StepSync {
+  unsigned long long ticket;
+  unsigned long long plan;       // step << 42 | flags | n_moves << 20 | rows for the cache CTAs
+  unsigned groups_done;
+  unsigned pad[11];
+  unsigned group[64];            // arrivals of each group of cache CTAs
+};
+constexpr unsigned long long kPlanReady = 1ull << 40, kPlanRefused = 1ull << 41;
+constexpr int kPlanEpochShift = 42;
+
+struct StepArgs {
+  WindowArgs w;
+  const unsigned long long* new_entries;   // predictor: {neurons to bring in, run}
+  const unsigned long long* act_entries;   // predictor: {active neurons, run}
+  int n_entries;
+  const int* predictor_run;
+  int* next_run;                  // bumped at the end (a predictor without a first stage needs it)
+  int32_t* n_act_out;
+  uint32_t* hit_rows;             // plan: row before the moves | neuron << 16, for the cache CTAs
+  const unsigned char* store;
+  unsigned char* cache;
+  const __half* x;
+  const float* gate_val;          // resident gate: gate pre-activations by neuron id
+  const __half* b_down;
+  float* p_member;                // partial sums of cache CTAs that form groups, [cta][d]
+  uint4 *p_hit, *p_new;           // tagged partial sums of cache CTAs (or groups) and fetch CTAs
+  float* y;
+  StepSync* sync;
+  int d, whole_cache, act;
+  float act_thr;
+  int n_cache_ctas, group_size, cache_stages, fetch_stages, fetch_rows_max;
+  unsigned wait_polls;
+  unsigned epoch;                 // steps before this one (filled in by the kernel)
+};
+
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ unsigned long long ld_acquire64(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+// Everything the CTA wrote before the preceding __syncthreads() is visible to whoever sees the
+// arrival (thread 0 only: one fence for the CTA instead of one per thread, which took 1-2 us).
+__device__ __forceinline__ bool arrive_last(unsigned* p, unsigned want) {
+  unsigned v;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(p) : "memory");
+  return v + 1 == want;
+}
+__device__ __forceinline__ void arrive(unsigned* p) {
+  asm volatile("red.add.release.gpu.global.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+__device__ __forceinline__ void publish(const StepArgs& a, unsigned long long v) {
+  v |= (unsigned long long)(a.epoch & ((1u << 22) - 1)) << kPlanEpochShift;
+  asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&a.sync->plan), "l"(v) : "memory");
+}
+// Exclusive prefixes of N words over the block and the block's sums; one barrier, so consecutive
+// calls need different `sums`.  Two counts up to 32768 can ride in one word (16 bits each).
+template <int N>
+__device__ __forceinline__ void step_scan(unsigned (&v)[N], unsigned (&total)[N],
+                                          unsigned (&sums)[N][kStepWarps]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned inc[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) inc[k] = v[k];
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const unsigned n = __shfl_up_sync(0xffffffffu, inc[k], o);
+      if (lane >= o) inc[k] += n;
+    }
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+    if (lane == 31) sums[k][warp] = inc[k];
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    const unsigned ws = sums[k][lane & (kStepWarps - 1)];
+    unsigned winc = ws;
+#pragma unroll
+    for (int o = 1; o < kStepWarps; o <<= 1) {
+      const unsigned n = __shfl_up_sync(0xffffffffu, winc, o);
+      if (lane >= o) winc += n;
+    }
+    total[k] = __shfl_sync(0xffffffffu, winc, kStepWarps - 1);
+    v[k] = __shfl_sync(0xffffffffu, winc - ws, warp) + inc[k] - v[k];
+  }
+}
+__device__ __forceinline__ void set_status(const StepArgs& a, int code) {
+  atomicCAS(a.w.counts + LIF_CNT_STATUS, LIF_OK, code);
+}
+// The thread's entries of the predictor run `run`.  This kernel may be resident while the score
+// kernel still runs; each entry is stored together with the number of its run, so a thread re-reads
+// its own until they carry it.  If they do not come (bounded), the kernel waits for its predecessor
+// and takes them as they are.
+__device__ __forceinline__ void read_entries(const unsigned long long* entries, int n, int run,
+                                             uint32_t (&mw)[kEntriesPerThread]) {
+  const int w0 = threadIdx.x * kEntriesPerThread;
+  auto read = [&](bool check) {
+    bool mine = true;
+#pragma unroll
+    for (int i = 0; i < kEntriesPerThread; ++i) {
+      mw[i] = 0u;
+      if (w0 + i < n) {
+        unsigned long long v;
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(entries + w0 + i)
+                     : "memory");
+        mw[i] = (uint32_t)v;
+        mine = mine && (!check || (int)(v >> 32) == run);
+      }
+    }
+    return mine;
+  };
+  int ok = 0;
+  for (int i = 0; i < kStepWatchPolls && !ok; ++i) ok = __syncthreads_and(read(true) ? 1 : 0);
+  if (!ok) {
+    pdl_wait();
+    read(false);
+  }
+}
+// Thread 0 waits for the plan; everyone gets it (0 if it did not come: an error is recorded).
+__device__ __forceinline__ unsigned long long wait_plan(const StepArgs& a,
+                                                        unsigned long long* shared) {
+  if (threadIdx.x == 0) {
+    unsigned long long v = 0;
+    bool there = false;
+    for (unsigned i = 0; i < kStepSpinLimit && !there; ++i) {
+      v = ld_acquire64(&a.sync->plan);
+      there = (v & kPlanReady) && v >> kPlanEpochShift == (a.epoch & ((1u << 22) - 1));
+    }
+    if (!there) {
+      set_status(a, LIF_ERR_TIMEOUT);
+      v = 0;
+    }
+    *shared = v;
+  }
+  __syncthreads();
+  return *shared;
+}
+
+// ---- window CTA ---------------------------------------------------------------------------------
+// The same plan as the window kernels (window.cu), held in shared memory: slot_of of every neuron
+// and row -> neuron, age of every row are read before the predictor's entries arrive (the window
+// state was last written by this layer's previous step), so between the entries and the flag there
+// are only shared-memory passes and block scans.  What the other CTAs need is written ahead of the
+// flag, the rest of the lists and the state behind it.
+size_t window_role_smem(int F, int cap) {
+  return 4 * (size_t)F + 8 * (size_t)cap + 4 * (size_t)((F + 31) / 32) + 64;
+}
+
+__device__ void window_role(const StepArgs& a, unsigned char* smem) {
+  __shared__ unsigned sums[3][1][kStepWarps];
+  __shared__ int hist[kMaxBudgetWindow + 1];
+  __shared__ int loads;
+  const WindowArgs& w = a.w;
+  const int tid = threadIdx.x, F = w.F;
+  unsigned short* slot_s = reinterpret_cast<unsigned short*>(smem);   // [F] row or kNoSlot
+  unsigned short* act_s = slot_s + F;                                 // [F] active ids, ascending
+  unsigned short* pid_s = act_s + F;                                  // [cap] row -> neuron
+  unsigned short* age_s = pid_s + w.cap;                              // [cap] steps since active
+  unsigned short* hole_s = age_s + w.cap;                             // [cap] freed rows, ascending
+  unsigned short* moved_s = hole_s + w.cap;                           // [cap] row - bound -> new row
+  uint32_t* bits = reinterpret_cast<uint32_t*>(moved_s + w.cap);      // [F / 32]
+
+  const int n = w.counts[LIF_CNT_NUM_USED];
+  const int t = w.counts[LIF_CNT_STEP];
+  const int stale_input = w.counts[LIF_CNT_STATUS] == LIF_ERR_TIMEOUT;   // see window.cu
+  const int t_end = t + w.keep - 1;
+  // (-1 becomes kNoSlot by itself)
+  for (int i0 = tid; i0 < F / 4; i0 += 8 * kStepThreads) {
+    int4 s[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (i0 + j * kStepThreads < F / 4) s[j] = reinterpret_cast<const int4*>(w.slot_of)[i0 + j * kStepThreads];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (i0 + j * kStepThreads < F / 4)
+        reinterpret_cast<ushort4*>(slot_s)[i0 + j * kStepThreads] =
+            make_ushort4((unsigned short)s[j].x, (unsigned short)s[j].y, (unsigned short)s[j].z,
+                         (unsigned short)s[j].w);
+  }
+  for (int s0 = tid; s0 < n; s0 += 4 * kStepThreads) {
+    int id[4], la[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) id[j] = s0 + j * kStepThreads < n ? w.pointers[s0 + j * kStepThreads] : 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) la[j] = s0 + j * kStepThreads < n ? w.last_active[id[j]] : 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (s0 + j * kStepThreads < n) {
+        pid_s[s0 + j * kStepThreads] = (unsigned short)id[j];
+        age_s[s0 + j * kStepThreads] = (unsigned short)min(65535, max(1, t_end - la[j]));
+      }
+  }
+  uint32_t mw[kEntriesPerThread];
+  read_entries(a.act_entries, a.n_entries, __ldcg(a.predictor_run), mw);
+  unsigned pre[1] = {0u}, tot[1];
+#pragma unroll
+  for (int i = 0; i < kEntriesPerThread; ++i) {
+    const int at = tid * kEntriesPerThread + i;
+    pre[0] += __popc(mw[i]);
+    if (at < (F + 31) / 32) bits[at] = mw[i];
+  }
+  step_scan<1>(pre, tot, sums[0]);                        // also publishes bits[] and the arrays
+  const int na = (int)tot[0];
+  {
+    int q = (int)pre[0];
+#pragma unroll 1
+    for (int i = 0; i < kEntriesPerThread; ++i)
+#pragma unroll 1
+      for (uint32_t m = mw[i]; m; m &= m - 1)
+        act_s[q++] = (unsigned short)((tid * kEntriesPerThread + i) * 32 + __ffs(m) - 1);
+  }
+  __syncthreads();
+  // each thread owns a run of consecutive rows and of consecutive active neurons
+  const int seg = (n + kStepThreads - 1) / kStepThreads;
+  const int s0 = min(n, tid * seg), s1 = min(n, s0 + seg);
+  const int qseg = (na + kStepThreads - 1) / kStepThreads;
+  const int q0 = min(na, tid * qseg), q1 = min(na, q0 + qseg);
+  auto idle_age = [&](int s) {       // 0: active now
+    const int id = pid_s[s];
+    return (bits[id >> 5] >> (id & 31)) & 1u ? 0 : (int)age_s[s];
+  };
+  int c_load = 0;
+  for (int q = q0; q < q1; ++q) c_load += slot_s[act_s[q]] == kNoSlot;
+  int k_eff = w.k;
+  if (w.budget > 0) {                // memory budget: shrink the window for this step if needed
+    if (tid <= kMaxBudgetWindow) hist[tid] = 0;
+    if (tid == 0) loads = 0;
+    __syncthreads();
+    for (int s = s0; s < s1; ++s) {
+      const int age = idle_age(s);
+      if (age > 0) atomicAdd(&hist[min(w.k, age)], 1);
+    }
+    if (c_load) atomicAdd(&loads, c_load);
+    __syncthreads();
+    k_eff = widest_window_that_fits(hist, w.k, n, loads, min(w.cap, w.budget));
+  }
+  const int limit = w.budget > 0 ? min(w.cap, w.budget) : w.cap;
+  int c_ev = 0;
+  for (int s = s0; s < s1; ++s) c_ev += idle_age(s) >= k_eff;
+  pre[0] = (unsigned)c_load | ((unsigned)c_ev << 16);
+  step_scan<1>(pre, tot, sums[1]);
+  const int n_load = (int)(tot[0] & 0xffff), n_evict = (int)(tot[0] >> 16);
+  const int n_kept = n - n_evict;
+  const int p_load0 = (int)(pre[0] & 0xffff), p_ev0 = (int)(pre[0] >> 16);
+  if (stale_input || n_kept + n_load > limit) {           // refuse before anything is changed
+    if (a.whole_cache)                                     // the FFN still runs over the rows in use
+      for (int s = tid; s < n; s += kStepThreads)
+        a.hit_rows[s] = (uint32_t)s | ((uint32_t)pid_s[s] << 16);
+    __syncthreads();
+    if (tid == 0) {
+      if (w.counts[LIF_CNT_STATUS] == LIF_OK) w.counts[LIF_CNT_STATUS] = LIF_ERR_CAPACITY;
+      w.counts[LIF_CNT_N_ACTIVE] = 0;
+      w.counts[LIF_CNT_N_EVICT] = 0;
+      w.counts[LIF_CNT_N_MOVES] = 0;
+      w.counts[LIF_CNT_N_LOAD] = 0;
+      w.counts[LIF_CNT_N_HITS] = 0;
+      w.counts[LIF_CNT_NUM_USED_BEFORE] = n;
+      w.counts[LIF_CNT_NUM_KEPT] = n;
+      publish(a, kPlanReady | kPlanRefused | (unsigned)(a.whole_cache ? n : 0));
+    }
+    pdl_wait();
+    return;
+  }
+  // freed rows taken by new neurons directly, and where the rows that must move begin
+  const int reuse = w.append_first ? min(n_evict, n_load) : 0;
+  const int bound = n - (n_evict - reuse);
+  int n_moves = 0, p_surv0 = 0;
+  if (bound < n) {
+    int c_surv = 0;
+    for (int s = max(s0, bound); s < s1; ++s) c_surv += idle_age(s) < k_eff;
+    pre[0] = (unsigned)c_surv;
+    step_scan<1>(pre, tot, sums[2]);
+    n_moves = (int)tot[0];
+    p_surv0 = (int)pre[0];
+  }
+  {
+    int p_ev = p_ev0;
+    for (int s = s0; s < s1; ++s) {
+      if (idle_age(s) >= k_eff) hole_s[p_ev++] = (unsigned short)s;
+      else if (a.whole_cache) a.hit_rows[s - p_ev] = (uint32_t)s | ((uint32_t)pid_s[s] << 16);
+    }
+  }
+  __syncthreads();
+  {
+    int p_surv = p_surv0;
+    for (int s = max(s0, bound); s < s1; ++s)
+      if (idle_age(s) < k_eff) {                           // surviving tail row: last one first
+        const int jm = n_moves - 1 - p_surv++;
+        const int dst = hole_s[reuse + jm];
+        w.move_src[jm] = s;
+        w.move_dst[jm] = dst;
+        moved_s[s - bound] = (unsigned short)dst;
+      }
+  }
+  auto new_row = [&](int p) { return p < n_load - reuse ? bound + p : (int)hole_s[n_load - 1 - p]; };
+  {
+    int p_load = p_load0;
+    for (int q = q0; q < q1; ++q) {
+      const int id = act_s[q], s = slot_s[id];
+      if (s == kNoSlot) {
+        w.load_slots[p_load] = new_row(p_load);
+        ++p_load;
+      } else if (!a.whole_cache) {
+        a.hit_rows[q - p_load] = (uint32_t)s | ((uint32_t)id << 16);
+      }
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const unsigned n_rows = a.whole_cache ? n_kept : na - n_load;
+    publish(a, kPlanReady | ((unsigned long long)n_moves << 20) | n_rows);
+  }
+
+  // ---- behind the flag: the public lists and the state ------------------------------------------
+  pdl_wait();                       // (speculative stamps come from the predictor's keep_tok)
+  {
+    int p_ev = p_ev0, p_surv = p_surv0;
+    for (int s = s0; s < s1; ++s) {
+      const int id = pid_s[s];
+      if (idle_age(s) >= k_eff) {
+        w.evict_ids[p_ev++] = id;
+        w.slot_of[id] = -1;
+      } else if (s >= bound) {
+        const int dst = hole_s[reuse + n_moves - 1 - p_surv++];
+        w.pointers[dst] = id;
+        w.slot_of[id] = dst;
+        w.bias[dst] = w.bias_up[id];
+      }
+      if (s >= n_kept + n_load) w.pointers[s] = -1;      // tail beyond the rows in use
+    }
+    int p_load = p_load0;
+    for (int q = q0; q < q1; ++q) {
+      const int id = act_s[q];
+      int s = slot_s[id];
+      w.last_active[id] = active_stamp(w, id, t, t_end);
+      if (s == kNoSlot) {
+        s = new_row(p_load);
+        w.load_ids[p_load++] = id;
+        w.slot_of[id] = s;
+        w.pointers[s] = id;
+        w.bias[s] = w.bias_up[id];
+      } else {
+        if (s >= bound) s = moved_s[s - bound];
+        w.hit_slots[q - p_load] = s;
+      }
+      w.active_slots[q] = s;
+      w.active_idx[q] = id;
+    }
+  }
+  if (tid == 0) {
+    *a.n_act_out = na;
+    w.counts[LIF_CNT_N_ACTIVE] = na;
+    w.counts[LIF_CNT_N_EVICT] = n_evict;
+    w.counts[LIF_CNT_N_MOVES] = n_moves;
+    w.counts[LIF_CNT_N_LOAD] = n_load;
+    w.counts[LIF_CNT_N_HITS] = na - n_load;
+    w.counts[LIF_CNT_NUM_USED_BEFORE] = n;
+    w.counts[LIF_CNT_NUM_KEPT] = n_kept;
+    w.counts[LIF_CNT_NUM_USED] = n_kept + n_load;
+    w.counts[LIF_CNT_STEP] = t + w.keep;
+    w.counts[LIF_CNT_K_EFF] = k_eff;
+    unsigned long long* totals = reinterpret_cast<unsigned long long*>(w.counts + CNT_TOTALS);
+    totals[0] += (unsigned long long)n_load * w.bundle_bytes;
+    totals[1] += (unsigned long long)n_moves;
+    totals[2] += (unsigned long long)na;
+    totals[3] += (unsigned long long)(n_kept + n_load);
+  }
+}
+
+// ---- shared by the cache and fetch CTAs ---------------------------------------------------------
+// acc += h * v for the thread's chunks of the down column
+__device__ __forceinline__ void axpy_row(float (&acc)[kStepChunks][8], const uint4* down, float h,
+                                         int nvec) {
+#pragma unroll
+  for (int k = 0; k < kStepChunks; ++k) {
+    const int c = threadIdx.x + k * kStepThreads;
+    if (c < nvec) {
+      float f[8];
+      unpack8(down[c], f);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) acc[k][e] = fmaf(h, f[e], acc[k][e]);
+    }
+  }
+}
+// A partial sum for the end of the step: every pair of values is stored as {v, tag, v, tag}, two
+// 8-byte words that are each written whole, with a tag of this step (step number + 1).  The reader
+// polls the words themselves, so there is no fence, no counter and no second round trip between
+// the last row and the sum (measured: 1.3 us from the last row to y instead of 3.5).  Pair e of
+// 8-column chunk c is word e * (d / 8) + c, so that a warp's stores are contiguous.
+__device__ __forceinline__ void store_tagged(uint4* dst, float v0, float v1, unsigned tag) {
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(dst),
+               "l"((unsigned long long)__float_as_uint(v0) | ((unsigned long long)tag << 32)),
+               "l"((unsigned long long)__float_as_uint(v1) | ((unsigned long long)tag << 32))
+               : "memory");
+}
+__device__ __forceinline__ ulonglong2 load_tagged(const uint4* src) {
+  ulonglong2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(src) : "memory");
+  return v;
+}
+__device__ __forceinline__ bool has_tag(const ulonglong2& v, unsigned tag) {
+  return (unsigned)(v.x >> 32) == tag && (unsigned)(v.y >> 32) == tag;
+}
+__device__ __forceinline__ void store_tagged_partial(const float (&acc)[kStepChunks][8], uint4* dst,
+                                                     int nvec, unsigned tag) {
+#pragma unroll
+  for (int k = 0; k < kStepChunks; ++k) {
+    const int c = threadIdx.x + k * kStepThreads;
+    if (c < nvec) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) store_tagged(dst + e * nvec + c, acc[k][2 * e], acc[k][2 * e + 1], tag);
+    }
+  }
+}
+__device__ __forceinline__ void store_partial(const float (&acc)[kStepChunks][8], float* dst, int nvec) {
+  float4* out = reinterpret_cast<float4*>(dst);
+#pragma unroll
+  for (int k = 0; k < kStepChunks; ++k) {
+    const int c = threadIdx.x + k * kStepThreads;
+    if (c < nvec) {
+      __stcg(out + 2 * c, make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]));
+      __stcg(out + 2 * c + 1, make_float4(acc[k][4], acc[k][5], acc[k][6], acc[k][7]));
+    }
+  }
+}
+template <int kGate>
+__device__ __forceinline__ float row_weight(const StepArgs& a, float b, float first, float second) {
+  if (kGate == LIF_GATE_BUNDLED) return apply_activation(first + b, a.act, a.act_thr) * second;
+  if (kGate == LIF_GATE_RESIDENT) return apply_activation(b, a.act, a.act_thr) * first;
+  return apply_activation(first + b, a.act, a.act_thr);
+}
+template <int kGate>
+__device__ __forceinline__ float row_scalar(const StepArgs& a, int id) {
+  return kGate == LIF_GATE_RESIDENT ? a.gate_val[id] : __half2float(a.w.bias_up[id]);
+}
+
+// ---- cache CTAs: row moves and the FFN of the rows that were already cached -------------------------
+// Rows are read where they were before the moves: a moved row's source is not overwritten before
+// all cache CTAs are done (append_first: not at all), so moves and FFN need no order.
+template <int kGate>
+__device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
+  constexpr int kVec = kGate == LIF_GATE_BUNDLED ? 3 : 2;
+  __shared__ __align__(8) uint64_t bars[16];
+  __shared__ float h_s[16], b_s[16];
+  __shared__ unsigned long long plan_s;
+  __shared__ int last_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int d = a.d, nvec = d >> 3, stages = a.cache_stages, nc = a.n_cache_ctas;
+  const unsigned row_bytes = 2u * kVec * d;
+  uint4* xs = reinterpret_cast<uint4*>(smem);              // [d]
+  unsigned char* rows = smem + (((size_t)d * 2 + 127) & ~(size_t)127);
+  if (tid == 0) {
+    for (int i = 0; i < stages; ++i) mbar_init(bars + i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  pdl_wait();
+  for (int i = tid; i < nvec; i += kStepThreads) xs[i] = reinterpret_cast<const uint4*>(a.x)[i];
+  const unsigned long long plan = wait_plan(a, &plan_s);
+  const int n = (int)(plan & 0xfffff), n_moves = (int)((plan >> 20) & 0xfffff);
+  const int cnt = c < n ? (n - c + nc - 1) / nc : 0;
+  float acc[kStepChunks][8];
+#pragma unroll
+  for (int k = 0; k < kStepChunks; ++k)
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[k][e] = 0.f;
+
+  unsigned parity = 0;
+  for (int r0 = 0; r0 < cnt || r0 == 0; r0 += stages) {
+    const int rc = min(stages, cnt - r0);
+    if (tid < rc) {
+      const uint32_t e = __ldcg(a.hit_rows + c + (r0 + tid) * nc);
+      mbar_expect_tx(bars + tid, row_bytes);
+      bulk_g2s(rows + (size_t)tid * row_bytes, a.cache + (size_t)(e & 0xffff) * row_bytes, row_bytes,
+               bars + tid);
+      b_s[tid] = row_scalar<kGate>(a, (int)(e >> 16));
+    }
+    if (r0 == 0) {                                         // the moves, while the first rows travel
+      const int row_vec = kVec * nvec;
+      for (int j = c; j < n_moves; j += nc) {
+        const uint4* src = reinterpret_cast<const uint4*>(a.cache) + (size_t)__ldcg(a.w.move_src + j) * row_vec;
+        uint4* dst = reinterpret_cast<uint4*>(a.cache) + (size_t)__ldcg(a.w.move_dst + j) * row_vec;
+        uint4 v[4];
+        for (int v0 = tid; v0 < row_vec; v0 += 4 * kStepThreads) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (v0 + u * kStepThreads < row_vec) v[u] = ld_stream16(src + v0 + u * kStepThreads);
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (v0 + u * kStepThreads < row_vec) dst[v0 + u * kStepThreads] = v[u];
+        }
+      }
+    }
+    __syncthreads();                                       // x and the rows' scalars
+    if (rc <= 0) break;
+    for (int i = warp; i < rc; i += kStepWarps) {          // a warp per row
+      bool landed = mbar_wait(bars + i, parity, a.wait_polls);
+      if (!landed) {                                       // flagged; its terms are left out
+        if (lane == 0) set_status(a, LIF_ERR_TIMEOUT);
+        mbar_wait(bars + i, parity);
+      }
+      const uint4* row = reinterpret_cast<const uint4*>(rows + (size_t)i * row_bytes);
+      float p = 0.f, p2 = 0.f;
+#pragma unroll 4
+      for (int v = lane; v < nvec; v += 32) {
+        float rf[8], xf[8];
+        unpack8(row[v], rf);
+        unpack8(xs[v], xf);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) p = fmaf(rf[e], xf[e], p);
+        if (kGate == LIF_GATE_BUNDLED) {
+          unpack8(row[nvec + v], rf);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) p2 = fmaf(rf[e], xf[e], p2);
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        p += __shfl_xor_sync(0xffffffffu, p, o);
+        if (kGate == LIF_GATE_BUNDLED) p2 += __shfl_xor_sync(0xffffffffu, p2, o);
+      }
+      if (lane == 0) h_s[i] = landed ? row_weight<kGate>(a, b_s[i], p, p2) : 0.f;
+    }
+    __syncthreads();
+    for (int i = 0; i < rc; ++i) {
+      const float h = h_s[i];
+      if (h != 0.f)
+        axpy_row(acc, reinterpret_cast<const uint4*>(rows + (size_t)i * row_bytes) + (kVec - 1) * nvec,
+                 h, nvec);
+    }
+    parity ^= 1u;
+    if (r0 + stages < cnt) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncthreads();                                     // rows are free for the next copies
+    }
+  }
+
+  // The CTA's partial; with many cache CTAs the last of each group of them adds the group's
+  // partials (in CTA order), so that few are left for the end of the step.
+  const int gs = a.group_size, g = c / gs;
+  if (gs == 1) {
+    if (cnt > 0) store_tagged_partial(acc, a.p_hit + (size_t)c * (d / 2), nvec, a.epoch + 1);
+    __syncthreads();
+  } else {
+    if (cnt > 0) store_partial(acc, a.p_member + (size_t)c * d, nvec);
+    __syncthreads();
+    const int members = min(gs, nc - g * gs);
+    if (tid == 0) last_s = arrive_last(&a.sync->group[g], (a.epoch + 1) * (unsigned)members);
+    __syncthreads();
+    if (!last_s) return;
+    const int have = min(members, max(0, n - g * gs));     // members with rows wrote a partial
+    if (have > 0)
+      for (int i = tid; i < d / 4; i += kStepThreads) {
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f), v[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+          if (m < have) v[m] = __ldcg(reinterpret_cast<const float4*>(a.p_member + (size_t)(g * gs + m) * d) + i);
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+          if (m < have) { s.x += v[m].x; s.y += v[m].y; s.z += v[m].z; s.w += v[m].w; }
+        uint4* dst = a.p_hit + (size_t)g * (d / 2) + (i & 1) * 2 * nvec + (i >> 1);
+        store_tagged(dst, s.x, s.y, a.epoch + 1);
+        store_tagged(dst + nvec, s.z, s.w, a.epoch + 1);
+      }
+  }
+  // (only the paper's cache order waits for this: the rows have been read and moved)
+  if (tid == 0) arrive(&a.sync->groups_done);
+}
+
+// ---- fetch CTAs: new bundles over the host link, their FFN terms, and the sum -----------------------
+// Fetch CTA f brings in entries f, f + kFetchCtas, ... of the load list, which is exactly the set
+// bits of the predictor's entries in ascending order; only the cache row comes from the plan.
+template <int kGate>
+__device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
+  constexpr int kVec = kGate == LIF_GATE_BUNDLED ? 3 : 2;
+  __shared__ __align__(8) uint64_t bars[16];
+  __shared__ unsigned sums[1][kStepWarps];
+  __shared__ float part[2][kStepWarps];
+  __shared__ unsigned long long plan_s;
+  __shared__ float2 red[kStepThreads];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int d = a.d, nvec = d >> 3, stages = a.fetch_stages;
+  constexpr int nf = kFetchCtas;
+  const unsigned row_bytes = 2u * kVec * d;
+  unsigned char* ring = smem;
+  unsigned short* ids = reinterpret_cast<unsigned short*>(ring + (size_t)stages * row_bytes);
+  unsigned short* dst_rows = ids + a.fetch_rows_max;
+  if (tid == 0) {
+    for (int i = 0; i < stages; ++i) mbar_init(bars + i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  uint32_t mw[kEntriesPerThread];
+  const int run = __ldcg(a.predictor_run);
+  read_entries(a.new_entries, a.n_entries, run, mw);
+  unsigned pre[1] = {0u}, tot[1];
+#pragma unroll
+  for (int i = 0; i < kEntriesPerThread; ++i) pre[0] += __popc(mw[i]);
+  step_scan<1>(pre, tot, sums);
+  auto issue = [&](int id, int st) {
+    mbar_expect_tx(bars + st, row_bytes);
+    bulk_g2s(ring + (size_t)st * row_bytes, a.store + (size_t)id * row_bytes, row_bytes, bars + st);
+  };
+  const int n_new = (int)tot[0];
+  int q = (int)pre[0];
+#pragma unroll
+  for (int i = 0; i < kEntriesPerThread; ++i)              // of the thread's bits, those of rank f mod nf
+    for (uint32_t m = mw[i]; m; m &= m - 1, ++q)
+      if (q % nf == f) {
+        const int id = (tid * kEntriesPerThread + i) * 32 + __ffs(m) - 1;
+        ids[q / nf] = (unsigned short)id;
+        if (q / nf < stages) issue(id, q / nf);            // the first ones by whoever finds them
+      }
+  int cnt = f < n_new ? (n_new - f + nf - 1) / nf : 0;
+  const int issued = min(stages, cnt);
+  pdl_wait();
+  uint4 xq[kStepChunks];
+#pragma unroll
+  for (int k = 0; k < kStepChunks; ++k) {
+    const int v = tid + k * kStepThreads;
+    xq[k] = v < nvec ? reinterpret_cast<const uint4*>(a.x)[v] : make_uint4(0, 0, 0, 0);
+  }
+  float acc[kStepChunks][8];
+#pragma unroll
+  for (int k = 0; k < kStepChunks; ++k)
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[k][e] = 0.f;
+
+  const unsigned long long plan = wait_plan(a, &plan_s);
+  const bool go = (plan & kPlanReady) && !(plan & kPlanRefused);
+  const int n_hit = (int)(plan & 0xfffff);
+  auto spin = [&](const unsigned* counter, unsigned per_step) {  // thread 0
+    const unsigned want = (a.epoch + 1) * per_step;
+    unsigned i = 0;
+    while ((int)(ld_acquire(counter) - want) < 0 && i < kStepSpinLimit) ++i;
+    if (i == kStepSpinLimit) set_status(a, LIF_ERR_TIMEOUT);
+  };
+  const int n_groups = (a.n_cache_ctas + a.group_size - 1) / a.group_size;
+  if (!go) {
+    // the update of this step was refused: nothing is brought in; let the copies land
+    if (tid == 0)
+      for (int i = 0; i < issued; ++i) mbar_wait(bars + i, 0);
+    cnt = 0;
+  } else {
+    for (int i = tid; i < cnt; i += kStepThreads)
+      dst_rows[i] = (unsigned short)__ldcg(a.w.load_slots + f + i * nf);
+    // in the paper's order the new rows' places may be rows the cache CTAs still read
+    if (!a.w.append_first && tid == 0) spin(&a.sync->groups_done, n_groups);
+  }
+  __syncthreads();
+  // The end of the step: every fetch CTA adds up a slice of the columns, in pairs, `width` of them
+  // side by side; the other threads share the partials.  Order: partials of the cached rows (read
+  // while the last row is on its way), then those of the fetch CTAs.
+  const unsigned tag = a.epoch + 1;
+  const int pairs = d >> 1, per = (pairs + nf - 1) / nf;
+  const int c0 = f * per, c1 = min(pairs, c0 + per);
+  int width = 32;
+  while (width < per && width < kStepThreads / 2) width *= 2;   // per <= 256
+  const int slices = kStepThreads / width;
+  const int slice = tid / width, col = c0 + tid % width;
+  const int have_hit = (min(n_hit, a.n_cache_ctas) + a.group_size - 1) / a.group_size;
+  const int have_new = go ? min(nf, n_new) : 0;
+  float2 sum = make_float2(0.f, 0.f);
+  int lost_sum = 0;
+  // adds this thread's partials from number t0 on; stops where they are not there after `limit` polls
+  auto add_partials = [&](const uint4* partials, int have, int t0, unsigned limit) {
+    if (col >= c1) return have;
+    for (; t0 < have; t0 += slices * kSumDepth) {
+      ulonglong2 v[kSumDepth];
+#pragma unroll
+      for (int k = 0; k < kSumDepth; ++k)                  // (past the end: the last one again)
+        v[k] = load_tagged(partials + (size_t)min(t0 + k * slices, have - 1) * pairs + col);
+      bool there = false;
+      for (unsigned polls = 0; polls < limit; ++polls) {
+        there = true;
+#pragma unroll
+        for (int k = 0; k < kSumDepth; ++k) there = there && has_tag(v[k], tag);
+        if (there || polls + 1 == limit) break;
+#pragma unroll
+        for (int k = 0; k < kSumDepth; ++k)                // again, those that were not there
+          if (!has_tag(v[k], tag))
+            v[k] = load_tagged(partials + (size_t)min(t0 + k * slices, have - 1) * pairs + col);
+      }
+      if (!there) return t0;
+#pragma unroll
+      for (int k = 0; k < kSumDepth; ++k)
+        if (t0 + k * slices < have) {
+          sum.x += __uint_as_float((unsigned)v[k].x);
+          sum.y += __uint_as_float((unsigned)v[k].y);
+        }
+    }
+    return have;
+  };
+  int t_hit = slice;
+
+  unsigned parity = 0;
+  for (int i = 0, st = 0; i < cnt; ++i) {
+    if (i == cnt - 1) t_hit = add_partials(a.p_hit, have_hit, t_hit, 1);
+    const uint4* row = reinterpret_cast<const uint4*>(ring + (size_t)st * row_bytes);
+    const bool landed = mbar_wait(bars + st, parity, a.wait_polls);
+    if (!landed) {                                         // flagged; its term is left out
+      if (tid == 0) set_status(a, LIF_ERR_TIMEOUT);
+      mbar_wait(bars + st, parity);
+    }
+    if (tid == 0) {
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                       a.cache + (size_t)dst_rows[i] * row_bytes), "r"(smem_u32(row)), "r"(row_bytes)
+                   : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    }
+    const float b = row_scalar<kGate>(a, ids[i]);
+    float p = 0.f, p2 = 0.f;
+#pragma unroll
+    for (int k = 0; k < kStepChunks; ++k) {
+      const int v = tid + k * kStepThreads;
+      if (v < nvec) {
+        float rf[8], xf[8];
+        unpack8(row[v], rf);
+        unpack8(xq[k], xf);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) p = fmaf(rf[e], xf[e], p);
+        if (kGate == LIF_GATE_BUNDLED) {
+          unpack8(row[nvec + v], rf);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) p2 = fmaf(rf[e], xf[e], p2);
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      p += __shfl_xor_sync(0xffffffffu, p, o);
+      if (kGate == LIF_GATE_BUNDLED) p2 += __shfl_xor_sync(0xffffffffu, p2, o);
+    }
+    if (lane == 0) {
+      part[0][warp] = p;
+      part[1][warp] = p2;
+    }
+    const int lost = __syncthreads_or(!landed);
+    float v1 = 0.f, v2 = 0.f;
+#pragma unroll
+    for (int w = 0; w < kStepWarps; ++w) {
+      v1 += part[0][w];
+      if (kGate == LIF_GATE_BUNDLED) v2 += part[1][w];
+    }
+    const float h = lost ? 0.f : row_weight<kGate>(a, b, v1, v2);
+    if (h != 0.f) axpy_row(acc, row + (kVec - 1) * nvec, h, nvec);
+    __syncthreads();                                       // the stage and part[] are free
+    if (tid == 0 && i + stages < cnt) {
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      issue(ids[i + stages], st);
+    }
+    if (++st == stages) {
+      st = 0;
+      parity ^= 1u;
+    }
+  }
+  if (cnt > 0) store_tagged_partial(acc, a.p_new + (size_t)f * (d / 2), nvec, tag);
+  if (add_partials(a.p_hit, have_hit, t_hit, kStepSpinLimit) < have_hit) lost_sum = 1;
+
+  if (add_partials(a.p_new, have_new, slice, kStepSpinLimit) < have_new) lost_sum = 1;
+  red[tid] = sum;
+  __syncthreads();
+  if (tid < width && col < c1) {
+    const int at = 4 * (col % nvec) + col / nvec;          // columns 2 * at, 2 * at + 1
+    float2 y = make_float2(0.f, 0.f);
+    if (a.b_down) y = __half22float2(*reinterpret_cast<const __half2*>(a.b_down + 2 * at));
+    for (int k = 0; k < slices; ++k) {
+      y.x += red[k * width + tid].x;
+      y.y += red[k * width + tid].y;
+    }
+    reinterpret_cast<float2*>(a.y)[at] = y;
+  }
+  if (lost_sum) set_status(a, LIF_ERR_TIMEOUT);
+  if (tid == 0) {
+    if (f == 0) advance_run(a.next_run, run);
+    // (shared memory must outlive the reads of the last rows' copies to the cache)
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+  }
+}
+
+template <int kGate>
+__global__ void __launch_bounds__(kStepThreads, 2) step_kernel(StepArgs a) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ unsigned part_s, epoch_s;
+  pdl_trigger();       // whatever follows waits for this kernel's end before it reads its results
+  if (threadIdx.x == 0) {
+    const unsigned long long ticket = atomicAdd(&a.sync->ticket, 1ull);
+    epoch_s = (unsigned)(ticket / gridDim.x);
+    part_s = (unsigned)(ticket % gridDim.x);
+  }
+  __syncthreads();
+  const int part = (int)part_s;
+  a.epoch = epoch_s;
+  if (part == 0) window_role(a, smem);
+  else if (part <= a.n_cache_ctas) cache_role<kGate>(a, part - 1, smem);
+  else fetch_role<kGate>(a, part - 1 - a.n_cache_ctas, smem);
+}
+
+using StepKernel = void (*)(StepArgs);
+StepKernel step_kernel_for(int gate_mode) {
+  if (gate_mode == LIF_GATE_BUNDLED) return step_kernel<LIF_GATE_BUNDLED>;
+  if (gate_mode == LIF_GATE_RESIDENT) return step_kernel<LIF_GATE_RESIDENT>;
+  return step_kernel<LIF_GATE_NONE>;
+}
+constexpr int kGroupMax = 8, kGroupsMax = 64;
+constexpr size_t kCacheRing = 128 * 1024, kFetchRing = 32 * 1024;
+
+}  // namespace
+
+size_t step_sync_bytes() { return sizeof(StepSync); }
+size_t step_tagged_bytes(const lif_layer_desc& D) {
+  return D.n_streams == 1 ? (size_t)(kGroupsMax + kFetchCtas) * D.d_model * 8 : 0;
+}
+
+// Shape of the launch, and whether the single launch applies: one input stream, ids and rows that
+// fit 16 bits and the predictor's entries two per thread (d_ff <= 32768), the window CTA's arrays in
+// shared memory.
+cudaError_t step_configure(lif_layer* L) {
+  const lif_layer_desc& D = L->desc;
+  L->step_ok = 0;
+  const int n_entries = new_mask_entries(D);
+  if (D.n_streams != 1 || n_entries > kEntriesPerThread * kStepThreads || D.d_ff > 32768 ||
+      new_mask_entry_bits(D) != 32 ||
+      D.window_k > 32767 || L->n_sm < 2 * kFetchCtas)
+    return cudaSuccess;
+  int dev = 0, max_smem = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  const size_t row = 2 * (size_t)row_elems(D);
+  const int nf = kFetchCtas;
+  auto stages = [&](size_t ring, int least) {
+    const int s = (int)(ring / row);
+    return s < least ? least : (s > 16 ? 16 : s);
+  };
+  // about eight rows of the cache per cache CTA: a third of them is active in a step
+  int nc = (D.capacity + 7) / 8;
+  if (nc < 8) nc = 8;
+  if (nc > L->n_sm - 1 - nf) nc = L->n_sm - 1 - nf;
+  L->step_cache_ctas = nc;
+  L->step_group = nc > kGroupsMax ? kGroupMax : 1;
+  L->step_cache_stages = stages(kCacheRing, 1);
+  // in the paper's cache order the bundles wait in the ring until the cache CTAs have read the rows
+  // they replace: twice the ring keeps the link busy meanwhile
+  L->step_fetch_stages = stages(D.append_first ? kFetchRing : 2 * kFetchRing, 2);
+  const size_t rows_max = ((size_t)D.d_ff + nf - 1) / nf;
+  const size_t need_w = window_role_smem(D.d_ff, D.capacity);
+  const size_t need_c = ((2 * (size_t)D.d_model + 127) & ~(size_t)127) + L->step_cache_stages * row;
+  const size_t need_f = L->step_fetch_stages * row + 4 * rows_max;
+  size_t smem = need_w > need_c ? need_w : need_c;
+  if (need_f > smem) smem = need_f;
+  cudaFuncAttributes at;
+  e = cudaFuncGetAttributes(&at, step_kernel_for(D.gate_mode));
+  if (e != cudaSuccess) return e;
+  if (smem + at.sharedSizeBytes > (size_t)max_smem) return cudaSuccess;
+  L->step_smem = smem;
+  e = cudaFuncSetAttribute(step_kernel_for(D.gate_mode), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           max_smem - (int)at.sharedSizeBytes);
+  if (e != cudaSuccess) return e;
+  L->step_ok = 1;
+  return cudaSuccess;
+}
+
+cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st) {
+  const lif_layer_desc& D = L->desc;
+  StepArgs a;
+  a.w = window_args(L, L->active_idx, L->n_tmp);
+  a.new_entries = L->new_mask_words;
+  a.n_entries = new_mask_entries(D);
+  a.act_entries = L->new_mask_words + a.n_entries;
+  a.predictor_run = L->counts + CNT_PREDICTOR_RUN;
+  a.next_run = (int*)(L->counts + CNT_PREDICTOR_RUN);
+  a.n_act_out = L->n_tmp;
+  a.hit_rows = L->hit_rows;
+  a.store = (const unsigned char*)L->dev_bundles;
+  a.cache = (unsigned char*)D.dev_cache;
+  a.x = x;
+  a.gate_val = L->gate_val;
+  a.b_down = (const __half*)D.dev_bias_down;
+  a.p_member = L->y_partial;
+  a.p_hit = (uint4*)L->step_tagged;
+  a.p_new = a.p_hit + (size_t)kGroupsMax * (D.d_model / 2);
+  a.y = y;
+  a.sync = (StepSync*)L->step_sync;
+  a.d = D.d_model;
+  a.whole_cache = D.ffn_mode == 1;
+  a.act = D.activation;
+  a.act_thr = D.activation_threshold;
+  a.n_cache_ctas = L->step_cache_ctas;
+  a.group_size = L->step_group;
+  a.cache_stages = L->step_cache_stages;
+  a.fetch_stages = L->step_fetch_stages;
+  a.fetch_rows_max = (D.d_ff + kFetchCtas - 1) / kFetchCtas;
+  a.wait_polls = L->wait_polls;
+  return launch_k(step_kernel_for(D.gate_mode), dim3(1 + a.n_cache_ctas + kFetchCtas),
+                  dim3(kStepThreads), L->step_smem, st, L->use_pdl, a);
+}
+
+}  // namespace lif

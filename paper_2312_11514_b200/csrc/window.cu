@@ -21,95 +21,15 @@
 // only the e - r freed rows left over are closed by moving old rows (those at or beyond
 // n - (e - r)).  Row moves and bundle writes then never touch the same row.
 #include "lif_internal.cuh"
+#include "window.cuh"
 
 namespace lif {
 namespace {
 
-// Three counters ride in one 64-bit scan, 21 bits each (d_ff < 2^21 is checked at creation).
-typedef unsigned long long u64;
-constexpr int kField = 21;
-constexpr u64 kFieldMask = (1ull << kField) - 1;
-__device__ __forceinline__ u64 pack3(int a, int b, int c) {
-  return (u64)a | ((u64)b << kField) | ((u64)c << (2 * kField));
-}
-__device__ __forceinline__ int field(u64 v, int i) { return (int)((v >> (i * kField)) & kFieldMask); }
-
-struct Scan {
-  u64 warp_sums[kWindowThreads / 32];
-};
-
-// exclusive prefix of v over the block (thread order); *total = block sum
-__device__ __forceinline__ u64 block_scan(u64 v, u64* total, Scan& sc) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  u64 inc = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    u64 n = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += n;
-  }
-  if (lane == 31) sc.warp_sums[warp] = inc;
-  __syncthreads();
-  u64 ws = sc.warp_sums[lane];   // 32 warps
-  u64 winc = ws;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    u64 n = __shfl_up_sync(0xffffffffu, winc, o);
-    if (lane >= o) winc += n;
-  }
-  const u64 base = __shfl_sync(0xffffffffu, winc - ws, warp);
-  *total = __shfl_sync(0xffffffffu, winc, 31);
-  __syncthreads();
-  return base + inc - v;
-}
-
-struct WindowArgs {
-  const int32_t* act;
-  const int32_t* n_act;
-  int32_t* counts;
-  int32_t *pointers, *slot_of, *last_active;
-  __half* bias;
-  const __half* bias_up;
-  int32_t *active_idx, *evict_ids, *evict_slots, *move_src, *move_dst, *load_ids, *load_slots,
-      *active_slots, *hit_slots;
-  int F, cap, k;
-  int budget;             // 0 = off; else rows the cache may hold (Appendix C memory budget)
-  // Speculative decoding (Section 4): the step holds consecutive tokens; the kept window ends
-  // with token `keep` of the step (keep = 1, keep_tok = nullptr: ordinary single-token update).
-  const int8_t* keep_tok; // [F] last kept token per neuron, -1 if active only in later tokens
-  int keep;
-  int append_first;       // stack the new neurons before deleting (see the header of this file)
-  int release_early;      // release the dependent kernel before this kernel's own wait
-  unsigned long long bundle_bytes;
-};
-
-// Memory-budgeted window (Appendix C, Persimmon 8B / Phi-2): hist[a] = cached rows that are not
-// active now and were last active a steps ago (a = 1 .. k, older ones in bin k).  Returns the
-// widest window k' <= k for which the rows kept plus the rows to load fit `limit`, at least 1.
-// Stamp of an active neuron: the time of the last kept token in which it is active (its old
-// stamp if it is active only beyond the kept token), but never below the oldest stamp still
-// inside the window that ends at t_end: this step does not delete it, the next one may.
-__device__ __forceinline__ int active_stamp(const WindowArgs& a, int id, int t, int t_end) {
-  if (!a.keep_tok) return t;
-  const int j = a.keep_tok[id];
-  return max(j >= 0 ? t + j : a.last_active[id], t_end - a.k + 1);
-}
-
-constexpr int kMaxBudgetWindow = 32;
 constexpr int kSegRegs = 12;    // general path: cached rows per thread kept in registers
 constexpr int kActRegs = 8;     // and active-list entries per thread
-__device__ __forceinline__ int widest_window_that_fits(const int* hist, int k, int n, int n_load,
-                                                       int limit) {
-  int evicted = 0;          // rows deleted under window kk = sum of hist[a], a >= kk
-  int kk = k;
-  for (; kk >= 1; --kk) {
-    evicted += hist[kk];
-    if (n - evicted + n_load <= limit) break;
-  }
-  return kk < 1 ? 1 : kk;
-}
-
 // General path: any cache size, active list read from memory.
-__device__ void window_update_generic(const WindowArgs& a, Scan& sc) {
+__device__ void window_update_generic(const WindowArgs& a, Scan<kWindowThreads>& sc) {
   const int tid = threadIdx.x;
   const int n = a.counts[LIF_CNT_NUM_USED];
   const int t = a.counts[LIF_CNT_STEP];
@@ -204,7 +124,7 @@ __device__ void window_update_generic(const WindowArgs& a, Scan& sc) {
       if (a.last_active[a.pointers[s]] <= stale_before) ++c_stale;
   }
   const int any_bad = __syncthreads_or(bad);
-  block_scan(pack3(c_load, c_back, c_stale), &tot, sc);
+  block_scan<kWindowThreads>(pack3(c_load, c_back, c_stale), &tot, sc);
   const int n_load = field(tot, 0);
   const int n_evict = field(tot, 2) - field(tot, 1);
   const int n_kept = n - n_evict;
@@ -265,7 +185,7 @@ __device__ void window_update_generic(const WindowArgs& a, Scan& sc) {
       c_surv += !f && s >= bound;
     }
   }
-  u64 pre = block_scan(pack3(c_ev, 0, c_surv), &tot, sc);
+  u64 pre = block_scan<kWindowThreads>(pack3(c_ev, 0, c_surv), &tot, sc);
   const int n_moves = field(tot, 2);          // surviving rows at or beyond the bound
   if (in_regs) {
     int p_ev = field(pre, 0), p_surv = field(pre, 2);
@@ -333,7 +253,7 @@ __device__ void window_update_generic(const WindowArgs& a, Scan& sc) {
   } else {
     for (int q = q0; q < q1; ++q) c_l += a.slot_of[a.act[q]] < 0;
   }
-  pre = block_scan(pack3(c_l, (q1 - q0) - c_l, 0), &tot, sc);
+  pre = block_scan<kWindowThreads>(pack3(c_l, (q1 - q0) - c_l, 0), &tot, sc);
   if (in_regs) {
     int p_l = field(pre, 0), p_h = field(pre, 1);
 #pragma unroll
@@ -399,7 +319,7 @@ __device__ void window_update_generic(const WindowArgs& a, Scan& sc) {
 }
 
 __global__ void __launch_bounds__(kWindowThreads) window_update_kernel(WindowArgs a) {
-  __shared__ Scan sc;
+  __shared__ Scan<kWindowThreads> sc;
   if (a.release_early) pdl_trigger();     // see window_plan_kernel
   pdl_wait();
   if (!a.release_early) pdl_trigger();
@@ -420,7 +340,7 @@ constexpr int kPlanMaxRows = kPlanSlots * kWindowThreads;
 __global__ void __launch_bounds__(kWindowThreads)
 window_plan_kernel(WindowArgs a, const uint32_t* __restrict__ mask_words, int nwords,
                    int32_t* n_act_out) {
-  __shared__ Scan sc;
+  __shared__ Scan<kWindowThreads> sc;
   __shared__ uint32_t bits[kWindowThreads];
   __shared__ int holes[kPlanMaxRows];
   __shared__ int newslot[kPlanMaxRows];
@@ -462,7 +382,7 @@ window_plan_kernel(WindowArgs a, const uint32_t* __restrict__ mask_words, int nw
   const int cnt = __popc(w);
   bits[tid] = w;
   u64 tot;
-  const int q_base = field(block_scan(pack3(cnt, 0, 0), &tot, sc), 0);   // also publishes bits[]
+  const int q_base = field(block_scan<kWindowThreads>(pack3(cnt, 0, 0), &tot, sc), 0);   // also publishes bits[]
   const int na = field(tot, 0);
   const int fast = __syncthreads_and(n <= kPlanMaxRows && cnt <= kPlanBits);
   if (!fast) {
@@ -528,7 +448,7 @@ window_plan_kernel(WindowArgs a, const uint32_t* __restrict__ mask_words, int nw
 #pragma unroll
   for (int j = 0; j < kPlanSlots; ++j)
     if (age[j] >= k_eff) evm |= 1u << j;
-  u64 pre = block_scan(pack3(c_load, __popc(evm), cnt - c_load), &tot, sc);
+  u64 pre = block_scan<kWindowThreads>(pack3(c_load, __popc(evm), cnt - c_load), &tot, sc);
   const int n_load = field(tot, 0), n_evict = field(tot, 1);
   const int n_kept = n - n_evict;
   int p_load = field(pre, 0), p_ev = field(pre, 1), p_hit = field(pre, 2);
@@ -554,7 +474,7 @@ window_plan_kernel(WindowArgs a, const uint32_t* __restrict__ mask_words, int nw
 #pragma unroll
   for (int j = 0; j < kPlanSlots; ++j)
     if (j < my_slots) c_surv += !((evm >> j) & 1u) && (s0 + j) >= bound;
-  pre = block_scan(pack3(c_surv, 0, 0), &tot, sc);
+  pre = block_scan<kWindowThreads>(pack3(c_surv, 0, 0), &tot, sc);
   const int n_moves = field(tot, 0);          // surviving rows at or beyond the bound
   int p_surv = field(pre, 0);
 
@@ -661,8 +581,8 @@ move_rows_kernel(uint4* __restrict__ cache, const int32_t* __restrict__ move_src
 
 __global__ void __launch_bounds__(kThreads)
 reset_kernel(int32_t* counts, int32_t* pointers, int32_t* slot_of, int32_t* last_active,
-             uint32_t* mask_words, unsigned long long* new_mask_words, int n_mask, int n_new, int F,
-             int cap) {
+             uint32_t* mask_words, unsigned long long* new_mask_words, uint32_t* step_sync, uint4* step_tagged,
+             int n_mask, int n_new, int n_sync, int n_tagged, int F, int cap) {
   const int i = blockIdx.x * kThreads + threadIdx.x;
   const int stride = gridDim.x * kThreads;
   // predictor runs are numbered from 1: no entry of new_mask_words carries a number in use
@@ -674,6 +594,8 @@ reset_kernel(int32_t* counts, int32_t* pointers, int32_t* slot_of, int32_t* last
   }
   for (int j = i; j < n_mask; j += stride) mask_words[j] = 0;
   for (int j = i; j < n_new; j += stride) new_mask_words[j] = 0ull;
+  for (int j = i; j < n_sync; j += stride) step_sync[j] = 0u;
+  for (int j = i; j < n_tagged; j += stride) step_tagged[j] = make_uint4(0, 0, 0, 0);
 }
 
 }  // namespace
@@ -681,13 +603,15 @@ reset_kernel(int32_t* counts, int32_t* pointers, int32_t* slot_of, int32_t* last
 cudaError_t launch_reset(lif_layer* L, cudaStream_t st) {
   const lif_layer_desc& D = L->desc;
   const int n_mask = (D.d_ff + kLogitTile - 1) / kLogitTile * (kLogitTile / 32);
-  reset_kernel<<<64, kThreads, 0, st>>>(L->counts, L->pointers, L->slot_of, L->last_active,
-                                        L->mask_words, L->new_mask_words, n_mask,
-                                        new_mask_entries(D), D.d_ff, D.capacity);
+  reset_kernel<<<296, kThreads, 0, st>>>(L->counts, L->pointers, L->slot_of, L->last_active,
+                                        L->mask_words, L->new_mask_words, L->step_sync,
+                                        (uint4*)L->step_tagged, n_mask,
+                                        2 * new_mask_entries(D), (int)(step_sync_bytes() / 4),
+                                        (int)(step_tagged_bytes(D) / 16), D.d_ff, D.capacity);
   return cudaGetLastError();
 }
 
-static WindowArgs window_args(lif_layer* L, const int32_t* act, const int32_t* n_act) {
+WindowArgs window_args(lif_layer* L, const int32_t* act, const int32_t* n_act) {
   const lif_layer_desc& D = L->desc;
   WindowArgs a;
   a.act = act;
