@@ -322,11 +322,12 @@ lif_status lif_decode_step(lif_layer* L, const void* dev_x, float* dev_y, void* 
     ev = L->tm_events + (size_t)(L->tm_cursor++) * kTimingEvents;
   if (ev) tm_record(ev[0], sc);
   bool ok;
-  // One input stream: predictor, then everything else in one launch, unless the caller times the
-  // phases or has set a knob of the separate kernels.
-  if (L->step_ok && !ev && L->fused_plan && L->split_ffn && L->fused_fetch &&
-      L->fetch_grid == L->n_sm && L->ffn_grid == L->n_sm && L->ffn_stages == L->ffn_stages_max) {
-    L->single_step = 1;
+  // The predictor, then everything else in one launch, unless the caller times the phases or has set
+  // a knob of the separate kernels.
+  if (L->step_ok && !ev && L->fused_plan && L->split_ffn && L->fused_fetch && L->early_fetch &&
+      L->fetch_grid == L->n_sm && L->ffn_grid == L->n_sm && L->ffn_stages == L->ffn_stages_max &&
+      !L->fb_parts_min && !L->fb_up_two_ctas) {
+    L->single_step = L->desc.n_streams == 1;
     ok = launch_predict(L, x, nullptr, L->active_idx, L->n_tmp, sc, nullptr, 0) == cudaSuccess;
     L->single_step = 0;
     ok = ok && launch_step(L, x, dev_y, sc) == cudaSuccess;

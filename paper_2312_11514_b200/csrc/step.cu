@@ -1,4 +1,4 @@
-// One launch for everything of a single-stream decode step behind the predictor: window update,
+// One launch for everything of a decode step behind the predictor: window update,
 // row moves, fetch of the new bundles, sparse FFN over cached and new rows, and the sum.
 //
 // The CTAs of the grid (one per SM) take parts of the step, in the order in which they start:
@@ -31,11 +31,9 @@ namespace {
 
 constexpr int kStepThreads = 512;
 constexpr int kStepWarps = kStepThreads / 32;
-constexpr int kStepChunks = 8192 / 8 / kStepThreads;   // 16-byte chunks per thread and vector
 constexpr int kEntriesPerThread = 2;                   // <= 1024 entries: d_ff <= 32768
 constexpr int kStepWatchPolls = 64;                    // about 30 us
 constexpr unsigned kStepSpinLimit = 1u << 20;          // polls of a counter: about a second
-constexpr int kSumDepth = 4;                           // partial sums per thread in flight
 constexpr int kFetchCtas = 16;
 constexpr unsigned short kNoSlot = 0xffff;
 
@@ -70,7 +68,7 @@ struct StepArgs {
   uint4 *p_hit, *p_new;           // tagged partial sums of cache CTAs (or groups) and fetch CTAs
   float* y;
   StepSync* sync;
-  int d, whole_cache, act;
+  int d, n_streams, whole_cache, act;
   float act_thr;
   int n_cache_ctas, group_size, cache_stages, fetch_stages, fetch_rows_max;
   unsigned wait_polls;
@@ -184,6 +182,10 @@ __device__ __forceinline__ unsigned long long wait_plan(const StepArgs& a,
   }
   __syncthreads();
   return *shared;
+}
+
+__host__ __device__ __forceinline__ size_t x_smem_bytes(int d, int S) {
+  return ((size_t)S * d * 2 + 127) & ~(size_t)127;
 }
 
 // ---- window CTA ---------------------------------------------------------------------------------
@@ -418,25 +420,67 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
 }
 
 // ---- shared by the cache and fetch CTAs ---------------------------------------------------------
-// acc += h * v for the thread's chunks of the down column
-__device__ __forceinline__ void axpy_row(float (&acc)[kStepChunks][8], const uint4* down, float h,
-                                         int nvec) {
+// kS streams (the layer's number rounded up to 1, 2, 4 or 8): a thread keeps kS x kChunks x 8 column
+// sums in registers, which is what limits n_streams * d_model.
+template <int kS>
+struct Shape {
+  static constexpr int kChunks = kS == 8 ? 1 : 2;          // 16-byte chunks per thread and vector
+  static constexpr int kDepth = kS == 1 ? 4 : 8;           // partial sums per thread in flight
+  static constexpr int kMaxD = kChunks * kStepThreads * 8;
+};
+template <int kS>
+struct Acc {
+  float v[kS][Shape<kS>::kChunks][8];
+  __device__ __forceinline__ Acc() {
 #pragma unroll
-  for (int k = 0; k < kStepChunks; ++k) {
+    for (int s = 0; s < kS; ++s)
+#pragma unroll
+      for (int k = 0; k < Shape<kS>::kChunks; ++k)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[s][k][e] = 0.f;
+  }
+};
+// acc += h[s] * v for the thread's chunks of the down column
+template <int kS>
+__device__ __forceinline__ void axpy_row(Acc<kS>& acc, const uint4* down, const float* h, int nvec) {
+#pragma unroll
+  for (int k = 0; k < Shape<kS>::kChunks; ++k) {
     const int c = threadIdx.x + k * kStepThreads;
     if (c < nvec) {
       float f[8];
       unpack8(down[c], f);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) acc[k][e] = fmaf(h, f[e], acc[k][e]);
+      for (int s = 0; s < kS; ++s) {
+        const float hs = h[s];
+        if (kS == 1 || hs != 0.f) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) acc.v[s][k][e] = fmaf(hs, f[e], acc.v[s][k][e]);
+        }
+      }
     }
   }
+}
+// p[s] += <row chunk, x[s] chunk>
+template <int kS>
+__device__ __forceinline__ void dot_chunk(float (&p)[kS], const uint4& row, const uint4* xs, int v,
+                                          int nvec, int S) {
+  float rf[8];
+  unpack8(row, rf);
+#pragma unroll
+  for (int s = 0; s < kS; ++s)
+    if (kS == 1 || s < S) {
+      float xf[8];
+      unpack8(xs[s * nvec + v], xf);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) p[s] = fmaf(rf[e], xf[e], p[s]);
+    }
 }
 // A partial sum for the end of the step: every pair of values is stored as {v, tag, v, tag}, two
 // 8-byte words that are each written whole, with a tag of this step (step number + 1).  The reader
 // polls the words themselves, so there is no fence, no counter and no second round trip between
 // the last row and the sum (measured: 1.3 us from the last row to y instead of 3.5).  Pair e of
-// 8-column chunk c is word e * (d / 8) + c, so that a warp's stores are contiguous.
+// 8-column chunk c is word e * (d / 8) + c of its stream's d / 2, so that a warp's stores are
+// contiguous.
 __device__ __forceinline__ void store_tagged(uint4* dst, float v0, float v1, unsigned tag) {
   asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(dst),
                "l"((unsigned long long)__float_as_uint(v0) | ((unsigned long long)tag << 32)),
@@ -451,27 +495,39 @@ __device__ __forceinline__ ulonglong2 load_tagged(const uint4* src) {
 __device__ __forceinline__ bool has_tag(const ulonglong2& v, unsigned tag) {
   return (unsigned)(v.x >> 32) == tag && (unsigned)(v.y >> 32) == tag;
 }
-__device__ __forceinline__ void store_tagged_partial(const float (&acc)[kStepChunks][8], uint4* dst,
-                                                     int nvec, unsigned tag) {
+template <int kS>
+__device__ __forceinline__ void store_tagged_partial(const Acc<kS>& acc, uint4* dst, int nvec, int S,
+                                                     unsigned tag) {
 #pragma unroll
-  for (int k = 0; k < kStepChunks; ++k) {
-    const int c = threadIdx.x + k * kStepThreads;
-    if (c < nvec) {
+  for (int s = 0; s < kS; ++s)
+    if (kS == 1 || s < S) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) store_tagged(dst + e * nvec + c, acc[k][2 * e], acc[k][2 * e + 1], tag);
+      for (int k = 0; k < Shape<kS>::kChunks; ++k) {
+        const int c = threadIdx.x + k * kStepThreads;
+        if (c < nvec) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            store_tagged(dst + (4 * s + e) * nvec + c, acc.v[s][k][2 * e], acc.v[s][k][2 * e + 1], tag);
+        }
+      }
     }
-  }
 }
-__device__ __forceinline__ void store_partial(const float (&acc)[kStepChunks][8], float* dst, int nvec) {
-  float4* out = reinterpret_cast<float4*>(dst);
+template <int kS>
+__device__ __forceinline__ void store_partial(const Acc<kS>& acc, float* dst, int nvec, int S) {
 #pragma unroll
-  for (int k = 0; k < kStepChunks; ++k) {
-    const int c = threadIdx.x + k * kStepThreads;
-    if (c < nvec) {
-      __stcg(out + 2 * c, make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]));
-      __stcg(out + 2 * c + 1, make_float4(acc[k][4], acc[k][5], acc[k][6], acc[k][7]));
+  for (int s = 0; s < kS; ++s)
+    if (kS == 1 || s < S) {
+      float4* out = reinterpret_cast<float4*>(dst) + (size_t)s * 2 * nvec;
+#pragma unroll
+      for (int k = 0; k < Shape<kS>::kChunks; ++k) {
+        const int c = threadIdx.x + k * kStepThreads;
+        const float(&v)[8] = acc.v[s][k];
+        if (c < nvec) {
+          __stcg(out + 2 * c, make_float4(v[0], v[1], v[2], v[3]));
+          __stcg(out + 2 * c + 1, make_float4(v[4], v[5], v[6], v[7]));
+        }
+      }
     }
-  }
 }
 template <int kGate>
 __device__ __forceinline__ float row_weight(const StepArgs& a, float b, float first, float second) {
@@ -479,6 +535,7 @@ __device__ __forceinline__ float row_weight(const StepArgs& a, float b, float fi
   if (kGate == LIF_GATE_RESIDENT) return apply_activation(b, a.act, a.act_thr) * first;
   return apply_activation(first + b, a.act, a.act_thr);
 }
+// the neuron's bias; resident gate (one stream): its gate value
 template <int kGate>
 __device__ __forceinline__ float row_scalar(const StepArgs& a, int id) {
   return kGate == LIF_GATE_RESIDENT ? a.gate_val[id] : __half2float(a.w.bias_up[id]);
@@ -487,33 +544,29 @@ __device__ __forceinline__ float row_scalar(const StepArgs& a, int id) {
 // ---- cache CTAs: row moves and the FFN of the rows that were already cached -------------------------
 // Rows are read where they were before the moves: a moved row's source is not overwritten before
 // all cache CTAs are done (append_first: not at all), so moves and FFN need no order.
-template <int kGate>
+template <int kGate, int kS>
 __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
   constexpr int kVec = kGate == LIF_GATE_BUNDLED ? 3 : 2;
   __shared__ __align__(8) uint64_t bars[16];
-  __shared__ float h_s[16], b_s[16];
+  __shared__ float h_s[16][kS], b_s[16];
   __shared__ unsigned long long plan_s;
   __shared__ int last_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int d = a.d, nvec = d >> 3, stages = a.cache_stages, nc = a.n_cache_ctas;
+  const int d = a.d, S = a.n_streams, nvec = d >> 3, stages = a.cache_stages, nc = a.n_cache_ctas;
   const unsigned row_bytes = 2u * kVec * d;
-  uint4* xs = reinterpret_cast<uint4*>(smem);              // [d]
-  unsigned char* rows = smem + (((size_t)d * 2 + 127) & ~(size_t)127);
+  uint4* xs = reinterpret_cast<uint4*>(smem);              // [S][d]
+  unsigned char* rows = smem + x_smem_bytes(d, S);
   if (tid == 0) {
     for (int i = 0; i < stages; ++i) mbar_init(bars + i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   pdl_wait();
-  for (int i = tid; i < nvec; i += kStepThreads) xs[i] = reinterpret_cast<const uint4*>(a.x)[i];
+  for (int i = tid; i < S * nvec; i += kStepThreads) xs[i] = reinterpret_cast<const uint4*>(a.x)[i];
   const unsigned long long plan = wait_plan(a, &plan_s);
   const int n = (int)(plan & 0xfffff), n_moves = (int)((plan >> 20) & 0xfffff);
   const int cnt = c < n ? (n - c + nc - 1) / nc : 0;
-  float acc[kStepChunks][8];
-#pragma unroll
-  for (int k = 0; k < kStepChunks; ++k)
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[k][e] = 0.f;
+  Acc<kS> acc;
 
   unsigned parity = 0;
   for (int r0 = 0; r0 < cnt || r0 == 0; r0 += stages) {
@@ -550,33 +603,32 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
         mbar_wait(bars + i, parity);
       }
       const uint4* row = reinterpret_cast<const uint4*>(rows + (size_t)i * row_bytes);
-      float p = 0.f, p2 = 0.f;
-#pragma unroll 4
+      float p[kS], p2[kS];
+#pragma unroll
+      for (int s = 0; s < kS; ++s) p[s] = p2[s] = 0.f;
+#pragma unroll 2
       for (int v = lane; v < nvec; v += 32) {
-        float rf[8], xf[8];
-        unpack8(row[v], rf);
-        unpack8(xs[v], xf);
+        dot_chunk<kS>(p, row[v], xs, v, nvec, S);
+        if (kGate == LIF_GATE_BUNDLED) dot_chunk<kS>(p2, row[nvec + v], xs, v, nvec, S);
+      }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) p = fmaf(rf[e], xf[e], p);
-        if (kGate == LIF_GATE_BUNDLED) {
-          unpack8(row[nvec + v], rf);
+      for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-          for (int e = 0; e < 8; ++e) p2 = fmaf(rf[e], xf[e], p2);
+        for (int s = 0; s < kS; ++s) {
+          p[s] += __shfl_xor_sync(0xffffffffu, p[s], o);
+          if (kGate == LIF_GATE_BUNDLED) p2[s] += __shfl_xor_sync(0xffffffffu, p2[s], o);
         }
-      }
+      if (lane == 0) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        p += __shfl_xor_sync(0xffffffffu, p, o);
-        if (kGate == LIF_GATE_BUNDLED) p2 += __shfl_xor_sync(0xffffffffu, p2, o);
+        for (int s = 0; s < kS; ++s)
+          h_s[i][s] = landed && s < S ? row_weight<kGate>(a, b_s[i], p[s], p2[s]) : 0.f;
       }
-      if (lane == 0) h_s[i] = landed ? row_weight<kGate>(a, b_s[i], p, p2) : 0.f;
     }
     __syncthreads();
     for (int i = 0; i < rc; ++i) {
-      const float h = h_s[i];
-      if (h != 0.f)
-        axpy_row(acc, reinterpret_cast<const uint4*>(rows + (size_t)i * row_bytes) + (kVec - 1) * nvec,
-                 h, nvec);
+      if (kS == 1 && h_s[i][0] == 0.f) continue;
+      axpy_row<kS>(acc, reinterpret_cast<const uint4*>(rows + (size_t)i * row_bytes) + (kVec - 1) * nvec,
+                   h_s[i], nvec);
     }
     parity ^= 1u;
     if (r0 + stages < cnt) {
@@ -588,11 +640,12 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
   // The CTA's partial; with many cache CTAs the last of each group of them adds the group's
   // partials (in CTA order), so that few are left for the end of the step.
   const int gs = a.group_size, g = c / gs;
+  const size_t width = (size_t)S * d;
   if (gs == 1) {
-    if (cnt > 0) store_tagged_partial(acc, a.p_hit + (size_t)c * (d / 2), nvec, a.epoch + 1);
+    if (cnt > 0) store_tagged_partial<kS>(acc, a.p_hit + (size_t)c * (width / 2), nvec, S, a.epoch + 1);
     __syncthreads();
   } else {
-    if (cnt > 0) store_partial(acc, a.p_member + (size_t)c * d, nvec);
+    if (cnt > 0) store_partial<kS>(acc, a.p_member + (size_t)c * width, nvec, S);
     __syncthreads();
     const int members = min(gs, nc - g * gs);
     if (tid == 0) last_s = arrive_last(&a.sync->group[g], (a.epoch + 1) * (unsigned)members);
@@ -600,15 +653,16 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
     if (!last_s) return;
     const int have = min(members, max(0, n - g * gs));     // members with rows wrote a partial
     if (have > 0)
-      for (int i = tid; i < d / 4; i += kStepThreads) {
+      for (int i = tid; i < (int)(width / 4); i += kStepThreads) {
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f), v[8];
 #pragma unroll
         for (int m = 0; m < 8; ++m)
-          if (m < have) v[m] = __ldcg(reinterpret_cast<const float4*>(a.p_member + (size_t)(g * gs + m) * d) + i);
+          if (m < have) v[m] = __ldcg(reinterpret_cast<const float4*>(a.p_member + (size_t)(g * gs + m) * width) + i);
 #pragma unroll
         for (int m = 0; m < 8; ++m)
           if (m < have) { s.x += v[m].x; s.y += v[m].y; s.z += v[m].z; s.w += v[m].w; }
-        uint4* dst = a.p_hit + (size_t)g * (d / 2) + (i & 1) * 2 * nvec + (i >> 1);
+        const int st = i / (2 * nvec), r = i - st * 2 * nvec;
+        uint4* dst = a.p_hit + (size_t)g * (width / 2) + (4 * st + (r & 1) * 2) * nvec + (r >> 1);
         store_tagged(dst, s.x, s.y, a.epoch + 1);
         store_tagged(dst + nvec, s.z, s.w, a.epoch + 1);
       }
@@ -620,19 +674,22 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
 // ---- fetch CTAs: new bundles over the host link, their FFN terms, and the sum -----------------------
 // Fetch CTA f brings in entries f, f + kFetchCtas, ... of the load list, which is exactly the set
 // bits of the predictor's entries in ascending order; only the cache row comes from the plan.
-template <int kGate>
+template <int kGate, int kS>
 __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   constexpr int kVec = kGate == LIF_GATE_BUNDLED ? 3 : 2;
+  constexpr int kDepth = Shape<kS>::kDepth;
   __shared__ __align__(8) uint64_t bars[16];
   __shared__ unsigned sums[1][kStepWarps];
-  __shared__ float part[2][kStepWarps];
+  __shared__ float part[2][kS][kStepWarps];
+  __shared__ float h_s[kS];
   __shared__ unsigned long long plan_s;
   __shared__ float2 red[kStepThreads];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int d = a.d, nvec = d >> 3, stages = a.fetch_stages;
+  const int d = a.d, S = a.n_streams, nvec = d >> 3, stages = a.fetch_stages;
   constexpr int nf = kFetchCtas;
   const unsigned row_bytes = 2u * kVec * d;
-  unsigned char* ring = smem;
+  uint4* xs = reinterpret_cast<uint4*>(smem);              // [S][d]
+  unsigned char* ring = smem + x_smem_bytes(d, S);
   unsigned short* ids = reinterpret_cast<unsigned short*>(ring + (size_t)stages * row_bytes);
   unsigned short* dst_rows = ids + a.fetch_rows_max;
   if (tid == 0) {
@@ -664,27 +721,12 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   int cnt = f < n_new ? (n_new - f + nf - 1) / nf : 0;
   const int issued = min(stages, cnt);
   pdl_wait();
-  uint4 xq[kStepChunks];
-#pragma unroll
-  for (int k = 0; k < kStepChunks; ++k) {
-    const int v = tid + k * kStepThreads;
-    xq[k] = v < nvec ? reinterpret_cast<const uint4*>(a.x)[v] : make_uint4(0, 0, 0, 0);
-  }
-  float acc[kStepChunks][8];
-#pragma unroll
-  for (int k = 0; k < kStepChunks; ++k)
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[k][e] = 0.f;
+  for (int i = tid; i < S * nvec; i += kStepThreads) xs[i] = reinterpret_cast<const uint4*>(a.x)[i];
+  Acc<kS> acc;
 
   const unsigned long long plan = wait_plan(a, &plan_s);
   const bool go = (plan & kPlanReady) && !(plan & kPlanRefused);
   const int n_hit = (int)(plan & 0xfffff);
-  auto spin = [&](const unsigned* counter, unsigned per_step) {  // thread 0
-    const unsigned want = (a.epoch + 1) * per_step;
-    unsigned i = 0;
-    while ((int)(ld_acquire(counter) - want) < 0 && i < kStepSpinLimit) ++i;
-    if (i == kStepSpinLimit) set_status(a, LIF_ERR_TIMEOUT);
-  };
   const int n_groups = (a.n_cache_ctas + a.group_size - 1) / a.group_size;
   if (!go) {
     // the update of this step was refused: nothing is brought in; let the copies land
@@ -695,45 +737,51 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     for (int i = tid; i < cnt; i += kStepThreads)
       dst_rows[i] = (unsigned short)__ldcg(a.w.load_slots + f + i * nf);
     // in the paper's order the new rows' places may be rows the cache CTAs still read
-    if (!a.w.append_first && tid == 0) spin(&a.sync->groups_done, n_groups);
+    if (!a.w.append_first && tid == 0) {
+      const unsigned want = (a.epoch + 1) * (unsigned)n_groups;
+      unsigned i = 0;
+      while ((int)(ld_acquire(&a.sync->groups_done) - want) < 0 && i < kStepSpinLimit) ++i;
+      if (i == kStepSpinLimit) set_status(a, LIF_ERR_TIMEOUT);
+    }
   }
   __syncthreads();
   // The end of the step: every fetch CTA adds up a slice of the columns, in pairs, `width` of them
-  // side by side; the other threads share the partials.  Order: partials of the cached rows (read
-  // while the last row is on its way), then those of the fetch CTAs.
+  // side by side; the other threads share the partials.  Order: partials of the cached rows (with
+  // one block of columns read while the last row is on its way), then those of the fetch CTAs.
   const unsigned tag = a.epoch + 1;
-  const int pairs = d >> 1, per = (pairs + nf - 1) / nf;
+  const int pairs = S * (d >> 1), per = (pairs + nf - 1) / nf;
   const int c0 = f * per, c1 = min(pairs, c0 + per);
   int width = 32;
-  while (width < per && width < kStepThreads / 2) width *= 2;   // per <= 256
+  while (width < per && width < kStepThreads / 2) width *= 2;
   const int slices = kStepThreads / width;
-  const int slice = tid / width, col = c0 + tid % width;
+  const int slice = tid / width;
   const int have_hit = (min(n_hit, a.n_cache_ctas) + a.group_size - 1) / a.group_size;
   const int have_new = go ? min(nf, n_new) : 0;
   float2 sum = make_float2(0.f, 0.f);
   int lost_sum = 0;
-  // adds this thread's partials from number t0 on; stops where they are not there after `limit` polls
-  auto add_partials = [&](const uint4* partials, int have, int t0, unsigned limit) {
+  // adds the thread's partials of column pair `col` from number t0 on; stops where they are not there
+  // after `limit` polls
+  auto add_partials = [&](const uint4* partials, int have, int col, int t0, unsigned limit) {
     if (col >= c1) return have;
-    for (; t0 < have; t0 += slices * kSumDepth) {
-      ulonglong2 v[kSumDepth];
+    for (; t0 < have; t0 += slices * kDepth) {
+      ulonglong2 v[kDepth];
 #pragma unroll
-      for (int k = 0; k < kSumDepth; ++k)                  // (past the end: the last one again)
+      for (int k = 0; k < kDepth; ++k)                     // (past the end: the last one again)
         v[k] = load_tagged(partials + (size_t)min(t0 + k * slices, have - 1) * pairs + col);
       bool there = false;
       for (unsigned polls = 0; polls < limit; ++polls) {
         there = true;
 #pragma unroll
-        for (int k = 0; k < kSumDepth; ++k) there = there && has_tag(v[k], tag);
+        for (int k = 0; k < kDepth; ++k) there = there && has_tag(v[k], tag);
         if (there || polls + 1 == limit) break;
 #pragma unroll
-        for (int k = 0; k < kSumDepth; ++k)                // again, those that were not there
+        for (int k = 0; k < kDepth; ++k)                   // again, those that were not there
           if (!has_tag(v[k], tag))
             v[k] = load_tagged(partials + (size_t)min(t0 + k * slices, have - 1) * pairs + col);
       }
       if (!there) return t0;
 #pragma unroll
-      for (int k = 0; k < kSumDepth; ++k)
+      for (int k = 0; k < kDepth; ++k)
         if (t0 + k * slices < have) {
           sum.x += __uint_as_float((unsigned)v[k].x);
           sum.y += __uint_as_float((unsigned)v[k].y);
@@ -745,7 +793,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
 
   unsigned parity = 0;
   for (int i = 0, st = 0; i < cnt; ++i) {
-    if (i == cnt - 1) t_hit = add_partials(a.p_hit, have_hit, t_hit, 1);
+    if (kS == 1 && i == cnt - 1) t_hit = add_partials(a.p_hit, have_hit, c0 + tid % width, t_hit, 1);
     const uint4* row = reinterpret_cast<const uint4*>(ring + (size_t)st * row_bytes);
     const bool landed = mbar_wait(bars + st, parity, a.wait_polls);
     if (!landed) {                                         // flagged; its term is left out
@@ -759,42 +807,56 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     }
     const float b = row_scalar<kGate>(a, ids[i]);
-    float p = 0.f, p2 = 0.f;
+    float p[kS], p2[kS];
 #pragma unroll
-    for (int k = 0; k < kStepChunks; ++k) {
+    for (int s = 0; s < kS; ++s) p[s] = p2[s] = 0.f;
+#pragma unroll
+    for (int k = 0; k < Shape<kS>::kChunks; ++k) {
       const int v = tid + k * kStepThreads;
       if (v < nvec) {
-        float rf[8], xf[8];
-        unpack8(row[v], rf);
-        unpack8(xq[k], xf);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) p = fmaf(rf[e], xf[e], p);
-        if (kGate == LIF_GATE_BUNDLED) {
-          unpack8(row[nvec + v], rf);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) p2 = fmaf(rf[e], xf[e], p2);
-        }
+        dot_chunk<kS>(p, row[v], xs, v, nvec, S);
+        if (kGate == LIF_GATE_BUNDLED) dot_chunk<kS>(p2, row[nvec + v], xs, v, nvec, S);
       }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      p += __shfl_xor_sync(0xffffffffu, p, o);
-      if (kGate == LIF_GATE_BUNDLED) p2 += __shfl_xor_sync(0xffffffffu, p2, o);
-    }
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int s = 0; s < kS; ++s) {
+        p[s] += __shfl_xor_sync(0xffffffffu, p[s], o);
+        if (kGate == LIF_GATE_BUNDLED) p2[s] += __shfl_xor_sync(0xffffffffu, p2[s], o);
+      }
     if (lane == 0) {
-      part[0][warp] = p;
-      part[1][warp] = p2;
+#pragma unroll
+      for (int s = 0; s < kS; ++s) {
+        part[0][s][warp] = p[s];
+        part[1][s][warp] = p2[s];
+      }
     }
     const int lost = __syncthreads_or(!landed);
-    float v1 = 0.f, v2 = 0.f;
+    const uint4* down = row + (kVec - 1) * nvec;
+    if (kS == 1) {
+      float v1 = 0.f, v2 = 0.f;
 #pragma unroll
-    for (int w = 0; w < kStepWarps; ++w) {
-      v1 += part[0][w];
-      if (kGate == LIF_GATE_BUNDLED) v2 += part[1][w];
+      for (int w = 0; w < kStepWarps; ++w) {
+        v1 += part[0][0][w];
+        if (kGate == LIF_GATE_BUNDLED) v2 += part[1][0][w];
+      }
+      const float h = lost ? 0.f : row_weight<kGate>(a, b, v1, v2);
+      if (h != 0.f) axpy_row<kS>(acc, down, &h, nvec);
+    } else {                                               // a warp per stream folds the 16 warps' sums
+      if (warp < kS) {
+        float v1 = part[0][warp][lane & (kStepWarps - 1)], v2 = part[1][warp][lane & (kStepWarps - 1)];
+#pragma unroll
+        for (int o = kStepWarps / 2; o > 0; o >>= 1) {
+          v1 += __shfl_xor_sync(0xffffffffu, v1, o);
+          v2 += __shfl_xor_sync(0xffffffffu, v2, o);
+        }
+        if (lane == 0) h_s[warp] = lost || warp >= S ? 0.f : row_weight<kGate>(a, b, v1, v2);
+      }
+      __syncthreads();
+      axpy_row<kS>(acc, down, h_s, nvec);
     }
-    const float h = lost ? 0.f : row_weight<kGate>(a, b, v1, v2);
-    if (h != 0.f) axpy_row(acc, row + (kVec - 1) * nvec, h, nvec);
-    __syncthreads();                                       // the stage and part[] are free
+    __syncthreads();                                       // the stage, part[] and h_s[] are free
     if (tid == 0 && i + stages < cnt) {
       asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -805,21 +867,29 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       parity ^= 1u;
     }
   }
-  if (cnt > 0) store_tagged_partial(acc, a.p_new + (size_t)f * (d / 2), nvec, tag);
-  if (add_partials(a.p_hit, have_hit, t_hit, kStepSpinLimit) < have_hit) lost_sum = 1;
-
-  if (add_partials(a.p_new, have_new, slice, kStepSpinLimit) < have_new) lost_sum = 1;
-  red[tid] = sum;
-  __syncthreads();
-  if (tid < width && col < c1) {
-    const int at = 4 * (col % nvec) + col / nvec;          // columns 2 * at, 2 * at + 1
-    float2 y = make_float2(0.f, 0.f);
-    if (a.b_down) y = __half22float2(*reinterpret_cast<const __half2*>(a.b_down + 2 * at));
-    for (int k = 0; k < slices; ++k) {
-      y.x += red[k * width + tid].x;
-      y.y += red[k * width + tid].y;
+  if (cnt > 0) store_tagged_partial<kS>(acc, a.p_new + (size_t)f * pairs, nvec, S, tag);
+  for (int cc = c0; cc < c1; cc += width) {
+    const int col = cc + tid % width;
+    if (cc > c0) {
+      sum = make_float2(0.f, 0.f);
+      t_hit = slice;
+      __syncthreads();                                     // red[] is free again
     }
-    reinterpret_cast<float2*>(a.y)[at] = y;
+    if (add_partials(a.p_hit, have_hit, col, t_hit, kStepSpinLimit) < have_hit) lost_sum = 1;
+    if (add_partials(a.p_new, have_new, col, slice, kStepSpinLimit) < have_new) lost_sum = 1;
+    red[tid] = sum;
+    __syncthreads();
+    if (tid < width && col < c1) {
+      const int s = kS == 1 ? 0 : col / (4 * nvec), r = kS == 1 ? col : col % (4 * nvec);
+      const int at = 4 * (r % nvec) + r / nvec;            // columns 2 * at, 2 * at + 1
+      float2 y = make_float2(0.f, 0.f);
+      if (a.b_down) y = __half22float2(*reinterpret_cast<const __half2*>(a.b_down + 2 * at));
+      for (int k = 0; k < slices; ++k) {
+        y.x += red[k * width + tid].x;
+        y.y += red[k * width + tid].y;
+      }
+      reinterpret_cast<float2*>(a.y + (size_t)s * d)[at] = y;
+    }
   }
   if (lost_sum) set_status(a, LIF_ERR_TIMEOUT);
   if (tid == 0) {
@@ -829,8 +899,8 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   }
 }
 
-template <int kGate>
-__global__ void __launch_bounds__(kStepThreads, 2) step_kernel(StepArgs a) {
+template <int kGate, int kS>
+__global__ void __launch_bounds__(kStepThreads, kS == 1 ? 2 : 1) step_kernel(StepArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ unsigned part_s, epoch_s;
   pdl_trigger();       // whatever follows waits for this kernel's end before it reads its results
@@ -843,71 +913,85 @@ __global__ void __launch_bounds__(kStepThreads, 2) step_kernel(StepArgs a) {
   const int part = (int)part_s;
   a.epoch = epoch_s;
   if (part == 0) window_role(a, smem);
-  else if (part <= a.n_cache_ctas) cache_role<kGate>(a, part - 1, smem);
-  else fetch_role<kGate>(a, part - 1 - a.n_cache_ctas, smem);
+  else if (part <= a.n_cache_ctas) cache_role<kGate, kS>(a, part - 1, smem);
+  else fetch_role<kGate, kS>(a, part - 1 - a.n_cache_ctas, smem);
 }
 
 using StepKernel = void (*)(StepArgs);
-StepKernel step_kernel_for(int gate_mode) {
-  if (gate_mode == LIF_GATE_BUNDLED) return step_kernel<LIF_GATE_BUNDLED>;
-  if (gate_mode == LIF_GATE_RESIDENT) return step_kernel<LIF_GATE_RESIDENT>;
-  return step_kernel<LIF_GATE_NONE>;
+StepKernel step_kernel_for(const lif_layer_desc& D) {
+  if (D.n_streams > 1) {
+    if (D.gate_mode != LIF_GATE_NONE) return nullptr;
+    if (D.n_streams == 2 && D.d_model <= Shape<2>::kMaxD) return step_kernel<LIF_GATE_NONE, 2>;
+    if (D.n_streams <= 4 && D.d_model <= Shape<4>::kMaxD) return step_kernel<LIF_GATE_NONE, 4>;
+    if (D.n_streams <= 8 && D.d_model <= Shape<8>::kMaxD) return step_kernel<LIF_GATE_NONE, 8>;
+    return nullptr;
+  }
+  if (D.gate_mode == LIF_GATE_BUNDLED) return step_kernel<LIF_GATE_BUNDLED, 1>;
+  if (D.gate_mode == LIF_GATE_RESIDENT) return step_kernel<LIF_GATE_RESIDENT, 1>;
+  return step_kernel<LIF_GATE_NONE, 1>;
 }
-constexpr int kGroupMax = 8, kGroupsMax = 64;
+constexpr int kGroupMax = 8, kUngroupedMax = 64, kUngroupedMaxStreams = 16;
 constexpr size_t kCacheRing = 128 * 1024, kFetchRing = 32 * 1024;
+
+// CTAs for the rows that are already cached, about a third of which are active in a step: with one
+// stream a CTA per eight rows of the cache; with several one per sixteen, because a CTA's partial is
+// as long as its streams' outputs together.
+int cache_ctas(const lif_layer_desc& D, int n_sm) {
+  const int per = D.n_streams > 1 ? 16 : 8, most = D.n_streams > 1 ? 64 : n_sm - 1 - kFetchCtas;
+  const int nc = (D.capacity + per - 1) / per;
+  return nc < 8 ? 8 : (nc > most ? most : nc);
+}
+// Tagged partials of cache CTAs (or of groups of them) that the fetch CTAs add up at the end.
+int hit_partials_max(const lif_layer_desc& D) {
+  return D.n_streams > 1 ? kUngroupedMaxStreams : kUngroupedMax;
+}
 
 }  // namespace
 
 size_t step_sync_bytes() { return sizeof(StepSync); }
 size_t step_tagged_bytes(const lif_layer_desc& D) {
-  return D.n_streams == 1 ? (size_t)(kGroupsMax + kFetchCtas) * D.d_model * 8 : 0;
+  return step_kernel_for(D) ? (size_t)(hit_partials_max(D) + kFetchCtas) * D.n_streams * D.d_model * 8 : 0;
 }
 
-// Shape of the launch, and whether the single launch applies: one input stream, ids and rows that
-// fit 16 bits and the predictor's entries two per thread (d_ff <= 32768), the window CTA's arrays in
-// shared memory.
+// Shape of the launch, and whether the single launch applies: streams x width in registers, ids and
+// rows that fit 16 bits and the predictor's entries two per thread (d_ff <= 32768), the window CTA's
+// arrays in shared memory.
 cudaError_t step_configure(lif_layer* L) {
   const lif_layer_desc& D = L->desc;
   L->step_ok = 0;
-  const int n_entries = new_mask_entries(D);
-  if (D.n_streams != 1 || n_entries > kEntriesPerThread * kStepThreads || D.d_ff > 32768 ||
-      new_mask_entry_bits(D) != 32 ||
-      D.window_k > 32767 || L->n_sm < 2 * kFetchCtas)
+  StepKernel kernel = step_kernel_for(D);
+  if (!kernel || new_mask_entries(D) > kEntriesPerThread * kStepThreads || D.d_ff > 32768 ||
+      new_mask_entry_bits(D) != 32 || D.window_k > 32767 || L->n_sm < 2 * kFetchCtas)
     return cudaSuccess;
   int dev = 0, max_smem = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  const size_t row = 2 * (size_t)row_elems(D);
-  const int nf = kFetchCtas;
-  auto stages = [&](size_t ring, int least) {
+  cudaFuncAttributes at;
+  e = cudaFuncGetAttributes(&at, kernel);
+  if (e != cudaSuccess) return e;
+  max_smem -= (int)at.sharedSizeBytes;
+  const size_t row = 2 * (size_t)row_elems(D), x = x_smem_bytes(D.d_model, D.n_streams);
+  const size_t ids = 4 * (((size_t)D.d_ff + kFetchCtas - 1) / kFetchCtas);
+  auto stages = [&](size_t ring, size_t other, int least) {
+    while (ring > row * least && ring + other > (size_t)max_smem) ring -= row;
     const int s = (int)(ring / row);
     return s < least ? least : (s > 16 ? 16 : s);
   };
-  // about eight rows of the cache per cache CTA: a third of them is active in a step
-  int nc = (D.capacity + 7) / 8;
-  if (nc < 8) nc = 8;
-  if (nc > L->n_sm - 1 - nf) nc = L->n_sm - 1 - nf;
-  L->step_cache_ctas = nc;
-  L->step_group = nc > kGroupsMax ? kGroupMax : 1;
-  L->step_cache_stages = stages(kCacheRing, 1);
+  L->step_cache_ctas = cache_ctas(D, L->n_sm);
+  L->step_group = L->step_cache_ctas > hit_partials_max(D) ? kGroupMax : 1;
+  L->step_cache_stages = stages(kCacheRing, x, 1);
   // in the paper's cache order the bundles wait in the ring until the cache CTAs have read the rows
   // they replace: twice the ring keeps the link busy meanwhile
-  L->step_fetch_stages = stages(D.append_first ? kFetchRing : 2 * kFetchRing, 2);
-  const size_t rows_max = ((size_t)D.d_ff + nf - 1) / nf;
-  const size_t need_w = window_role_smem(D.d_ff, D.capacity);
-  const size_t need_c = ((2 * (size_t)D.d_model + 127) & ~(size_t)127) + L->step_cache_stages * row;
-  const size_t need_f = L->step_fetch_stages * row + 4 * rows_max;
-  size_t smem = need_w > need_c ? need_w : need_c;
+  L->step_fetch_stages = stages(D.append_first ? kFetchRing : 2 * kFetchRing, x + ids, 2);
+  size_t smem = window_role_smem(D.d_ff, D.capacity);
+  const size_t need_c = x + L->step_cache_stages * row, need_f = x + L->step_fetch_stages * row + ids;
+  if (need_c > smem) smem = need_c;
   if (need_f > smem) smem = need_f;
-  cudaFuncAttributes at;
-  e = cudaFuncGetAttributes(&at, step_kernel_for(D.gate_mode));
-  if (e != cudaSuccess) return e;
-  if (smem + at.sharedSizeBytes > (size_t)max_smem) return cudaSuccess;
+  if (smem > (size_t)max_smem) return cudaSuccess;
   L->step_smem = smem;
-  e = cudaFuncSetAttribute(step_kernel_for(D.gate_mode), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           max_smem - (int)at.sharedSizeBytes);
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
   if (e != cudaSuccess) return e;
   L->step_ok = 1;
   return cudaSuccess;
@@ -931,10 +1015,11 @@ cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st
   a.b_down = (const __half*)D.dev_bias_down;
   a.p_member = L->y_partial;
   a.p_hit = (uint4*)L->step_tagged;
-  a.p_new = a.p_hit + (size_t)kGroupsMax * (D.d_model / 2);
+  a.p_new = a.p_hit + (size_t)hit_partials_max(D) * D.n_streams * (D.d_model / 2);
   a.y = y;
   a.sync = (StepSync*)L->step_sync;
   a.d = D.d_model;
+  a.n_streams = D.n_streams;
   a.whole_cache = D.ffn_mode == 1;
   a.act = D.activation;
   a.act_thr = D.activation_threshold;
@@ -944,7 +1029,7 @@ cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st
   a.fetch_stages = L->step_fetch_stages;
   a.fetch_rows_max = (D.d_ff + kFetchCtas - 1) / kFetchCtas;
   a.wait_polls = L->wait_polls;
-  return launch_k(step_kernel_for(D.gate_mode), dim3(1 + a.n_cache_ctas + kFetchCtas),
+  return launch_k(step_kernel_for(D), dim3(1 + a.n_cache_ctas + kFetchCtas),
                   dim3(kStepThreads), L->step_smem, st, L->use_pdl, a);
 }
 
