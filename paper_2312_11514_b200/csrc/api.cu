@@ -169,7 +169,9 @@ lif_status lif_create_layer(const lif_layer_desc* desc, lif_layer** out) {
 
   int dev = 0;
   bool ok = cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&L->n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+            cudaDeviceGetAttribute(&L->n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&L->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) ==
+                cudaSuccess;
   ok = ok && ffn_configure(L) == cudaSuccess;
   L->fb_up_two_ctas = 0;
   L->early_fetch = 1;

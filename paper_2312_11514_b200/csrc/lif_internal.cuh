@@ -78,12 +78,13 @@ struct lif_layer {
   int fb_ksplit, fb_kps, fb_up_partitions, fb_parts_min, fb_up_group, fb_up_two_ctas;
   size_t fb_up_smem, fb_down_smem;
   // single-launch decode step (step.cu); step_ok = 0: it does not apply to this layer
-  int step_ok, step_cache_ctas, step_group, step_cache_stages, step_fetch_stages;
+  int step_ok, step_cache_ctas, step_sum_ctas, step_group, step_cache_stages, step_fetch_stages;
   size_t step_smem;
   uint32_t* hit_rows;         // plan of the step: rows (before the moves) and neurons of the hits
   uint32_t* step_sync;        // its counters
   uint32_t* step_tagged;      // its tagged partial sums (no tag of a step to come)
   int n_sm;
+  int max_smem;       // shared memory a CTA can opt in to
   int z_ctas;         // CTAs of the first predictor stage
   int ffn_grid;       // CTAs of the sparse-FFN kernel
   int ffn_stages;     // bundles in flight per CTA
@@ -175,6 +176,10 @@ cudaError_t launch_fetch_ffn(lif_layer* L, const __half* x, float* partial, cuda
 size_t step_sync_bytes();
 size_t step_tagged_bytes(const lif_layer_desc& D);
 cudaError_t predict_configure(const lif_layer* L);
+// several input streams (predict_multi.cu)
+cudaError_t predict_multi_configure(const lif_layer* L);
+cudaError_t launch_predict_multi(lif_layer* L, const __half* x, float* logits, int32_t* active_idx,
+                                 int32_t* n_active, cudaStream_t st, cudaEvent_t* ev, int compact);
 cudaError_t step_configure(lif_layer* L);
 cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st);
 cudaError_t launch_refill(lif_layer* L, cudaStream_t st);
@@ -300,6 +305,22 @@ __device__ __forceinline__ void unpack8(const uint4& v, float* f) {
     f[2 * i] = t.x;
     f[2 * i + 1] = t.y;
   }
+}
+
+// c + a * b for two fp32 values at once (each rounded as fmaf rounds it)
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(r)
+      : "l"(*reinterpret_cast<unsigned long long*>(&a)), "l"(*reinterpret_cast<unsigned long long*>(&b)),
+        "l"(*reinterpret_cast<unsigned long long*>(&c)));
+  return *reinterpret_cast<float2*>(&r);
+}
+// eight fp16 values -> four pairs of fp32
+__device__ __forceinline__ void unpack8(const uint4& v, float2* f) {
+  const __half2* h = reinterpret_cast<const __half2*>(&v);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) f[i] = __half22float2(h[i]);
 }
 
 // ---- mbarrier + bulk asynchronous copy (TMA, CTA-local, no multicast) -------------------------

@@ -1,4 +1,5 @@
-// Low-rank sparsity predictor (Section 3.1, "Anticipating ReLU Sparsity"; Appendix B):
+// Low-rank sparsity predictor (Section 3.1, "Anticipating ReLU Sparsity"; Appendix B), one input
+// stream (several: predict_multi.cu):
 // scores = x.A.B + c, active iff score > theta, compacted to an ascending index list.
 //
 // Both stages are HBM-bound GEMVs over fp16 factors with fp32 accumulation:
@@ -13,8 +14,7 @@
 namespace lif {
 namespace {
 
-// ---- stage 1: z_partial[cta][s][j] = sum_{m in rows(cta)} x[s][m] * A[m][j] -------------
-template <int S>
+// ---- stage 1: z_partial[cta][j] = sum_{m in rows(cta)} x[m] * A[m][j] -------------
 __global__ void __launch_bounds__(kThreads)
 predict_z_kernel(const __half* __restrict__ x, const __half* __restrict__ A, int d, int r,
                  int rows_per_cta, int staged, float* __restrict__ z_partial) {
@@ -27,11 +27,9 @@ predict_z_kernel(const __half* __restrict__ x, const __half* __restrict__ A, int
   const int m0 = blockIdx.x * rows_per_cta;
   const int m1 = min(d, m0 + rows_per_cta);
 
-  float acc[S][8];
+  float acc[8];
 #pragma unroll
-  for (int s = 0; s < S; ++s)
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[s][e] = 0.f;
+  for (int e = 0; e < 8; ++e) acc[e] = 0.f;
 
   // A is a weight: the thread's first 8 rows go into registers and the next `staged` into its own
   // slots of shared memory before the dependency wait, x (possibly written by the previous kernel)
@@ -56,12 +54,9 @@ predict_z_kernel(const __half* __restrict__ x, const __half* __restrict__ A, int
       if (m < m1) {
         float af[8];
         unpack8(aq[u], af);
+        const float xs = __half2float(x[m]);
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const float xs = __half2float(x[(size_t)s * d + m]);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) acc[s][e] = fmaf(xs, af[e], acc[s][e]);
-        }
+        for (int e = 0; e < 8; ++e) acc[e] = fmaf(xs, af[e], acc[e]);
       }
     }
     own_copies_wait();
@@ -71,46 +66,36 @@ predict_z_kernel(const __half* __restrict__ x, const __half* __restrict__ A, int
       if (m < m1) {
         float af[8];
         unpack8(staged_rows[u * kThreads + tid], af);
+        const float xs = __half2float(x[m]);
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const float xs = __half2float(x[(size_t)s * d + m]);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) acc[s][e] = fmaf(xs, af[e], acc[s][e]);
-        }
+        for (int e = 0; e < 8; ++e) acc[e] = fmaf(xs, af[e], acc[e]);
       }
     }
 #pragma unroll 4
     for (int m = m0 + rl + (8 + staged) * nrl; m < m1; m += nrl) {
       float af[8];
       unpack8(ld_stream16(A + (size_t)m * r + cg * 8), af);
+      const float xs = __half2float(x[m]);
 #pragma unroll
-      for (int s = 0; s < S; ++s) {
-        const float xs = __half2float(x[(size_t)s * d + m]);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[s][e] = fmaf(xs, af[e], acc[s][e]);
-      }
+      for (int e = 0; e < 8; ++e) acc[e] = fmaf(xs, af[e], acc[e]);
     }
   }
-  // fold the row lanes, one stream at a time (8 KB of shared memory)
+  // fold the row lanes (8 KB of shared memory)
+  if (rl < nrl) {
 #pragma unroll
-  for (int s = 0; s < S; ++s) {
-    if (rl < nrl) {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) red[rl * r + cg * 8 + e] = acc[s][e];
-    }
-    __syncthreads();
-    for (int j = tid; j < r; j += kThreads) {
-      float v = 0.f;
-      for (int l = 0; l < nrl; ++l) v += red[l * r + j];
-      z_partial[((size_t)blockIdx.x * S + s) * r + j] = v;
-    }
-    __syncthreads();
+    for (int e = 0; e < 8; ++e) red[rl * r + cg * 8 + e] = acc[e];
+  }
+  __syncthreads();
+  for (int j = tid; j < r; j += kThreads) {
+    float v = 0.f;
+    for (int l = 0; l < nrl; ++l) v += red[l * r + j];
+    z_partial[(size_t)blockIdx.x * r + j] = v;
   }
 }
 
 // ---- stage 2: scores, threshold, bit mask; last CTA compacts ------------------------------
 // kSpec: also record per neuron the last token < keep in which it is active (speculative mode).
-template <int S, bool kSpec>
+template <bool kSpec>
 __global__ void __launch_bounds__(kThreads)
 predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* __restrict__ B,
                       const float* __restrict__ c, float theta, int r, int F,
@@ -118,7 +103,7 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
                       int* __restrict__ active_idx, int* __restrict__ n_active, int compact,
                       int8_t* __restrict__ keep_tok, int keep, const int32_t* __restrict__ slot_of,
                       unsigned long long* new_mask_words, int* predictor_run, int staged) {
-  extern __shared__ __align__(16) float zs[];   // [S][r], then the rows of B beyond the first 128
+  extern __shared__ __align__(16) float zs[];   // [r], then the rows of B beyond the first 128
   __shared__ float red[16][kLogitTile];
   __shared__ int warp_sums[kThreads / 32];
   __shared__ int is_last;
@@ -135,7 +120,7 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
     bq[u] = (col < F && j < r) ? ld_stream16(B + (size_t)j * F + col) : make_uint4(0, 0, 0, 0);
   }
   // the next rows go into the thread's own slots of shared memory (see predict_z_kernel)
-  uint4* staged_rows = reinterpret_cast<uint4*>(zs + S * r) + tid;
+  uint4* staged_rows = reinterpret_cast<uint4*>(zs + r) + tid;
   for (int u = 0; u < staged; ++u) {
     const int j = rs + 16 * (8 + u);
     if (col < F && j < r) copy_async16(staged_rows + u * kThreads, B + (size_t)j * F + col);
@@ -152,45 +137,24 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
   pdl_trigger();
   pdl_wait();
   const int run = (tid < kLogitTile && (tid & 31) == 0) ? __ldcg(predictor_run) : 0;
-  if (S == 1) {
-    // one stream: every partial of a sum is requested before the first is used (one memory
-    // round trip instead of several); the additions keep their order
-    for (int i = tid; i < S * r; i += kThreads) {
-      float t[kMaxZPartials];
+  // every partial of a sum is requested before the first is used (one memory round trip instead of
+  // several); the additions keep their order
+  for (int i = tid; i < r; i += kThreads) {
+    float t[kMaxZPartials];
 #pragma unroll
-      for (int p = 0; p < kMaxZPartials; ++p)
-        t[p] = p < P ? __ldcg(z_partial + (size_t)p * S * r + i) : 0.f;
-      float v = 0.f;
+    for (int p = 0; p < kMaxZPartials; ++p)
+      t[p] = p < P ? __ldcg(z_partial + (size_t)p * r + i) : 0.f;
+    float v = 0.f;
 #pragma unroll
-      for (int p = 0; p < kMaxZPartials; ++p)
-        if (p < P) v += t[p];
-      zs[i] = v;
-    }
-  } else {
-    // several streams: S * r sums per CTA; four per thread at a time keep 32 loads in flight
-    // (same order of additions per sum)
-    for (int i0 = tid; i0 < S * r; i0 += 4 * kThreads) {
-      float v[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-      for (int p = 0; p < P; ++p) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = i0 + u * kThreads;
-          if (i < S * r) v[u] += __ldcg(z_partial + (size_t)p * S * r + i);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (i0 + u * kThreads < S * r) zs[i0 + u * kThreads] = v[u];
-    }
+    for (int p = 0; p < kMaxZPartials; ++p)
+      if (p < P) v += t[p];
+    zs[i] = v;
   }
   __syncthreads();
 
-  float acc[S][8];
+  float acc[8];
 #pragma unroll
-  for (int s = 0; s < S; ++s)
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[s][e] = 0.f;
+  for (int e = 0; e < 8; ++e) acc[e] = 0.f;
   for (int j0 = 0; j0 < r; j0 += 128) {
     if (j0 > 0) {
       if (j0 == 128) own_copies_wait();
@@ -208,35 +172,26 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
       if (j < r) {
         float bf[8];
         unpack8(bq[u], bf);
+        const float zz = zs[j];
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const float zz = zs[s * r + j];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) acc[s][e] = fmaf(zz, bf[e], acc[s][e]);
-        }
+        for (int e = 0; e < 8; ++e) acc[e] = fmaf(zz, bf[e], acc[e]);
       }
     }
   }
 
+#pragma unroll
+  for (int e = 0; e < 8; ++e) red[rs][cg * 8 + e] = acc[e];
+  __syncthreads();
   bool active = false;
-  int last_kept = -1;        // speculative mode: last token < keep in which the neuron is active
+  if (tid < kLogitTile && my_col < F) {
+    float v = 0.f;
 #pragma unroll
-  for (int s = 0; s < S; ++s) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) red[rs][cg * 8 + e] = acc[s][e];
-    __syncthreads();
-    if (tid < kLogitTile && my_col < F) {
-      float v = 0.f;
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v += red[k][tid];
-      v += my_c;
-      if (logits) logits[(size_t)s * F + my_col] = v;
-      active = active || (v > theta);
-      if (kSpec && v > theta && s < keep) last_kept = s;
-    }
-    __syncthreads();
+    for (int k = 0; k < 16; ++k) v += red[k][tid];
+    v += my_c;
+    if (logits) logits[my_col] = v;
+    active = v > theta;
+    if (kSpec) keep_tok[my_col] = (int8_t)(active && keep > 0 ? 0 : -1);
   }
-  if (kSpec && tid < kLogitTile && my_col < F) keep_tok[my_col] = (int8_t)last_kept;
   if (tid < kLogitTile) {
     const unsigned m = __ballot_sync(0xffffffffu, active);
     const unsigned mn = __ballot_sync(0xffffffffu, active && my_row < 0);
@@ -274,12 +229,11 @@ int logit_staged_rows(const lif_layer_desc& D) {
   return rows < 0 ? 0 : (rows > kMaxStaged ? kMaxStaged : rows);
 }
 
-template <int S>
-cudaError_t launch_predict_s(lif_layer* L, const __half* x, float* logits, int32_t* active_idx,
+cudaError_t launch_predict_single(lif_layer* L, const __half* x, float* logits, int32_t* active_idx,
                              int32_t* n_active, cudaStream_t st, cudaEvent_t* ev, int compact) {
   const lif_layer_desc& D = L->desc;
   const int z_staged = z_staged_rows(D);
-  cudaError_t e = launch_k2(predict_z_kernel<S>, dim3(L->z_ctas), dim3(kThreads),
+  cudaError_t e = launch_k2(predict_z_kernel, dim3(L->z_ctas), dim3(kThreads),
                            (size_t)z_staged * kThreads * 16, st, L->use_pdl, L->single_step,
                            x, (const __half*)D.dev_pred_A, D.d_model, D.rank,
                            z_rows_per_cta(D.d_model), z_staged, L->z_partial);
@@ -287,8 +241,8 @@ cudaError_t launch_predict_s(lif_layer* L, const __half* x, float* logits, int32
   if (ev) tm_record(ev[1], st);
   const int grid = (D.d_ff + kLogitTile - 1) / kLogitTile;
   const int staged = logit_staged_rows(D);
-  const size_t smem = (size_t)S * D.rank * sizeof(float) + (size_t)staged * kThreads * 16;
-  auto kernel = L->keep_tok ? predict_logits_kernel<S, true> : predict_logits_kernel<S, false>;
+  const size_t smem = (size_t)D.rank * sizeof(float) + (size_t)staged * kThreads * 16;
+  auto kernel = L->keep_tok ? predict_logits_kernel<true> : predict_logits_kernel<false>;
   e = launch_k2(kernel, dim3(grid), dim3(kThreads), smem, st, L->use_pdl, L->single_step,
                (const float*)L->z_partial, L->z_ctas, (const __half*)D.dev_pred_B, D.dev_pred_c,
                D.threshold_logit, D.rank, D.d_ff, logits, L->mask_words,
@@ -299,34 +253,20 @@ cudaError_t launch_predict_s(lif_layer* L, const __half* x, float* logits, int32
   return e;
 }
 
-// Opt-ins of the kernels for S streams (once per layer).
-template <int S>
-cudaError_t predict_configure_s() {
-  const void* kernels[3] = {(const void*)predict_z_kernel<S>, (const void*)predict_logits_kernel<S, false>,
-                            (const void*)predict_logits_kernel<S, true>};
+}  // namespace
+
+// Opt-ins of the kernels (once per layer).
+cudaError_t predict_configure(const lif_layer* L) {
+  if (L->desc.n_streams > 1) return predict_multi_configure(L);
+  const void* kernels[3] = {(const void*)predict_z_kernel, (const void*)predict_logits_kernel<false>,
+                            (const void*)predict_logits_kernel<true>};
   for (const void* k : kernels) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kMaxStaged * kThreads * 16 +
-                                             (k == kernels[0] ? 0 : S * kMaxRank * (int)sizeof(float)));
+                                             (k == kernels[0] ? 0 : kMaxRank * (int)sizeof(float)));
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
-}
-
-}  // namespace
-
-cudaError_t predict_configure(const lif_layer* L) {
-  switch (L->desc.n_streams) {
-    case 1: return predict_configure_s<1>();
-    case 2: return predict_configure_s<2>();
-    case 3: return predict_configure_s<3>();
-    case 4: return predict_configure_s<4>();
-    case 5: return predict_configure_s<5>();
-    case 6: return predict_configure_s<6>();
-    case 7: return predict_configure_s<7>();
-    case 8: return predict_configure_s<8>();
-  }
-  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_predict_one(lif_layer* L, int kernel, const __half* x, cudaStream_t st) {
@@ -338,12 +278,12 @@ cudaError_t launch_predict_one(lif_layer* L, int kernel, const __half* x, cudaSt
                                      L->fused_plan ? 0 : 1, false)
                : cudaErrorInvalidValue;
   if (kernel == LIF_KERNEL_PREDICT_Z)
-    return launch_k(predict_z_kernel<1>, dim3(L->z_ctas), dim3(kThreads),
+    return launch_k(predict_z_kernel, dim3(L->z_ctas), dim3(kThreads),
                     (size_t)z_staged_rows(D) * kThreads * 16, st, L->use_pdl, x,
                     (const __half*)D.dev_pred_A, D.d_model, D.rank, z_rows_per_cta(D.d_model),
                     z_staged_rows(D), L->z_partial);
   const int grid = (D.d_ff + kLogitTile - 1) / kLogitTile;
-  return launch_k(L->keep_tok ? predict_logits_kernel<1, true> : predict_logits_kernel<1, false>,
+  return launch_k(L->keep_tok ? predict_logits_kernel<true> : predict_logits_kernel<false>,
                   dim3(grid), dim3(kThreads),
                   (size_t)D.rank * sizeof(float) + (size_t)logit_staged_rows(D) * kThreads * 16, st, L->use_pdl, (const float*)L->z_partial,
                   L->z_ctas, (const __half*)D.dev_pred_B, D.dev_pred_c, D.threshold_logit, D.rank,
@@ -357,17 +297,9 @@ cudaError_t launch_predict(lif_layer* L, const __half* x, float* logits, int32_t
                            int32_t* n_active, cudaStream_t st, cudaEvent_t* ev, int compact) {
   if (L->desc.gate_mode == LIF_GATE_RESIDENT)
     return launch_gate_predict(L, x, logits, active_idx, n_active, st, ev, compact);
-  switch (L->desc.n_streams) {
-    case 1: return launch_predict_s<1>(L, x, logits, active_idx, n_active, st, ev, compact);
-    case 2: return launch_predict_s<2>(L, x, logits, active_idx, n_active, st, ev, compact);
-    case 3: return launch_predict_s<3>(L, x, logits, active_idx, n_active, st, ev, compact);
-    case 4: return launch_predict_s<4>(L, x, logits, active_idx, n_active, st, ev, compact);
-    case 5: return launch_predict_s<5>(L, x, logits, active_idx, n_active, st, ev, compact);
-    case 6: return launch_predict_s<6>(L, x, logits, active_idx, n_active, st, ev, compact);
-    case 7: return launch_predict_s<7>(L, x, logits, active_idx, n_active, st, ev, compact);
-    case 8: return launch_predict_s<8>(L, x, logits, active_idx, n_active, st, ev, compact);
-  }
-  return cudaErrorInvalidValue;
+  return L->desc.n_streams == 1
+             ? launch_predict_single(L, x, logits, active_idx, n_active, st, ev, compact)
+             : launch_predict_multi(L, x, logits, active_idx, n_active, st, ev, compact);
 }
 
 }  // namespace lif

@@ -6,12 +6,13 @@
 //                          predictor's entries; publishes the plan with one flag
 //   cache CTAs   (middle)  wait for the plan; row moves, then the FFN terms of the rows that were
 //                          already cached (bulk copies into shared memory, a warp per row)
-//   fetch CTAs   (last)    find the new neurons themselves in the predictor's entries, bring their
+//   fetch CTAs   (then)    find the new neurons themselves in the predictor's entries, bring their
 //                          bundles over the host link through a ring of bulk copies, add their FFN
-//                          terms from shared memory, copy them to their cache rows, and in the end
-//                          add up all partial sums
-// A CTA waits only for CTAs that took their parts before it (the fetch CTAs also for one
-// another, at the very end, when nothing else is left to run), every wait is bounded, and every CTA
+//                          terms from shared memory, copy them to their cache rows, and (one stream) in
+//                          the end add up all partial sums
+//   sum CTAs     (last)    with several streams add up the partial sums
+// A CTA waits only for CTAs that took their parts before it (with one stream the fetch CTAs also for
+// one another, at the very end, when nothing else is left to run), every wait is bounded, and every CTA
 // makes its arrivals on all paths, so the counters are complete whatever happened.
 //
 // Why one launch: the parts run side by side without an event or a stream of their own (five
@@ -70,7 +71,7 @@ struct StepArgs {
   StepSync* sync;
   int d, n_streams, whole_cache, act;
   float act_thr;
-  int n_cache_ctas, group_size, cache_stages, fetch_stages, fetch_rows_max;
+  int n_cache_ctas, n_sum_ctas, group_size, cache_stages, fetch_stages, fetch_rows_max;
   unsigned wait_polls;
   unsigned epoch;                 // steps before this one (filled in by the kernel)
 };
@@ -425,7 +426,7 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
 template <int kS>
 struct Shape {
   static constexpr int kChunks = kS == 8 ? 1 : 2;          // 16-byte chunks per thread and vector
-  static constexpr int kDepth = kS == 1 ? 4 : 8;           // partial sums per thread in flight
+  static constexpr int kDepth = kS == 1 ? 4 : 12;          // partial sums per thread in flight
   static constexpr int kMaxD = kChunks * kStepThreads * 8;
 };
 template <int kS>
@@ -614,10 +615,11 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-        for (int s = 0; s < kS; ++s) {
-          p[s] += __shfl_xor_sync(0xffffffffu, p[s], o);
-          if (kGate == LIF_GATE_BUNDLED) p2[s] += __shfl_xor_sync(0xffffffffu, p2[s], o);
-        }
+        for (int s = 0; s < kS; ++s)
+          if (kS == 1 || s < S) {
+            p[s] += __shfl_xor_sync(0xffffffffu, p[s], o);
+            if (kGate == LIF_GATE_BUNDLED) p2[s] += __shfl_xor_sync(0xffffffffu, p2[s], o);
+          }
       if (lane == 0) {
 #pragma unroll
         for (int s = 0; s < kS; ++s)
@@ -671,19 +673,142 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
   if (tid == 0) arrive(&a.sync->groups_done);
 }
 
+// ---- the sum: CTA `index` of `n` adds up a slice of the columns, in pairs, in a fixed order ----------
+// `width` pairs are side by side; the other threads share the partials: those of the cached rows, then
+// those of the fetch CTAs.
+template <int kS>
+struct Summer {
+  static constexpr int kDepth = Shape<kS>::kDepth;
+  const StepArgs& a;
+  const unsigned tag;
+  const int pairs, have_hit, have;
+  int c0, c1, width, slices, slice, t_next, lost;
+  float2 v_sum;
+
+  __device__ __forceinline__ Summer(const StepArgs& args, int index, int n, int n_hit, int n_new)
+      : a(args), tag(args.epoch + 1), pairs(args.n_streams * (args.d >> 1)),
+        have_hit((min(n_hit, args.n_cache_ctas) + args.group_size - 1) / args.group_size),
+        have(have_hit + n_new), lost(0), v_sum(make_float2(0.f, 0.f)) {
+    const int per = (pairs + n - 1) / n;
+    c0 = index * per;
+    c1 = min(pairs, c0 + per);
+    width = 32;
+    while (width < per && width < kStepThreads / 2) width *= 2;
+    slices = kStepThreads / width;
+    slice = threadIdx.x / width;
+    t_next = slice;
+  }
+  // (past the end: the last one again)
+  __device__ __forceinline__ const uint4* at(int t, int end, int col) const {
+    t = min(t, end - 1);
+    return (t < have_hit ? a.p_hit + (size_t)t * pairs : a.p_new + (size_t)(t - have_hit) * pairs) + col;
+  }
+  // adds the thread's partials of column pair `col` up to number `end`; stops where they are not there
+  // after `limit` polls
+  __device__ __forceinline__ void add(int end, int col, unsigned limit) {
+    if (col >= c1) return;
+    for (; t_next < end; t_next += slices * kDepth) {
+      ulonglong2 v[kDepth];
+#pragma unroll
+      for (int k = 0; k < kDepth; ++k) v[k] = load_tagged(at(t_next + k * slices, end, col));
+      bool there = false;
+      for (unsigned polls = 0; polls < limit; ++polls) {
+        there = true;
+#pragma unroll
+        for (int k = 0; k < kDepth; ++k) there = there && has_tag(v[k], tag);
+        if (there || polls + 1 == limit) break;
+#pragma unroll
+        for (int k = 0; k < kDepth; ++k)                   // again, those that were not there
+          if (!has_tag(v[k], tag)) v[k] = load_tagged(at(t_next + k * slices, end, col));
+      }
+      if (!there) {
+        lost = 1;
+        return;
+      }
+#pragma unroll
+      for (int k = 0; k < kDepth; ++k)
+        if (t_next + k * slices < end) {
+          v_sum.x += __uint_as_float((unsigned)v[k].x);
+          v_sum.y += __uint_as_float((unsigned)v[k].y);
+        }
+    }
+    lost = 0;
+    t_next = end <= slice ? slice : slice + (end - slice + slices - 1) / slices * slices;
+  }
+  // red: kStepThreads values in shared memory
+  __device__ __forceinline__ void finish(float2* red) {
+    const int tid = threadIdx.x, nvec = a.d >> 3;
+    for (int cc = c0; cc < c1; cc += width) {
+      const int col = cc + tid % width;
+      if (cc > c0) {
+        v_sum = make_float2(0.f, 0.f);
+        t_next = slice;
+        __syncthreads();                                   // red[] is free again
+      }
+      add(have, col, kStepSpinLimit);
+      if (lost) set_status(a, LIF_ERR_TIMEOUT);
+      red[tid] = v_sum;
+      __syncthreads();
+      if (tid < width && col < c1) {
+        const int s = kS == 1 ? 0 : col / (4 * nvec), r = kS == 1 ? col : col % (4 * nvec);
+        const int to = 4 * (r % nvec) + r / nvec;          // columns 2 * to, 2 * to + 1
+        float2 y = make_float2(0.f, 0.f);
+        if (a.b_down) y = __half22float2(*reinterpret_cast<const __half2*>(a.b_down + 2 * to));
+        for (int k = 0; k < slices; ++k) {
+          y.x += red[k * width + tid].x;
+          y.y += red[k * width + tid].y;
+        }
+        reinterpret_cast<float2*>(a.y + (size_t)s * a.d)[to] = y;
+      }
+    }
+  }
+};
+
+constexpr size_t kSumSmem = kStepThreads * sizeof(float2);
+
+// ---- sum CTAs (several streams) ------------------------------------------------------------------
+// The outputs of several streams are too long for the fetch CTAs to add up at the end (measured at
+// 5 x 4096: 6.5 us).  These CTAs wait for one word of each fetch CTA's partial, with pauses, so that
+// they do not load the memory system meanwhile, and then read everything at once.
+template <int kS>
+__device__ void sum_role(const StepArgs& a, int index, unsigned char* smem) {
+  __shared__ unsigned long long plan_s;
+  const int tid = threadIdx.x;
+  uint32_t mw[kEntriesPerThread];
+  unsigned n[1] = {0u}, tot[1];
+  __shared__ unsigned sums[1][kStepWarps];
+  read_entries(a.new_entries, a.n_entries, __ldcg(a.predictor_run), mw);
+#pragma unroll
+  for (int i = 0; i < kEntriesPerThread; ++i) n[0] += __popc(mw[i]);
+  step_scan<1>(n, tot, sums);
+  pdl_wait();
+  const unsigned long long plan = wait_plan(a, &plan_s);
+  const bool go = (plan & kPlanReady) && !(plan & kPlanRefused);
+  Summer<kS> sum(a, index, a.n_sum_ctas, (int)(plan & 0xfffff), go ? min(kFetchCtas, (int)tot[0]) : 0);
+  const size_t pairs = (size_t)a.n_streams * (a.d >> 1);
+  if (tid < sum.have - sum.have_hit) {
+    bool there = false;
+    for (unsigned polls = 0; !there && polls < kStepSpinLimit; ++polls) {
+      there = has_tag(load_tagged(a.p_new + (tid + 1) * pairs - 1), sum.tag);
+      if (!there) __nanosleep(100);
+    }
+  }
+  __syncthreads();
+  sum.finish(reinterpret_cast<float2*>(smem));             // kSumSmem bytes
+}
+
 // ---- fetch CTAs: new bundles over the host link, their FFN terms, and the sum -----------------------
 // Fetch CTA f brings in entries f, f + kFetchCtas, ... of the load list, which is exactly the set
 // bits of the predictor's entries in ascending order; only the cache row comes from the plan.
 template <int kGate, int kS>
 __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   constexpr int kVec = kGate == LIF_GATE_BUNDLED ? 3 : 2;
-  constexpr int kDepth = Shape<kS>::kDepth;
   __shared__ __align__(8) uint64_t bars[16];
   __shared__ unsigned sums[1][kStepWarps];
   __shared__ float part[2][kS][kStepWarps];
   __shared__ float h_s[kS];
   __shared__ unsigned long long plan_s;
-  __shared__ float2 red[kStepThreads];
+  __shared__ float2 red[kS == 1 ? kStepThreads : 1];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int d = a.d, S = a.n_streams, nvec = d >> 3, stages = a.fetch_stages;
   constexpr int nf = kFetchCtas;
@@ -745,55 +870,15 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     }
   }
   __syncthreads();
-  // The end of the step: every fetch CTA adds up a slice of the columns, in pairs, `width` of them
-  // side by side; the other threads share the partials.  Order: partials of the cached rows (with
-  // one block of columns read while the last row is on its way), then those of the fetch CTAs.
+  // One stream: the fetch CTAs also add up all partial sums (the cached rows' while the last row is on
+  // its way).  Several: that is for the sum CTAs.
   const unsigned tag = a.epoch + 1;
-  const int pairs = S * (d >> 1), per = (pairs + nf - 1) / nf;
-  const int c0 = f * per, c1 = min(pairs, c0 + per);
-  int width = 32;
-  while (width < per && width < kStepThreads / 2) width *= 2;
-  const int slices = kStepThreads / width;
-  const int slice = tid / width;
-  const int have_hit = (min(n_hit, a.n_cache_ctas) + a.group_size - 1) / a.group_size;
-  const int have_new = go ? min(nf, n_new) : 0;
-  float2 sum = make_float2(0.f, 0.f);
-  int lost_sum = 0;
-  // adds the thread's partials of column pair `col` from number t0 on; stops where they are not there
-  // after `limit` polls
-  auto add_partials = [&](const uint4* partials, int have, int col, int t0, unsigned limit) {
-    if (col >= c1) return have;
-    for (; t0 < have; t0 += slices * kDepth) {
-      ulonglong2 v[kDepth];
-#pragma unroll
-      for (int k = 0; k < kDepth; ++k)                     // (past the end: the last one again)
-        v[k] = load_tagged(partials + (size_t)min(t0 + k * slices, have - 1) * pairs + col);
-      bool there = false;
-      for (unsigned polls = 0; polls < limit; ++polls) {
-        there = true;
-#pragma unroll
-        for (int k = 0; k < kDepth; ++k) there = there && has_tag(v[k], tag);
-        if (there || polls + 1 == limit) break;
-#pragma unroll
-        for (int k = 0; k < kDepth; ++k)                   // again, those that were not there
-          if (!has_tag(v[k], tag))
-            v[k] = load_tagged(partials + (size_t)min(t0 + k * slices, have - 1) * pairs + col);
-      }
-      if (!there) return t0;
-#pragma unroll
-      for (int k = 0; k < kDepth; ++k)
-        if (t0 + k * slices < have) {
-          sum.x += __uint_as_float((unsigned)v[k].x);
-          sum.y += __uint_as_float((unsigned)v[k].y);
-        }
-    }
-    return have;
-  };
-  int t_hit = slice;
+  const size_t pairs = (size_t)S * (d >> 1);
+  Summer<kS> sum(a, f, nf, n_hit, go ? min(nf, n_new) : 0);
 
   unsigned parity = 0;
   for (int i = 0, st = 0; i < cnt; ++i) {
-    if (kS == 1 && i == cnt - 1) t_hit = add_partials(a.p_hit, have_hit, c0 + tid % width, t_hit, 1);
+    if (kS == 1 && i == cnt - 1) sum.add(sum.have_hit, sum.c0 + tid % sum.width, 1);
     const uint4* row = reinterpret_cast<const uint4*>(ring + (size_t)st * row_bytes);
     const bool landed = mbar_wait(bars + st, parity, a.wait_polls);
     if (!landed) {                                         // flagged; its term is left out
@@ -821,10 +906,11 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-      for (int s = 0; s < kS; ++s) {
-        p[s] += __shfl_xor_sync(0xffffffffu, p[s], o);
-        if (kGate == LIF_GATE_BUNDLED) p2[s] += __shfl_xor_sync(0xffffffffu, p2[s], o);
-      }
+      for (int s = 0; s < kS; ++s)
+        if (kS == 1 || s < S) {
+          p[s] += __shfl_xor_sync(0xffffffffu, p[s], o);
+          if (kGate == LIF_GATE_BUNDLED) p2[s] += __shfl_xor_sync(0xffffffffu, p2[s], o);
+        }
     if (lane == 0) {
 #pragma unroll
       for (int s = 0; s < kS; ++s) {
@@ -868,30 +954,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     }
   }
   if (cnt > 0) store_tagged_partial<kS>(acc, a.p_new + (size_t)f * pairs, nvec, S, tag);
-  for (int cc = c0; cc < c1; cc += width) {
-    const int col = cc + tid % width;
-    if (cc > c0) {
-      sum = make_float2(0.f, 0.f);
-      t_hit = slice;
-      __syncthreads();                                     // red[] is free again
-    }
-    if (add_partials(a.p_hit, have_hit, col, t_hit, kStepSpinLimit) < have_hit) lost_sum = 1;
-    if (add_partials(a.p_new, have_new, col, slice, kStepSpinLimit) < have_new) lost_sum = 1;
-    red[tid] = sum;
-    __syncthreads();
-    if (tid < width && col < c1) {
-      const int s = kS == 1 ? 0 : col / (4 * nvec), r = kS == 1 ? col : col % (4 * nvec);
-      const int at = 4 * (r % nvec) + r / nvec;            // columns 2 * at, 2 * at + 1
-      float2 y = make_float2(0.f, 0.f);
-      if (a.b_down) y = __half22float2(*reinterpret_cast<const __half2*>(a.b_down + 2 * at));
-      for (int k = 0; k < slices; ++k) {
-        y.x += red[k * width + tid].x;
-        y.y += red[k * width + tid].y;
-      }
-      reinterpret_cast<float2*>(a.y + (size_t)s * d)[at] = y;
-    }
-  }
-  if (lost_sum) set_status(a, LIF_ERR_TIMEOUT);
+  if (kS == 1) sum.finish(red);
   if (tid == 0) {
     if (f == 0) advance_run(a.next_run, run);
     // (shared memory must outlive the reads of the last rows' copies to the cache)
@@ -914,7 +977,8 @@ __global__ void __launch_bounds__(kStepThreads, kS == 1 ? 2 : 1) step_kernel(Ste
   a.epoch = epoch_s;
   if (part == 0) window_role(a, smem);
   else if (part <= a.n_cache_ctas) cache_role<kGate, kS>(a, part - 1, smem);
-  else fetch_role<kGate, kS>(a, part - 1 - a.n_cache_ctas, smem);
+  else if (part <= a.n_cache_ctas + kFetchCtas) fetch_role<kGate, kS>(a, part - 1 - a.n_cache_ctas, smem);
+  else if (kS > 1) sum_role<kS>(a, part - 1 - a.n_cache_ctas - kFetchCtas, smem);
 }
 
 using StepKernel = void (*)(StepArgs);
@@ -940,6 +1004,11 @@ int cache_ctas(const lif_layer_desc& D, int n_sm) {
   const int per = D.n_streams > 1 ? 16 : 8, most = D.n_streams > 1 ? 64 : n_sm - 1 - kFetchCtas;
   const int nc = (D.capacity + per - 1) / per;
   return nc < 8 ? 8 : (nc > most ? most : nc);
+}
+// CTAs that add up the outputs of several streams: 128 pairs of columns each.
+int sum_ctas(const lif_layer_desc& D) {
+  const int n = (D.n_streams * D.d_model / 2 + 127) / 128;
+  return n > 48 ? 48 : n;
 }
 // Tagged partials of cache CTAs (or of groups of them) that the fetch CTAs add up at the end.
 int hit_partials_max(const lif_layer_desc& D) {
@@ -980,6 +1049,7 @@ cudaError_t step_configure(lif_layer* L) {
     return s < least ? least : (s > 16 ? 16 : s);
   };
   L->step_cache_ctas = cache_ctas(D, L->n_sm);
+  L->step_sum_ctas = D.n_streams > 1 ? sum_ctas(D) : 0;
   L->step_group = L->step_cache_ctas > hit_partials_max(D) ? kGroupMax : 1;
   L->step_cache_stages = stages(kCacheRing, x, 1);
   // in the paper's cache order the bundles wait in the ring until the cache CTAs have read the rows
@@ -989,6 +1059,7 @@ cudaError_t step_configure(lif_layer* L) {
   const size_t need_c = x + L->step_cache_stages * row, need_f = x + L->step_fetch_stages * row + ids;
   if (need_c > smem) smem = need_c;
   if (need_f > smem) smem = need_f;
+  if (D.n_streams > 1 && smem < kSumSmem) smem = kSumSmem;
   if (smem > (size_t)max_smem) return cudaSuccess;
   L->step_smem = smem;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
@@ -1024,12 +1095,13 @@ cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st
   a.act = D.activation;
   a.act_thr = D.activation_threshold;
   a.n_cache_ctas = L->step_cache_ctas;
+  a.n_sum_ctas = L->step_sum_ctas;
   a.group_size = L->step_group;
   a.cache_stages = L->step_cache_stages;
   a.fetch_stages = L->step_fetch_stages;
   a.fetch_rows_max = (D.d_ff + kFetchCtas - 1) / kFetchCtas;
   a.wait_polls = L->wait_polls;
-  return launch_k(step_kernel_for(D), dim3(1 + a.n_cache_ctas + kFetchCtas),
+  return launch_k(step_kernel_for(D), dim3(1 + a.n_cache_ctas + kFetchCtas + a.n_sum_ctas),
                   dim3(kStepThreads), L->step_smem, st, L->use_pdl, a);
 }
 
