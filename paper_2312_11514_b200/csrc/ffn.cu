@@ -144,16 +144,9 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_ffn_kernel(FfnArgs a) {
       float p = 0.f, p2 = 0.f;
 #pragma unroll 4
       for (int c = lane; c < nvec; c += 32) {
-        float uf[8], xf[8];
-        unpack8(up[c], uf);
-        unpack8(reinterpret_cast<const uint4*>(xs)[c], xf);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) p = fmaf(uf[e], xf[e], p);
-        if (kGate == LIF_GATE_BUNDLED) {       // first vector = gate row, second = up row
-          unpack8(up[nvec + c], uf);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) p2 = fmaf(uf[e], xf[e], p2);
-        }
+        const uint4 xv = reinterpret_cast<const uint4*>(xs)[c];
+        p = dot8(up[c], xv, p);
+        if (kGate == LIF_GATE_BUNDLED) p2 = dot8(up[nvec + c], xv, p2);   // gate row, then up row
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);

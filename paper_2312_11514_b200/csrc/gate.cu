@@ -73,17 +73,11 @@ gate_scores_kernel(const __half* __restrict__ x, const __half* __restrict__ gate
     for (int j = 0; j < kDepth; ++j) {
       const int c = lane + 32 * (g0 + j);
       if (c < nvec) {
-        float wf[kRowsPerWarp][8];
-#pragma unroll
-        for (int q = 0; q < kRowsPerWarp; ++q) unpack8(w[j][q], wf[q]);
 #pragma unroll
         for (int s = 0; s < S; ++s) {
-          float xf[8];
-          unpack8(xs[s * nvec + c], xf);
+          const uint4 xv = xs[s * nvec + c];
 #pragma unroll
-          for (int q = 0; q < kRowsPerWarp; ++q)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[q][s] = fmaf(wf[q][e], xf[e], acc[q][s]);
+          for (int q = 0; q < kRowsPerWarp; ++q) acc[q][s] = dot8(w[j][q], xv, acc[q][s]);
         }
       }
       load_group(w[j], g0 + j + kDepth);     // past the end of the row: no load, zeros

@@ -37,15 +37,14 @@ __device__ __forceinline__ void compact_mask_last_cta(const uint32_t* mask_words
                                                       int* __restrict__ n_active, int* warp_sums,
                                                       int* is_last) {
   const int tid = threadIdx.x;
-  __threadfence();
   __syncthreads();
-  if (tid == 0) {
-    const int t = atomicAdd(ticket, 1);
+  if (tid == 0) {     // releases the CTA's words, acquires the others' (one fence, not one per thread)
+    int t;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(t) : "l"(ticket) : "memory");
     *is_last = (t == (int)gridDim.x - 1);
   }
   __syncthreads();
   if (!*is_last) return;
-  __threadfence();
 
   const int wpt = (nwords + kThreads - 1) / kThreads;
   const int w0 = min(nwords, tid * wpt), w1 = min(nwords, w0 + wpt);

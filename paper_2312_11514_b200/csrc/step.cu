@@ -465,16 +465,9 @@ __device__ __forceinline__ void axpy_row(Acc<kS>& acc, const uint4* down, const 
 template <int kS>
 __device__ __forceinline__ void dot_chunk(float (&p)[kS], const uint4& row, const uint4* xs, int v,
                                           int nvec, int S) {
-  float rf[8];
-  unpack8(row, rf);
 #pragma unroll
   for (int s = 0; s < kS; ++s)
-    if (kS == 1 || s < S) {
-      float xf[8];
-      unpack8(xs[s * nvec + v], xf);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) p[s] = fmaf(rf[e], xf[e], p[s]);
-    }
+    if (kS == 1 || s < S) p[s] = dot8(row, xs[s * nvec + v], p[s]);
 }
 // A partial sum for the end of the step: every pair of values is stored as {v, tag, v, tag}, two
 // 8-byte words that are each written whole, with a tag of this step (step number + 1).  The reader
@@ -861,14 +854,16 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   } else {
     for (int i = tid; i < cnt; i += kStepThreads)
       dst_rows[i] = (unsigned short)__ldcg(a.w.load_slots + f + i * nf);
-    // in the paper's order the new rows' places may be rows the cache CTAs still read
-    if (!a.w.append_first && tid == 0) {
-      const unsigned want = (a.epoch + 1) * (unsigned)n_groups;
-      unsigned i = 0;
-      while ((int)(ld_acquire(&a.sync->groups_done) - want) < 0 && i < kStepSpinLimit) ++i;
-      if (i == kStepSpinLimit) set_status(a, LIF_ERR_TIMEOUT);
-    }
   }
+  // In the paper's order the new rows' places may be rows that the cache CTAs still read: the first
+  // ringful of bundles stays in the ring until they are done, its FFN terms are computed meanwhile.
+  const int held = a.w.append_first ? 0 : min(cnt, stages);
+  auto store_row = [&](int i, int st) {                    // thread 0
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                     a.cache + (size_t)dst_rows[i] * row_bytes),
+                 "r"(smem_u32(ring + (size_t)st * row_bytes)), "r"(row_bytes) : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+  };
   __syncthreads();
   // One stream: the fetch CTAs also add up all partial sums (the cached rows' while the last row is on
   // its way).  Several: that is for the sum CTAs.
@@ -885,12 +880,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       if (tid == 0) set_status(a, LIF_ERR_TIMEOUT);
       mbar_wait(bars + st, parity);
     }
-    if (tid == 0) {
-      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
-                       a.cache + (size_t)dst_rows[i] * row_bytes), "r"(smem_u32(row)), "r"(row_bytes)
-                   : "memory");
-      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-    }
+    if (tid == 0 && i >= held) store_row(i, st);
     const float b = row_scalar<kGate>(a, ids[i]);
     float p[kS], p2[kS];
 #pragma unroll
@@ -943,10 +933,18 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       axpy_row<kS>(acc, down, h_s, nvec);
     }
     __syncthreads();                                       // the stage, part[] and h_s[] are free
-    if (tid == 0 && i + stages < cnt) {
+    if (tid == 0 && i == held - 1) {
+      const unsigned want = (a.epoch + 1) * (unsigned)n_groups;
+      unsigned n = 0;
+      while ((int)(ld_acquire(&a.sync->groups_done) - want) < 0 && n < kStepSpinLimit) ++n;
+      if (n == kStepSpinLimit) set_status(a, LIF_ERR_TIMEOUT);
+      for (int j = 0; j < held; ++j) store_row(j, j);
+    }
+    const int again = i == held - 1 ? 0 : i;               // rows again .. i may be replaced
+    if (tid == 0 && i >= held - 1 && again + stages < cnt) {
       asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      issue(ids[i + stages], st);
+      for (int j = again; j <= i && j + stages < cnt; ++j) issue(ids[j + stages], j % stages);
     }
     if (++st == stages) {
       st = 0;
