@@ -186,7 +186,8 @@ lif_status lif_create_layer(const lif_layer_desc* desc, lif_layer** out) {
     L->split_ffn = 1;
     L->fused_plan = window_plan_supported(*desc) ? 1 : 0;
     L->fused_fetch = 1;
-    ok = step_configure(L) == cudaSuccess && predict_configure(L) == cudaSuccess;
+    ok = step_configure(L) == cudaSuccess && predict_configure(L) == cudaSuccess &&
+         fetch_configure(L) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&L->ev_plan, cudaEventDisableTiming) == cudaSuccess;
     if (ok && cudaEventCreateWithFlags(&L->ev_fetch, cudaEventDisableTiming) != cudaSuccess) {
       cudaEventDestroy(L->ev_plan);
@@ -345,8 +346,7 @@ lif_status lif_decode_step(lif_layer* L, const void* dev_x, float* dev_y, void* 
   // Otherwise the plain fetch takes that place on the compute stream, and the second stream, if
   // there is one, carries the row moves.
   const bool split = L->split_ffn && L->desc.n_streams == 1;
-  // (in speculative mode the load list is a subset of the predictor's mask: no early start)
-  L->watch_chain = L->use_pdl && fetch_ffn_can_watch(L) && L->desc.spec_keep == 0 &&
+  L->watch_chain = L->use_pdl && fetch_ffn_can_watch(L) &&
                    (split ? sf != sc : L->early_fetch != 0);
   if (L->fused_plan) {
     ok = launch_predict(L, x, nullptr, L->active_idx, L->n_tmp, sc, ev, 0) == cudaSuccess;
@@ -371,7 +371,7 @@ lif_status lif_decode_step(lif_layer* L, const void* dev_x, float* dev_y, void* 
       ok = ok && cudaEventRecord(L->ev_fetch, sf) == cudaSuccess;
     }
     if (ev) tm_record(ev[5], sc);
-    ok = ok && launch_fetch_early(L, sc, kEarlyWatch) == cudaSuccess;
+    ok = ok && launch_fetch_early(L, sc) == cudaSuccess;
     if (ev) tm_record(ev[6], sc);
     if (moves_aside) ok = ok && cudaStreamWaitEvent(sc, L->ev_fetch, 0) == cudaSuccess;
     L->ends_step = 1;

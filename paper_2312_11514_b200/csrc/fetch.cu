@@ -1,8 +1,6 @@
 // Bringing in new neurons (Section 3.3 item 2): gather the bundles of the newly needed
 // neurons from the full store in mapped pinned host memory (standing in for flash) into
-// their cache rows.  The kernel reads host memory directly: every warp instruction reads 512
-// contiguous bytes of one bundle with 16-byte loads, and each thread keeps several loads in
-// flight so the link sees enough outstanding requests.  Bound: host-link bandwidth.
+// their cache rows.  The kernels read host memory directly.  Bound: host-link bandwidth.
 #include "lif_internal.cuh"
 #include "mask_compact.cuh"
 
@@ -40,15 +38,6 @@ __device__ __forceinline__ void gather_rows(const uint4* __restrict__ src_base,
       if (v < row_vec) dst[v] = buf[i];
     }
   }
-}
-
-__global__ void __launch_bounds__(kThreads)
-fetch_kernel(const uint4* __restrict__ store, uint4* __restrict__ cache,
-             const int32_t* __restrict__ load_ids, const int32_t* __restrict__ load_slots,
-             const int32_t* __restrict__ counts, int row_vec) {
-  pdl_wait();
-  pdl_trigger();
-  gather_rows(store, cache, load_ids, load_slots, counts[LIF_CNT_N_LOAD], row_vec);
 }
 
 // Fetch and FFN of the new rows in one kernel (single stream, row = up | down of at most
@@ -109,46 +98,54 @@ constexpr int kWatchPolls = 64;     // about 30 us of polling at most
 struct EarlyPick {
   int mode, n, id;
 };
+// Thread t owns a run of consecutive entries, which begins here (at most four of them: nwords <= 1024
+// in the forms that read entries).
+__device__ __forceinline__ int entries_begin(const EarlySource& src) {
+  return min(src.nwords, (int)threadIdx.x * ((src.nwords + kThreads - 1) / kThreads));
+}
+__device__ __forceinline__ bool read_entries(const EarlySource& src, int want_tag, bool check,
+                                             uint32_t (&mw)[4]) {
+  const int w0 = entries_begin(src);
+  const int w1 = min(src.nwords, w0 + (src.nwords + kThreads - 1) / kThreads);
+  bool all_mine = true;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    mw[i] = 0u;
+    if (w0 + i < w1) {
+      unsigned long long v;
+      asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(src.entries + w0 + i) : "memory");
+      mw[i] = (uint32_t)v;
+      all_mine = all_mine && (!check || (int)(v >> 32) == want_tag);
+    }
+  }
+  return all_mine;
+}
+// Resident while the predictor may still be running (all of its CTAs are: it released the window
+// kernel, which released this one, only after every one of them had started).  Every entry is
+// stored together with the number of the predictor run that wrote it (one 8-byte store), and that
+// number was fixed before the run began, so each thread simply re-reads its own entries until all of
+// them carry it: one read tells both that they are there and what they hold.  Bounded; if they do
+// not come the kernel waits for its predecessors, and whatever it read is checked against the window
+// kernel's list after the wait, so no result depends on this phase.
+__device__ __forceinline__ bool watch_entries(const EarlySource& src, uint32_t (&mw)[4]) {
+  const int run = __ldcg(src.predictor_run);
+  int ok = 0;
+  for (int i = 0; i < kWatchPolls && !ok; ++i)
+    ok = __syncthreads_and(read_entries(src, run, true, mw) ? 1 : 0);
+  return ok != 0;
+}
 template <int kEarlyT>
 __device__ __forceinline__ EarlyPick early_pick(const EarlySource& src, int want, int* scan_sums,
                                                 int* first_id) {
   const int tid = threadIdx.x;
   int kEarly = kEarlyT;
-  // thread t owns a run of consecutive words of the mask of neurons to bring in
-  const int wpt = (src.nwords + kThreads - 1) / kThreads;
-  const int w0 = min(src.nwords, tid * wpt), w1 = min(src.nwords, w0 + wpt);
-  uint32_t mw[4] = {0u, 0u, 0u, 0u};               // nwords <= 1024 in the mask-driven forms
-  auto read_words = [&](int want_tag, bool check) {
-    bool all_mine = true;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      mw[i] = 0u;
-      if (w0 + i < w1) {
-        unsigned long long v;
-        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(src.entries + w0 + i)
-                     : "memory");
-        mw[i] = (uint32_t)v;
-        all_mine = all_mine && (!check || (int)(v >> 32) == want_tag);
-      }
-    }
-    return all_mine;
-  };
+  uint32_t mw[4] = {0u, 0u, 0u, 0u};
   if (kEarlyT == kEarlyWatch) {
-    // Resident while the predictor may still be running (all of its CTAs are: it released the
-    // window kernel, which released this one, only after every one of them had started).  Every
-    // mask word is stored together with the number of the predictor run that wrote it (one
-    // 8-byte store), and that number was fixed before the run began, so each thread simply
-    // re-reads its own words until all of them carry it: one read tells both that the words are
-    // there and what they hold.  Bounded; if the words do not come the kernel waits for its
-    // predecessors like kEarlyNone, and whatever it read is checked against the window kernel's
-    // list after the wait, so no result depends on this phase.
-    const int run = __ldcg(src.predictor_run);
-    int ok = 0;
-    for (int i = 0; i < kWatchPolls && !ok; ++i) ok = __syncthreads_and(read_words(run, true) ? 1 : 0);
-    kEarly = ok ? kEarlyMask : kEarlyNone;
+    kEarly = watch_entries(src, mw) ? kEarlyMask : kEarlyNone;
   } else if (kEarlyT == kEarlyMask) {
-    read_words(0, false);                          // final before the kernel ahead passed its wait
+    read_entries(src, 0, false, mw);               // final before the kernel ahead passed its wait
   }
+  const int w0 = entries_begin(src);
   if (kEarly == kEarlyNone) {
     pdl_wait();
     pdl_trigger();
@@ -308,74 +305,119 @@ __global__ void __launch_bounds__(kThreads) fetch_ffn_kernel(FetchFfnArgs a) {
   }
 }
 
-// The plain fetch with the same early start as fetch_ffn_kernel (used where that kernel does not
-// apply: several input streams, three-vector bundles).  CTA c's first unit is slice c % slices
-// of row c / slices of the load list; its host loads are issued ahead of the dependency wait
-// and held in registers until the window kernel's list says where the row goes.  The units
-// after the first come from the list.
+// The fetch as a kernel of its own: a few CTAs bring bundles through a ring of bulk copies in shared
+// memory, host memory -> stage -> cache row, without a register on the way.  CTA c brings in entries
+// c, c + G, ... of the load list.
+//   kEarlyNone   everything from the window kernel's lists, behind the dependency wait
+//   kEarlyWatch  the window kernel is ahead and the predictor may still be running: the ids come
+//                from the predictor's entries (the load list is exactly their set bits in ascending
+//                order), and the first bundles travel while the window kernel runs; behind the wait
+//                the count is compared with the list (0 when the step was refused) and the rows come
+//                from it.
+// Few CTAs: about 200 KB of host reads in flight fill the link (16 CTAs reach the 51 GB/s that 148
+// reach), and the rest of the chip keeps its latency and bandwidth: with host loads on all SMs the
+// window kernel behind the predictor of 8 streams took 52-69 us (39 now), and an FFN beside the fetch
+// did not pay.  `window` copies are in flight per CTA, 24 KB at least; two more stages hold rows that
+// are being stored.
+constexpr int kRingCtas = 16;
+constexpr size_t kRingWindow = 24 * 1024;
+constexpr int kRingList = 1024;      // ids and rows kept in shared memory at a time
+
+struct RingArgs {
+  const unsigned char* store;
+  unsigned char* cache;
+  const int32_t* load_ids;           // nullptr: bundle j of the store is entry j of the list
+  const int32_t* load_slots;
+  int32_t* counts;
+  unsigned row_bytes;
+  int stages, window;
+  EarlySource early;
+};
+
 template <int kEarlyT>
-__global__ void __launch_bounds__(kThreads)
-fetch_early_kernel(const uint4* __restrict__ store, uint4* __restrict__ cache,
-                   const int32_t* __restrict__ load_ids, const int32_t* __restrict__ load_slots,
-                   int row_vec, EarlySource early) {
+__global__ void __launch_bounds__(kThreads) fetch_ring_kernel(RingArgs a) {
+  extern __shared__ __align__(128) unsigned char ring[];
+  __shared__ __align__(8) uint64_t bars[16];
   __shared__ int scan_sums[kThreads / 32];
-  __shared__ int first_id;
-  constexpr int kSlice = kThreads * kFetchUnroll;
-  const int slices = (row_vec + kSlice - 1) / kSlice;
-  const int j0 = blockIdx.x / slices;
-  const int v0 = (blockIdx.x % slices) * kSlice + threadIdx.x;
-  const EarlyPick pk = early_pick<kEarlyT>(early, j0, scan_sums, &first_id);
-  uint4 buf[kFetchUnroll];
-  auto host_loads = [&](int id) {
-    const uint4* src = store + (size_t)id * row_vec;
-#pragma unroll
-    for (int i = 0; i < kFetchUnroll; ++i) {
-      const int v = v0 + i * kThreads;
-      if (v < row_vec) buf[i] = ld_stream16(src + v);
-    }
+  int32_t* ids = reinterpret_cast<int32_t*>(ring + (size_t)a.stages * a.row_bytes);
+  int32_t* rows = ids + kRingList;
+  const int tid = threadIdx.x, c = blockIdx.x, G = gridDim.x;
+  if (tid == 0) {
+    for (int i = 0; i < a.stages; ++i) mbar_init(bars + i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  auto issue = [&](int id, int k) {                  // copy number k of this CTA
+    uint64_t* bar = bars + k % a.stages;
+    mbar_expect_tx(bar, a.row_bytes);
+    bulk_g2s(ring + (size_t)(k % a.stages) * a.row_bytes, a.store + (size_t)id * a.row_bytes, a.row_bytes, bar);
   };
-  int n = pk.n, id = -1;
-  const bool mine = j0 < n;
-  if (mine) {
-    id = pk.mode == kEarlyMask ? pk.id : __ldcg(load_ids + j0);
-    host_loads(id);
-  }
-  if (pk.mode != kEarlyNone) {
-    pdl_wait();
-    pdl_trigger();
-  }
-  if (pk.mode == kEarlyMask) {
-    // the window kernel's list is the reference (see fetch_ffn_kernel)
-    const int n_plan = __ldcg(early.counts + LIF_CNT_N_LOAD);
-    const bool stale = n_plan != n || (mine && __ldcg(load_ids + j0) != id);
-    n = n_plan;
-    if (j0 < n && stale) host_loads(__ldcg(load_ids + j0));
-  }
-  if (j0 < n) {
-    uint4* dst = cache + (size_t)load_slots[j0] * row_vec;
+  auto landed = [&](int k) {                         // thread 0
+    if (mbar_wait(bars + k % a.stages, (unsigned)(k / a.stages) & 1u)) return;
+    atomicCAS(a.counts + LIF_CNT_STATUS, LIF_OK, LIF_ERR_TIMEOUT);
+  };
+  int known = 0, n_early = 0;                        // entries of this CTA found early; of all CTAs
+  if (kEarlyT == kEarlyWatch) {
+    uint32_t mw[4];
+    if (watch_entries(a.early, mw)) {                // also orders the barriers' initialisation
+      int cnt = 0;
 #pragma unroll
-    for (int i = 0; i < kFetchUnroll; ++i) {
-      const int v = v0 + i * kThreads;
-      if (v < row_vec) dst[v] = buf[i];
+      for (int i = 0; i < 4; ++i) cnt += __popc(mw[i]);
+      int q = block_exclusive_scan_256(cnt, &n_early, scan_sums);
+      const int w0 = entries_begin(a.early);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        for (uint32_t m = mw[i]; m; m &= m - 1, ++q)
+          if (q % G == c && q / G < kRingList) {
+            const int id = (w0 + i) * a.early.word_bits + __ffs(m) - 1;
+            ids[q / G] = id;
+            if (q / G < a.window) issue(id, q / G);
+          }
+      known = n_early > c ? min(kRingList, (n_early - c + G - 1) / G) : 0;
+    }
+  } else {
+    __syncthreads();
+  }
+  pdl_wait();
+  pdl_trigger();
+  int issued = min(known, a.window), used = 0;       // copies so far: asked for, done with
+  const int n = __ldcg(a.counts + LIF_CNT_N_LOAD);
+  if (known && n != n_early) {                       // not this step's: let them land, start over
+    if (tid == 0)
+      for (; used < issued; ++used) landed(used);
+    used = issued;
+    known = 0;
+  }
+  const int mine = n > c ? (n - c + G - 1) / G : 0;
+  for (int i0 = 0; i0 < mine; i0 += kRingList) {
+    const int m = min(kRingList, mine - i0);
+    __syncthreads();
+    for (int i = tid; i < m; i += kThreads) {
+      const int j = c + (i0 + i) * G;
+      if (i0 || i >= known) ids[i] = a.load_ids ? __ldcg(a.load_ids + j) : j;
+      rows[i] = __ldcg(a.load_slots + j);
+    }
+    __syncthreads();
+    if (tid == 0) {
+      int asked = i0 == 0 && known ? issued : 0;     // entries of this batch already asked for
+      for (; asked < min(m, a.window); ++asked, ++issued) {
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        issue(ids[asked], issued);
+      }
+      for (int i = 0; i < m; ++i, ++used) {
+        landed(used);
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                         a.cache + (size_t)rows[i] * a.row_bytes),
+                     "r"(smem_u32(ring + (size_t)(used % a.stages) * a.row_bytes)), "r"(a.row_bytes) : "memory");
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        if (asked < m) {                             // its stage was stored two rows ago
+          asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+          issue(ids[asked++], issued++);
+        }
+      }
     }
   }
-  const long long units = (long long)n * slices;
-  for (long long u = (long long)blockIdx.x + gridDim.x; u < units; u += gridDim.x) {
-    const int j = (int)(u / slices);
-    const int w0 = (int)(u % slices) * kSlice + threadIdx.x;
-    const uint4* src = store + (size_t)load_ids[j] * row_vec;
-    uint4* dst = cache + (size_t)load_slots[j] * row_vec;
-#pragma unroll
-    for (int i = 0; i < kFetchUnroll; ++i) {
-      const int v = w0 + i * kThreads;
-      if (v < row_vec) buf[i] = ld_stream16(src + v);
-    }
-#pragma unroll
-    for (int i = 0; i < kFetchUnroll; ++i) {
-      const int v = w0 + i * kThreads;
-      if (v < row_vec) dst[v] = buf[i];
-    }
-  }
+  if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -500,13 +542,6 @@ cudaError_t launch_refill(lif_layer* L, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_fetch(lif_layer* L, cudaStream_t st) {
-  return launch_k(fetch_kernel, dim3(L->fetch_grid), dim3(kThreads), 0, st, L->use_pdl,
-                  (const uint4*)L->dev_bundles, (uint4*)L->desc.dev_cache,
-                  (const int32_t*)L->load_ids, (const int32_t*)L->load_slots,
-                  (const int32_t*)L->counts, row_elems(L->desc) / 8);
-}
-
 static EarlySource early_source(const lif_layer* L) {
   EarlySource e;
   e.entries = L->new_mask_words;
@@ -517,26 +552,49 @@ static EarlySource early_source(const lif_layer* L) {
   return e;
 }
 
-// The plain fetch behind the window kernel (or the row moves) on the same stream, started early
-// (`early` as for launch_fetch_ffn).
-cudaError_t launch_fetch_early(lif_layer* L, cudaStream_t st, int early) {
-  if (early >= kEarlyMask && !fetch_ffn_can_watch(L)) early = kEarlyNone;
-  if (early == kEarlyNone) return launch_fetch(L, st);
-  auto kernel = early == kEarlyWatch  ? fetch_early_kernel<kEarlyWatch>
-                : early == kEarlyMask ? fetch_early_kernel<kEarlyMask>
-                                      : fetch_early_kernel<kEarlyLists>;
-  return launch_k(kernel, dim3(L->fetch_grid), dim3(kThreads), 0, st, L->use_pdl,
-                  (const uint4*)L->dev_bundles, (uint4*)L->desc.dev_cache,
-                  (const int32_t*)L->load_ids, (const int32_t*)L->load_slots,
-                  row_elems(L->desc) / 8, early_source(L));
+int fetch_ring_ctas(const lif_layer* L) {
+  return L->fetch_grid == L->n_sm ? kRingCtas : L->fetch_grid;   // (unless the knob is set)
+}
+
+static cudaError_t launch_ring(lif_layer* L, const int32_t* ids, bool watch, cudaStream_t st) {
+  RingArgs a;
+  a.store = (const unsigned char*)L->dev_bundles;
+  a.cache = (unsigned char*)L->desc.dev_cache;
+  a.load_ids = ids;
+  a.load_slots = L->load_slots;
+  a.counts = L->counts;
+  a.row_bytes = 2u * row_elems(L->desc);
+  int window = (int)((kRingWindow + a.row_bytes - 1) / a.row_bytes);
+  a.window = window < 2 ? 2 : (window > 14 ? 14 : window);
+  a.stages = a.window + 2;
+  a.early = early_source(L);
+  return launch_k(watch ? fetch_ring_kernel<kEarlyWatch> : fetch_ring_kernel<kEarlyNone>,
+                  dim3(fetch_ring_ctas(L)), dim3(kThreads),
+                  (size_t)a.stages * a.row_bytes + 2 * kRingList * 4, st, L->use_pdl, a);
+}
+
+cudaError_t fetch_configure(const lif_layer* L) {
+  for (auto k : {fetch_ring_kernel<kEarlyWatch>, fetch_ring_kernel<kEarlyNone>}) {
+    cudaFuncAttributes at;
+    cudaError_t e = cudaFuncGetAttributes(&at, k);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               L->max_smem - (int)at.sharedSizeBytes);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_fetch(lif_layer* L, cudaStream_t st) { return launch_ring(L, L->load_ids, false, st); }
+
+// The fetch behind the window kernel (or the row moves) on the same stream, started early where the
+// predictor's entries can be watched.
+cudaError_t launch_fetch_early(lif_layer* L, cudaStream_t st) {
+  return launch_ring(L, L->load_ids, fetch_ffn_can_watch(L), st);
 }
 
 // File-backed store: staging row j (bundle load_ids[j], read by the host) -> cache row load_slots[j].
-cudaError_t launch_fetch_staged(lif_layer* L, cudaStream_t st) {
-  return launch_k(fetch_kernel, dim3(L->fetch_grid), dim3(kThreads), 0, st, L->use_pdl,
-                  (const uint4*)L->dev_bundles, (uint4*)L->desc.dev_cache, (const int32_t*)nullptr,
-                  (const int32_t*)L->load_slots, (const int32_t*)L->counts, row_elems(L->desc) / 8);
-}
+cudaError_t launch_fetch_staged(lif_layer* L, cudaStream_t st) { return launch_ring(L, nullptr, false, st); }
 
 bool fetch_ffn_supported(const lif_layer* L) {
   const lif_layer_desc& D = L->desc;

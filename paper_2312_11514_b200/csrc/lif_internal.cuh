@@ -149,9 +149,11 @@ cudaError_t launch_moves(lif_layer* L, cudaStream_t st, cudaEvent_t* ev = nullpt
                          bool release_early = false);
 cudaError_t launch_fetch(lif_layer* L, cudaStream_t st);
 cudaError_t launch_fetch_staged(lif_layer* L, cudaStream_t st);
-cudaError_t launch_fetch_early(lif_layer* L, cudaStream_t st, int early);
+cudaError_t launch_fetch_early(lif_layer* L, cudaStream_t st);
+cudaError_t fetch_configure(const lif_layer* L);
 bool fetch_ffn_supported(const lif_layer* L);
 bool fetch_ffn_can_watch(const lif_layer* L);
+int fetch_ring_ctas(const lif_layer* L);           // CTAs of the fetch as a kernel of its own
 int gate_predict_tile();                           // neurons per CTA of the resident-gate predictor
 // entries of new_mask_words and the neurons each one covers
 inline int new_mask_entry_bits(const lif_layer_desc& D) {
