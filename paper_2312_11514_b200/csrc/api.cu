@@ -39,7 +39,7 @@ Workspace plan_workspace(const lif_layer_desc& d, int ffn_grid_max) {
   w.new_mask_words = take((size_t)new_mask_entries(d) * 2 * 8);
   w.keep_tok = take(d.spec_keep > 0 ? F : 0);
   w.h_rows = take(d.n_streams > 1 ? (size_t)kBatchedMaxKSplit * F * 8 * 4 *
-                                        (d.gate_mode == LIF_GATE_BUNDLED ? 2 : 1)
+                                        (d.gate_mode == LIF_GATE_BUNDLED ? 2 : 1) * 2   // (two lists)
                                   : 0);
   w.gate_val = take(d.gate_mode == LIF_GATE_RESIDENT ? S * F * 4 : 0);
   w.hit_rows = take(F * 4);
@@ -48,6 +48,7 @@ Workspace plan_workspace(const lif_layer_desc& d, int ffn_grid_max) {
   size_t partial_rows = (size_t)ffn_grid_max;
   if (ffn_batched_supported(d) && (size_t)kBatchedMaxPartitions * S > partial_rows)
     partial_rows = (size_t)kBatchedMaxPartitions * S;
+  if (ffn_batched_supported(d)) partial_rows += (size_t)kBatchedMaxPartitions * S;   // two lists
   w.y_partial = take(partial_rows * d.d_model * 4);
   w.total = off;
   return w;
@@ -364,18 +365,27 @@ lif_status lif_decode_step(lif_layer* L, const void* dev_x, float* dev_y, void* 
   if (L->watch_chain) {
     // compute stream: ... window kernel -> (row moves) -> fetch, resident early -> FFN
     L->watch_chain = 0;
-    if (moves_aside) {                 // the moves touch other rows than the fetch: beside it
+    // beside it, given a second stream: the moves where they touch other rows than the fetch, and the
+    // tensor-core FFN of the rows that were already cached
+    const bool hits_aside = sf != sc && L->fb_ok && L->desc.ffn_mode == 0 && L->split_ffn;
+    if (moves_aside || hits_aside) {
       ok = ok && cudaEventRecord(L->ev_plan, sc) == cudaSuccess;
       ok = ok && cudaStreamWaitEvent(sf, L->ev_plan, 0) == cudaSuccess;
-      ok = ok && launch_moves(L, sf, ev) == cudaSuccess;
+      if (moves_aside) ok = ok && launch_moves(L, sf, ev) == cudaSuccess;
+      if (ev && hits_aside) tm_record(ev[7], sf);
+      if (hits_aside) ok = ok && launch_ffn_batched_hits(L, x, sf, moves_aside && L->use_pdl) == cudaSuccess;
+      if (ev && hits_aside) tm_record(ev[8], sf);
       ok = ok && cudaEventRecord(L->ev_fetch, sf) == cudaSuccess;
     }
     if (ev) tm_record(ev[5], sc);
     ok = ok && launch_fetch_early(L, sc) == cudaSuccess;
     if (ev) tm_record(ev[6], sc);
-    if (moves_aside) ok = ok && cudaStreamWaitEvent(sc, L->ev_fetch, 0) == cudaSuccess;
+    if (moves_aside && !hits_aside) ok = ok && cudaStreamWaitEvent(sc, L->ev_fetch, 0) == cudaSuccess;
     L->ends_step = 1;
-    if (L->desc.ffn_mode == 0)
+    if (hits_aside) {
+      ok = ok && launch_ffn_batched_new(L, x, dev_y, sc, L->ev_fetch) == cudaSuccess;
+      if (ev) tm_record(ev[9], sc);
+    } else if (L->desc.ffn_mode == 0)
       ok = ok && launch_ffn(L, x, L->active_slots, L->counts + LIF_CNT_N_ACTIVE, nullptr, dev_y,
                             false, sc, ev) == cudaSuccess;
     else

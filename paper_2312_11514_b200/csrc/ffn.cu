@@ -207,14 +207,14 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_ffn_kernel(FfnArgs a) {
 }
 
 // y[m] = (accumulate ? y[m] : b_down[m]) + sum over set 0 then set 1 of the CTA partials
-// (set j holds min(G, *n_j) partials; set 1 is optional).  A CTA owns 8 float4 columns (one
+// (set 0 holds min(G, *n0) partials, set 1, which is optional, min(G1, *n1)).  A CTA owns 8 float4 columns (one
 // 128-byte line per partial) x 32 slices of the partial index; each slice adds its partials
 // in ascending order, then the slices are added in ascending order: a fixed summation order.
 constexpr int kSumThreads = 256;
 constexpr int kSumCols = 8;                     // float4 columns per CTA
 __global__ void __launch_bounds__(kSumThreads)
 ffn_reduce_kernel(const float* __restrict__ p0, const int32_t* __restrict__ n0,
-                  const float* __restrict__ p1, const int32_t* __restrict__ n1, int G,
+                  const float* __restrict__ p1, const int32_t* __restrict__ n1, int G, int G1,
                   const __half* __restrict__ b_down, int b_period, float* __restrict__ y, int d,
                   int accumulate, int n_cap, int* next_run_after_wait) {
   __shared__ float4 red[32][kSumCols];
@@ -239,7 +239,7 @@ ffn_reduce_kernel(const float* __restrict__ p0, const int32_t* __restrict__ n0,
   if (next_run_after_wait && blockIdx.x == 0 && tid == 0)
     advance_run(next_run_after_wait, run);
   // counts as the kernels that wrote the partials clamp them: [0, n_cap]
-  const int v0 = min(G, max(0, min(*n0, n_cap))), v1 = p1 ? min(G, max(0, min(*n1, n_cap))) : 0;
+  const int v0 = min(G, max(0, min(*n0, n_cap))), v1 = p1 ? min(G1, max(0, min(*n1, n_cap))) : 0;
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
   if (in) {
     // batches of 10 partials per thread (two sets of up to 148 over 32 slices), a batch's loads
@@ -362,7 +362,7 @@ cudaError_t launch_ffn(lif_layer* L, const __half* x, const int32_t* slots, cons
     if (ev && s == D.n_streams - 1) tm_record(ev[8], st);
     e = launch_k(ffn_reduce_kernel, dim3((d / 4 + kSumCols - 1) / kSumCols), dim3(kSumThreads), 0, st, L->use_pdl,
                  (const float*)L->y_partial, n, (const float*)nullptr, (const int32_t*)nullptr,
-                 L->ffn_grid, (const __half*)D.dev_bias_down, d, y + (size_t)s * d, d,
+                 L->ffn_grid, 0, (const __half*)D.dev_bias_down, d, y + (size_t)s * d, d,
                  accumulate ? 1 : 0, D.capacity,
                  L->ends_step && s == D.n_streams - 1 ? (int*)(L->counts + CNT_PREDICTOR_RUN) : (int*)nullptr);
     if (e != cudaSuccess) return e;
@@ -396,7 +396,7 @@ cudaError_t launch_one(lif_layer* L, int kernel, const __half* x, float* y, cuda
     case LIF_KERNEL_FFN_SUM:
       return launch_k(ffn_reduce_kernel, dim3((d / 4 + kSumCols - 1) / kSumCols), dim3(kSumThreads), 0, st,
                       L->use_pdl, (const float*)p0, cnt + LIF_CNT_N_HITS, (const float*)p1,
-                      cnt + LIF_CNT_N_LOAD, L->ffn_grid, (const __half*)D.dev_bias_down, d, y, d, 0,
+                      cnt + LIF_CNT_N_LOAD, L->ffn_grid, L->ffn_grid, (const __half*)D.dev_bias_down, d, y, d, 0,
                       D.capacity, (int*)nullptr);
     default:
       return cudaErrorInvalidValue;
@@ -405,11 +405,12 @@ cudaError_t launch_one(lif_layer* L, int kernel, const __half* x, float* y, cuda
                   L->use_pdl, a);
 }
 
-cudaError_t launch_partial_sum(lif_layer* L, const float* partial, const int32_t* n,
-                               int partitions, int width, float* y, cudaStream_t st) {
+cudaError_t launch_partial_sum(lif_layer* L, const float* p0, const int32_t* n0, int parts0,
+                               const float* p1, const int32_t* n1, int parts1, int width, float* y,
+                               cudaStream_t st) {
   return launch_k(ffn_reduce_kernel, dim3((width / 4 + kSumCols - 1) / kSumCols),
-                  dim3(kSumThreads), 0, st, L->use_pdl, partial, n, (const float*)nullptr,
-                  (const int32_t*)nullptr, partitions, (const __half*)L->desc.dev_bias_down,
+                  dim3(kSumThreads), 0, st, L->use_pdl, p0, n0, p1, n1, parts0, parts1,
+                  (const __half*)L->desc.dev_bias_down,
                   L->desc.d_model, y, width, 0, L->desc.capacity,
                   L->ends_step ? (int*)(L->counts + CNT_PREDICTOR_RUN) : (int*)nullptr);
 }
@@ -461,7 +462,7 @@ cudaError_t launch_fetch_and_ffn_split(lif_layer* L, const __half* x, float* y, 
   }
   if (fork && (e = cudaStreamWaitEvent(st, L->ev_fetch, 0)) != cudaSuccess) return e;
   e = launch_k(ffn_reduce_kernel, dim3((d / 4 + kSumCols - 1) / kSumCols), dim3(kSumThreads), 0,
-               st, L->use_pdl, (const float*)p0, hit.n, (const float*)p1, miss.n, L->ffn_grid,
+               st, L->use_pdl, (const float*)p0, hit.n, (const float*)p1, miss.n, L->ffn_grid, L->ffn_grid,
                (const __half*)D.dev_bias_down, d, y, d, 0, D.capacity,
                (int*)(L->counts + CNT_PREDICTOR_RUN));
   if (ev) tm_record(ev[9], st);
@@ -604,7 +605,7 @@ extern "C" lif_status lif_sparse_ffn_static(const void* dev_matrix, int32_t n_ro
   sparse_ffn_kernel<LIF_GATE_NONE><<<grid, kThreads, ffn_smem_bytes(d_model, stages), st>>>(a);
   if (cudaGetLastError() != cudaSuccess) return LIF_ERR_CUDA;
   ffn_reduce_kernel<<<(d_model / 4 + kSumCols - 1) / kSumCols, kSumThreads, 0, st>>>(
-      sd.scratch->partial, dev_n_slots, nullptr, nullptr, grid, (const __half*)dev_bias_down,
+      sd.scratch->partial, dev_n_slots, nullptr, nullptr, grid, 0, (const __half*)dev_bias_down,
       d_model, dev_y, d_model, 0, n_rows, (int*)nullptr);
   return cudaGetLastError() == cudaSuccess ? LIF_OK : LIF_ERR_CUDA;
 }

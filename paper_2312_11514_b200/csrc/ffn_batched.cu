@@ -511,9 +511,19 @@ cudaError_t ffn_batched_configure(lif_layer* L) {
   return cudaSuccess;
 }
 
-cudaError_t launch_ffn_batched(lif_layer* L, const __half* x, const int32_t* slots,
-                               const int32_t* n, const int32_t* base, float* y, cudaStream_t st) {
+// The two phases over one list of rows.  set 0 / 1: which half of the scratch memory they use; ctas:
+// how many SMs they may take.  *partitions: partials written per (stream, column) at most.
+static cudaError_t launch_phases(lif_layer* L, const __half* x, const int32_t* slots, const int32_t* n,
+                                 const int32_t* base, int set, int ctas, cudaStream_t st, int pdl,
+                                 float** partials, int* partitions) {
   const lif_layer_desc& D = L->desc;
+  const size_t h_block = (size_t)kBatchedMaxKSplit * D.d_ff * 8;   // floats of one phase-A output
+  const int vecs = D.gate_mode == LIF_GATE_BUNDLED ? 2 : 1;
+  float* h = L->h_rows + (size_t)set * vecs * h_block;
+  auto share = [&](int parts, int whole) {           // partitions that fit `ctas`
+    const int p = ctas / parts > 0 ? ctas / parts : 1;
+    return p < whole ? p : whole;
+  };
   BatchedArgs a;
   a.cache = (const __half*)D.dev_cache;
   a.bias = L->bias;
@@ -521,17 +531,17 @@ cudaError_t launch_ffn_batched(lif_layer* L, const __half* x, const int32_t* slo
   a.slots = slots;
   a.n = n;
   a.base = base;
-  a.H = L->h_rows;
-  a.y_partial = L->y_partial;
+  a.H = h;
+  a.y_partial = L->y_partial + (size_t)set * kBatchedMaxPartitions * D.n_streams * D.d_model;
   a.status = L->counts + LIF_CNT_STATUS;
   a.d = D.d_model;
   a.S = D.n_streams;
   a.parts = L->fb_parts;
-  a.partitions = L->fb_partitions;
+  a.partitions = share(L->fb_parts, L->fb_partitions);
   a.cols_per_part = L->fb_cols;
   a.ksplit = L->fb_ksplit;
   a.k_per_split = L->fb_kps;
-  a.up_partitions = L->fb_up_partitions;
+  a.up_partitions = share(L->fb_ksplit, L->fb_up_partitions);
   a.up_group = L->fb_up_group;
   a.h_stride = (size_t)D.d_ff * 8;
   a.act = D.activation;
@@ -548,25 +558,63 @@ cudaError_t launch_ffn_batched(lif_layer* L, const __half* x, const int32_t* slo
   a.rows = D.capacity;
   a.wait_polls = L->wait_polls;
   a.stages = L->fb_up_stages;
-  cudaError_t e = launch_k(ffn_batched_up_kernel, dim3(L->fb_up_partitions * L->fb_ksplit),
-                           dim3(kThreads), L->fb_up_smem, st, L->use_pdl, a);
+  *partials = a.y_partial;
+  *partitions = a.partitions;
+  cudaError_t e = launch_k(ffn_batched_up_kernel, dim3(a.up_partitions * L->fb_ksplit),
+                           dim3(kThreads), L->fb_up_smem, st, pdl, a);
   if (e != cudaSuccess) return e;
   if (D.gate_mode == LIF_GATE_BUNDLED) {           // second pass of phase A: the up rows
-    float* h2 = L->h_rows + (size_t)kBatchedMaxKSplit * D.d_ff * 8;
-    a.H = h2;
+    a.H = h + h_block;
     a.vec_off = D.d_model;
     a.add_bias = 0;
-    e = launch_k(ffn_batched_up_kernel, dim3(L->fb_up_partitions * L->fb_ksplit), dim3(kThreads),
+    e = launch_k(ffn_batched_up_kernel, dim3(a.up_partitions * L->fb_ksplit), dim3(kThreads),
                  L->fb_up_smem, st, L->use_pdl, a);
     if (e != cudaSuccess) return e;
-    a.H = L->h_rows;
-    a.H2 = h2;
+    a.H = h;
+    a.H2 = h + h_block;
   }
   a.stages = 32;
-  e = launch_k(ffn_batched_down_kernel, dim3(L->fb_parts * L->fb_partitions), dim3(kThreads),
-               L->fb_down_smem, st, L->use_pdl, a);
+  return launch_k(ffn_batched_down_kernel, dim3(L->fb_parts * a.partitions), dim3(kThreads),
+                  L->fb_down_smem, st, L->use_pdl, a);
+}
+
+cudaError_t launch_ffn_batched(lif_layer* L, const __half* x, const int32_t* slots,
+                               const int32_t* n, const int32_t* base, float* y, cudaStream_t st) {
+  float* p;
+  int parts;
+  cudaError_t e = launch_phases(L, x, slots, n, base, 0, 1 << 20, st, L->use_pdl, &p, &parts);
   if (e != cudaSuccess) return e;
-  return launch_partial_sum(L, L->y_partial, n, L->fb_partitions, D.n_streams * D.d_model, y, st);
+  return launch_partial_sum(L, p, n, parts, nullptr, nullptr, 0, L->desc.n_streams * L->desc.d_model, y, st);
+}
+
+// Around the fetch: the rows that were already cached need nothing of it, and the fetch leaves all but
+// a few SMs free, so their FFN runs beside it; behind it there are only the new rows (8 streams at
+// 7168 x 28672: 840 of 5500 rows; up, down and sum 54 -> 25 us behind the last row).
+static int ctas_beside_the_fetch(const lif_layer* L) {
+  const int n = L->n_sm - fetch_ring_ctas(L);
+  return n > L->n_sm / 2 ? n : L->n_sm / 2;
+}
+cudaError_t launch_ffn_batched_hits(lif_layer* L, const __half* x, cudaStream_t st, int pdl) {
+  float* p;
+  int parts;
+  return launch_phases(L, x, L->hit_slots, L->counts + LIF_CNT_N_HITS, nullptr, 0,
+                       ctas_beside_the_fetch(L), st, pdl, &p, &parts);
+}
+cudaError_t launch_ffn_batched_new(lif_layer* L, const __half* x, float* y, cudaStream_t st,
+                                   cudaEvent_t hits_done) {
+  float* p;
+  int parts;
+  const int32_t* cnt = L->counts;
+  // (not a dependent launch: resident early, its CTAs would keep the SMs from the kernels beside the
+  // fetch; measured 543 instead of 500 us per layer-step)
+  cudaError_t e = launch_phases(L, x, L->load_slots, cnt + LIF_CNT_N_LOAD, nullptr, 1, 1 << 20, st,
+                                0, &p, &parts);
+  if (e != cudaSuccess) return e;
+  if ((e = cudaStreamWaitEvent(st, hits_done, 0)) != cudaSuccess) return e;
+  const int hit_parts = ctas_beside_the_fetch(L) / L->fb_parts;
+  return launch_partial_sum(L, L->y_partial, cnt + LIF_CNT_N_HITS,
+                            hit_parts < L->fb_partitions ? hit_parts : L->fb_partitions, p,
+                            cnt + LIF_CNT_N_LOAD, parts, L->desc.n_streams * L->desc.d_model, y, st);
 }
 
 }  // namespace lif

@@ -204,13 +204,20 @@ cudaError_t launch_predict_one(lif_layer* L, int kernel, const __half* x, cudaSt
 cudaError_t ffn_configure(lif_layer* L);
 constexpr int kBatchedMaxPartitions = 128;
 constexpr int kBatchedMaxKSplit = 8;
-// y[i] = b_down[i % d_model] + sum_{p < min(partitions, *n)} partial[p][i], i < width
-cudaError_t launch_partial_sum(lif_layer* L, const float* partial, const int32_t* n,
-                               int partitions, int width, float* y, cudaStream_t st);
+// y[i] = b_down[i % d_model] + sum_{p < min(parts0, *n0)} p0[p][i] + the same of set 1 (p1 may be
+// nullptr), i < width
+cudaError_t launch_partial_sum(lif_layer* L, const float* p0, const int32_t* n0, int parts0,
+                               const float* p1, const int32_t* n1, int parts1, int width, float* y,
+                               cudaStream_t st);
 bool ffn_batched_supported(const lif_layer_desc& D);
 cudaError_t ffn_batched_configure(lif_layer* L);
 cudaError_t launch_ffn_batched(lif_layer* L, const __half* x, const int32_t* slots,
                                const int32_t* n, const int32_t* base, float* y, cudaStream_t st);
+// The FFN of a decode step of several streams around the fetch: launch_ffn_batched_hits (the rows that
+// were already cached, on a stream beside the fetch), then launch_ffn_batched_new behind both.
+cudaError_t launch_ffn_batched_hits(lif_layer* L, const __half* x, cudaStream_t st, int pdl);
+cudaError_t launch_ffn_batched_new(lif_layer* L, const __half* x, float* y, cudaStream_t st,
+                                   cudaEvent_t hits_done);
 size_t ffn_smem_for(const lif_layer* L, int stages);
 
 // Launch with (pdl) or without the programmatic-stream-serialization attribute.  A kernel
