@@ -60,21 +60,10 @@ predict_z_kernel(const __half* __restrict__ x, const __half* __restrict__ A, int
       }
     }
     own_copies_wait();
-#pragma unroll 4
-    for (int u = 0; u < staged; ++u) {
-      const int m = m0 + rl + (8 + u) * nrl;
-      if (m < m1) {
-        float af[8];
-        unpack8(staged_rows[u * kThreads + tid], af);
-        const float xs = __half2float(x[m]);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] = fmaf(xs, af[e], acc[e]);
-      }
-    }
-#pragma unroll 4
-    for (int m = m0 + rl + (8 + staged) * nrl; m < m1; m += nrl) {
+#pragma unroll 2
+    for (int u = 0, m = m0 + rl + 8 * nrl; m < m1; ++u, m += nrl) {
       float af[8];
-      unpack8(ld_stream16(A + (size_t)m * r + cg * 8), af);
+      unpack8(u < staged ? staged_rows[u * kThreads + tid] : ld_stream16(A + (size_t)m * r + cg * 8), af);
       const float xs = __half2float(x[m]);
 #pragma unroll
       for (int e = 0; e < 8; ++e) acc[e] = fmaf(xs, af[e], acc[e]);
@@ -133,9 +122,11 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
   const int my_row = (tid < kLogitTile && my_col < F) ? slot_of[my_col] : 0;
   // Released before this kernel's own wait: what follows (the window kernel or the single-launch
   // step) reads ahead of its wait only the window state, complete before stage 1 passed its own
-  // wait and released this kernel, and entries that carry this run's number.
-  pdl_trigger();
+  // wait and released this kernel, and entries that carry this run's number.  (A compacting run is
+  // followed by a kernel that can do nothing before its list: no early release, 0.6 us a call.)
+  if (!compact) pdl_trigger();
   pdl_wait();
+  if (compact) pdl_trigger();
   const int run = (tid < kLogitTile && (tid & 31) == 0) ? __ldcg(predictor_run) : 0;
   // every partial of a sum is requested before the first is used (one memory round trip instead of
   // several); the additions keep their order
@@ -202,10 +193,12 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
       const unsigned long long e = (unsigned long long)mn | ((unsigned long long)(unsigned)run << 32);
       asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(
                        new_mask_words + blockIdx.x * (kLogitTile / 32) + (tid >> 5)), "l"(e) : "memory");
-      const unsigned long long ea = (unsigned long long)m | ((unsigned long long)(unsigned)run << 32);
-      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(
-                       new_mask_words + (gridDim.x + blockIdx.x) * (kLogitTile / 32) + (tid >> 5)),
-                   "l"(ea) : "memory");
+      if (!compact) {     // and the active ones themselves, for the single-launch step
+        const unsigned long long ea = (unsigned long long)m | ((unsigned long long)(unsigned)run << 32);
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(
+                         new_mask_words + (gridDim.x + blockIdx.x) * (kLogitTile / 32) + (tid >> 5)),
+                     "l"(ea) : "memory");
+      }
     }
   }
 
