@@ -22,7 +22,12 @@
 // copies each reach the same 49.8 GB/s as 148 CTAs).  More in flight does not read faster, it only
 // queues up in front of everything else: with host loads in flight on all SMs a dependent load
 // beside them takes 1800 cycles instead of 290, and an HBM stream of the whole chip falls from 3.6
-// to 0.9 TB/s (2.3 TB/s with 16 CTAs and two copies each).
+// to 0.9 TB/s (2.7 TB/s with 32 CTAs and one copy each).
+// Why 32 with all but one stage of the ring in flight, asked for when a row has landed and not when it
+// is done with: the copies of one SM share its rate and land together, so with 16 CTAs and two wide
+// rows each the last two rows were worked on one after the other behind the link.  Layers of 4544 and
+// 768 columns 79 -> 77.7 and 16.2 -> 15.9 us, three streams at 1544 47.7 -> 46.7; 16 CTAs asked the
+// same way lose 5% to the gap between a landing and the next request, 24 lose 2%.
 #include "lif_internal.cuh"
 #include "mask_compact.cuh"
 #include "window.cuh"
@@ -35,7 +40,7 @@ constexpr int kStepWarps = kStepThreads / 32;
 constexpr int kEntriesPerThread = 2;                   // <= 1024 entries: d_ff <= 32768
 constexpr int kStepWatchPolls = 64;                    // about 30 us
 constexpr unsigned kStepSpinLimit = 1u << 20;          // polls of a counter: about a second
-constexpr int kFetchCtas = 16;
+constexpr int kFetchCtas = 32;
 constexpr unsigned short kNoSlot = 0xffff;
 
 // Counters of the layer's steps.  They only grow: the ticket tells the step as well as the part, and
@@ -827,6 +832,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     bulk_g2s(ring + (size_t)st * row_bytes, a.store + (size_t)id * row_bytes, row_bytes, bars + st);
   };
   const int n_new = (int)tot[0];
+  const int first = a.w.append_first ? stages - 1 : stages;
   int q = (int)pre[0];
 #pragma unroll
   for (int i = 0; i < kEntriesPerThread; ++i)              // of the thread's bits, those of rank f mod nf
@@ -834,10 +840,10 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       if (q % nf == f) {
         const int id = (tid * kEntriesPerThread + i) * 32 + __ffs(m) - 1;
         ids[q / nf] = (unsigned short)id;
-        if (q / nf < stages) issue(id, q / nf);            // the first ones by whoever finds them
+        if (q / nf < first) issue(id, q / nf);             // the first ones by whoever finds them
       }
   int cnt = f < n_new ? (n_new - f + nf - 1) / nf : 0;
-  const int issued = min(stages, cnt);
+  const int issued = min(first, cnt);
   pdl_wait();
   for (int i = tid; i < S * nvec; i += kStepThreads) xs[i] = reinterpret_cast<const uint4*>(a.x)[i];
   Acc<kS> acc;
@@ -880,7 +886,14 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       if (tid == 0) set_status(a, LIF_ERR_TIMEOUT);
       mbar_wait(bars + st, parity);
     }
-    if (tid == 0 && i >= held) store_row(i, st);
+    if (tid == 0 && i >= held) {
+      if (held == 0 && i + stages - 1 < cnt) {             // the stage of row i - 1 is free
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        issue(ids[i + stages - 1], st == 0 ? stages - 1 : st - 1);
+      }
+      store_row(i, st);
+    }
     const float b = row_scalar<kGate>(a, ids[i]);
     float p[kS], p2[kS];
 #pragma unroll
@@ -941,7 +954,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       for (int j = 0; j < held; ++j) store_row(j, j);
     }
     const int again = i == held - 1 ? 0 : i;               // rows again .. i may be replaced
-    if (tid == 0 && i >= held - 1 && again + stages < cnt) {
+    if (tid == 0 && held > 0 && i >= held - 1 && again + stages < cnt) {
       asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       for (int j = again; j <= i && j + stages < cnt; ++j) issue(ids[j + stages], j % stages);
