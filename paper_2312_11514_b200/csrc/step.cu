@@ -832,7 +832,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     bulk_g2s(ring + (size_t)st * row_bytes, a.store + (size_t)id * row_bytes, row_bytes, bars + st);
   };
   const int n_new = (int)tot[0];
-  const int first = a.w.append_first ? stages - 1 : stages;
+  const int first = stages - 1;                            // rows in flight at a time
   int q = (int)pre[0];
 #pragma unroll
   for (int i = 0; i < kEntriesPerThread; ++i)              // of the thread's bits, those of rank f mod nf
@@ -861,14 +861,23 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     for (int i = tid; i < cnt; i += kStepThreads)
       dst_rows[i] = (unsigned short)__ldcg(a.w.load_slots + f + i * nf);
   }
-  // In the paper's order the new rows' places may be rows that the cache CTAs still read: the first
-  // ringful of bundles stays in the ring until they are done, its FFN terms are computed meanwhile.
-  const int held = a.w.append_first ? 0 : min(cnt, stages);
+  // In the paper's order the new rows' places may be rows that the cache CTAs still read: the bundles
+  // stay in the ring until they are done, or until a stage is needed again; their FFN terms are computed
+  // meanwhile.
+  bool released = a.w.append_first;                        // thread 0
   auto store_row = [&](int i, int st) {                    // thread 0
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
                      a.cache + (size_t)dst_rows[i] * row_bytes),
                  "r"(smem_u32(ring + (size_t)st * row_bytes)), "r"(row_bytes) : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+  };
+  auto release = [&](int rows) {                           // thread 0; rows 0 .. rows - 1 are held
+    const unsigned want = (a.epoch + 1) * (unsigned)n_groups;
+    unsigned n = 0;
+    while ((int)(ld_acquire(&a.sync->groups_done) - want) < 0 && n < kStepSpinLimit) ++n;
+    if (n == kStepSpinLimit) set_status(a, LIF_ERR_TIMEOUT);
+    for (int j = 0; j < rows; ++j) store_row(j, j);
+    released = true;
   };
   __syncthreads();
   // One stream: the fetch CTAs also add up all partial sums (the cached rows' while the last row is on
@@ -886,13 +895,14 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       if (tid == 0) set_status(a, LIF_ERR_TIMEOUT);
       mbar_wait(bars + st, parity);
     }
-    if (tid == 0 && i >= held) {
-      if (held == 0 && i + stages - 1 < cnt) {             // the stage of row i - 1 is free
+    if (tid == 0) {
+      if (i + stages - 1 < cnt) {                          // the stage of row i - 1 is free once it is stored
+        if (i > 0 && !released) release(i);
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         issue(ids[i + stages - 1], st == 0 ? stages - 1 : st - 1);
       }
-      store_row(i, st);
+      if (released) store_row(i, st);
     }
     const float b = row_scalar<kGate>(a, ids[i]);
     float p[kS], p2[kS];
@@ -946,25 +956,13 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       axpy_row<kS>(acc, down, h_s, nvec);
     }
     __syncthreads();                                       // the stage, part[] and h_s[] are free
-    if (tid == 0 && i == held - 1) {
-      const unsigned want = (a.epoch + 1) * (unsigned)n_groups;
-      unsigned n = 0;
-      while ((int)(ld_acquire(&a.sync->groups_done) - want) < 0 && n < kStepSpinLimit) ++n;
-      if (n == kStepSpinLimit) set_status(a, LIF_ERR_TIMEOUT);
-      for (int j = 0; j < held; ++j) store_row(j, j);
-    }
-    const int again = i == held - 1 ? 0 : i;               // rows again .. i may be replaced
-    if (tid == 0 && held > 0 && i >= held - 1 && again + stages < cnt) {
-      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      for (int j = again; j <= i && j + stages < cnt; ++j) issue(ids[j + stages], j % stages);
-    }
     if (++st == stages) {
       st = 0;
       parity ^= 1u;
     }
   }
   if (cnt > 0) store_tagged_partial<kS>(acc, a.p_new + (size_t)f * pairs, nvec, S, tag);
+  if (tid == 0 && cnt > 0 && !released) release(cnt);
   if (kS == 1) sum.finish(red);
   if (tid == 0) {
     if (f == 0) advance_run(a.next_run, run);
@@ -1063,8 +1061,7 @@ cudaError_t step_configure(lif_layer* L) {
   L->step_sum_ctas = D.n_streams > 1 ? sum_ctas(D) : 0;
   L->step_group = L->step_cache_ctas > hit_partials_max(D) ? kGroupMax : 1;
   L->step_cache_stages = stages(kCacheRing, x, 1);
-  // in the paper's cache order the bundles wait in the ring until the cache CTAs have read the rows
-  // they replace: twice the ring keeps the link busy meanwhile
+  // (paper's cache order: bundles wait in the ring, see fetch_role; twice the ring keeps the link busy)
   L->step_fetch_stages = stages(D.append_first ? kFetchRing : 2 * kFetchRing, x + ids, 2);
   size_t smem = window_role_smem(D.d_ff, D.capacity);
   const size_t need_c = x + L->step_cache_stages * row, need_f = x + L->step_fetch_stages * row + ids;
