@@ -1,0 +1,79 @@
+"""The decode step at the edges of its single-launch form (one stream, or several whose sums fit a
+CTA's registers), of the kernels beyond them, and of the multi-stream predictor: widths and stream
+counts on both sides of each limit, ranks around the two forms of the first predictor stage, fewer new
+neurons than fetch CTAs, more than a ring holds, refused updates."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2312_11514_b200 import binding as B
+from paper_2312_11514_b200 import workloads as W
+
+import parity_util as P
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _steps(cfg, **kw):
+    gpu, ora = P.make_layer_pair(cfg, 0, b_down=True, **kw)
+    X = W.make_inputs(cfg, device=DEV)
+    y = torch.empty(cfg.n_streams, cfg.d_model, dtype=torch.float32, device=DEV)
+    sc, sf = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    loads = []
+    for t in range(cfg.steps):
+        B.lif_decode_step(gpu.handle, X[t], y, sc, sf)
+        loads.append(len(P.check_decode_step(gpu, ora, X[t].cpu().numpy(), y)["load_ids"]))
+        P.compare_cache_rows(gpu, ora)
+    gpu.close()
+    return loads
+
+
+@pytest.mark.parametrize("append_first", [0, 1])
+@pytest.mark.parametrize("S,d,F,r,fire,gate_mode", [
+    (1, 8, 64, 8, 0.20, 0),            # one 16-byte piece per vector
+    (1, 4104, 1032, 120, 0.10, 0),     # a thread's second piece begins; tail of the entries
+    (1, 8192, 520, 16, 0.10, 1),       # widest rows, three vectors: the smallest ring
+    (1, 520, 32768, 136, 0.02, 0),     # most neurons, most cache CTAs (grouped partials)
+    (1, 520, 32768, 8, 0.0005, 2),     # fewer new neurons than fetch CTAs, some steps none
+    (2, 8192, 520, 128, 0.10, 0),      # two streams: any width
+    (3, 1032, 2056, 248, 0.10, 0),     # three in the four-stream form, rank not a multiple of 16
+    (4, 8192, 264, 24, 0.10, 0),
+    (5, 4096, 1032, 128, 0.06, 0),     # widest row of the eight-stream form
+    (5, 4112, 1032, 128, 0.06, 0),     # beyond it: tensor cores, cached rows beside the fetch
+    (7, 1040, 4104, 2048, 0.03, 0),    # largest rank
+    (8, 4096, 2056, 120, 0.05, 0),
+    (8, 7168, 1032, 256, 0.05, 0),
+    (4, 1040, 2056, 40, 0.08, 2),      # resident gate, several streams
+])
+def test_decode_step_at_the_edges(S, d, F, r, fire, gate_mode, append_first):
+    act, thr = (B.ACT_FATRELU, 0.05) if gate_mode else (B.ACT_RELU, 0.0)
+    cfg = W.LifConfig("edges", 1, d, F, r, 2, S, 7, fire, 1.0, 0.7, 0.7, 71)
+    loads = _steps(cfg, capacity=F if F <= 2056 else None, append_first=append_first,
+                   gate_mode=gate_mode, activation=act, act_threshold=thr)
+    assert sum(loads) > 0
+
+
+@pytest.mark.parametrize("S", [1, 3])
+def test_a_refused_update_brings_nothing_in_and_the_next_step_follows_the_oracle(S):
+    cfg = W.LifConfig("refused", 1, 1032, 4096, 32, 3, S, 8, 0.04, 1.0, 0.8, 0.6, 72)
+    gpu, ora = P.make_layer_pair(cfg, 0, b_down=True, append_first=1, capacity=1500)
+    X = W.make_inputs(cfg, device=DEV)
+    y = torch.empty(S, cfg.d_model, dtype=torch.float32, device=DEV)
+    sc, sf = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for t in range(cfg.steps):
+        B.lif_decode_step(gpu.handle, X[t], y, sc, sf)
+        P.check_decode_step(gpu, ora, X[t].cpu().numpy(), y)
+        before = gpu.lists()
+        B.lif_decode_step(gpu.handle, (X[t] * 30).half(), y, sc, sf)   # about half of all neurons
+        after = gpu.lists()
+        assert after["status"] == B.LIF_ERR_CAPACITY and len(after["load_ids"]) == 0
+        for key in ("pointers", "slot_of", "last_active", "num_used", "step"):
+            np.testing.assert_array_equal(after[key], before[key])
+        P.compare_cache_rows(gpu, ora)
+        want = np.tile(gpu.keep["bias_down"].float().cpu().numpy(), (S, 1))
+        np.testing.assert_array_equal(y.cpu().numpy(), want)
+        B.lif_clear_status(gpu.handle)
+    gpu.close()
