@@ -14,12 +14,16 @@ extern "C" {
 #endif
 
 /* Launch-shape knobs (defaults in parentheses); they change speed, never results beyond the
- * order of floating-point partial sums.  Set them before capturing a graph. */
+ * order of floating-point partial sums.  Set them before capturing a graph.  Except for
+ * LIF_TUNE_DEPENDENT_LAUNCH and LIF_TUNE_WAIT_POLLS they concern the separate kernels: a layer whose
+ * decode step runs as one launch behind the predictor uses them once such a knob is moved from its
+ * default (and while lif_timing_enable records). */
 enum {
   LIF_TUNE_DEPENDENT_LAUNCH = 0, /* (1) programmatic dependent launch along the compute stream */
   LIF_TUNE_SPLIT_FFN = 1,        /* (1) lif_decode_step runs the FFN of already-cached rows
                                     while the fetch copies, then the FFN of the new rows */
-  LIF_TUNE_FETCH_CTAS = 2,       /* (SM count) CTAs of the fetch kernel, 1..4096 */
+  LIF_TUNE_FETCH_CTAS = 2,       /* (SM count; the fetch as a kernel of its own: 16) CTAs of the fetch
+                                    kernel, 1..4096 */
   LIF_TUNE_FFN_CTAS = 3,         /* (SM count) CTAs of the sparse-FFN kernel, 1..256 */
   LIF_TUNE_FFN_STAGES = 4,       /* (as many as fit, at most 16) bundles in flight per CTA;
                                     fewer stages let several CTAs share an SM */
@@ -68,7 +72,7 @@ lif_status lif_timing_read(lif_layer* layer, float* host_us_sums /* [LIF_PHASE_L
                            int32_t* host_n_steps);
 
 /* Profiling aid: enqueue exactly one kernel of the decode step, with the launch shape
- * lif_decode_step uses, on the layer's current lists (valid after a completed step; these
+ * lif_decode_step uses when it launches separate kernels, on the layer's current lists (valid after a completed step; these
  * kernels do not change the window state, so they can be replayed).  dev_x as for
  * lif_decode_step; dev_y is written only by LIF_KERNEL_FFN_SUM.  n_streams must be 1. */
 enum {
