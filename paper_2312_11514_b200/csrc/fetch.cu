@@ -565,6 +565,8 @@ static cudaError_t launch_ring(lif_layer* L, const int32_t* ids, bool watch, cud
   a.counts = L->counts;
   a.row_bytes = 2u * row_elems(L->desc);
   int window = (int)((kRingWindow + a.row_bytes - 1) / a.row_bytes);
+  if (watch)         // what travels while the window kernel runs has nowhere to go yet: as deep as it gets
+    window = (int)((L->max_smem - 2048 - 2 * kRingList * 4) / a.row_bytes) - 2;
   a.window = window < 2 ? 2 : (window > 14 ? 14 : window);
   a.stages = a.window + 2;
   a.early = early_source(L);

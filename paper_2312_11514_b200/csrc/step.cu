@@ -832,7 +832,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     bulk_g2s(ring + (size_t)st * row_bytes, a.store + (size_t)id * row_bytes, row_bytes, bars + st);
   };
   const int n_new = (int)tot[0];
-  const int first = stages - 1;                            // rows in flight at a time
+  const int first = a.w.append_first ? stages - 1 : max(1, stages / 2 - 1);   // rows in flight at a time
   int q = (int)pre[0];
 #pragma unroll
   for (int i = 0; i < kEntriesPerThread; ++i)              // of the thread's bits, those of rank f mod nf
@@ -896,11 +896,13 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       mbar_wait(bars + st, parity);
     }
     if (tid == 0) {
-      if (i + stages - 1 < cnt) {                          // the stage of row i - 1 is free once it is stored
-        if (i > 0 && !released) release(i);
-        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        issue(ids[i + stages - 1], st == 0 ? stages - 1 : st - 1);
+      if (i + first < cnt) {
+        if (i + first >= stages) {                         // a row before i was in that stage: stored first
+          if (!released) release(i);
+          asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        }
+        issue(ids[i + first], st + first < stages ? st + first : st + first - stages);
       }
       if (released) store_row(i, st);
     }
