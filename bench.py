@@ -419,7 +419,7 @@ def measure(args, config_name, steps, warmup, rank, world, local, detail):
                     "host_link_bytes_per_step": fetched / K},
             # per layer-step: z, scores (or the gate kernel alone), window, moves, fetch (one stream:
             # with the new rows' FFN terms), FFN of cached rows (several streams: up + down), sum
-            "gpu_launches": ((7 if S == 1 else 8) - (1 if gate_mode == B.GATE_RESIDENT else 0)
+            "gpu_launches": ((3 if S == 1 else 10) - (1 if gate_mode == B.GATE_RESIDENT else 0)
                              + (1 if gate_mode == B.GATE_BUNDLED else 0)) * n_launch,
             "roofline": {"kernel": "sparse_ffn_kernel" if S == 1 else
                                    "ffn_batched_up_kernel + ffn_batched_down_kernel + ffn_reduce_kernel",
@@ -439,7 +439,7 @@ def measure(args, config_name, steps, warmup, rank, world, local, detail):
                                  "last token") + f", {reps} replays, CUDA events",
                          "other_launches": split},
             "host_link": {"kernel": "fetch_ffn_kernel" if S == 1 and gate_mode != B.GATE_BUNDLED
-                                    else "fetch_kernel", "bound": "host_link", "achieved": fetch_gbs,
+                                    else "fetch_ring_kernel", "bound": "host_link", "achieved": fetch_gbs,
                           "peak": link_peak, "unit": "GB/s", "frac": fetch_gbs / link_peak,
                           "peak_kind": "of measured (1 GiB pinned cudaMemcpyAsync, this run)",
                           "bytes_per_launch": fetch_bytes, "us_per_launch": kernel_us["fetch"],
