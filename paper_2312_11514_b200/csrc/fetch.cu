@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(kThreads) fetch_ring_kernel(RingArgs a) {
   };
   auto landed = [&](int k) {                         // thread 0
     if (mbar_wait(bars + k % a.stages, (unsigned)(k / a.stages) & 1u)) return;
-    atomicCAS(a.counts + LIF_CNT_STATUS, LIF_OK, LIF_ERR_TIMEOUT);
+    flag_timeout(a.counts + LIF_CNT_STATUS);
   };
   int known = 0, n_early = 0;                        // entries of this CTA found early; of all CTAs
   if (kEarlyT == kEarlyWatch) {

@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_ffn_kernel(FfnArgs a) {
       // bounded chance to land (they target this CTA's shared memory), and leave.  The
       // partial is not written.
       if (tid == 0) {
-        atomicCAS(a.status, LIF_OK, LIF_ERR_TIMEOUT);
+        flag_timeout(a.status);
         for (int i = 0; i < rc; ++i) mbar_wait(bars + i, parity);
       }
       __syncthreads();

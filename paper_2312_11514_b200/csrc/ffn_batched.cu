@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_batched_up_kernel(BatchedArgs
     *reinterpret_cast<float4*>(red + (warp * 32 + lane) * 4) = make_float4(c[0], c[1], c[2], c[3]);
     if (__syncthreads_or(timed_out)) {
       if (tid == 0) {
-        atomicCAS(a.status, LIF_OK, LIF_ERR_TIMEOUT);
+        flag_timeout(a.status);
         drain_ring(bars, stages, G, g, groups_in_ring);
       }
       __syncthreads();
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_batched_down_kernel(BatchedAr
     if (!mbar_wait(bars + st0, parity, a.wait_polls)) timed_out = 1;
     if (__syncthreads_or(timed_out)) {
       if (tid == 0) {
-        atomicCAS(a.status, LIF_OK, LIF_ERR_TIMEOUT);
+        flag_timeout(a.status);
         drain_ring(bars, stages, kGroup, g, stages / kGroup);
       }
       __syncthreads();

@@ -260,6 +260,12 @@ cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sme
 }
 
 #ifdef __CUDACC__
+// A wait ran out.  Recorded over any other condition: this one also refuses further window updates,
+// so it must not go unrecorded because the status word already names a harmless one.
+static_assert(LIF_ERR_TIMEOUT > LIF_ERR_CUDA && LIF_ERR_TIMEOUT > LIF_ERR_STATE &&
+              LIF_ERR_TIMEOUT > LIF_ERR_CAPACITY && LIF_ERR_TIMEOUT > LIF_ERR_INVALID_ARG,
+              "flag_timeout: the largest status");
+__device__ __forceinline__ void flag_timeout(int32_t* status) { atomicMax(status, LIF_ERR_TIMEOUT); }
 // The next predictor run gets a number of its own (0 stays 0: see CNT_NO_RUN).
 // `now`: the number of the run that ends, read when it began (reading it here would put a memory
 // round trip at the end of the kernel).

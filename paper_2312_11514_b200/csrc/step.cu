@@ -138,9 +138,7 @@ __device__ __forceinline__ void step_scan(unsigned (&v)[N], unsigned (&total)[N]
     v[k] = __shfl_sync(0xffffffffu, winc - ws, warp) + inc[k] - v[k];
   }
 }
-__device__ __forceinline__ void set_status(const StepArgs& a, int code) {
-  atomicCAS(a.w.counts + LIF_CNT_STATUS, LIF_OK, code);
-}
+__device__ __forceinline__ void timed_out(const StepArgs& a) { flag_timeout(a.w.counts + LIF_CNT_STATUS); }
 // The thread's entries of the predictor run `run`.  This kernel may be resident while the score
 // kernel still runs; each entry is stored together with the number of its run, so a thread re-reads
 // its own until they carry it.  If they do not come (bounded), the kernel waits for its predecessor
@@ -181,7 +179,7 @@ __device__ __forceinline__ unsigned long long wait_plan(const StepArgs& a,
       there = (v & kPlanReady) && v >> kPlanEpochShift == (a.epoch & ((1u << 22) - 1));
     }
     if (!there) {
-      set_status(a, LIF_ERR_TIMEOUT);
+      timed_out(a);
       v = 0;
     }
     *shared = v;
@@ -306,7 +304,7 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
         a.hit_rows[s] = (uint32_t)s | ((uint32_t)pid_s[s] << 16);
     __syncthreads();
     if (tid == 0) {
-      if (w.counts[LIF_CNT_STATUS] == LIF_OK) w.counts[LIF_CNT_STATUS] = LIF_ERR_CAPACITY;
+      atomicCAS(w.counts + LIF_CNT_STATUS, LIF_OK, LIF_ERR_CAPACITY);   // (another CTA may flag a wait)
       w.counts[LIF_CNT_N_ACTIVE] = 0;
       w.counts[LIF_CNT_N_EVICT] = 0;
       w.counts[LIF_CNT_N_MOVES] = 0;
@@ -598,7 +596,7 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
     for (int i = warp; i < rc; i += kStepWarps) {          // a warp per row
       bool landed = mbar_wait(bars + i, parity, a.wait_polls);
       if (!landed) {                                       // flagged; its terms are left out
-        if (lane == 0) set_status(a, LIF_ERR_TIMEOUT);
+        if (lane == 0) timed_out(a);
         mbar_wait(bars + i, parity);
       }
       const uint4* row = reinterpret_cast<const uint4*>(rows + (size_t)i * row_bytes);
@@ -744,7 +742,7 @@ struct Summer {
         __syncthreads();                                   // red[] is free again
       }
       add(have, col, kStepSpinLimit);
-      if (lost) set_status(a, LIF_ERR_TIMEOUT);
+      if (lost) timed_out(a);
       red[tid] = v_sum;
       __syncthreads();
       if (tid < width && col < c1) {
@@ -875,7 +873,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     const unsigned want = (a.epoch + 1) * (unsigned)n_groups;
     unsigned n = 0;
     while ((int)(ld_acquire(&a.sync->groups_done) - want) < 0 && n < kStepSpinLimit) ++n;
-    if (n == kStepSpinLimit) set_status(a, LIF_ERR_TIMEOUT);
+    if (n == kStepSpinLimit) timed_out(a);
     for (int j = 0; j < rows; ++j) store_row(j, j);
     released = true;
   };
@@ -892,7 +890,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     const uint4* row = reinterpret_cast<const uint4*>(ring + (size_t)st * row_bytes);
     const bool landed = mbar_wait(bars + st, parity, a.wait_polls);
     if (!landed) {                                         // flagged; its term is left out
-      if (tid == 0) set_status(a, LIF_ERR_TIMEOUT);
+      if (tid == 0) timed_out(a);
       mbar_wait(bars + st, parity);
     }
     if (tid == 0) {
