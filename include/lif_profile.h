@@ -37,11 +37,11 @@ enum {
                                     fetch kernel also adds the FFN terms of the rows it brings
                                     in (needs fetch CTAs = FFN CTAs, bundles of two vectors) */
   LIF_TUNE_WAIT_POLLS = 9,       /* (2^22) test aid: poll limit of the FIRST wait on each bulk
-                                    copy in the sparse-FFN kernels, >= 0 (0: give up without
-                                    polling).  When it runs out the CTA sets LIF_ERR_TIMEOUT,
-                                    then waits for its copies with the full limit before it
-                                    returns, so 0 makes the error path run with nothing left in
-                                    flight */
+                                    copy in the sparse-FFN, fetch and step kernels, >= 0 (0:
+                                    give up without polling).  When it runs out the CTA sets
+                                    LIF_ERR_TIMEOUT, then waits for its copies with the full
+                                    limit before it goes on, so 0 makes the error path run with
+                                    nothing left in flight */
   LIF_TUNE_EARLY_FETCH = 10      /* (1) lif_decode_step where the fetch is a kernel of its own
                                     (several input streams, three-vector bundles): it runs on
                                     the compute stream directly behind the window kernel, is

@@ -319,6 +319,10 @@ __global__ void __launch_bounds__(kThreads) fetch_ffn_kernel(FetchFfnArgs a) {
 // window kernel behind the predictor of 8 streams took 52-69 us (39 now), and an FFN beside the fetch
 // did not pay.  `window` copies are in flight per CTA, 24 KB at least; two more stages hold rows that
 // are being stored.
+// The window state already names the rows when this kernel runs, so every one of them is filled whatever
+// happens: a copy that does not land in time is flagged, the copies in flight get another bounded chance
+// (they write this CTA's shared memory), the ring is given up, and that row and the CTA's later ones are
+// copied with plain loads.
 constexpr int kRingCtas = 16;
 constexpr size_t kRingWindow = 24 * 1024;
 constexpr int kRingList = 1024;      // ids and rows kept in shared memory at a time
@@ -331,6 +335,7 @@ struct RingArgs {
   int32_t* counts;
   unsigned row_bytes;
   int stages, window;
+  unsigned wait_polls;               // poll limit of the first wait on each copy (kWaitLimit)
   EarlySource early;
 };
 
@@ -352,9 +357,14 @@ __global__ void __launch_bounds__(kThreads) fetch_ring_kernel(RingArgs a) {
     mbar_expect_tx(bar, a.row_bytes);
     bulk_g2s(ring + (size_t)(k % a.stages) * a.row_bytes, a.store + (size_t)id * a.row_bytes, a.row_bytes, bar);
   };
-  auto landed = [&](int k) {                         // thread 0
-    if (mbar_wait(bars + k % a.stages, (unsigned)(k / a.stages) & 1u)) return;
-    flag_timeout(a.counts + LIF_CNT_STATUS);
+  auto landed = [&](int k, unsigned polls) {         // thread 0
+    return mbar_wait(bars + k % a.stages, (unsigned)(k / a.stages) & 1u, polls);
+  };
+  auto copy_row = [&](int id, int row) {             // thread 0, without the ring
+    const uint4* src = reinterpret_cast<const uint4*>(a.store + (size_t)id * a.row_bytes);
+    uint4* dst = reinterpret_cast<uint4*>(a.cache + (size_t)row * a.row_bytes);
+#pragma unroll 4
+    for (unsigned v = 0; v < a.row_bytes / 16; ++v) dst[v] = ld_stream16(src + v);
   };
   int known = 0, n_early = 0;                        // entries of this CTA found early; of all CTAs
   if (kEarlyT == kEarlyWatch) {
@@ -381,10 +391,17 @@ __global__ void __launch_bounds__(kThreads) fetch_ring_kernel(RingArgs a) {
   pdl_wait();
   pdl_trigger();
   int issued = min(known, a.window), used = 0;       // copies so far: asked for, done with
+  bool lost = false;                                 // thread 0: the ring has been given up
+  auto give_up = [&]() {                             // thread 0
+    flag_timeout(a.counts + LIF_CNT_STATUS);
+    for (int k = used; k < issued; ++k) landed(k, kWaitLimit);
+    lost = true;
+  };
   const int n = __ldcg(a.counts + LIF_CNT_N_LOAD);
   if (known && n != n_early) {                       // not this step's: let them land, start over
     if (tid == 0)
-      for (; used < issued; ++used) landed(used);
+      for (; used < issued && !lost; ++used)
+        if (!landed(used, a.wait_polls)) give_up();
     used = issued;
     known = 0;
   }
@@ -400,12 +417,16 @@ __global__ void __launch_bounds__(kThreads) fetch_ring_kernel(RingArgs a) {
     __syncthreads();
     if (tid == 0) {
       int asked = i0 == 0 && known ? issued : 0;     // entries of this batch already asked for
-      for (; asked < min(m, a.window); ++asked, ++issued) {
+      for (; asked < min(m, a.window) && !lost; ++asked, ++issued) {
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         issue(ids[asked], issued);
       }
       for (int i = 0; i < m; ++i, ++used) {
-        landed(used);
+        if (!lost && !landed(used, a.wait_polls)) give_up();
+        if (lost) {
+          copy_row(ids[i], rows[i]);
+          continue;
+        }
         asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
                          a.cache + (size_t)rows[i] * a.row_bytes),
                      "r"(smem_u32(ring + (size_t)(used % a.stages) * a.row_bytes)), "r"(a.row_bytes) : "memory");
@@ -569,6 +590,7 @@ static cudaError_t launch_ring(lif_layer* L, const int32_t* ids, bool watch, cud
     window = (int)((L->max_smem - 2048 - 2 * kRingList * 4) / a.row_bytes) - 2;
   a.window = window < 2 ? 2 : (window > 14 ? 14 : window);
   a.stages = a.window + 2;
+  a.wait_polls = L->wait_polls;
   a.early = early_source(L);
   return launch_k(watch ? fetch_ring_kernel<kEarlyWatch> : fetch_ring_kernel<kEarlyNone>,
                   dim3(fetch_ring_ctas(L)), dim3(kThreads),

@@ -92,7 +92,7 @@ struct lif_layer {
   size_t ffn_smem;    // dynamic shared memory of the sparse-FFN kernel
   int fetch_grid;     // CTAs of the fetch kernel
   int move_grid;
-  unsigned wait_polls; // poll limit of the first wait on each bulk copy in the FFN kernels
+  unsigned wait_polls; // poll limit of the first wait on each bulk copy
   int early_fetch;    // knob: the plain fetch of lif_decode_step starts early behind the window kernel
   int ends_step;      // set by lif_decode_step: the FFN's last kernel advances the run number
   int single_step;    // set by lif_decode_step: the single-launch step follows the predictor

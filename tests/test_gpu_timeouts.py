@@ -44,3 +44,68 @@ def test_a_timeout_is_recorded_over_another_condition():
     assert after["status"] == B.LIF_ERR_TIMEOUT and after["step"] == before["step"]
     np.testing.assert_array_equal(after["pointers"], before["pointers"])
     gpu.close()
+
+
+def _rows_after_the_step(gpu, ora):
+    """The window state and every cached row are the oracle's after a step that timed out."""
+    g = gpu.lists()
+    assert g["status"] == B.LIF_ERR_TIMEOUT
+    lists = ora.cache.window_update(g["active_idx"])
+    ora.cache.insert(lists, ora.bundles, ora.bias_up)
+    for key in P.LIST_KEYS:
+        np.testing.assert_array_equal(g[key], lists[key], err_msg=key)
+    np.testing.assert_array_equal(g["pointers"], ora.cache.pointers)
+    np.testing.assert_array_equal(g["slot_of"], ora.cache.slot_of)
+    P.compare_cache_rows(gpu, ora)
+    return lists
+
+
+@pytest.mark.parametrize("d,n_new", [(264, "many"), (8192, "few")])
+def test_bundles_whose_copies_are_given_up_are_fetched_all_the_same(d, n_new):
+    # a cold start, so that a CTA has more rows than its ring holds, or wide rows: two in flight
+    cfg = W.LifConfig("fetch", 1, d, 4096 if n_new == "many" else 512, 16, 3, 1, 4, 0.15, 1.0, 0.8, 0.6, 92)
+    gpu, ora = P.make_layer_pair(cfg, 0, b_down=True, capacity=cfg.d_ff)
+    X, bufs = W.make_inputs(cfg, device=DEV), P.make_bufs(gpu)
+    B.lif_predict(gpu.handle, X[0], None, bufs["act"], bufs["n_act"])
+    B.lif_window_update(gpu.handle, bufs["act"], bufs["n_act"])
+    B.lif_set_tuning(gpu.handle, B.TUNE_WAIT_POLLS, 0)
+    B.lif_fetch_bundles(gpu.handle)
+    B.lif_set_tuning(gpu.handle, B.TUNE_WAIT_POLLS, POLLS)
+    assert len(_rows_after_the_step(gpu, ora)["load_ids"]) > (16 * 14 if n_new == "many" else 16)
+    B.lif_clear_status(gpu.handle)
+    P.staged_step(gpu, ora, X[1], bufs)
+    gpu.close()
+
+
+@pytest.mark.parametrize("append_first", [0, 1])
+def test_early_copies_given_up_beyond_the_single_launch(append_first):
+    # three streams with a resident gate: the fetch is a kernel of its own and starts early
+    gpu, ora, X, y, streams = _layer(S=3, gate_mode=B.GATE_RESIDENT, activation=B.ACT_FATRELU,
+                                     act_threshold=0.05, append_first=append_first)
+    B.lif_set_tuning(gpu.handle, B.TUNE_WAIT_POLLS, 0)
+    B.lif_decode_step(gpu.handle, X[3], y, *streams)
+    B.lif_set_tuning(gpu.handle, B.TUNE_WAIT_POLLS, POLLS)
+    _rows_after_the_step(gpu, ora)
+    B.lif_clear_status(gpu.handle)
+    B.lif_decode_step(gpu.handle, X[4], y, *streams)
+    P.check_decode_step(gpu, ora, X[4].cpu().numpy(), y)
+    gpu.close()
+
+
+def test_staged_bundles_of_a_file_store_whose_copies_are_given_up(tmp_path):
+    cfg = W.LifConfig("file", 1, 264, 1000, 16, 3, 1, 6, 0.15, 1.0, 0.8, 0.6, 93)
+    path = str(tmp_path / "bundles.bin")
+    gpu, ora = P.make_layer_pair(cfg, 0, b_down=True, store_file=path)
+    store = B.lif_store_open(path, cfg.d_ff, 4 * cfg.d_model, n_threads=4, direct_io=False)
+    X = W.make_inputs(cfg, device=DEV)
+    y = torch.empty(1, cfg.d_model, dtype=torch.float32, device=DEV)
+    B.lif_set_tuning(gpu.handle, B.TUNE_WAIT_POLLS, 0)
+    B.lif_decode_step_store(gpu.handle, store, X[0], y)
+    B.lif_set_tuning(gpu.handle, B.TUNE_WAIT_POLLS, POLLS)
+    _rows_after_the_step(gpu, ora)
+    B.lif_clear_status(gpu.handle)
+    B.lif_decode_step_store(gpu.handle, store, X[1], y)
+    P.check_decode_step(gpu, ora, X[1].cpu().numpy(), y)
+    P.compare_cache_rows(gpu, ora)
+    B.lif_store_close(store)
+    gpu.close()
