@@ -853,7 +853,11 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   if (!go) {
     // the update of this step was refused: nothing is brought in; let the copies land
     if (tid == 0)
-      for (int i = 0; i < issued; ++i) mbar_wait(bars + i, 0);
+      for (int i = 0; i < issued; ++i)
+        if (!mbar_wait(bars + i, 0, a.wait_polls)) {
+          timed_out(a);
+          mbar_wait(bars + i, 0);
+        }
     cnt = 0;
   } else {
     for (int i = tid; i < cnt; i += kStepThreads)
@@ -885,15 +889,12 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   Summer<kS> sum(a, f, nf, n_hit, go ? min(nf, n_new) : 0);
 
   unsigned parity = 0;
+  int from = cnt;                                          // first row that was not waited for any longer
   for (int i = 0, st = 0; i < cnt; ++i) {
     if (kS == 1 && i == cnt - 1) sum.add(sum.have_hit, sum.c0 + tid % sum.width, 1);
     const uint4* row = reinterpret_cast<const uint4*>(ring + (size_t)st * row_bytes);
     const bool landed = mbar_wait(bars + st, parity, a.wait_polls);
-    if (!landed) {                                         // flagged; its term is left out
-      if (tid == 0) timed_out(a);
-      mbar_wait(bars + st, parity);
-    }
-    if (tid == 0) {
+    if (tid == 0 && landed) {
       if (i + first < cnt) {
         if (i + first >= stages) {                         // a row before i was in that stage: stored first
           if (!released) release(i);
@@ -931,7 +932,15 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
         part[1][s][warp] = p2[s];
       }
     }
-    const int lost = __syncthreads_or(!landed);
+    if (__syncthreads_or(!landed)) {                       // flagged; this term and the later ones are left out
+      if (tid == 0) {                                      // what is in flight gets another bounded chance
+        timed_out(a);
+        const int asked = min(cnt, i + first + (landed ? 1 : 0));
+        for (int j = i; j < asked; ++j) mbar_wait(bars + j % stages, (unsigned)(j / stages) & 1u);
+      }
+      from = i;
+      break;
+    }
     const uint4* down = row + (kVec - 1) * nvec;
     if (kS == 1) {
       float v1 = 0.f, v2 = 0.f;
@@ -940,7 +949,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
         v1 += part[0][0][w];
         if (kGate == LIF_GATE_BUNDLED) v2 += part[1][0][w];
       }
-      const float h = lost ? 0.f : row_weight<kGate>(a, b, v1, v2);
+      const float h = row_weight<kGate>(a, b, v1, v2);
       if (h != 0.f) axpy_row<kS>(acc, down, &h, nvec);
     } else {                                               // a warp per stream folds the 16 warps' sums
       if (warp < kS) {
@@ -950,7 +959,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
           v1 += __shfl_xor_sync(0xffffffffu, v1, o);
           v2 += __shfl_xor_sync(0xffffffffu, v2, o);
         }
-        if (lane == 0) h_s[warp] = lost || warp >= S ? 0.f : row_weight<kGate>(a, b, v1, v2);
+        if (lane == 0) h_s[warp] = warp >= S ? 0.f : row_weight<kGate>(a, b, v1, v2);
       }
       __syncthreads();
       axpy_row<kS>(acc, down, h_s, nvec);
@@ -962,7 +971,17 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     }
   }
   if (cnt > 0) store_tagged_partial<kS>(acc, a.p_new + (size_t)f * pairs, nvec, S, tag);
-  if (tid == 0 && cnt > 0 && !released) release(cnt);
+  if (tid == 0 && cnt > 0 && !released) release(from);
+  if (from < cnt) {
+    // The window state already names these rows, so they are filled all the same, with plain loads and
+    // without the ring (in the paper's order thread 0 has waited until their places are free).
+    __syncthreads();
+    for (int i = from; i < cnt; ++i) {
+      const uint4* src = reinterpret_cast<const uint4*>(a.store + (size_t)ids[i] * row_bytes);
+      uint4* dst = reinterpret_cast<uint4*>(a.cache + (size_t)dst_rows[i] * row_bytes);
+      for (int v = tid; v < kVec * nvec; v += kStepThreads) dst[v] = ld_stream16(src + v);
+    }
+  }
   if (kS == 1) sum.finish(red);
   if (tid == 0) {
     if (f == 0) advance_run(a.next_run, run);

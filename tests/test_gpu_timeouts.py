@@ -109,3 +109,27 @@ def test_staged_bundles_of_a_file_store_whose_copies_are_given_up(tmp_path):
     P.compare_cache_rows(gpu, ora)
     B.lif_store_close(store)
     gpu.close()
+
+
+@pytest.mark.parametrize("append_first", [0, 1])
+@pytest.mark.parametrize("S,d,gate_mode", [
+    (1, 264, B.GATE_NONE),           # a ring of 16 stages
+    (1, 8192, B.GATE_BUNDLED),       # two stages of 48 KB
+    (1, 1032, B.GATE_RESIDENT),
+    (5, 1032, B.GATE_NONE),
+])
+def test_the_single_launch_fills_rows_whose_copies_it_gave_up(S, d, gate_mode, append_first):
+    act, thr = (B.ACT_FATRELU, 0.05) if gate_mode else (B.ACT_RELU, 0.0)
+    gpu, ora, X, y, streams = _layer(S=S, steps=0, d=d, F=1024 if d == 8192 else 4096, gate_mode=gate_mode,
+                                     activation=act, act_threshold=thr, append_first=append_first)
+    for t in range(6):               # cold (more rows than a ring) and warm (rows of others move) in turn
+        lost = t % 2 == 0
+        B.lif_set_tuning(gpu.handle, B.TUNE_WAIT_POLLS, 0 if lost else POLLS)
+        B.lif_decode_step(gpu.handle, X[t], y, *streams)
+        if lost:
+            _rows_after_the_step(gpu, ora)
+            B.lif_clear_status(gpu.handle)
+        else:
+            P.check_decode_step(gpu, ora, X[t].cpu().numpy(), y)
+            P.compare_cache_rows(gpu, ora)
+    gpu.close()
