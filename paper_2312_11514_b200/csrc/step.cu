@@ -593,11 +593,13 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
     }
     __syncthreads();                                       // x and the rows' scalars
     if (rc <= 0) break;
+    int lost = 0;
     for (int i = warp; i < rc; i += kStepWarps) {          // a warp per row
-      bool landed = mbar_wait(bars + i, parity, a.wait_polls);
+      const bool landed = __all_sync(0xffffffffu, mbar_wait(bars + i, parity, a.wait_polls));
       if (!landed) {                                       // flagged; its terms are left out
+        lost = 1;
         if (lane == 0) timed_out(a);
-        mbar_wait(bars + i, parity);
+        mbar_wait(bars + i, parity);                       // another bounded chance to land
       }
       const uint4* row = reinterpret_cast<const uint4*>(rows + (size_t)i * row_bytes);
       float p[kS], p2[kS];
@@ -622,12 +624,13 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
           h_s[i][s] = landed && s < S ? row_weight<kGate>(a, b_s[i], p[s], p2[s]) : 0.f;
       }
     }
-    __syncthreads();
+    lost = __syncthreads_or(lost);
     for (int i = 0; i < rc; ++i) {
       if (kS == 1 && h_s[i][0] == 0.f) continue;
       axpy_row<kS>(acc, reinterpret_cast<const uint4*>(rows + (size_t)i * row_bytes) + (kVec - 1) * nvec,
                    h_s[i], nvec);
     }
+    if (lost) break;                                       // nothing more into stages that may be written late
     parity ^= 1u;
     if (r0 + stages < cnt) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

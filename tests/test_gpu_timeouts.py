@@ -133,3 +133,23 @@ def test_the_single_launch_fills_rows_whose_copies_it_gave_up(S, d, gate_mode, a
             P.check_decode_step(gpu, ora, X[t].cpu().numpy(), y)
             P.compare_cache_rows(gpu, ora)
     gpu.close()
+
+
+def test_cached_rows_whose_copies_were_given_up_leave_the_layer_usable():
+    # every neuron active: 1024 cached rows of 32 KB, three rounds of a cache CTA's ring
+    cfg = W.LifConfig("rounds", 1, 8192, 1024, 16, 3, 1, 3, 0.3, 0.3, 0.5, 0.6, 94)
+    gpu, ora = P.make_layer_pair(cfg, 0, capacity=cfg.d_ff, theta=-1e30, b_down=True)
+    X = W.make_inputs(cfg, device=DEV)
+    y = torch.empty(1, cfg.d_model, dtype=torch.float32, device=DEV)
+    B.lif_decode_step(gpu.handle, X[0], y)
+    P.check_decode_step(gpu, ora, X[0].cpu().numpy(), y)
+    B.lif_set_tuning(gpu.handle, B.TUNE_WAIT_POLLS, 0)
+    B.lif_decode_step(gpu.handle, X[1], y)
+    B.lif_set_tuning(gpu.handle, B.TUNE_WAIT_POLLS, POLLS)
+    assert len(_rows_after_the_step(gpu, ora)["hit_slots"]) == cfg.d_ff
+    want = gpu.keep["bias_down"].float().cpu().numpy()[None]     # no CTA went past its first round
+    np.testing.assert_array_equal(y.cpu().numpy(), want)
+    B.lif_clear_status(gpu.handle)
+    B.lif_decode_step(gpu.handle, X[2], y)
+    P.check_decode_step(gpu, ora, X[2].cpu().numpy(), y)
+    gpu.close()
