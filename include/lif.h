@@ -17,7 +17,7 @@
  *    sticky device status word and reported by lif_get_stats: a cache overflow or a bad neuron
  *    id (the window update of that step is refused, the window state untouched); a row index
  *    outside the cache given to the sparse FFN (the row is not read and contributes nothing); a
- *    bounded wait on a copy that ran out (LIF_ERR_TIMEOUT: that call's output lacks some rows'
+ *    bounded wait that ran out (LIF_ERR_TIMEOUT: that call's output lacks some rows'
  *    terms; the window bookkeeping stays consistent, and while this status stands every
  *    further window update is refused — lif_clear_status resumes).  The first condition stands
  *    until it is cleared, except that LIF_ERR_TIMEOUT takes the place of any other.
@@ -395,7 +395,9 @@ lif_status lif_snapshot_bytes(lif_layer* layer, size_t* out_bytes);
 lif_status lif_snapshot(lif_layer* layer, void* host_buf, size_t bytes);
 lif_status lif_restore(lif_layer* layer, const void* host_buf, size_t bytes);
 
-/* Clears the sticky device status word. */
+/* Clears the sticky device status word.  Where the wait that ran out (LIF_ERR_TIMEOUT) may have kept a
+ * step from filling or moving a row that its window update names, every cached row is first read from
+ * the bundle store again.  Order the layer's next call behind this one. */
 lif_status lif_clear_status(lif_layer* layer, void* stream);
 
 #ifdef __cplusplus

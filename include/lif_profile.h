@@ -15,7 +15,7 @@ extern "C" {
 
 /* Launch-shape knobs (defaults in parentheses); they change speed, never results beyond the
  * order of floating-point partial sums.  Set them before capturing a graph.  Except for
- * LIF_TUNE_DEPENDENT_LAUNCH and LIF_TUNE_WAIT_POLLS they concern the separate kernels: a layer whose
+ * LIF_TUNE_DEPENDENT_LAUNCH and the two poll limits they concern the separate kernels: a layer whose
  * decode step runs as one launch behind the predictor uses them once such a knob is moved from its
  * default (and while lif_timing_enable records). */
 enum {
@@ -42,12 +42,16 @@ enum {
                                     LIF_ERR_TIMEOUT, then waits for its copies with the full
                                     limit before it goes on, so 0 makes the error path run with
                                     nothing left in flight */
-  LIF_TUNE_EARLY_FETCH = 10      /* (1) lif_decode_step where the fetch is a kernel of its own
+  LIF_TUNE_EARLY_FETCH = 10,     /* (1) lif_decode_step where the fetch is a kernel of its own
                                     (several input streams, three-vector bundles): it runs on
                                     the compute stream directly behind the window kernel, is
                                     resident while the predictor still runs and issues its first
                                     host loads from the predictor's masks; 0: it waits for the
                                     window kernel's lists on the fetch stream */
+  LIF_TUNE_STEP_POLLS = 11       /* (2^20) test aid: poll limit of the waits of a single-launch step's
+                                    CTAs for one another, >= 0.  0: all of them give up at once,
+                                    nothing is moved or brought in and the step ends with
+                                    LIF_ERR_TIMEOUT */
 };
 lif_status lif_set_tuning(lif_layer* layer, int32_t key, int32_t value);
 

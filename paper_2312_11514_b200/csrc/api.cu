@@ -184,6 +184,7 @@ lif_status lif_create_layer(const lif_layer_desc* desc, lif_layer** out) {
     L->move_grid = L->n_sm;
     L->use_pdl = 1;
     L->wait_polls = kWaitLimit;
+    L->spin_limit = kStepSpinLimit;
     L->split_ffn = 1;
     L->fused_plan = window_plan_supported(*desc) ? 1 : 0;
     L->fused_fetch = 1;
@@ -573,6 +574,10 @@ lif_status lif_set_tuning(lif_layer* L, int32_t key, int32_t value) {
       if (value < 0) return LIF_ERR_INVALID_ARG;
       L->wait_polls = (unsigned)value;
       return LIF_OK;
+    case LIF_TUNE_STEP_POLLS:
+      if (value < 0) return LIF_ERR_INVALID_ARG;
+      L->spin_limit = (unsigned)value;
+      return LIF_OK;
     case LIF_TUNE_FFN_STAGES:
       if (value < 1 || value > L->ffn_stages_max) return LIF_ERR_INVALID_ARG;
       L->ffn_stages = value;
@@ -735,9 +740,9 @@ lif_status lif_get_stats(lif_layer* L, lif_stats* o) {
 
 lif_status lif_clear_status(lif_layer* L, void* stream) {
   if (!L) return LIF_ERR_INVALID_ARG;
-  return cudaMemsetAsync(L->counts + LIF_CNT_STATUS, 0, 4, (cudaStream_t)stream) == cudaSuccess
-             ? LIF_OK
-             : LIF_ERR_CUDA;
+  // (rows are read again by neuron id: only the single-launch step asks for that, and a layer with a
+  // staging buffer does not run it)
+  return launch_clear_status(L, (cudaStream_t)stream) == cudaSuccess ? LIF_OK : LIF_ERR_CUDA;
 }
 
 lif_status lif_probe_host_read(const void* host_src, void* dev_dst, size_t bytes,

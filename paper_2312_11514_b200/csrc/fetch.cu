@@ -554,7 +554,32 @@ refill_kernel(const uint4* __restrict__ store, uint4* __restrict__ cache,
   gather_rows(store, cache, pointers, nullptr, counts[LIF_CNT_NUM_USED], row_vec);
 }
 
+// lif_clear_status: the rows first, where a step named rows that not all of its CTAs filled or moved; the
+// last CTA clears the words.
+__global__ void __launch_bounds__(kThreads)
+clear_status_kernel(const uint4* __restrict__ store, uint4* __restrict__ cache,
+                    const int32_t* __restrict__ pointers, int32_t* counts, int row_vec) {
+  if (__ldcg(counts + CNT_ROWS_SUSPECT) == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) counts[LIF_CNT_STATUS] = LIF_OK;
+    return;
+  }
+  gather_rows(store, cache, pointers, nullptr, counts[LIF_CNT_NUM_USED], row_vec);
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicAdd(counts + CNT_TICKET_CLEAR, 1) == (int)gridDim.x - 1) {
+    counts[CNT_TICKET_CLEAR] = 0;
+    counts[CNT_ROWS_SUSPECT] = 0;
+    counts[LIF_CNT_STATUS] = LIF_OK;
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_clear_status(lif_layer* L, cudaStream_t st) {
+  clear_status_kernel<<<L->n_sm, kThreads, 0, st>>>((const uint4*)L->dev_bundles,
+                                                    (uint4*)L->desc.dev_cache, L->pointers, L->counts,
+                                                    row_elems(L->desc) / 8);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_refill(lif_layer* L, cudaStream_t st) {
   refill_kernel<<<L->fetch_grid, kThreads, 0, st>>>((const uint4*)L->dev_bundles,

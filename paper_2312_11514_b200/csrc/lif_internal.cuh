@@ -16,6 +16,8 @@ enum {
   CNT_PREDICTOR_RUN = 17,   // number of the predictor run whose masks are (being) written; advanced
                             // by the kernel that ends a decode step, or by the run that compacts
   CNT_NO_RUN = 18,          // always 0: runs that no step consumes are tagged with it
+  CNT_ROWS_SUSPECT = 19,    // 1: a step committed a plan that not all of its CTAs carried out
+  CNT_TICKET_CLEAR = 20,    // "last block done" counter of the kernel that clears the status
   CNT_TOTALS = 32           // four uint64: bytes_fetched, rows_moved, rows_active, rows_cached
 };
 
@@ -34,6 +36,7 @@ inline int z_cta_count(int d_model) {
 constexpr int kLogitTile = 128;     // neurons per CTA in the second predictor stage
 constexpr int kMaxStreams = 8;
 constexpr int kMaxRank = 2048;
+constexpr unsigned kStepSpinLimit = 1u << 20;   // polls of a wait of one CTA for another: about a second
 constexpr int kTimingEvents = 10;   // z0 z1 s1 w1 m1 | f0 f1 | g0 g1 r1
 
 struct Workspace {
@@ -93,6 +96,7 @@ struct lif_layer {
   int fetch_grid;     // CTAs of the fetch kernel
   int move_grid;
   unsigned wait_polls; // poll limit of the first wait on each bulk copy
+  unsigned spin_limit; // poll limit of the waits of a step's CTAs for one another
   int early_fetch;    // knob: the plain fetch of lif_decode_step starts early behind the window kernel
   int ends_step;      // set by lif_decode_step: the FFN's last kernel advances the run number
   int single_step;    // set by lif_decode_step: the single-launch step follows the predictor
@@ -185,6 +189,8 @@ cudaError_t launch_predict_multi(lif_layer* L, const __half* x, float* logits, i
 cudaError_t step_configure(lif_layer* L);
 cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st);
 cudaError_t launch_refill(lif_layer* L, cudaStream_t st);
+// status word <- LIF_OK, after a refill where a step's CTAs gave up (CNT_ROWS_SUSPECT)
+cudaError_t launch_clear_status(lif_layer* L, cudaStream_t st);
 cudaError_t launch_probe(const void* dev_src_alias, void* dev_dst, size_t bytes, size_t chunk,
                          int grid, cudaStream_t st);
 cudaError_t launch_probe_read(const void* dev_src, size_t bytes, void* dev_sink, int grid, int pdl,

@@ -11,6 +11,9 @@
 //                          terms from shared memory, copy them to their cache rows, and (one stream) in
 //                          the end add up all partial sums
 //   sum CTAs     (last)    with several streams add up the partial sums
+// A CTA whose wait for the plan runs out moves or brings in nothing, although the window CTA commits the
+// state that names those rows.  Like every wait that runs out it flags LIF_ERR_TIMEOUT, which refuses further
+// updates, and it marks the rows as suspect, so that clearing the status reads them from the store again.
 // A CTA waits only for CTAs that took their parts before it (with one stream the fetch CTAs also for
 // one another, at the very end, when nothing else is left to run), every wait is bounded, and every CTA
 // makes its arrivals on all paths, so the counters are complete whatever happened.
@@ -39,7 +42,6 @@ constexpr int kStepThreads = 512;
 constexpr int kStepWarps = kStepThreads / 32;
 constexpr int kEntriesPerThread = 2;                   // <= 1024 entries: d_ff <= 32768
 constexpr int kStepWatchPolls = 64;                    // about 30 us
-constexpr unsigned kStepSpinLimit = 1u << 20;          // polls of a counter: about a second
 constexpr int kFetchCtas = 32;
 constexpr unsigned short kNoSlot = 0xffff;
 
@@ -77,7 +79,8 @@ struct StepArgs {
   int d, n_streams, whole_cache, act;
   float act_thr;
   int n_cache_ctas, n_sum_ctas, group_size, cache_stages, fetch_stages, fetch_rows_max;
-  unsigned wait_polls;
+  unsigned wait_polls;            // of the first wait for a bulk copy
+  unsigned spin_limit;            // of a wait for another CTA
   unsigned epoch;                 // steps before this one (filled in by the kernel)
 };
 
@@ -139,6 +142,11 @@ __device__ __forceinline__ void step_scan(unsigned (&v)[N], unsigned (&total)[N]
   }
 }
 __device__ __forceinline__ void timed_out(const StepArgs& a) { flag_timeout(a.w.counts + LIF_CNT_STATUS); }
+// ... on something without which this CTA cannot fill or move the rows that the plan gives it
+__device__ __forceinline__ void plan_not_carried_out(const StepArgs& a) {
+  a.w.counts[CNT_ROWS_SUSPECT] = 1;
+  timed_out(a);
+}
 // The thread's entries of the predictor run `run`.  This kernel may be resident while the score
 // kernel still runs; each entry is stored together with the number of its run, so a thread re-reads
 // its own until they carry it.  If they do not come (bounded), the kernel waits for its predecessor
@@ -174,12 +182,12 @@ __device__ __forceinline__ unsigned long long wait_plan(const StepArgs& a,
   if (threadIdx.x == 0) {
     unsigned long long v = 0;
     bool there = false;
-    for (unsigned i = 0; i < kStepSpinLimit && !there; ++i) {
+    for (unsigned i = 0; i < a.spin_limit && !there; ++i) {
       v = ld_acquire64(&a.sync->plan);
       there = (v & kPlanReady) && v >> kPlanEpochShift == (a.epoch & ((1u << 22) - 1));
     }
     if (!there) {
-      timed_out(a);
+      plan_not_carried_out(a);
       v = 0;
     }
     *shared = v;
@@ -744,7 +752,7 @@ struct Summer {
         t_next = slice;
         __syncthreads();                                   // red[] is free again
       }
-      add(have, col, kStepSpinLimit);
+      add(have, col, a.spin_limit);
       if (lost) timed_out(a);
       red[tid] = v_sum;
       __syncthreads();
@@ -787,7 +795,7 @@ __device__ void sum_role(const StepArgs& a, int index, unsigned char* smem) {
   const size_t pairs = (size_t)a.n_streams * (a.d >> 1);
   if (tid < sum.have - sum.have_hit) {
     bool there = false;
-    for (unsigned polls = 0; !there && polls < kStepSpinLimit; ++polls) {
+    for (unsigned polls = 0; !there && polls < a.spin_limit; ++polls) {
       there = has_tag(load_tagged(a.p_new + (tid + 1) * pairs - 1), sum.tag);
       if (!there) __nanosleep(100);
     }
@@ -879,8 +887,8 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   auto release = [&](int rows) {                           // thread 0; rows 0 .. rows - 1 are held
     const unsigned want = (a.epoch + 1) * (unsigned)n_groups;
     unsigned n = 0;
-    while ((int)(ld_acquire(&a.sync->groups_done) - want) < 0 && n < kStepSpinLimit) ++n;
-    if (n == kStepSpinLimit) timed_out(a);
+    while ((int)(ld_acquire(&a.sync->groups_done) - want) < 0 && n < a.spin_limit) ++n;
+    if (n == a.spin_limit) plan_not_carried_out(a);        // rows may be overwritten before they have moved
     for (int j = 0; j < rows; ++j) store_row(j, j);
     released = true;
   };
@@ -1131,6 +1139,7 @@ cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st
   a.fetch_stages = L->step_fetch_stages;
   a.fetch_rows_max = (D.d_ff + kFetchCtas - 1) / kFetchCtas;
   a.wait_polls = L->wait_polls;
+  a.spin_limit = L->spin_limit;
   return launch_k(step_kernel_for(D), dim3(1 + a.n_cache_ctas + kFetchCtas + a.n_sum_ctas),
                   dim3(kStepThreads), L->step_smem, st, L->use_pdl, a);
 }

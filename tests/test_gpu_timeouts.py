@@ -86,7 +86,7 @@ def test_early_copies_given_up_beyond_the_single_launch(append_first):
     B.lif_decode_step(gpu.handle, X[3], y, *streams)
     B.lif_set_tuning(gpu.handle, B.TUNE_WAIT_POLLS, POLLS)
     _rows_after_the_step(gpu, ora)
-    B.lif_clear_status(gpu.handle)
+    B.lif_clear_status(gpu.handle, streams[0])
     B.lif_decode_step(gpu.handle, X[4], y, *streams)
     P.check_decode_step(gpu, ora, X[4].cpu().numpy(), y)
     gpu.close()
@@ -128,7 +128,7 @@ def test_the_single_launch_fills_rows_whose_copies_it_gave_up(S, d, gate_mode, a
         B.lif_decode_step(gpu.handle, X[t], y, *streams)
         if lost:
             _rows_after_the_step(gpu, ora)
-            B.lif_clear_status(gpu.handle)
+            B.lif_clear_status(gpu.handle, streams[0])
         else:
             P.check_decode_step(gpu, ora, X[t].cpu().numpy(), y)
             P.compare_cache_rows(gpu, ora)
@@ -152,4 +152,66 @@ def test_cached_rows_whose_copies_were_given_up_leave_the_layer_usable():
     B.lif_clear_status(gpu.handle)
     B.lif_decode_step(gpu.handle, X[2], y)
     P.check_decode_step(gpu, ora, X[2].cpu().numpy(), y)
+    gpu.close()
+
+
+@pytest.mark.parametrize("S,gate_mode,ffn_mode,append_first", [
+    (1, B.GATE_NONE, 0, 0), (1, B.GATE_NONE, 0, 1), (1, B.GATE_NONE, 1, 0), (1, B.GATE_BUNDLED, 0, 0),
+    (1, B.GATE_BUNDLED, 0, 1), (4, B.GATE_NONE, 0, 0), (4, B.GATE_NONE, 0, 1)])
+def test_rows_named_by_a_step_whose_parts_gave_up_are_read_again_when_the_status_is_cleared(
+        S, gate_mode, ffn_mode, append_first):
+    # Every wait of a CTA for another gives up at once: the window CTA commits the plan, no row of it is
+    # moved or brought in.  No copy is left behind: those asked for ahead of the plan are waited for.
+    gpu, ora, X, y, streams = _layer(S=S, steps=0 if ffn_mode else 4, gate_mode=gate_mode, ffn_mode=ffn_mode,
+                                     append_first=append_first)
+    for t in range(4 if ffn_mode else 0):
+        B.lif_decode_step(gpu.handle, X[t], y, *streams)
+        lists = ora.cache.window_update(gpu.lists()["active_idx"])
+        ora.cache.insert(lists, ora.bundles, ora.bias_up)
+    P.compare_cache_rows(gpu, ora)
+    B.lif_set_tuning(gpu.handle, B.TUNE_STEP_POLLS, 0)
+    B.lif_decode_step(gpu.handle, X[4], y, *streams)
+    B.lif_set_tuning(gpu.handle, B.TUNE_STEP_POLLS, 1 << 20)
+    g = gpu.lists()
+    assert g["status"] == B.LIF_ERR_TIMEOUT
+    lists = ora.cache.window_update(g["active_idx"])
+    ora.cache.insert(lists, ora.bundles, ora.bias_up)
+    for key in P.LIST_KEYS:
+        np.testing.assert_array_equal(g[key], lists[key], err_msg=key)
+    assert len(lists["load_ids"]) > 0 and (append_first or len(lists["move_src"]) > 0)
+    rows = gpu.cache[torch.tensor(lists["load_slots"], device=DEV).long()].cpu().numpy()
+    assert not np.array_equal(rows, ora.bundles[lists["load_ids"]])          # nothing has come in
+    B.lif_decode_step(gpu.handle, X[5], y, *streams)                         # refused
+    after = gpu.lists()
+    assert after["status"] == B.LIF_ERR_TIMEOUT and after["step"] == g["step"]
+    np.testing.assert_array_equal(after["pointers"], g["pointers"])
+    B.lif_clear_status(gpu.handle, streams[0])
+    torch.cuda.synchronize()
+    P.compare_cache_rows(gpu, ora)
+    B.lif_decode_step(gpu.handle, X[5], y, *streams)
+    g = gpu.lists()
+    assert g["status"] == B.LIF_OK
+    if ffn_mode == 0:
+        P.check_decode_step(gpu, ora, X[5].cpu().numpy(), y)
+    else:                                                                    # FFN over every cached row
+        lists = ora.cache.window_update(g["active_idx"])
+        ora.cache.insert(lists, ora.bundles, ora.bias_up)
+        ref, flips = P.ffn_reference(ora, np.arange(ora.cache.num_used), X[5].cpu().numpy())
+        P.assert_y_close(y.cpu().numpy().astype(np.float64), ref, flips)
+    P.compare_cache_rows(gpu, ora)
+    with pytest.raises(B.LifError):
+        B.lif_set_tuning(gpu.handle, B.TUNE_STEP_POLLS, -1)
+    gpu.close()
+
+
+def test_clearing_another_status_leaves_the_cached_rows_alone():
+    gpu, ora, X, y, streams = _layer()
+    marked = torch.full_like(gpu.cache[0], 7.0)
+    gpu.cache[0].copy_(marked)
+    bad = torch.tensor([-1], dtype=torch.int32, device=DEV)
+    B.lif_sparse_ffn(gpu.handle, X[0], bad, torch.ones(1, dtype=torch.int32, device=DEV), y)
+    assert B.lif_get_stats(gpu.handle).status == B.LIF_ERR_INVALID_ARG
+    B.lif_clear_status(gpu.handle)
+    assert B.lif_get_stats(gpu.handle).status == B.LIF_OK
+    assert torch.equal(gpu.cache[0], marked)
     gpu.close()
