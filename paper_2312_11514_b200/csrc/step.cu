@@ -555,13 +555,14 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
   __shared__ __align__(8) uint64_t bars[16];
   __shared__ float h_s[16][kS], b_s[16];
   __shared__ unsigned long long plan_s;
-  __shared__ int last_s;
+  __shared__ int last_s, lost_s;       // (lost_s: as a barrier's reduction 0.4 us a step more)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int d = a.d, S = a.n_streams, nvec = d >> 3, stages = a.cache_stages, nc = a.n_cache_ctas;
   const unsigned row_bytes = 2u * kVec * d;
   uint4* xs = reinterpret_cast<uint4*>(smem);              // [S][d]
   unsigned char* rows = smem + x_smem_bytes(d, S);
   if (tid == 0) {
+    lost_s = 0;
     for (int i = 0; i < stages; ++i) mbar_init(bars + i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -601,11 +602,10 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
     }
     __syncthreads();                                       // x and the rows' scalars
     if (rc <= 0) break;
-    int lost = 0;
     for (int i = warp; i < rc; i += kStepWarps) {          // a warp per row
       const bool landed = __all_sync(0xffffffffu, mbar_wait(bars + i, parity, a.wait_polls));
       if (!landed) {                                       // flagged; its terms are left out
-        lost = 1;
+        lost_s = 1;
         if (lane == 0) timed_out(a);
         mbar_wait(bars + i, parity);                       // another bounded chance to land
       }
@@ -632,13 +632,13 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
           h_s[i][s] = landed && s < S ? row_weight<kGate>(a, b_s[i], p[s], p2[s]) : 0.f;
       }
     }
-    lost = __syncthreads_or(lost);
+    __syncthreads();
     for (int i = 0; i < rc; ++i) {
       if (kS == 1 && h_s[i][0] == 0.f) continue;
       axpy_row<kS>(acc, reinterpret_cast<const uint4*>(rows + (size_t)i * row_bytes) + (kVec - 1) * nvec,
                    h_s[i], nvec);
     }
-    if (lost) break;                                       // nothing more into stages that may be written late
+    if (lost_s) break;                                     // nothing more into stages that may be written late
     parity ^= 1u;
     if (r0 + stages < cnt) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
