@@ -8,15 +8,14 @@
 //                          already cached (bulk copies into shared memory, a warp per row)
 //   fetch CTAs   (then)    find the new neurons themselves in the predictor's entries, bring their
 //                          bundles over the host link through a ring of bulk copies, add their FFN
-//                          terms from shared memory, copy them to their cache rows, and (one stream) in
-//                          the end add up all partial sums
-//   sum CTAs     (last)    with several streams add up the partial sums
+//                          terms from shared memory, copy them to their cache rows
+//   sum CTAs     (last)    add up the partial sums
 // A CTA whose wait for the plan runs out moves or brings in nothing, although the window CTA commits the
 // state that names those rows.  Like every wait that runs out it flags LIF_ERR_TIMEOUT, which refuses further
 // updates, and it marks the rows as suspect, so that clearing the status reads them from the store again.
-// A CTA waits only for CTAs that took their parts before it (with one stream the fetch CTAs also for
-// one another, at the very end, when nothing else is left to run), every wait is bounded, and every CTA
-// makes its arrivals on all paths, so the counters are complete whatever happened.
+// A CTA waits only for CTAs that took their parts before it and are therefore running, so a step ends
+// however few of its CTAs fit the chip at a time beside other streams' kernels; every wait is bounded,
+// and every CTA makes its arrivals on all paths, so the counters are complete whatever happened.
 //
 // Why one launch: the parts run side by side without an event or a stream of their own (five
 // launches and two event pairs less per layer-step), and the fetch does not wait for the window
@@ -773,10 +772,17 @@ struct Summer {
 
 constexpr size_t kSumSmem = kStepThreads * sizeof(float2);
 
-// ---- sum CTAs (several streams) ------------------------------------------------------------------
-// The outputs of several streams are too long for the fetch CTAs to add up at the end (measured at
-// 5 x 4096: 6.5 us).  These CTAs wait for one word of each fetch CTA's partial, with pauses, so that
-// they do not load the memory system meanwhile, and then read everything at once.
+// ---- sum CTAs ----------------------------------------------------------------------------------------
+// They wait for a word of the fetch CTAs' partials, with pauses, so that they do not load the memory
+// system while the rows travel.  Several streams: for one of each CTA, to read everything at once.  One
+// stream: for one of the CTA with the fewest rows, adding the cached rows' partials meanwhile if they come
+// first, and then they take what is missing as it comes: a single round trip from the last partial,
+// whichever it is, to y.  With at most two rows per fetch CTA the whole wait is a few microseconds and a
+// poll of that word ahead of the partials is what is noticed: 352 x 944, 10 new rows, 2 layers 33.9 us with
+// it and 31.6 without, tiny 29.2 and 27.0; with more rows there is no difference (4096 x 16384, 8 layers
+// 386-388 us) and the memory system is left alone while they travel.
+// (With one stream the fetch CTAs themselves used to do this, waiting for one another.  These CTAs, the
+// same number at 1024 columns and more, measure the same or better: 768 x 3072, 4 layers 65.4 -> 62.8 us.)
 template <int kS>
 __device__ void sum_role(const StepArgs& a, int index, unsigned char* smem) {
   __shared__ unsigned long long plan_s;
@@ -793,7 +799,15 @@ __device__ void sum_role(const StepArgs& a, int index, unsigned char* smem) {
   const bool go = (plan & kPlanReady) && !(plan & kPlanRefused);
   Summer<kS> sum(a, index, a.n_sum_ctas, (int)(plan & 0xfffff), go ? min(kFetchCtas, (int)tot[0]) : 0);
   const size_t pairs = (size_t)a.n_streams * (a.d >> 1);
-  if (tid < sum.have - sum.have_hit) {
+  const int n_new = sum.have - sum.have_hit, n_load = (int)tot[0];
+  if (kS == 1) {
+    for (unsigned polls = 0; n_load > 2 * kFetchCtas && polls < a.spin_limit; ++polls) {
+      const int there = tid == 0 && (n_new == 0 || has_tag(load_tagged(a.p_new + n_new * pairs - 1), sum.tag));
+      sum.add(sum.have_hit, sum.c0 + tid % sum.width, 1);
+      if (__syncthreads_or(there)) break;
+      __nanosleep(100);
+    }
+  } else if (tid < n_new) {
     bool there = false;
     for (unsigned polls = 0; !there && polls < a.spin_limit; ++polls) {
       there = has_tag(load_tagged(a.p_new + (tid + 1) * pairs - 1), sum.tag);
@@ -804,7 +818,7 @@ __device__ void sum_role(const StepArgs& a, int index, unsigned char* smem) {
   sum.finish(reinterpret_cast<float2*>(smem));             // kSumSmem bytes
 }
 
-// ---- fetch CTAs: new bundles over the host link, their FFN terms, and the sum -----------------------
+// ---- fetch CTAs: new bundles over the host link and their FFN terms ---------------------------------
 // Fetch CTA f brings in entries f, f + kFetchCtas, ... of the load list, which is exactly the set
 // bits of the predictor's entries in ascending order; only the cache row comes from the plan.
 template <int kGate, int kS>
@@ -815,7 +829,6 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   __shared__ float part[2][kS][kStepWarps];
   __shared__ float h_s[kS];
   __shared__ unsigned long long plan_s;
-  __shared__ float2 red[kS == 1 ? kStepThreads : 1];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int d = a.d, S = a.n_streams, nvec = d >> 3, stages = a.fetch_stages;
   constexpr int nf = kFetchCtas;
@@ -859,7 +872,6 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
 
   const unsigned long long plan = wait_plan(a, &plan_s);
   const bool go = (plan & kPlanReady) && !(plan & kPlanRefused);
-  const int n_hit = (int)(plan & 0xfffff);
   const int n_groups = (a.n_cache_ctas + a.group_size - 1) / a.group_size;
   if (!go) {
     // the update of this step was refused: nothing is brought in; let the copies land
@@ -893,16 +905,9 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     released = true;
   };
   __syncthreads();
-  // One stream: the fetch CTAs also add up all partial sums (the cached rows' while the last row is on
-  // its way).  Several: that is for the sum CTAs.
-  const unsigned tag = a.epoch + 1;
-  const size_t pairs = (size_t)S * (d >> 1);
-  Summer<kS> sum(a, f, nf, n_hit, go ? min(nf, n_new) : 0);
-
   unsigned parity = 0;
   int from = cnt;                                          // first row that was not waited for any longer
   for (int i = 0, st = 0; i < cnt; ++i) {
-    if (kS == 1 && i == cnt - 1) sum.add(sum.have_hit, sum.c0 + tid % sum.width, 1);
     const uint4* row = reinterpret_cast<const uint4*>(ring + (size_t)st * row_bytes);
     const bool landed = mbar_wait(bars + st, parity, a.wait_polls);
     if (tid == 0 && landed) {
@@ -981,7 +986,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       parity ^= 1u;
     }
   }
-  if (cnt > 0) store_tagged_partial<kS>(acc, a.p_new + (size_t)f * pairs, nvec, S, tag);
+  if (cnt > 0) store_tagged_partial<kS>(acc, a.p_new + (size_t)f * S * (d >> 1), nvec, S, a.epoch + 1);
   if (tid == 0 && cnt > 0 && !released) release(from);
   if (from < cnt) {
     // The window state already names these rows, so they are filled all the same, with plain loads and
@@ -993,7 +998,6 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       for (int v = tid; v < kVec * nvec; v += kStepThreads) dst[v] = ld_stream16(src + v);
     }
   }
-  if (kS == 1) sum.finish(red);
   if (tid == 0) {
     if (f == 0) advance_run(a.next_run, run);
     // (shared memory must outlive the reads of the last rows' copies to the cache)
@@ -1017,7 +1021,7 @@ __global__ void __launch_bounds__(kStepThreads, kS == 1 ? 2 : 1) step_kernel(Ste
   if (part == 0) window_role(a, smem);
   else if (part <= a.n_cache_ctas) cache_role<kGate, kS>(a, part - 1, smem);
   else if (part <= a.n_cache_ctas + kFetchCtas) fetch_role<kGate, kS>(a, part - 1 - a.n_cache_ctas, smem);
-  else if (kS > 1) sum_role<kS>(a, part - 1 - a.n_cache_ctas - kFetchCtas, smem);
+  else sum_role<kS>(a, part - 1 - a.n_cache_ctas - kFetchCtas, smem);
 }
 
 using StepKernel = void (*)(StepArgs);
@@ -1036,20 +1040,23 @@ StepKernel step_kernel_for(const lif_layer_desc& D) {
 constexpr int kGroupMax = 8, kUngroupedMax = 64, kUngroupedMaxStreams = 16;
 constexpr size_t kCacheRing = 128 * 1024, kFetchRing = 32 * 1024;
 
+// CTAs that add up the outputs: 16 pairs of columns or more each, which leaves 16 slices of the partials to
+// a CTA's threads (several streams: 128 pairs).
+int sum_ctas(const lif_layer_desc& D) {
+  const int per = D.n_streams > 1 ? 128 : 16, most = D.n_streams > 1 ? 48 : 32;
+  const int n = (D.n_streams * D.d_model / 2 + per - 1) / per;
+  return n > most ? most : n;
+}
 // CTAs for the rows that are already cached, about a third of which are active in a step: with one
 // stream a CTA per eight rows of the cache; with several one per sixteen, because a CTA's partial is
 // as long as its streams' outputs together.
 int cache_ctas(const lif_layer_desc& D, int n_sm) {
-  const int per = D.n_streams > 1 ? 16 : 8, most = D.n_streams > 1 ? 64 : n_sm - 1 - kFetchCtas;
+  const int per = D.n_streams > 1 ? 16 : 8;
+  const int most = D.n_streams > 1 ? 64 : n_sm - 1 - kFetchCtas - sum_ctas(D);
   const int nc = (D.capacity + per - 1) / per;
   return nc < 8 ? 8 : (nc > most ? most : nc);
 }
-// CTAs that add up the outputs of several streams: 128 pairs of columns each.
-int sum_ctas(const lif_layer_desc& D) {
-  const int n = (D.n_streams * D.d_model / 2 + 127) / 128;
-  return n > 48 ? 48 : n;
-}
-// Tagged partials of cache CTAs (or of groups of them) that the fetch CTAs add up at the end.
+// Tagged partials of cache CTAs (or of groups of them) that the sum CTAs add up.
 int hit_partials_max(const lif_layer_desc& D) {
   return D.n_streams > 1 ? kUngroupedMaxStreams : kUngroupedMax;
 }
@@ -1088,7 +1095,7 @@ cudaError_t step_configure(lif_layer* L) {
     return s < least ? least : (s > 16 ? 16 : s);
   };
   L->step_cache_ctas = cache_ctas(D, L->n_sm);
-  L->step_sum_ctas = D.n_streams > 1 ? sum_ctas(D) : 0;
+  L->step_sum_ctas = sum_ctas(D);
   L->step_group = L->step_cache_ctas > hit_partials_max(D) ? kGroupMax : 1;
   L->step_cache_stages = stages(kCacheRing, x, 1);
   // (paper's cache order: bundles wait in the ring, see fetch_role; twice the ring keeps the link busy)
@@ -1097,7 +1104,7 @@ cudaError_t step_configure(lif_layer* L) {
   const size_t need_c = x + L->step_cache_stages * row, need_f = x + L->step_fetch_stages * row + ids;
   if (need_c > smem) smem = need_c;
   if (need_f > smem) smem = need_f;
-  if (D.n_streams > 1 && smem < kSumSmem) smem = kSumSmem;
+  if (smem < kSumSmem) smem = kSumSmem;
   if (smem > (size_t)max_smem) return cudaSuccess;
   L->step_smem = smem;
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);

@@ -77,3 +77,32 @@ def test_a_refused_update_brings_nothing_in_and_the_next_step_follows_the_oracle
         np.testing.assert_array_equal(y.cpu().numpy(), want)
         B.lif_clear_status(gpu.handle)
     gpu.close()
+
+
+def test_steps_of_more_layers_than_the_chip_holds_at_a_time():
+    # Eight layers on streams of their own and of several priorities: their steps together have more CTAs
+    # than there are SMs, and rows of 16 KB leave room for one CTA on an SM.  Every CTA of a step must get by
+    # without those that have not started yet; outputs and state are those of the layers run one by one.
+    cfg = W.LifConfig("together", 8, 4096, 2048, 32, 3, 1, 10, 0.08, 1.0, 0.8, 0.6, 73)
+    pairs = [P.make_layer_pair(cfg, l, b_down=True, append_first=l % 2) for l in range(cfg.n_layers)]
+    X = W.make_inputs(cfg, device=DEV)
+    greatest = torch.cuda.Stream.priority_range()[1]
+    streams = [torch.cuda.Stream(priority=max(greatest, -(l % 4))) for l in range(cfg.n_layers)]
+    y = torch.empty(2, cfg.steps, cfg.n_layers, cfg.d_model, dtype=torch.float32, device=DEV)
+    state = []
+    for together in (0, 1):
+        torch.cuda.synchronize()
+        for t in range(cfg.steps):
+            for l, (gpu, _) in enumerate(pairs):
+                B.lif_decode_step(gpu.handle, X[t], y[together, t, l], streams[l if together else 0], None)
+        torch.cuda.synchronize()
+        state.append([gpu.lists() for gpu, _ in pairs])
+        for gpu, _ in pairs:
+            B.lif_reset(gpu.handle)
+    assert torch.equal(y[0], y[1])
+    for one, other in zip(*state):
+        assert one["status"] == other["status"] == B.LIF_OK and one["step"] == cfg.steps
+        for key in ("pointers", "slot_of", "last_active"):
+            np.testing.assert_array_equal(one[key], other[key])
+    for gpu, _ in pairs:
+        gpu.close()
