@@ -209,9 +209,10 @@ scores_multi_kernel(const float* __restrict__ z_partial, int P, const __half* __
   const int n = tid & (kLogitTile - 1), my_col = blockIdx.x * kLogitTile + n;
   const float my_c = my_col < F ? c[my_col] : 0.f;
   const int my_row = my_col < F ? slot_of[my_col] : 0;
-  // released before this kernel's own wait: see predict_logits_kernel
-  pdl_trigger();
+  // released before this kernel's own wait, unless it compacts: see predict_logits_kernel
+  if (!compact) pdl_trigger();
   pdl_wait();
+  if (compact) pdl_trigger();
   const int run = (tid < kLogitTile && (tid & 31) == 0) ? __ldcg(predictor_run) : 0;
   if (P == 1) {                                              // z is finished: all loads in flight
     for (int j = tid; j < r; j += kThreads) {
