@@ -337,11 +337,16 @@ lif_status lif_sum_peer_outputs(const float* const* dev_partials, int32_t n_peer
                                 size_t n_floats, void* stream);
 
 /* One token through the layer: predict -> window update -> fetch -> sparse FFN (ffn_mode
- * selects the rows).  Two streams let the bundle fetch overlap the part of the FFN that does
- * not need the new rows; which of the two kernels runs on `fetch_stream` is the library's
- * choice (ordering is by events inside the call).  The compute stream ends up ordered after
- * everything, so consecutive calls on the same streams are safe.  Passing the same stream
- * twice runs the step serially. */
+ * selects the rows).  Everything behind the predictor is one kernel on `compute_stream`, in which
+ * window update, fetch and FFN run side by side and which does not use `fetch_stream`, for one input
+ * stream and, with plain bundles, for two (any width), up to four (d_model <= 8192) and up to eight
+ * (d_model <= 4096), where d_ff <= 32768 and the window arrays (about 4*d_ff + 8*capacity bytes)
+ * fit the shared memory of a CTA.  Otherwise the step is several kernels: a second stream lets the
+ * bundle fetch overlap the part of the FFN that does not need the new rows (which of them runs
+ * on `fetch_stream` is the library's choice, ordering is by events inside the call), and passing
+ * the same stream twice runs them serially.  Either way the compute stream ends up ordered
+ * after everything, so consecutive calls on the same streams are safe.  Different layers may be
+ * stepped at the same time on different streams. */
 lif_status lif_decode_step(lif_layer* layer, const void* dev_x, float* dev_y,
                            void* compute_stream, void* fetch_stream);
 

@@ -69,7 +69,8 @@ enum {
 
 /* Profiling aid: with n_steps > 0, the next n_steps calls of lif_decode_step record CUDA
  * events around every kernel (host-side event objects, no device memory); n_steps = 0 turns
- * it off and frees the events.  lif_timing_read synchronises the device and returns, per
+ * it off and frees the events.  A step that is recorded runs as separate kernels also where it
+ * would otherwise be one launch behind the predictor, so the phases are not that launch's.  lif_timing_read synchronises the device and returns, per
  * phase, the summed device time in microseconds over the steps recorded since enabling. */
 lif_status lif_timing_enable(lif_layer* layer, int32_t n_steps);
 lif_status lif_timing_read(lif_layer* layer, float* host_us_sums /* [LIF_PHASE_LEN] */,

@@ -1,5 +1,6 @@
 // C ABI of liblif.so: argument checking, workspace carve-up and stream/event orchestration.
-// Every step of the path runs in the kernels of predict.cu / window.cu / fetch.cu / ffn.cu.
+// Every step of the path runs in the kernels of predict*.cu / gate.cu / step.cu, or of window.cu /
+// fetch.cu / ffn*.cu where the calls are made one by one or the single launch does not apply.
 #include <new>
 
 #include "lif_internal.cuh"

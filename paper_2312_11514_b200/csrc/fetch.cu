@@ -49,6 +49,9 @@ __device__ __forceinline__ void gather_rows(const uint4* __restrict__ src_base,
 // their sum do not depend on scheduling.  Where the kernel ahead is the row-move kernel, the
 // first bundle's host loads are issued before the dependency wait: the list and the counts were
 // final before that kernel passed its own wait, while the cache rows may still be moving.
+// A decode step runs it only where it is not one launch behind the predictor (step.cu): d_ff above 32768
+// (without the mask-driven forms), window arrays that exceed a CTA's shared memory, a knob or
+// lif_timing_enable.
 constexpr int kFusedChunks = 4;     // 8-column chunks per thread and half row: d_model <= 8192
 
 // The predictor's entries of neurons to bring in, and where the run number lives.

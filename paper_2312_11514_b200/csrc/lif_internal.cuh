@@ -178,14 +178,15 @@ inline int new_mask_entries(const lif_layer_desc& D) {
 enum { kEarlyNone = 0, kEarlyLists = 1, kEarlyMask = 2, kEarlyWatch = 3 };
 cudaError_t launch_fetch_ffn(lif_layer* L, const __half* x, float* partial, cudaStream_t st,
                              int early);
-// Everything of a single-stream decode step behind the predictor, in one launch (step.cu).
-size_t step_sync_bytes();
-size_t step_tagged_bytes(const lif_layer_desc& D);
 cudaError_t predict_configure(const lif_layer* L);
 // several input streams (predict_multi.cu)
 cudaError_t predict_multi_configure(const lif_layer* L);
 cudaError_t launch_predict_multi(lif_layer* L, const __half* x, float* logits, int32_t* active_idx,
                                  int32_t* n_active, cudaStream_t st, cudaEvent_t* ev, int compact);
+// Everything of a decode step behind the predictor, in one launch (step.cu): one input stream, or several
+// as long as their output fits a CTA's registers.
+size_t step_sync_bytes();
+size_t step_tagged_bytes(const lif_layer_desc& D);
 cudaError_t step_configure(lif_layer* L);
 cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st);
 cudaError_t launch_refill(lif_layer* L, cudaStream_t st);

@@ -65,9 +65,6 @@ struct WindowArgs {
   unsigned long long bundle_bytes;
 };
 
-// Memory-budgeted window (Appendix C, Persimmon 8B / Phi-2): hist[a] = cached rows that are not
-// active now and were last active a steps ago (a = 1 .. k, older ones in bin k).  Returns the
-// widest window k' <= k for which the rows kept plus the rows to load fit `limit`, at least 1.
 // Stamp of an active neuron: the time of the last kept token in which it is active (its old
 // stamp if it is active only beyond the kept token), but never below the oldest stamp still
 // inside the window that ends at t_end: this step does not delete it, the next one may.
@@ -79,6 +76,9 @@ __device__ __forceinline__ int active_stamp(const WindowArgs& a, int id, int t, 
 
 WindowArgs window_args(lif_layer* L, const int32_t* act, const int32_t* n_act);
 
+// Memory-budgeted window (Appendix C, Persimmon 8B / Phi-2): hist[a] = cached rows that are not
+// active now and were last active a steps ago (a = 1 .. k, older ones in bin k).  Returns the
+// widest window k' <= k for which the rows kept plus the rows to load fit `limit`, at least 1.
 constexpr int kMaxBudgetWindow = 32;
 __device__ __forceinline__ int widest_window_that_fits(const int* hist, int k, int n, int n_load,
                                                        int limit) {
