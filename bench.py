@@ -8,10 +8,11 @@ sparse FFN, every layer, one token per step) on seeded synthetic data.
 One step = one decode token through all layers of the configuration.  `value` is tokens/s
 with the decode inputs resident in HBM (the bundle store stays in pinned host memory: reading
 it is part of the method); `e2e` passes pinned HOST inputs/outputs through
-lif_graph_launch_host.  A token is one CUDA graph (lif_graph_capture).  Per-kernel durations
-for the roofline come from a further pass after the timed tokens: for each kernel, a graph of
-that one kernel on every layer (the lists of the last token) is replayed and timed with CUDA
-events.  With --gpus N > 1 and no torchrun environment the script starts its own N ranks.
+lif_graph_launch_host.  A token is one CUDA graph (lif_graph_capture).  With one input stream a
+layer-step is the predictor and step_kernel, which cannot be replayed alone (it updates the
+window): its time for the roofline is the layer-step's less the predictor's.  The durations of
+the other kernels come from a further pass after the timed tokens: for each, a graph of that one
+kernel on every layer (the lists of the last token) is replayed and timed with CUDA events.  With --gpus N > 1 and no torchrun environment the script starts its own N ranks.
 """
 from __future__ import annotations
 
@@ -33,8 +34,8 @@ NOMINAL_HBM_GBS = 8000.0
 # dram__bytes_read.sum + dram__bytes_write.sum over algorithmic bytes of sparse_ffn_kernel, from
 # the ncu capture summarised under profiles/ (set to None when that kernel changes)
 FFN_TRAFFIC_RATIO = 1.003
-# fetch_ffn_kernel: bytes read from system memory per bundle byte, same kind of capture
-FETCH_TRAFFIC_RATIO = 1.000
+# step_kernel: bytes read from system memory per bundle byte, same kind of capture
+STEP_LINK_TRAFFIC_RATIO = 1.000
 FALLBACK_HBM_GBS = 6650.0
 _LINK_PEAK = {}          # measured pinned host -> device rate per local device, GB/s
 
@@ -312,7 +313,7 @@ def measure(args, config_name, steps, warmup, rank, world, local, detail):
                      for kind, name in enumerate(B.KERNELS)
                      if not (gate_mode == B.GATE_RESIDENT and name == "predict_z")}
         if not detail:
-            launchers = {k: v for k, v in launchers.items() if k in ("fetch", "ffn_active", "ffn_hits", "ffn_new")}
+            launchers = {k: v for k, v in launchers.items() if k in ("predict_z", "predict_scores", "fetch", "ffn_active", "ffn_hits", "ffn_new")}
         if args.append_first == 0 and "ffn_cache" in launchers:
             pass      # rows [0, num_used) are the cache in both orders once a step is complete
     else:
@@ -367,8 +368,7 @@ def measure(args, config_name, steps, warmup, rank, world, local, detail):
         all_bytes = (n_act_l * (beta + row_extra) + L * S * 6 * d) / L
         all_gbs = all_bytes / (kernel_us["ffn_active"] * 1e-6) / 1e9
         if S == 1:
-            # the launch the decode step makes: the rows that were already cached (the new rows'
-            # terms are added by the fetch kernel, or by a second launch for three-vector bundles)
+            # sparse_ffn_kernel over the rows that were already cached
             ffn_bytes = (n_hit_l * (beta + row_extra) + L * 6 * d) / L
             ffn_us = kernel_us["ffn_hits"]
         else:
@@ -376,29 +376,66 @@ def measure(args, config_name, steps, warmup, rank, world, local, detail):
         ffn_gbs = ffn_bytes / (ffn_us * 1e-6) / 1e9
         fetch_bytes = n_load_l * beta / L
         fetch_gbs = fetch_bytes / (kernel_us["fetch"] * 1e-6) / 1e9
-        predictor = None
-        if detail or S > 1:
-            if gate_mode == B.GATE_RESIDENT:       # gate matrix + bias in, gate values out
-                pred_bytes = 2 * cfg.d_ff * d + 2 * cfg.d_ff + 4 * S * cfg.d_ff
-                pred_us = kernel_us["predict"] if S > 1 else kernel_us["predict_scores"]
-            else:
-                pred_bytes = 2 * cfg.rank * (d + cfg.d_ff) + 4 * cfg.d_ff
-                pred_us = kernel_us["predict"] if S > 1 else kernel_us["predict_z"] + kernel_us["predict_scores"]
-            pred_gbs = pred_bytes / (pred_us * 1e-6) / 1e9
-            predictor = {"bound": "hbm", "achieved": pred_gbs, "unit": "GB/s", "frac": pred_gbs / peak,
-                         "bytes_per_launch": pred_bytes, "us_per_launch": pred_us}
-        split = None
+        if gate_mode == B.GATE_RESIDENT:       # gate matrix + bias in, gate values out
+            pred_bytes = 2 * cfg.d_ff * d + 2 * cfg.d_ff + 4 * S * cfg.d_ff
+            pred_us = kernel_us["predict"] if S > 1 else kernel_us["predict_scores"]
+        else:
+            pred_bytes = 2 * cfg.rank * (d + cfg.d_ff) + 4 * cfg.d_ff
+            pred_us = kernel_us["predict"] if S > 1 else kernel_us["predict_z"] + kernel_us["predict_scores"]
+        pred_gbs = pred_bytes / (pred_us * 1e-6) / 1e9
+        predictor = {"bound": "hbm", "achieved": pred_gbs, "unit": "GB/s", "frac": pred_gbs / peak,
+                     "bytes_per_launch": pred_bytes, "us_per_launch": pred_us}
+        link = {"bound": "host_link", "peak": link_peak, "unit": "GB/s",
+                "peak_kind": "of measured (1 GiB pinned cudaMemcpyAsync, this run)"}
+        separate = None
         if S == 1:
-            split = {"all_active_rows": {"GBs": all_gbs, "us_per_launch": kernel_us["ffn_active"],
-                                         "bytes_per_launch": all_bytes, "frac": all_gbs / peak},
-                     "new_rows_GBs": (n_load_l * (beta + row_extra) / L + 6 * d) / (kernel_us["ffn_new"] * 1e-6) / 1e9}
+            # the kernel that runs: window update, row moves, fetch, FFN and sum in one launch
+            step_bytes = fetched / (K * L)
+            step_us = ms_total * 1e3 / (K * L) - pred_us
+            step_gbs = step_bytes / (step_us * 1e-6) / 1e9
+            roofline = {"kernel": "step_kernel" if not args.tune else
+                                  "everything behind the predictor (a knob may select separate kernels)", **link, "achieved": step_gbs, "frac": step_gbs / link_peak,
+                        "bytes_per_launch": step_bytes, "us_per_launch": step_us,
+                        "traffic": STEP_LINK_TRAFFIC_RATIO * step_bytes
+                                   if STEP_LINK_TRAFFIC_RATIO and not gate_mode else None,
+                        "traffic_how": "system-memory bytes read per bundle byte from the ncu capture in "
+                                       "profiles/step_kernel_opt6p7b_12layers.md, times this run's bundle "
+                                       "bytes per launch",
+                        "how": "bundle bytes of a layer-step over the layer-step's time in the timed tokens "
+                               "less the predictor's (replayed alone): the boundaries around both (and, with "
+                               "--shard neurons, the exchange) count as the step kernel's"}
+            host_link = dict(roofline)
+            separate = {"note": "not launched by lif_decode_step at this shape: the staged calls' and the knobs' "
+                                "kernels, replayed on the last token's lists",
+                        "fetch": {"kernel": "fetch_ffn_kernel" if gate_mode != B.GATE_BUNDLED
+                                            else "fetch_ring_kernel",
+                                  "GBs": fetch_gbs, "us_per_launch": kernel_us["fetch"],
+                                  "bytes_per_launch": fetch_bytes, "frac": fetch_gbs / link_peak},
+                        "ffn_cached_rows": {"kernel": "sparse_ffn_kernel", "GBs": ffn_gbs, "us_per_launch": ffn_us,
+                                            "bytes_per_launch": ffn_bytes, "frac": ffn_gbs / peak,
+                                            "traffic": FFN_TRAFFIC_RATIO * ffn_bytes
+                                                       if FFN_TRAFFIC_RATIO and not gate_mode else None}}
+            separate.update({"all_active_rows": {"GBs": all_gbs, "us_per_launch": kernel_us["ffn_active"],
+                                                 "bytes_per_launch": all_bytes, "frac": all_gbs / peak},
+                             "new_rows_GBs": (n_load_l * (beta + row_extra) / L + 6 * d) / (kernel_us["ffn_new"] * 1e-6) / 1e9})
             if "ffn_cache" in kernel_us:
                 # the same kernel over every cached row (Section 3.3 item 3 as written)
                 cache_bytes = (n_used_l * (beta + row_extra) + L * 6 * d) / L
                 cache_gbs = cache_bytes / (kernel_us["ffn_cache"] * 1e-6) / 1e9
-                split["whole_cache"] = {"GBs": cache_gbs, "us_per_launch": kernel_us["ffn_cache"],
-                                        "bytes_per_launch": cache_bytes, "frac": cache_gbs / peak,
-                                        "rows_per_launch": n_used_l / L}
+                separate["whole_cache"] = {"GBs": cache_gbs, "us_per_launch": kernel_us["ffn_cache"],
+                                           "bytes_per_launch": cache_bytes, "frac": cache_gbs / peak,
+                                           "rows_per_launch": n_used_l / L}
+        else:
+            roofline = {"kernel": "ffn_batched_up_kernel + ffn_batched_down_kernel + ffn_reduce_kernel",
+                        "bound": "hbm", "achieved": ffn_gbs, "peak": peak, "unit": "GB/s", "frac": ffn_gbs / peak,
+                        "peak_kind": f"of {peak_kind}", "frac_of_nominal_8TBs": ffn_gbs / NOMINAL_HBM_GBS,
+                        "traffic": None, "us_per_launch": ffn_us, "bytes_per_launch": ffn_bytes,
+                        "how": "graph of these kernels on every layer, over the active rows of the last token "
+                               "(the decode step runs them over the cached rows beside the fetch and over the "
+                               f"new rows behind it), {reps} replays, CUDA events"}
+            host_link = {"kernel": "fetch_ring_kernel", **link, "achieved": fetch_gbs,
+                         "frac": fetch_gbs / link_peak, "bytes_per_launch": fetch_bytes,
+                         "us_per_launch": kernel_us["fetch"], "traffic": None}
         out = {
             "metric": METRIC, "value": whole_job_tokens_per_s(K, 1 if sharded else world, ms_total), "unit": UNIT,
             "n_gpus": world, "steps": K, "warmup": Wm, "ms_per_step": ms_total / K,
@@ -410,7 +447,7 @@ def measure(args, config_name, steps, warmup, rank, world, local, detail):
                                       "deletions first, then new neurons stacked (Section 3.3 as written)",
                        "l2": "per-token working set (all layers' window caches, "
                              f"{s1[3] / n_tok * beta / 2**20:.0f} MiB) exceeds the 126 MB L2",
-                       "bundle_store": "pinned host memory, read by the fetch kernel",
+                       "bundle_store": "pinned host memory, read by the kernels",
                        "parallelism": f"one sequence, neurons of every layer split over {world} GPUs, "
                                       f"partial outputs summed after every layer ({args.exchange})"
                                       if sharded else "independent sequence per GPU"},
@@ -421,32 +458,9 @@ def measure(args, config_name, steps, warmup, rank, world, local, detail):
             # several: window, moves, fetch, up + down for cached and for new rows, sum
             "gpu_launches": ((3 if S == 1 else 10) - (1 if gate_mode == B.GATE_RESIDENT else 0)
                              + (2 if gate_mode == B.GATE_BUNDLED and S > 1 else 0)) * n_launch,
-            "roofline": {"kernel": "sparse_ffn_kernel" if S == 1 else
-                                   "ffn_batched_up_kernel + ffn_batched_down_kernel + ffn_reduce_kernel",
-                         "bound": "hbm",
-                         "achieved": ffn_gbs, "peak": peak, "unit": "GB/s", "frac": ffn_gbs / peak,
-                         "peak_kind": f"of {peak_kind}", "frac_of_nominal_8TBs": ffn_gbs / NOMINAL_HBM_GBS,
-                         "traffic": FFN_TRAFFIC_RATIO * ffn_bytes
-                                    if FFN_TRAFFIC_RATIO and S == 1 and not gate_mode else None,
-                         "traffic_how": "dram read+write bytes per algorithmic byte from the ncu capture in "
-                                        "profiles/sparse_ffn_kernel_opt6p7b_12layers.md (12 layers, "
-                                        "277-463 rows per launch), scaled by this run's rows per launch",
-                         "us_per_launch": ffn_us,
-                         "bytes_per_launch": ffn_bytes,
-                         "how": ("graph of this kernel on every layer, over the rows of the last token "
-                                 "that were already cached (the decode step's launch)" if S == 1 else
-                                 "graph of these kernels on every layer, over the active rows of the "
-                                 "last token") + f", {reps} replays, CUDA events",
-                         "other_launches": split},
-            "host_link": {"kernel": "fetch_ffn_kernel" if S == 1 and gate_mode != B.GATE_BUNDLED
-                                    else "fetch_ring_kernel", "bound": "host_link", "achieved": fetch_gbs,
-                          "peak": link_peak, "unit": "GB/s", "frac": fetch_gbs / link_peak,
-                          "peak_kind": "of measured (1 GiB pinned cudaMemcpyAsync, this run)",
-                          "bytes_per_launch": fetch_bytes, "us_per_launch": kernel_us["fetch"],
-                          "traffic": FETCH_TRAFFIC_RATIO * fetch_bytes if S == 1 and not gate_mode else None,
-                          "traffic_how": "system-memory bytes read per algorithmic byte from the ncu capture "
-                                         "in profiles/fetch_ffn_kernel_opt6p7b_12layers.md, scaled by this "
-                                         "run's rows per launch"},
+            "roofline": roofline,
+            "host_link": host_link,
+            "separate_kernels": separate,
             "predictor": predictor,
             "kernel_us_per_launch": kernel_us,
             "per_token": {"rows_active": rows_active / K, "rows_loaded": fetched / beta / K,
@@ -496,7 +510,7 @@ def run_kernel_loop(args):
         for h in handles:
             B.lif_set_tuning(h, getattr(B, "TUNE_" + key.upper()), int(value))
     L, S, d = len(layers), cfg.n_streams, cfg.d_model
-    X = _inputs(cfg, args.warmup, dev, W)
+    X = _inputs(cfg, args.warmup + 1, dev, W)
     Y = torch.empty(L, S, d, dtype=torch.float32, device=dev)
     dev_x = torch.empty(S, d, dtype=torch.float16, device=dev)
     sc, sf = torch.cuda.Stream(), torch.cuda.Stream()
@@ -511,12 +525,16 @@ def run_kernel_loop(args):
            "fetch": B.CNT_N_LOAD, "ffn_api": B.CNT_N_ACTIVE}.get(args.kernel_loop)
     rows = [int(l.counts[cnt]) for l in layers] if cnt is not None else None
     for l in range(L):
-        if args.kernel_loop == "ffn_api":     # lif_sparse_ffn over the active rows, any stream count
+        if args.kernel_loop == "step":        # the rows are known afterwards: brought in, active
+            B.lif_decode_step(handles[l], X[args.warmup], Y[l], sc, sf)
+        elif args.kernel_loop == "ffn_api":     # lif_sparse_ffn over the active rows, any stream count
             B.lif_sparse_ffn(handles[l], dev_x, layers[l]._view("active_slots", cfg.d_ff),
                              layers[l].counts[B.CNT_N_ACTIVE:], Y[l], sc)
         else:
             B.lif_profile_launch(handles[l], B.KERNELS.index(args.kernel_loop), dev_x, Y[l], sc)
     torch.cuda.synchronize()
+    if args.kernel_loop == "step":
+        rows = [[int(l.counts[B.CNT_N_LOAD]), int(l.counts[B.CNT_N_ACTIVE])] for l in layers]
     print(json.dumps({"kernel": args.kernel_loop, "layers": L, "warmup_tokens": args.warmup,
                       "rows_per_launch": rows,
                       "bundle_bytes": (3 if gate_mode == 1 else 2) * d * 2}), flush=True)
@@ -964,7 +982,8 @@ def main():
     ap.add_argument("--kernel-loop", default=None,
                     help="profiling aid: after the warm-up tokens launch this kernel once per layer "
                          "(predict_z, predict_scores, fetch, ffn_active, ffn_hits, ffn_new, ffn_sum; "
-                         "ffn_api = lif_sparse_ffn over the active rows, for any number of streams)")
+                         "ffn_api = lif_sparse_ffn over the active rows, for any number of streams; step = "
+                         "lif_decode_step with the next token, as plain launches)")
     ap.add_argument("--sweep-k", default=None,
                     help="comma-separated window sizes: memory-latency trade-off, one line per k")
     args = ap.parse_args()
