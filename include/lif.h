@@ -17,8 +17,8 @@
  *    sticky device status word and reported by lif_get_stats: a cache overflow or a bad neuron
  *    id (the window update of that step is refused, the window state untouched); a row index
  *    outside the cache given to the sparse FFN (the row is not read and contributes nothing); a
- *    bounded wait that ran out (LIF_ERR_TIMEOUT: that call's output lacks some rows'
- *    terms; the window bookkeeping stays consistent, and while this status stands every
+ *    bounded wait that ran out (LIF_ERR_TIMEOUT: that call's output is not to be used,
+ *    some rows' terms are missing or an earlier call's; the window bookkeeping stays consistent, and while this status stands every
  *    further window update is refused — lif_clear_status resumes).  The first condition stands
  *    until it is cleared, except that LIF_ERR_TIMEOUT takes the place of any other.
  *  - fp16 = IEEE binary16; accumulations are fp32.
@@ -267,7 +267,7 @@ lif_status lif_sparse_ffn(lif_layer* layer, const void* dev_x, const int32_t* de
  * Conditions only the kernels can see go to a status word inside the same array, which stays
  * set until it is read: lif_sparse_ffn_static_status synchronises the device, copies the word
  * (a lif_status: LIF_OK, LIF_ERR_INVALID_ARG for a refused row or count, LIF_ERR_TIMEOUT for a
- * bounded wait that ran out — the output of that call then lacks some rows' terms) to
+ * bounded wait that ran out — the output of that call is then not to be used) to
  * *host_status and, with clear != 0, resets it.  It allocates nothing either. */
 #define LIF_STATIC_MAX_D_MODEL 8192
 lif_status lif_sparse_ffn_static(const void* dev_matrix, int32_t n_rows, const void* dev_bias,
