@@ -17,10 +17,11 @@
  *    sticky device status word and reported by lif_get_stats: a cache overflow or a bad neuron
  *    id (the window update of that step is refused, the window state untouched); a row index
  *    outside the cache given to the sparse FFN (the row is not read and contributes nothing); a
- *    bounded wait that ran out (LIF_ERR_TIMEOUT: that call's output is not to be used,
- *    some rows' terms are missing or an earlier call's; the window bookkeeping stays consistent, and while this status stands every
- *    further window update is refused — lif_clear_status resumes).  The first condition stands
- *    until it is cleared, except that LIF_ERR_TIMEOUT takes the place of any other.
+ *    bounded wait that ran out (LIF_ERR_TIMEOUT: that call's output is not to be used, some rows'
+ *    terms are missing or an earlier call's; the window bookkeeping stays consistent, and while
+ *    this status stands every further window update is refused — lif_clear_status resumes).
+ *    The first condition stands until it is cleared, except that LIF_ERR_TIMEOUT takes the
+ *    place of any other.
  *  - fp16 = IEEE binary16; accumulations are fp32.
  *  - All counts the kernels need (n_active, n_load, ...) stay in device memory; no call
  *    needs them on the host to launch the next one.

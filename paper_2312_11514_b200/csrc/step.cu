@@ -1080,7 +1080,7 @@ cudaError_t step_configure(lif_layer* L) {
   L->step_ok = 0;
   StepKernel kernel = step_kernel_for(D);
   if (!kernel || new_mask_entries(D) > kEntriesPerThread * kStepThreads || D.d_ff > 32768 ||
-      new_mask_entry_bits(D) != 32 || D.window_k > 32767 || L->n_sm < 2 * kFetchCtas)
+      new_mask_entry_bits(D) != 32 || D.window_k > 32767 || L->n_sm < 3 * kFetchCtas)   // (sum CTAs: <= 48)
     return cudaSuccess;
   int dev = 0, max_smem = 0;
   cudaError_t e = cudaGetDevice(&dev);
