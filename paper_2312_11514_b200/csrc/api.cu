@@ -37,7 +37,7 @@ Workspace plan_workspace(const lif_layer_desc& d, int ffn_grid_max) {
   w.n_tmp = take(64);
   w.z_partial = take(z_ctas * S * d.rank * 4);
   w.mask_words = take(n_mask * 4);
-  w.new_mask_words = take((size_t)new_mask_entries(d) * 2 * 8);
+  w.new_mask_words = take(tagged_words(d) * 8);
   w.keep_tok = take(d.spec_keep > 0 ? F : 0);
   w.h_rows = take(d.n_streams > 1 ? (size_t)kBatchedMaxKSplit * F * 8 * 4 *
                                         (d.gate_mode == LIF_GATE_BUNDLED ? 2 : 1) * 2   // (two lists)
@@ -712,7 +712,7 @@ lif_status lif_restore(lif_layer* L, const void* host_buf, size_t bytes) {
     in += p[i].bytes;
   }
   // entries of predictor runs after the snapshot must not be taken for those of the next run
-  if (cudaMemset(L->new_mask_words, 0, (size_t)new_mask_entries(L->desc) * 2 * 8) != cudaSuccess ||
+  if (cudaMemset(L->new_mask_words, 0, tagged_words(L->desc) * 8) != cudaSuccess ||
       launch_refill(L, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
     cudaGetLastError();
     return LIF_ERR_CUDA;

@@ -58,7 +58,7 @@ gate_scores_kernel(const __half* __restrict__ x, const __half* __restrict__ gate
   for (int j = 0; j < kDepth; ++j) load_group(w[j], j);
   pdl_wait();
   pdl_trigger();
-  const int run = tid == 0 ? __ldcg(predictor_run) : 0;
+  const int run = __ldcg(predictor_run);
   for (int c = tid; c < S * nvec; c += kThreads) xs[c] = reinterpret_cast<const uint4*>(x)[c];
   __syncthreads();
 
@@ -97,6 +97,7 @@ gate_scores_kernel(const __half* __restrict__ x, const __half* __restrict__ gate
   if (lane < kRowsPerWarp) {
     const int i = i0 + lane;
     bool active = false;
+    float value = 0.f;
     if (i < F) {
       const float b = __half2float(bias[i]);
 #pragma unroll
@@ -106,13 +107,20 @@ gate_scores_kernel(const __half* __restrict__ x, const __half* __restrict__ gate
         for (int q = 0; q < kRowsPerWarp; ++q)
           if (q == lane) v = acc[q][s];
         v += b;
+        value = v;
         gate_val[(size_t)s * F + i] = v;
         if (logits) logits[(size_t)s * F + i] = v;
         active = active || (v > theta);
       }
     }
     // (the window state of the previous step is final long before this kernel starts)
-    act_flag[warp * kRowsPerWarp + lane] = active ? (slot_of[i] < 0 ? 3 : 1) : 0;
+    const int row = active ? slot_of[i] : 0;
+    act_flag[warp * kRowsPerWarp + lane] = active ? (row < 0 ? 3 : 1) : 0;
+    if (S == 1 && !compact && active) {                    // for the single-launch step
+      unsigned long long* words = new_mask_words + 2 * gridDim.x + i;
+      if (row >= 0) store_with_run(words, (uint32_t)row, run);
+      store_with_run(words + F, __float_as_uint(value), run);
+    }
   }
   __syncthreads();
   if (warp == 0) {
@@ -129,13 +137,8 @@ gate_scores_kernel(const __half* __restrict__ x, const __half* __restrict__ gate
       }
       // this CTA's neurons to bring in, with the run's number, in one store (one entry per CTA):
       // a fetch kernel that is already resident re-reads the entry until the number is the run's
-      const unsigned long long e = (unsigned long long)mn | ((unsigned long long)(unsigned)run << 32);
-      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(new_mask_words + blockIdx.x), "l"(e)
-                   : "memory");
-      // likewise the active neurons themselves
-      const unsigned long long ea = (unsigned long long)m | ((unsigned long long)(unsigned)run << 32);
-      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(new_mask_words + gridDim.x + blockIdx.x),
-                   "l"(ea) : "memory");
+      store_with_run(new_mask_words + blockIdx.x, mn, run);
+      store_with_run(new_mask_words + gridDim.x + blockIdx.x, m, run);   // likewise the active neurons
     }
   }
   if (!compact) return;     // the consumer reads the bit mask itself

@@ -69,7 +69,9 @@ struct lif_layer {
   // Neurons predicted active that have no cache row yet, as 64-bit entries {bits, run}: the low
   // half holds the bits of 32 consecutive neurons (of one predictor CTA's neurons, where those
   // are fewer), the high half the number of the predictor run that stored it (one store).
-  // A second block of as many entries holds the active neurons themselves in the same form.
+  // A second block of as many entries holds the active neurons themselves in the same form.  Behind
+  // it a word per neuron, {cache row, run}, written where a neuron is active and cached; with a
+  // resident gate another one, {gate value, run}, written where it is active (one stream).
   unsigned long long* new_mask_words;
   int8_t* keep_tok;   // [d_ff] last kept token per neuron (speculative mode)
   float* y_partial;
@@ -166,6 +168,12 @@ inline int new_mask_entry_bits(const lif_layer_desc& D) {
 inline int new_mask_entries(const lif_layer_desc& D) {
   if (D.gate_mode == LIF_GATE_RESIDENT) return (D.d_ff + gate_predict_tile() - 1) / gate_predict_tile();
   return (D.d_ff + kLogitTile - 1) / kLogitTile * (kLogitTile / 32);
+}
+// 64-bit words of the new_mask_words block: two blocks of entries, {row, run} and {gate value, run}
+inline size_t row_words_at(const lif_layer_desc& D) { return 2 * (size_t)new_mask_entries(D); }
+inline size_t gate_words_at(const lif_layer_desc& D) { return row_words_at(D) + D.d_ff; }
+inline size_t tagged_words(const lif_layer_desc& D) {
+  return gate_words_at(D) + (D.gate_mode == LIF_GATE_RESIDENT ? D.d_ff : 0);
 }
 // early: what the kernel may do before its own dependency wait.  kEarlyLists: the lists were
 // final before the kernel ahead of this one passed its wait, so the first bundle's host loads
@@ -293,6 +301,13 @@ __device__ __forceinline__ float apply_activation(float v, int act, float thr) {
 // Let the next kernel of the stream start its prologue.
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// {low, run}: a value and the number of the predictor run that it belongs to, written whole, so that a
+// kernel that is resident early can re-read the word until it carries the number
+__device__ __forceinline__ void store_with_run(unsigned long long* at, uint32_t low, int run) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(at),
+               "l"((unsigned long long)low | ((unsigned long long)(unsigned)run << 32)) : "memory");
 }
 
 // 16-byte streaming load (no L1 allocation) of data that is read once: weights, bundles in

@@ -127,7 +127,7 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
   if (!compact) pdl_trigger();
   pdl_wait();
   if (compact) pdl_trigger();
-  const int run = (tid < kLogitTile && (tid & 31) == 0) ? __ldcg(predictor_run) : 0;
+  const int run = tid < kLogitTile ? __ldcg(predictor_run) : 0;
   // every partial of a sum is requested before the first is used (one memory round trip instead of
   // several); the additions keep their order
   for (int i = tid; i < r; i += kThreads) {
@@ -190,16 +190,12 @@ predict_logits_kernel(const float* __restrict__ z_partial, int P, const __half* 
       mask_words[blockIdx.x * (kLogitTile / 32) + (tid >> 5)] = m;
       // the bits together with this run's number, in one store: a fetch kernel that is already
       // resident re-reads the entry until the number is the run's
-      const unsigned long long e = (unsigned long long)mn | ((unsigned long long)(unsigned)run << 32);
-      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(
-                       new_mask_words + blockIdx.x * (kLogitTile / 32) + (tid >> 5)), "l"(e) : "memory");
-      if (!compact) {     // and the active ones themselves, for the single-launch step
-        const unsigned long long ea = (unsigned long long)m | ((unsigned long long)(unsigned)run << 32);
-        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(
-                         new_mask_words + (gridDim.x + blockIdx.x) * (kLogitTile / 32) + (tid >> 5)),
-                     "l"(ea) : "memory");
-      }
+      store_with_run(new_mask_words + blockIdx.x * (kLogitTile / 32) + (tid >> 5), mn, run);
+      if (!compact)       // and the active ones themselves, for the single-launch step
+        store_with_run(new_mask_words + (gridDim.x + blockIdx.x) * (kLogitTile / 32) + (tid >> 5), m, run);
     }
+    if (!compact && active && my_row >= 0)                 // ... with the row of each that has one
+      store_with_run(new_mask_words + 2 * gridDim.x * (kLogitTile / 32) + my_col, (uint32_t)my_row, run);
   }
 
   if (!compact) return;     // the consumer reads the bit mask itself

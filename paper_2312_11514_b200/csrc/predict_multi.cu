@@ -213,7 +213,7 @@ scores_multi_kernel(const float* __restrict__ z_partial, int P, const __half* __
   if (!compact) pdl_trigger();
   pdl_wait();
   if (compact) pdl_trigger();
-  const int run = (tid < kLogitTile && (tid & 31) == 0) ? __ldcg(predictor_run) : 0;
+  const int run = tid < kLogitTile ? __ldcg(predictor_run) : 0;
   if (P == 1) {                                              // z is finished: all loads in flight
     for (int j = tid; j < r; j += kThreads) {
       float v[S];
@@ -305,12 +305,12 @@ scores_multi_kernel(const float* __restrict__ z_partial, int P, const __half* __
     if ((tid & 31) == 0) {
       mask_words[blockIdx.x * (kLogitTile / 32) + (tid >> 5)] = m;
       // entries of the neurons to bring in and of the active ones, each with this run's number
-      const unsigned long long tag = (unsigned long long)(unsigned)run << 32;
       unsigned long long* at = new_mask_words + blockIdx.x * (kLogitTile / 32) + (tid >> 5);
-      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(at), "l"(tag | mn) : "memory");
-      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(at + gridDim.x * (kLogitTile / 32)),
-                   "l"(tag | m) : "memory");
+      store_with_run(at, mn, run);
+      store_with_run(at + gridDim.x * (kLogitTile / 32), m, run);
     }
+    if (!compact && ((m >> (tid & 31)) & 1u) && my_row >= 0)
+      store_with_run(new_mask_words + 2 * gridDim.x * (kLogitTile / 32) + my_col, (uint32_t)my_row, run);
   }
   if (!compact) return;     // the consumer reads the bit mask itself
   compact_mask_last_cta(mask_words, gridDim.x * (kLogitTile / 32), ticket, active_idx, n_active,

@@ -4,12 +4,21 @@
 // The CTAs of the grid (one per SM) take parts of the step, in the order in which they start:
 //   window CTA   (first)   the plan of Section 3.3: lists, counters and state, from the
 //                          predictor's entries; publishes the plan with one flag
-//   cache CTAs   (middle)  wait for the plan; row moves, then the FFN terms of the rows that were
-//                          already cached (bulk copies into shared memory, a warp per row)
-//   fetch CTAs   (then)    find the new neurons themselves in the predictor's entries, bring their
-//                          bundles over the host link through a ring of bulk copies, add their FFN
-//                          terms from shared memory, copy them to their cache rows
+//   cache CTAs   (middle)  find the active rows that are already cached in the predictor's entries,
+//                          add their FFN terms (bulk copies into shared memory, a warp per row); the
+//                          plan's row moves
+//   fetch CTAs   (then)    find the new neurons in the predictor's entries, bring their bundles over
+//                          the host link through a ring of bulk copies, add their FFN terms from
+//                          shared memory, copy them to their cache rows
 //   sum CTAs     (last)    add up the partial sums
+// The terms of the output wait for the predictor's entries only, which carry the row of every cached
+// neuron; the plan (3 us behind them) is needed for the places of new and moved rows, and by the sum,
+// which leaves the terms out when the update was refused.  With the terms behind the plan a token of two
+// 512 x 2048 layers took 28.4 us, 26.6 now; eight of 4096 x 16384 386-391 us, 380-383 now.
+// (The FFN over every cached row takes its rows from the plan.)
+// x, like the window state, was complete before every kernel ahead of this one passed its own wait, so
+// it is read (past L1) ahead of this kernel's wait, which comes 2-4 us behind the last entry where
+// host reads are in flight.
 // A CTA whose wait for the plan runs out moves or brings in nothing, although the window CTA commits the
 // state that names those rows.  Like every wait that runs out it flags LIF_ERR_TIMEOUT, which refuses further
 // updates, and it marks the rows as suspect, so that clearing the status reads them from the store again.
@@ -49,19 +58,25 @@ constexpr unsigned short kNoSlot = 0xffff;
 // to be put back at the end.
 struct StepSync {
   unsigned long long ticket;
-  unsigned long long plan;       // step << 42 | flags | n_moves << 20 | rows for the cache CTAs
+  unsigned long long plan;       // step << 50 | flags | n_load << 32 | n_moves << 16 | rows for the cache CTAs
   unsigned groups_done;
   unsigned pad[11];
   unsigned group[64];            // arrivals of each group of cache CTAs
 };
-constexpr unsigned long long kPlanReady = 1ull << 40, kPlanRefused = 1ull << 41;
-constexpr int kPlanEpochShift = 42;
+constexpr unsigned long long kPlanReady = 1ull << 48, kPlanRefused = 1ull << 49;
+constexpr int kPlanEpochShift = 50;
+constexpr unsigned kPlanEpochMask = (1u << 14) - 1;
+__device__ __forceinline__ int plan_rows(unsigned long long v) { return (int)(v & 0xffff); }
+__device__ __forceinline__ int plan_moves(unsigned long long v) { return (int)((v >> 16) & 0xffff); }
+__device__ __forceinline__ int plan_loads(unsigned long long v) { return (int)((v >> 32) & 0xffff); }
 
 struct StepArgs {
   WindowArgs w;
   const unsigned long long* new_entries;   // predictor: {neurons to bring in, run}
   const unsigned long long* act_entries;   // predictor: {active neurons, run}
   int n_entries;
+  const unsigned long long* row_words;     // predictor: {cache row, run} of the active cached neurons
+  const unsigned long long* gate_words;    // resident gate: {gate value, run} of the active neurons
   const int* predictor_run;
   int* next_run;                  // bumped at the end (a predictor without a first stage needs it)
   int32_t* n_act_out;
@@ -77,7 +92,7 @@ struct StepArgs {
   StepSync* sync;
   int d, n_streams, whole_cache, act;
   float act_thr;
-  int n_cache_ctas, n_sum_ctas, group_size, cache_stages, fetch_stages, fetch_rows_max;
+  int n_cache_ctas, n_sum_ctas, group_size, cache_stages, fetch_stages, fetch_rows_max, hits_max;
   unsigned wait_polls;            // of the first wait for a bulk copy
   unsigned spin_limit;            // of a wait for another CTA
   unsigned epoch;                 // steps before this one (filled in by the kernel)
@@ -103,8 +118,11 @@ __device__ __forceinline__ bool arrive_last(unsigned* p, unsigned want) {
 __device__ __forceinline__ void arrive(unsigned* p) {
   asm volatile("red.add.release.gpu.global.u32 [%0], 1;" ::"l"(p) : "memory");
 }
+__device__ __forceinline__ bool is_plan(const StepArgs& a, unsigned long long v) {
+  return (v & kPlanReady) && v >> kPlanEpochShift == (a.epoch & kPlanEpochMask);
+}
 __device__ __forceinline__ void publish(const StepArgs& a, unsigned long long v) {
-  v |= (unsigned long long)(a.epoch & ((1u << 22) - 1)) << kPlanEpochShift;
+  v |= (unsigned long long)(a.epoch & kPlanEpochMask) << kPlanEpochShift;
   asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&a.sync->plan), "l"(v) : "memory");
 }
 // Exclusive prefixes of N words over the block and the block's sums; one barrier, so consecutive
@@ -146,26 +164,32 @@ __device__ __forceinline__ void plan_not_carried_out(const StepArgs& a) {
   a.w.counts[CNT_ROWS_SUSPECT] = 1;
   timed_out(a);
 }
+__device__ __forceinline__ unsigned long long ld_relaxed64(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
 // The thread's entries of the predictor run `run`.  This kernel may be resident while the score
 // kernel still runs; each entry is stored together with the number of its run, so a thread re-reads
 // its own until they carry it.  If they do not come (bounded), the kernel waits for its predecessor
-// and takes them as they are.
-__device__ __forceinline__ void read_entries(const unsigned long long* entries, int n, int run,
-                                             uint32_t (&mw)[kEntriesPerThread]) {
+// and takes them as they are: false, and then the other words of the run need no check either.
+template <int N>
+__device__ __forceinline__ bool read_entries(const unsigned long long* const (&entries)[N], int n, int run,
+                                             uint32_t (&mw)[N][kEntriesPerThread]) {
   const int w0 = threadIdx.x * kEntriesPerThread;
   auto read = [&](bool check) {
     bool mine = true;
 #pragma unroll
-    for (int i = 0; i < kEntriesPerThread; ++i) {
-      mw[i] = 0u;
-      if (w0 + i < n) {
-        unsigned long long v;
-        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(entries + w0 + i)
-                     : "memory");
-        mw[i] = (uint32_t)v;
-        mine = mine && (!check || (int)(v >> 32) == run);
+    for (int k = 0; k < N; ++k)
+#pragma unroll
+      for (int i = 0; i < kEntriesPerThread; ++i) {
+        mw[k][i] = 0u;
+        if (w0 + i < n) {
+          const unsigned long long v = ld_relaxed64(entries[k] + w0 + i);
+          mw[k][i] = (uint32_t)v;
+          mine = mine && (!check || (int)(v >> 32) == run);
+        }
       }
-    }
     return mine;
   };
   int ok = 0;
@@ -174,6 +198,7 @@ __device__ __forceinline__ void read_entries(const unsigned long long* entries, 
     pdl_wait();
     read(false);
   }
+  return ok != 0;
 }
 // Thread 0 waits for the plan; everyone gets it (0 if it did not come: an error is recorded).
 __device__ __forceinline__ unsigned long long wait_plan(const StepArgs& a,
@@ -183,7 +208,7 @@ __device__ __forceinline__ unsigned long long wait_plan(const StepArgs& a,
     bool there = false;
     for (unsigned i = 0; i < a.spin_limit && !there; ++i) {
       v = ld_acquire64(&a.sync->plan);
-      there = (v & kPlanReady) && v >> kPlanEpochShift == (a.epoch & ((1u << 22) - 1));
+      there = is_plan(a, v);
     }
     if (!there) {
       plan_not_carried_out(a);
@@ -253,8 +278,9 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
         age_s[s0 + j * kStepThreads] = (unsigned short)min(65535, max(1, t_end - la[j]));
       }
   }
-  uint32_t mw[kEntriesPerThread];
-  read_entries(a.act_entries, a.n_entries, __ldcg(a.predictor_run), mw);
+  uint32_t act_w[1][kEntriesPerThread];
+  read_entries<1>({a.act_entries}, a.n_entries, __ldcg(a.predictor_run), act_w);
+  const uint32_t(&mw)[kEntriesPerThread] = act_w[0];
   unsigned pre[1] = {0u}, tot[1];
 #pragma unroll
   for (int i = 0; i < kEntriesPerThread; ++i) {
@@ -371,7 +397,7 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
   __syncthreads();
   if (tid == 0) {
     const unsigned n_rows = a.whole_cache ? n_kept : na - n_load;
-    publish(a, kPlanReady | ((unsigned long long)n_moves << 20) | n_rows);
+    publish(a, kPlanReady | ((unsigned long long)n_load << 32) | ((unsigned long long)n_moves << 16) | n_rows);
   }
 
   // ---- behind the flag: the public lists and the state ------------------------------------------
@@ -539,65 +565,134 @@ __device__ __forceinline__ float row_weight(const StepArgs& a, float b, float fi
   if (kGate == LIF_GATE_RESIDENT) return apply_activation(b, a.act, a.act_thr) * first;
   return apply_activation(first + b, a.act, a.act_thr);
 }
+// The low half of a word that the predictor run `run` stores beside its entries, once it is there (it is
+// stored with the entry: a poll or two).  checked = false: as it is (see read_entries).
+__device__ __forceinline__ uint32_t word_of_run(const StepArgs& a, const unsigned long long* at, int run,
+                                                bool checked) {
+  unsigned long long v = checked ? 0ull : ld_relaxed64(at);
+  bool there = !checked;
+  for (unsigned i = 0; i < a.spin_limit && !there; ++i) {
+    v = ld_relaxed64(at);
+    there = (int)(v >> 32) == run;
+  }
+  if (!there) {                                            // (row 0, gate value 0)
+    timed_out(a);
+    v = 0;
+  }
+  return (uint32_t)v;
+}
 // the neuron's bias; resident gate (one stream): its gate value
 template <int kGate>
-__device__ __forceinline__ float row_scalar(const StepArgs& a, int id) {
-  return kGate == LIF_GATE_RESIDENT ? a.gate_val[id] : __half2float(a.w.bias_up[id]);
+__device__ __forceinline__ float row_scalar(const StepArgs& a, int id, int run, bool checked) {
+  return kGate == LIF_GATE_RESIDENT ? __uint_as_float(word_of_run(a, a.gate_words + id, run, checked))
+                                    : __half2float(a.w.bias_up[id]);
+}
+// x of every stream into shared memory, past L1: it may hold lines of an earlier token's
+__device__ __forceinline__ void load_x(const StepArgs& a, uint4* xs) {
+  for (int i = threadIdx.x; i < a.n_streams * (a.d >> 3); i += kStepThreads)
+    xs[i] = __ldcg(reinterpret_cast<const uint4*>(a.x) + i);
 }
 
 // ---- cache CTAs: row moves and the FFN of the rows that were already cached -------------------------
 // Rows are read where they were before the moves: a moved row's source is not overwritten before
-// all cache CTAs are done (append_first: not at all), so moves and FFN need no order.
+// all cache CTAs are done (append_first: not at all), so moves and FFN need no order.  The moves come
+// first in the paper's order, where the new rows wait for them, and last otherwise.
+// CTA c adds the hits of rank c, c + nc, ... (ascending neuron ids): the set bits of the predictor's
+// entries of active neurons that its entries of new ones lack.
 template <int kGate, int kS>
 __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
   constexpr int kVec = kGate == LIF_GATE_BUNDLED ? 3 : 2;
   __shared__ __align__(8) uint64_t bars[16];
   __shared__ float h_s[16][kS], b_s[16];
   __shared__ unsigned long long plan_s;
+  __shared__ unsigned sums[1][kStepWarps];
   __shared__ int last_s, lost_s;       // (lost_s: as a barrier's reduction 0.4 us a step more)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int d = a.d, S = a.n_streams, nvec = d >> 3, stages = a.cache_stages, nc = a.n_cache_ctas;
   const unsigned row_bytes = 2u * kVec * d;
   uint4* xs = reinterpret_cast<uint4*>(smem);              // [S][d]
   unsigned char* rows = smem + x_smem_bytes(d, S);
+  unsigned short* hits = reinterpret_cast<unsigned short*>(rows + (size_t)stages * row_bytes);
   if (tid == 0) {
     lost_s = 0;
     for (int i = 0; i < stages; ++i) mbar_init(bars + i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  pdl_wait();
-  for (int i = tid; i < S * nvec; i += kStepThreads) xs[i] = reinterpret_cast<const uint4*>(a.x)[i];
-  const unsigned long long plan = wait_plan(a, &plan_s);
-  const int n = (int)(plan & 0xfffff), n_moves = (int)((plan >> 20) & 0xfffff);
-  const int cnt = c < n ? (n - c + nc - 1) / nc : 0;
+  const int run = __ldcg(a.predictor_run);
+  bool checked = false;
+  int n, n_moves = 0;
+  if (a.whole_cache) {
+    pdl_wait();                                            // (gate values of every row)
+    const unsigned long long plan = wait_plan(a, &plan_s);
+    n = plan_rows(plan);
+    n_moves = plan_moves(plan);
+  } else {
+    // one thread watches one entry: the whole CTA re-reading all of them beside the score kernel cost it
+    // 1 us at 4096 x 16384
+    for (int i = 0; tid == 0 && i < 2 * kStepWatchPolls; ++i) {
+      if ((int)(ld_relaxed64(a.new_entries + a.n_entries - 1) >> 32) == run) break;
+      __nanosleep(100);
+    }
+    __syncthreads();
+    uint32_t mw[2][kEntriesPerThread];
+    checked = read_entries<2>({a.act_entries, a.new_entries}, a.n_entries, run, mw);
+    unsigned pre[1] = {0u}, tot[1];
+#pragma unroll
+    for (int i = 0; i < kEntriesPerThread; ++i) pre[0] += __popc(mw[0][i] & ~mw[1][i]);
+    step_scan<1>(pre, tot, sums);
+    n = (int)tot[0];
+    unsigned q = pre[0];
+#pragma unroll
+    for (int i = 0; i < kEntriesPerThread; ++i)
+      for (uint32_t m = mw[0][i] & ~mw[1][i]; m; m &= m - 1, ++q) {
+        const unsigned j = q / (unsigned)nc;
+        if (q - j * nc == (unsigned)c && j < (unsigned)a.hits_max)
+          hits[j] = (unsigned short)((tid * kEntriesPerThread + i) * 32 + __ffs(m) - 1);
+      }
+    __syncthreads();
+  }
+  auto move_rows = [&]() {
+    const int row_vec = kVec * nvec;
+    for (int j = c; j < n_moves; j += nc) {
+      const uint4* src = reinterpret_cast<const uint4*>(a.cache) + (size_t)__ldcg(a.w.move_src + j) * row_vec;
+      uint4* dst = reinterpret_cast<uint4*>(a.cache) + (size_t)__ldcg(a.w.move_dst + j) * row_vec;
+      uint4 v[4];
+      for (int v0 = tid; v0 < row_vec; v0 += 4 * kStepThreads) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (v0 + u * kStepThreads < row_vec) v[u] = ld_stream16(src + v0 + u * kStepThreads);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (v0 + u * kStepThreads < row_vec) dst[v0 + u * kStepThreads] = v[u];
+      }
+    }
+  };
+  const int cnt = c < n ? min(a.hits_max, (n - c + nc - 1) / nc) : 0;
   Acc<kS> acc;
 
   unsigned parity = 0;
   for (int r0 = 0; r0 < cnt || r0 == 0; r0 += stages) {
     const int rc = min(stages, cnt - r0);
     if (tid < rc) {
-      const uint32_t e = __ldcg(a.hit_rows + c + (r0 + tid) * nc);
-      mbar_expect_tx(bars + tid, row_bytes);
-      bulk_g2s(rows + (size_t)tid * row_bytes, a.cache + (size_t)(e & 0xffff) * row_bytes, row_bytes,
-               bars + tid);
-      b_s[tid] = row_scalar<kGate>(a, (int)(e >> 16));
-    }
-    if (r0 == 0) {                                         // the moves, while the first rows travel
-      const int row_vec = kVec * nvec;
-      for (int j = c; j < n_moves; j += nc) {
-        const uint4* src = reinterpret_cast<const uint4*>(a.cache) + (size_t)__ldcg(a.w.move_src + j) * row_vec;
-        uint4* dst = reinterpret_cast<uint4*>(a.cache) + (size_t)__ldcg(a.w.move_dst + j) * row_vec;
-        uint4 v[4];
-        for (int v0 = tid; v0 < row_vec; v0 += 4 * kStepThreads) {
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (v0 + u * kStepThreads < row_vec) v[u] = ld_stream16(src + v0 + u * kStepThreads);
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (v0 + u * kStepThreads < row_vec) dst[v0 + u * kStepThreads] = v[u];
-        }
+      int id, row;
+      if (a.whole_cache) {
+        const uint32_t e = __ldcg(a.hit_rows + c + (r0 + tid) * nc);
+        id = (int)(e >> 16);
+        row = (int)(e & 0xffff);
+      } else {
+        id = hits[r0 + tid];
+        row = (int)word_of_run(a, a.row_words + id, run, checked);
       }
+      mbar_expect_tx(bars + tid, row_bytes);
+      bulk_g2s(rows + (size_t)tid * row_bytes, a.cache + (size_t)row * row_bytes, row_bytes, bars + tid);
+      b_s[tid] = kGate == LIF_GATE_RESIDENT && a.whole_cache ? a.gate_val[id]
+                                                             : row_scalar<kGate>(a, id, run, checked);
+    }
+    if (r0 == 0) load_x(a, xs);                            // while the first rows travel
+    if (r0 == 0 && !a.w.append_first) {                    // ... and the moves
+      if (!a.whole_cache) n_moves = plan_moves(wait_plan(a, &plan_s));
+      move_rows();
     }
     __syncthreads();                                       // x and the rows' scalars
     if (rc <= 0) break;
@@ -649,6 +744,7 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
   // partials (in CTA order), so that few are left for the end of the step.
   const int gs = a.group_size, g = c / gs;
   const size_t width = (size_t)S * d;
+  bool last = true;
   if (gs == 1) {
     if (cnt > 0) store_tagged_partial<kS>(acc, a.p_hit + (size_t)c * (width / 2), nvec, S, a.epoch + 1);
     __syncthreads();
@@ -658,9 +754,9 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
     const int members = min(gs, nc - g * gs);
     if (tid == 0) last_s = arrive_last(&a.sync->group[g], (a.epoch + 1) * (unsigned)members);
     __syncthreads();
-    if (!last_s) return;
+    last = last_s;
     const int have = min(members, max(0, n - g * gs));     // members with rows wrote a partial
-    if (have > 0)
+    if (last && have > 0)
       for (int i = tid; i < (int)(width / 4); i += kStepThreads) {
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f), v[8];
 #pragma unroll
@@ -676,7 +772,11 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
       }
   }
   // (only the paper's cache order waits for this: the rows have been read and moved)
-  if (tid == 0) arrive(&a.sync->groups_done);
+  if (tid == 0 && last) arrive(&a.sync->groups_done);
+  if (a.w.append_first) {                                  // (plan_s was not used before)
+    n_moves = plan_moves(wait_plan(a, &plan_s));
+    move_rows();
+  }
 }
 
 // ---- the sum: CTA `index` of `n` adds up a slice of the columns, in pairs, in a fixed order ----------
@@ -787,19 +887,12 @@ template <int kS>
 __device__ void sum_role(const StepArgs& a, int index, unsigned char* smem) {
   __shared__ unsigned long long plan_s;
   const int tid = threadIdx.x;
-  uint32_t mw[kEntriesPerThread];
-  unsigned n[1] = {0u}, tot[1];
-  __shared__ unsigned sums[1][kStepWarps];
-  read_entries(a.new_entries, a.n_entries, __ldcg(a.predictor_run), mw);
-#pragma unroll
-  for (int i = 0; i < kEntriesPerThread; ++i) n[0] += __popc(mw[i]);
-  step_scan<1>(n, tot, sums);
-  pdl_wait();
+  const int run = __ldcg(a.predictor_run);
   const unsigned long long plan = wait_plan(a, &plan_s);
-  const bool go = (plan & kPlanReady) && !(plan & kPlanRefused);
-  Summer<kS> sum(a, index, a.n_sum_ctas, (int)(plan & 0xfffff), go ? min(kFetchCtas, (int)tot[0]) : 0);
+  const int n_load = plan_loads(plan);                     // (0: refused)
+  Summer<kS> sum(a, index, a.n_sum_ctas, plan_rows(plan), min(kFetchCtas, n_load));
   const size_t pairs = (size_t)a.n_streams * (a.d >> 1);
-  const int n_new = sum.have - sum.have_hit, n_load = (int)tot[0];
+  const int n_new = sum.have - sum.have_hit;
   if (kS == 1) {
     for (unsigned polls = 0; n_load > 2 * kFetchCtas && polls < a.spin_limit; ++polls) {
       const int there = tid == 0 && (n_new == 0 || has_tag(load_tagged(a.p_new + n_new * pairs - 1), sum.tag));
@@ -816,11 +909,15 @@ __device__ void sum_role(const StepArgs& a, int index, unsigned char* smem) {
   }
   __syncthreads();
   sum.finish(reinterpret_cast<float2*>(smem));             // kSumSmem bytes
+  // (by the CTA that started last: every other one has read the number by now)
+  if (index == a.n_sum_ctas - 1 && tid == 0) advance_run(a.next_run, run);
 }
 
 // ---- fetch CTAs: new bundles over the host link and their FFN terms ---------------------------------
 // Fetch CTA f brings in entries f, f + kFetchCtas, ... of the load list, which is exactly the set
-// bits of the predictor's entries in ascending order; only the cache row comes from the plan.
+// bits of the predictor's entries in ascending order; only the cache row comes from the plan.  A bundle
+// stays in the ring until its row is known and, in the paper's order, until the cache CTAs have read and
+// moved what was there; its FFN term is computed meanwhile.
 template <int kGate, int kS>
 __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   constexpr int kVec = kGate == LIF_GATE_BUNDLED ? 3 : 2;
@@ -828,7 +925,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   __shared__ unsigned sums[1][kStepWarps];
   __shared__ float part[2][kS][kStepWarps];
   __shared__ float h_s[kS];
-  __shared__ unsigned long long plan_s;
+  __shared__ int count_s, go_s;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int d = a.d, S = a.n_streams, nvec = d >> 3, stages = a.fetch_stages;
   constexpr int nf = kFetchCtas;
@@ -836,15 +933,15 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   uint4* xs = reinterpret_cast<uint4*>(smem);              // [S][d]
   unsigned char* ring = smem + x_smem_bytes(d, S);
   unsigned short* ids = reinterpret_cast<unsigned short*>(ring + (size_t)stages * row_bytes);
-  unsigned short* dst_rows = ids + a.fetch_rows_max;
   if (tid == 0) {
     for (int i = 0; i < stages; ++i) mbar_init(bars + i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  uint32_t mw[kEntriesPerThread];
+  uint32_t new_w[1][kEntriesPerThread];
   const int run = __ldcg(a.predictor_run);
-  read_entries(a.new_entries, a.n_entries, run, mw);
+  const bool checked = read_entries<1>({a.new_entries}, a.n_entries, run, new_w);
+  const uint32_t(&mw)[kEntriesPerThread] = new_w[0];
   unsigned pre[1] = {0u}, tot[1];
 #pragma unroll
   for (int i = 0; i < kEntriesPerThread; ++i) pre[0] += __popc(mw[i]);
@@ -864,64 +961,69 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
         ids[q / nf] = (unsigned short)id;
         if (q / nf < first) issue(id, q / nf);             // the first ones by whoever finds them
       }
-  int cnt = f < n_new ? (n_new - f + nf - 1) / nf : 0;
-  const int issued = min(first, cnt);
-  pdl_wait();
-  for (int i = tid; i < S * nvec; i += kStepThreads) xs[i] = reinterpret_cast<const uint4*>(a.x)[i];
+  const int cnt = f < n_new ? (n_new - f + nf - 1) / nf : 0;
+  int issued = min(first, cnt);                            // thread 0 from here on
+  load_x(a, xs);
   Acc<kS> acc;
 
-  const unsigned long long plan = wait_plan(a, &plan_s);
-  const bool go = (plan & kPlanReady) && !(plan & kPlanRefused);
+  int go = -1, stored = 0;                                 // thread 0: 1 / 0 once the plan says so; rows stored,
+  int place = 0;                                           // the place of the next one
+  bool moved = a.w.append_first;
   const int n_groups = (a.n_cache_ctas + a.group_size - 1) / a.group_size;
-  if (!go) {
-    // the update of this step was refused: nothing is brought in; let the copies land
-    if (tid == 0)
-      for (int i = 0; i < issued; ++i)
-        if (!mbar_wait(bars + i, 0, a.wait_polls)) {
-          timed_out(a);
-          mbar_wait(bars + i, 0);
-        }
-    cnt = 0;
-  } else {
-    for (int i = tid; i < cnt; i += kStepThreads)
-      dst_rows[i] = (unsigned short)__ldcg(a.w.load_slots + f + i * nf);
+  // Thread 0: asks whether new rows may be stored, or (wait) until they may; then stores those below `upto`.
+  auto learn = [&](bool wait) {
+    const unsigned limit = wait ? a.spin_limit : min(1u, a.spin_limit);
+    for (unsigned n = 0; n < limit && go < 0; ++n) {
+      const unsigned long long v = ld_acquire64(&a.sync->plan);
+      if (is_plan(a, v)) go = !(v & kPlanRefused);
+    }
+    if (go > 0) place = __ldcg(a.w.load_slots + f + stored * nf);
+    for (unsigned n = 0; n < limit && go > 0 && !moved; ++n)
+      moved = (int)(ld_acquire(&a.sync->groups_done) - (a.epoch + 1) * (unsigned)n_groups) >= 0;
+    if (wait && (go < 0 || (go > 0 && !moved))) {          // rows stay as they are, or are overwritten too early
+      plan_not_carried_out(a);
+      if (go < 0) go = 0;
+      moved = true;
+    }
+  };
+  auto store_rows = [&](int upto) {
+    for (; go > 0 && moved && stored < upto; ++stored) {
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                       a.cache + (size_t)place * row_bytes),
+                   "r"(smem_u32(ring + (size_t)(stored % stages) * row_bytes)), "r"(row_bytes) : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      if (stored + 1 < cnt) place = __ldcg(a.w.load_slots + f + (stored + 1) * nf);
+    }
+  };
+  if (tid == 0) {
+    count_s = cnt;
+    if (kS > 1 && cnt > 0) learn(true);                   // (3 streams at 1544 columns: 46.2 us a step, 46.6 without)
   }
-  // In the paper's order the new rows' places may be rows that the cache CTAs still read: the bundles
-  // stay in the ring until they are done, or until a stage is needed again; their FFN terms are computed
-  // meanwhile.
-  bool released = a.w.append_first;                        // thread 0
-  auto store_row = [&](int i, int st) {                    // thread 0
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
-                     a.cache + (size_t)dst_rows[i] * row_bytes),
-                 "r"(smem_u32(ring + (size_t)st * row_bytes)), "r"(row_bytes) : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-  };
-  auto release = [&](int rows) {                           // thread 0; rows 0 .. rows - 1 are held
-    const unsigned want = (a.epoch + 1) * (unsigned)n_groups;
-    unsigned n = 0;
-    while ((int)(ld_acquire(&a.sync->groups_done) - want) < 0 && n < a.spin_limit) ++n;
-    if (n == a.spin_limit) plan_not_carried_out(a);        // rows may be overwritten before they have moved
-    for (int j = 0; j < rows; ++j) store_row(j, j);
-    released = true;
-  };
   __syncthreads();
   unsigned parity = 0;
   int from = cnt;                                          // first row that was not waited for any longer
-  for (int i = 0, st = 0; i < cnt; ++i) {
+  for (int i = 0, st = 0; i < from; ++i) {
     const uint4* row = reinterpret_cast<const uint4*>(ring + (size_t)st * row_bytes);
     const bool landed = mbar_wait(bars + st, parity, a.wait_polls);
-    if (tid == 0 && landed) {
-      if (i + first < cnt) {
-        if (i + first >= stages) {                         // a row before i was in that stage: stored first
-          if (!released) release(i);
+    if (tid == 0 && landed && i + first < cnt) {           // the next one, in the stage of an earlier row?
+      const bool reuse = i + first >= stages;
+      if (go < 0 || (go > 0 && !moved)) {
+        learn(reuse);
+        store_rows(i);
+      }
+      if (go) {
+        if (reuse) {
           asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         }
         issue(ids[i + first], st + first < stages ? st + first : st + first - stages);
+        ++issued;
+      } else {
+        count_s = issued;                                  // refused: nothing more is brought in
       }
-      if (released) store_row(i, st);
     }
-    const float b = row_scalar<kGate>(a, ids[i]);
+    if (tid == 0 && landed && i + 1 < from) store_rows(i + 1);   // (the last one behind the partial sum)
+    const float b = row_scalar<kGate>(a, ids[i], run, checked);
     float p[kS], p2[kS];
 #pragma unroll
     for (int s = 0; s < kS; ++s) p[s] = p2[s] = 0.f;
@@ -951,12 +1053,12 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     if (__syncthreads_or(!landed)) {                       // flagged; this term and the later ones are left out
       if (tid == 0) {                                      // what is in flight gets another bounded chance
         timed_out(a);
-        const int asked = min(cnt, i + first + (landed ? 1 : 0));
-        for (int j = i; j < asked; ++j) mbar_wait(bars + j % stages, (unsigned)(j / stages) & 1u);
+        for (int j = i; j < issued; ++j) mbar_wait(bars + j % stages, (unsigned)(j / stages) & 1u);
       }
       from = i;
       break;
     }
+    from = min(from, count_s);
     const uint4* down = row + (kVec - 1) * nvec;
     if (kS == 1) {
       float v1 = 0.f, v2 = 0.f;
@@ -987,22 +1089,23 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     }
   }
   if (cnt > 0) store_tagged_partial<kS>(acc, a.p_new + (size_t)f * S * (d >> 1), nvec, S, a.epoch + 1);
-  if (tid == 0 && cnt > 0 && !released) release(from);
+  if (tid == 0) {
+    if (cnt > 0 && (go < 0 || (go > 0 && !moved))) learn(true);
+    store_rows(from);
+    go_s = go;
+  }
   if (from < cnt) {
     // The window state already names these rows, so they are filled all the same, with plain loads and
     // without the ring (in the paper's order thread 0 has waited until their places are free).
     __syncthreads();
-    for (int i = from; i < cnt; ++i) {
+    for (int i = from; i < cnt && go_s > 0; ++i) {
       const uint4* src = reinterpret_cast<const uint4*>(a.store + (size_t)ids[i] * row_bytes);
-      uint4* dst = reinterpret_cast<uint4*>(a.cache + (size_t)dst_rows[i] * row_bytes);
+      uint4* dst = reinterpret_cast<uint4*>(a.cache + (size_t)__ldcg(a.w.load_slots + f + i * nf) * row_bytes);
       for (int v = tid; v < kVec * nvec; v += kStepThreads) dst[v] = ld_stream16(src + v);
     }
   }
-  if (tid == 0) {
-    if (f == 0) advance_run(a.next_run, run);
-    // (shared memory must outlive the reads of the last rows' copies to the cache)
-    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-  }
+  // (shared memory must outlive the reads of the last rows' copies to the cache)
+  if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
 // (One stream: two CTAs per SM, 64 registers and 0-4 bytes spilled, so that small layers' steps on several
@@ -1092,7 +1195,7 @@ cudaError_t step_configure(lif_layer* L) {
   if (e != cudaSuccess) return e;
   max_smem -= (int)at.sharedSizeBytes;
   const size_t row = 2 * (size_t)row_elems(D), x = x_smem_bytes(D.d_model, D.n_streams);
-  const size_t ids = 4 * (((size_t)D.d_ff + kFetchCtas - 1) / kFetchCtas);
+  const size_t ids = 2 * (((size_t)D.d_ff + kFetchCtas - 1) / kFetchCtas);
   auto stages = [&](size_t ring, size_t other, int least) {
     while (ring > row * least && ring + other > (size_t)max_smem) ring -= row;
     const int s = (int)(ring / row);
@@ -1101,11 +1204,12 @@ cudaError_t step_configure(lif_layer* L) {
   L->step_cache_ctas = cache_ctas(D, L->n_sm);
   L->step_sum_ctas = sum_ctas(D);
   L->step_group = L->step_cache_ctas > hit_partials_max(D) ? kGroupMax : 1;
-  L->step_cache_stages = stages(kCacheRing, x, 1);
+  const size_t hits = 2 * (((size_t)D.capacity + L->step_cache_ctas - 1) / L->step_cache_ctas);
+  L->step_cache_stages = stages(kCacheRing, x + hits, 1);
   // (paper's cache order: bundles wait in the ring, see fetch_role; twice the ring keeps the link busy)
   L->step_fetch_stages = stages(D.append_first ? kFetchRing : 2 * kFetchRing, x + ids, 2);
   size_t smem = window_role_smem(D.d_ff, D.capacity);
-  const size_t need_c = x + L->step_cache_stages * row, need_f = x + L->step_fetch_stages * row + ids;
+  const size_t need_c = x + L->step_cache_stages * row + hits, need_f = x + L->step_fetch_stages * row + ids;
   if (need_c > smem) smem = need_c;
   if (need_f > smem) smem = need_f;
   if (smem < kSumSmem) smem = kSumSmem;
@@ -1124,6 +1228,8 @@ cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st
   a.new_entries = L->new_mask_words;
   a.n_entries = new_mask_entries(D);
   a.act_entries = L->new_mask_words + a.n_entries;
+  a.row_words = L->new_mask_words + row_words_at(D);
+  a.gate_words = L->new_mask_words + gate_words_at(D);
   a.predictor_run = L->counts + CNT_PREDICTOR_RUN;
   a.next_run = (int*)(L->counts + CNT_PREDICTOR_RUN);
   a.n_act_out = L->n_tmp;
@@ -1149,6 +1255,7 @@ cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st
   a.cache_stages = L->step_cache_stages;
   a.fetch_stages = L->step_fetch_stages;
   a.fetch_rows_max = (D.d_ff + kFetchCtas - 1) / kFetchCtas;
+  a.hits_max = (D.capacity + a.n_cache_ctas - 1) / a.n_cache_ctas;
   a.wait_polls = L->wait_polls;
   a.spin_limit = L->spin_limit;
   return launch_k(step_kernel_for(D), dim3(1 + a.n_cache_ctas + kFetchCtas + a.n_sum_ctas),

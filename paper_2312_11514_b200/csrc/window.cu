@@ -606,7 +606,7 @@ cudaError_t launch_reset(lif_layer* L, cudaStream_t st) {
   reset_kernel<<<296, kThreads, 0, st>>>(L->counts, L->pointers, L->slot_of, L->last_active,
                                         L->mask_words, L->new_mask_words, L->step_sync,
                                         (uint4*)L->step_tagged, n_mask,
-                                        2 * new_mask_entries(D), (int)(step_sync_bytes() / 4),
+                                        (int)tagged_words(D), (int)(step_sync_bytes() / 4),
                                         (int)(step_tagged_bytes(D) / 16), D.d_ff, D.capacity);
   return cudaGetLastError();
 }

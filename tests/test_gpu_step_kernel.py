@@ -2,6 +2,8 @@
 CTA's registers), of the kernels beyond them, and of the multi-stream predictor: widths and stream
 counts on both sides of each limit, ranks around the two forms of the first predictor stage, fewer new
 neurons than fetch CTAs, more than a ring holds, refused updates."""
+import copy
+
 import numpy as np
 import pytest
 import torch
@@ -106,3 +108,30 @@ def test_steps_of_more_layers_than_the_chip_holds_at_a_time():
             np.testing.assert_array_equal(one[key], other[key])
     for gpu, _ in pairs:
         gpu.close()
+
+
+@pytest.mark.parametrize("S,gate_mode,append_first", [(1, 0, 0), (1, 2, 1), (3, 0, 1)])
+def test_other_tokens_after_a_restore_do_not_meet_words_of_runs_of_the_same_number(S, gate_mode, append_first):
+    # the rows and gate values that the predictor stores beside its entries carry its run's number, which a
+    # restore puts back: with other tokens the same numbers belong to other rows
+    act, thr = (B.ACT_FATRELU, 0.05) if gate_mode else (B.ACT_RELU, 0.0)
+    cfg = W.LifConfig("again", 1, 520, 4096, 32, 3, S, 9, 0.08, 1.0, 0.3, 0.95, 74)
+    gpu, ora = P.make_layer_pair(cfg, 0, b_down=True, append_first=append_first, gate_mode=gate_mode,
+                                 activation=act, act_threshold=thr)
+    X = W.make_inputs(cfg, device=DEV)
+    y = torch.empty(S, cfg.d_model, dtype=torch.float32, device=DEV)
+    torch.cuda.synchronize()
+
+    def run(tokens):
+        for t in tokens:
+            B.lif_decode_step(gpu.handle, X[t], y)
+            P.check_decode_step(gpu, ora, X[t].cpu().numpy(), y)
+            P.compare_cache_rows(gpu, ora)
+
+    run(range(3))
+    snap, cache = B.lif_snapshot(gpu.handle), copy.deepcopy(ora.cache)
+    run(range(3, 6))
+    B.lif_restore(gpu.handle, snap)
+    ora.cache = cache
+    run(range(6, 9))
+    gpu.close()
