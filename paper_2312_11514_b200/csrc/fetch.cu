@@ -338,6 +338,7 @@ struct RingArgs {
   int32_t* counts;
   unsigned row_bytes;
   int stages, window;
+  int list_max;                      // entries that load_ids has room for
   unsigned wait_polls;               // poll limit of the first wait on each copy (kWaitLimit)
   EarlySource early;
 };
@@ -393,6 +394,21 @@ __global__ void __launch_bounds__(kThreads) fetch_ring_kernel(RingArgs a) {
   }
   pdl_wait();
   pdl_trigger();
+  const int n = __ldcg(a.counts + LIF_CNT_N_LOAD);
+  if (kEarlyT == kEarlyNone) {
+    // the first ids come with the count and are asked for by the threads that read them: one round trip
+    // and a barrier less ahead of the link
+    const int j = c + tid * G;
+    if (tid < a.window && j < a.list_max) {
+      const int id = a.load_ids ? __ldcg(a.load_ids + j) : j;
+      if (j < n) {
+        ids[tid] = id;
+        issue(id, tid);
+      }
+    }
+    known = n > c ? min(a.window, (n - c + G - 1) / G) : 0;
+    n_early = n;
+  }
   int issued = min(known, a.window), used = 0;       // copies so far: asked for, done with
   bool lost = false;                                 // thread 0: the ring has been given up
   auto give_up = [&]() {                             // thread 0
@@ -400,7 +416,6 @@ __global__ void __launch_bounds__(kThreads) fetch_ring_kernel(RingArgs a) {
     for (int k = used; k < issued; ++k) landed(k, kWaitLimit);
     lost = true;
   };
-  const int n = __ldcg(a.counts + LIF_CNT_N_LOAD);
   if (known && n != n_early) {                       // not this step's: let them land, start over
     if (tid == 0)
       for (; used < issued && !lost; ++used)
@@ -617,6 +632,7 @@ static cudaError_t launch_ring(lif_layer* L, const int32_t* ids, bool watch, cud
   if (watch)         // what travels while the window kernel runs has nowhere to go yet: as deep as it gets
     window = (int)((L->max_smem - 2048 - 2 * kRingList * 4) / a.row_bytes) - 2;
   a.window = window < 2 ? 2 : (window > 14 ? 14 : window);
+  a.list_max = L->desc.capacity;
   a.stages = a.window + 2;
   a.wait_polls = L->wait_polls;
   a.early = early_source(L);
