@@ -15,7 +15,7 @@ extern "C" {
 
 /* Launch-shape knobs (defaults in parentheses); they change speed, never results beyond the
  * order of floating-point partial sums.  Set them before capturing a graph.  Except for
- * LIF_TUNE_DEPENDENT_LAUNCH and the two poll limits they concern the separate kernels: a layer whose
+ * LIF_TUNE_DEPENDENT_LAUNCH and the poll limits they concern the separate kernels: a layer whose
  * decode step runs as one launch behind the predictor uses them once such a knob is moved from its
  * default (and while lif_timing_enable records). */
 enum {
@@ -48,17 +48,20 @@ enum {
                                     resident while the predictor still runs and issues its first
                                     host loads from the predictor's masks; 0: it waits for the
                                     window kernel's lists on the fetch stream */
-  LIF_TUNE_STEP_POLLS = 11       /* (2^20) test aid: poll limit of the waits of a single-launch step's
+  LIF_TUNE_STEP_POLLS = 11,      /* (2^20) test aid: poll limit of the waits of a single-launch step's
                                     CTAs for one another, >= 0.  0: all of them give up at once,
                                     nothing is moved or brought in and the step ends with
                                     LIF_ERR_TIMEOUT */
+  LIF_TUNE_PREDICTOR_POLLS = 12  /* (2^20) test aid: poll limit of the predictor's second stage waiting
+                                    for a value of its first, >= 0.  0: one look; the call ends with
+                                    LIF_ERR_TIMEOUT and takes no neuron whose score it lacks for active */
 };
 lif_status lif_set_tuning(lif_layer* layer, int32_t key, int32_t value);
 
 /* Phases timed by lif_timing_* (one CUDA event pair each, inside lif_decode_step). */
 enum {
-  LIF_PHASE_PREDICT_Z = 0,      /* x.A partial sums */
-  LIF_PHASE_PREDICT_SCORES = 1, /* scores, threshold, compaction */
+  LIF_PHASE_PREDICT_Z = 0,      /* (nothing: both stages of the predictor are one launch) */
+  LIF_PHASE_PREDICT_SCORES = 1, /* predictor: x.A, scores, threshold, compaction */
   LIF_PHASE_WINDOW = 2,         /* window bookkeeping kernel */
   LIF_PHASE_MOVES = 3,          /* row moves */
   LIF_PHASE_FETCH = 4,          /* bundle fetch (on the fetch stream) */
@@ -81,8 +84,9 @@ lif_status lif_timing_read(lif_layer* layer, float* host_us_sums /* [LIF_PHASE_L
  * kernels do not change the window state, so they can be replayed).  dev_x as for
  * lif_decode_step; dev_y is written only by LIF_KERNEL_FFN_SUM.  n_streams must be 1. */
 enum {
-  LIF_KERNEL_PREDICT_Z = 0,  /* LIF_ERR_STATE with LIF_GATE_RESIDENT (no first stage) */
-  LIF_KERNEL_PREDICT_SCORES = 1, /* LIF_GATE_RESIDENT: the gate-projection kernel */
+  LIF_KERNEL_PREDICT_Z = 0,  /* the first stage's CTAs of the predictor alone; LIF_ERR_STATE with
+                                LIF_GATE_RESIDENT (no first stage) */
+  LIF_KERNEL_PREDICT_SCORES = 1, /* the second stage's alone; LIF_GATE_RESIDENT: the gate-projection kernel */
   LIF_KERNEL_FETCH = 2,      /* re-copies this step's new bundles (and, where the decode step
                                 fuses it, recomputes their FFN partials) */
   LIF_KERNEL_FFN_ACTIVE = 3, /* sparse FFN kernel over all active rows */

@@ -1,5 +1,5 @@
 // C ABI of liblif.so: argument checking, workspace carve-up and stream/event orchestration.
-// Every step of the path runs in the kernels of predict*.cu / gate.cu / step.cu, or of window.cu /
+// Every step of the path runs in the kernels of predict.cu / gate.cu / step.cu, or of window.cu /
 // fetch.cu / ffn*.cu where the calls are made one by one or the single launch does not apply.
 #include <new>
 
@@ -18,7 +18,6 @@ Workspace plan_workspace(const lif_layer_desc& d, int ffn_grid_max) {
     return at;
   };
   const size_t F = d.d_ff, cap = d.capacity, S = d.n_streams;
-  const size_t z_ctas = z_cta_count(d.d_model);
   const size_t n_mask = (F + kLogitTile - 1) / kLogitTile * (kLogitTile / 32);
   w.counts = take(LIF_CNT_LEN * 4);
   w.pointers = take(cap * 4);
@@ -35,7 +34,6 @@ Workspace plan_workspace(const lif_layer_desc& d, int ffn_grid_max) {
   w.active_slots = take(F * 4);
   w.hit_slots = take(F * 4);
   w.n_tmp = take(64);
-  w.z_partial = take(z_ctas * S * d.rank * 4);
   w.mask_words = take(n_mask * 4);
   w.new_mask_words = take(tagged_words(d) * 8);
   w.keep_tok = take(d.spec_keep > 0 ? F : 0);
@@ -44,6 +42,7 @@ Workspace plan_workspace(const lif_layer_desc& d, int ffn_grid_max) {
                                   : 0);
   w.gate_val = take(d.gate_mode == LIF_GATE_RESIDENT ? S * F * 4 : 0);
   w.hit_rows = take(F * 4);
+  w.row_stamps = take(cap * 4);
   w.step_sync = take(step_sync_bytes());
   w.step_tagged = take(step_tagged_bytes(d));
   size_t partial_rows = (size_t)ffn_grid_max;
@@ -158,10 +157,10 @@ lif_status lif_create_layer(const lif_layer_desc* desc, lif_layer** out) {
   L->active_slots = (int32_t*)(b + ws.active_slots);
   L->hit_slots = (int32_t*)(b + ws.hit_slots);
   L->n_tmp = (int32_t*)(b + ws.n_tmp);
-  L->z_partial = (float*)(b + ws.z_partial);
   L->mask_words = (uint32_t*)(b + ws.mask_words);
   L->new_mask_words = (unsigned long long*)(b + ws.new_mask_words);
   L->hit_rows = (uint32_t*)(b + ws.hit_rows);
+  L->row_stamps = (int32_t*)(b + ws.row_stamps);
   L->step_sync = (uint32_t*)(b + ws.step_sync);
   L->step_tagged = (uint32_t*)(b + ws.step_tagged);
   L->keep_tok = desc->spec_keep > 0 ? (int8_t*)(b + ws.keep_tok) : nullptr;
@@ -179,13 +178,13 @@ lif_status lif_create_layer(const lif_layer_desc* desc, lif_layer** out) {
   L->early_fetch = 1;
   ok = ok && ffn_batched_configure(L) == cudaSuccess;
   if (ok) {
-    L->z_ctas = z_cta_count(desc->d_model);
     L->ffn_grid = L->n_sm < ffn_grid_upper_bound() ? L->n_sm : ffn_grid_upper_bound();
     L->fetch_grid = L->n_sm;
     L->move_grid = L->n_sm;
     L->use_pdl = 1;
     L->wait_polls = kWaitLimit;
     L->spin_limit = kStepSpinLimit;
+    L->predictor_polls = kStepSpinLimit;
     L->split_ffn = 1;
     L->fused_plan = window_plan_supported(*desc) ? 1 : 0;
     L->fused_fetch = 1;
@@ -435,8 +434,10 @@ lif_status lif_decode_token_host(lif_layer* const* layers, int32_t n_layers, con
   if (cudaMemcpyAsync(dev_x, host_x, per * 2, cudaMemcpyHostToDevice, sc) != cudaSuccess)
     return LIF_ERR_CUDA;
   for (int l = 0; l < n_layers; ++l) {
+    layers[l]->input_late = l == 0;
     lif_status s = lif_decode_step(layers[l], dev_x, dev_y + (size_t)l * per, compute_stream,
                                    fetch_stream);
+    layers[l]->input_late = 0;
     if (s != LIF_OK) return s;
   }
   if (cudaMemcpyAsync(host_y, dev_y, per * 4 * n_layers, cudaMemcpyDeviceToHost, sc) !=
@@ -472,8 +473,11 @@ lif_status lif_graph_capture(lif_layer* const* layers, int32_t n_layers, void* d
     return LIF_ERR_CUDA;
   }
   lif_status s = LIF_OK;
-  for (int l = 0; l < n_layers && s == LIF_OK; ++l)
+  for (int l = 0; l < n_layers && s == LIF_OK; ++l) {
+    layers[l]->input_late = l == 0;
     s = lif_decode_step(layers[l], dev_x, dev_y + (size_t)l * per, compute_stream, fetch_stream);
+    layers[l]->input_late = 0;
+  }
   cudaError_t e = cudaStreamEndCapture(sc, &g->graph);   // always end, also after an error
   if (s == LIF_OK && e == cudaSuccess && cudaGraphInstantiate(&g->exec, g->graph, 0) == cudaSuccess) {
     *out = g;
@@ -578,6 +582,10 @@ lif_status lif_set_tuning(lif_layer* L, int32_t key, int32_t value) {
     case LIF_TUNE_STEP_POLLS:
       if (value < 0) return LIF_ERR_INVALID_ARG;
       L->spin_limit = (unsigned)value;
+      return LIF_OK;
+    case LIF_TUNE_PREDICTOR_POLLS:
+      if (value < 0) return LIF_ERR_INVALID_ARG;
+      L->predictor_polls = (unsigned)value;
       return LIF_OK;
     case LIF_TUNE_FFN_STAGES:
       if (value < 1 || value > L->ffn_stages_max) return LIF_ERR_INVALID_ARG;
@@ -711,8 +719,11 @@ lif_status lif_restore(lif_layer* L, const void* host_buf, size_t bytes) {
     }
     in += p[i].bytes;
   }
-  // entries of predictor runs after the snapshot must not be taken for those of the next run
-  if (cudaMemset(L->new_mask_words, 0, tagged_words(L->desc) * 8) != cudaSuccess ||
+  // entries of predictor runs after the snapshot must not be taken for those of the next run; the stamps by
+  // row are those of another state
+  const int32_t no_step = -1;
+  if (cudaMemcpy(L->counts + CNT_ROW_STAMPS, &no_step, 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemset(L->new_mask_words, 0, tagged_words(L->desc) * 8) != cudaSuccess ||
       launch_refill(L, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
     cudaGetLastError();
     return LIF_ERR_CUDA;

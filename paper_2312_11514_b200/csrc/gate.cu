@@ -142,7 +142,7 @@ gate_scores_kernel(const __half* __restrict__ x, const __half* __restrict__ gate
     }
   }
   if (!compact) return;     // the consumer reads the bit mask itself
-  compact_mask_last_cta(mask_words, nwords, ticket, active_idx, n_active, warp_sums, &is_last);
+  compact_mask_last_cta(mask_words, nwords, gridDim.x, ticket, active_idx, n_active, warp_sums, &is_last);
   // every CTA has read this run's number: the next run gets one of its own (in a decode step
   // the kernel that ends the step does this)
   if (is_last && tid == 0) advance_run(predictor_run, run);

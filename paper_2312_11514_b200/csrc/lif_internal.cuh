@@ -18,20 +18,21 @@ enum {
   CNT_NO_RUN = 18,          // always 0: runs that no step consumes are tagged with it
   CNT_ROWS_SUSPECT = 19,    // 1: a step committed a plan that not all of its CTAs carried out
   CNT_TICKET_CLEAR = 20,    // "last block done" counter of the kernel that clears the status
+  CNT_ROW_STAMPS = 21,      // step whose stamps row_stamps holds (all rows in use)
+  CNT_PREDICTOR_TICKETS = 22,   // uint64: CTAs of the predictor that have started, every launch as many
   CNT_TOTALS = 32           // four uint64: bytes_fetched, rows_moved, rows_active, rows_cached
 };
 
 constexpr int kNever = -(1 << 30);  // last_active stamp of a neuron never predicted active
 constexpr int kThreads = 256;
 constexpr int kWindowThreads = 1024;
-// rows of A per CTA in the first predictor stage: about 32 CTAs, so stage 2 folds few partials
-inline int z_rows_per_cta(int d_model) {
+// rows of A per part of the first predictor stage's sums: about 32 parts
+inline int z_rows_per_part(int d_model) {
   const int rows = ((d_model + 31) / 32 + 31) / 32 * 32;
   return rows < 32 ? 32 : rows;
 }
-constexpr int kMaxZPartials = 32;   // z_cta_count() never exceeds it
-inline int z_cta_count(int d_model) {
-  return (d_model + z_rows_per_cta(d_model) - 1) / z_rows_per_cta(d_model);
+inline int z_part_count(int d_model) {
+  return (d_model + z_rows_per_part(d_model) - 1) / z_rows_per_part(d_model);
 }
 constexpr int kLogitTile = 128;     // neurons per CTA in the second predictor stage
 constexpr int kMaxStreams = 8;
@@ -42,8 +43,8 @@ constexpr int kTimingEvents = 10;   // z0 z1 s1 w1 m1 | f0 f1 | g0 g1 r1
 struct Workspace {
   // offsets in bytes from the workspace base; every block 256-byte aligned
   size_t counts, pointers, slot_of, last_active, bias, active_idx, evict_ids, evict_slots,
-      move_src, move_dst, load_ids, load_slots, active_slots, hit_slots, n_tmp, z_partial,
-      mask_words, new_mask_words, keep_tok, h_rows, gate_val, hit_rows, step_sync, step_tagged, y_partial, total;
+      move_src, move_dst, load_ids, load_slots, active_slots, hit_slots, n_tmp,
+      mask_words, new_mask_words, keep_tok, h_rows, gate_val, hit_rows, row_stamps, step_sync, step_tagged, y_partial, total;
 };
 
 // fp16 elements per bundle / cache row: up | down, preceded by the gate row when it is bundled
@@ -64,14 +65,14 @@ struct lif_layer {
   __half* bias;
   int32_t *active_idx, *evict_ids, *evict_slots, *move_src, *move_dst, *load_ids, *load_slots,
       *active_slots, *hit_slots, *n_tmp;
-  float* z_partial;
   uint32_t* mask_words;
   // Neurons predicted active that have no cache row yet, as 64-bit entries {bits, run}: the low
   // half holds the bits of 32 consecutive neurons (of one predictor CTA's neurons, where those
   // are fewer), the high half the number of the predictor run that stored it (one store).
   // A second block of as many entries holds the active neurons themselves in the same form.  Behind
   // it a word per neuron, {cache row, run}, written where a neuron is active and cached; with a
-  // resident gate another one, {gate value, run}, written where it is active (one stream).
+  // resident gate another one, {gate value, run}, written where it is active (one stream), else the
+  // predictor's z = x.A, [S][rank] words {value, launch of the predictor}.
   unsigned long long* new_mask_words;
   int8_t* keep_tok;   // [d_ff] last kept token per neuron (speculative mode)
   float* y_partial;
@@ -85,12 +86,12 @@ struct lif_layer {
   // single-launch decode step (step.cu); step_ok = 0: it does not apply to this layer
   int step_ok, step_cache_ctas, step_sum_ctas, step_group, step_cache_stages, step_fetch_stages;
   size_t step_smem;
+  int32_t* row_stamps;        // [cap] last_active by row (see CNT_ROW_STAMPS)
   uint32_t* hit_rows;         // plan of the step: rows (before the moves) and neurons of the hits
   uint32_t* step_sync;        // its counters
   uint32_t* step_tagged;      // its tagged partial sums (no tag of a step to come)
   int n_sm;
   int max_smem;       // shared memory a CTA can opt in to
-  int z_ctas;         // CTAs of the first predictor stage
   int ffn_grid;       // CTAs of the sparse-FFN kernel
   int ffn_stages;     // bundles in flight per CTA
   int ffn_stages_max; // what fits the shared memory of one CTA
@@ -99,6 +100,8 @@ struct lif_layer {
   int move_grid;
   unsigned wait_polls; // poll limit of the first wait on each bulk copy
   unsigned spin_limit; // poll limit of the waits of a step's CTAs for one another
+  int input_late;      // set while the first layer of a token is enqueued: its input comes from a copy
+  unsigned predictor_polls;   // ... of the predictor's score CTAs for z
   int early_fetch;    // knob: the plain fetch of lif_decode_step starts early behind the window kernel
   int ends_step;      // set by lif_decode_step: the FFN's last kernel advances the run number
   int single_step;    // set by lif_decode_step: the single-launch step follows the predictor
@@ -169,11 +172,13 @@ inline int new_mask_entries(const lif_layer_desc& D) {
   if (D.gate_mode == LIF_GATE_RESIDENT) return (D.d_ff + gate_predict_tile() - 1) / gate_predict_tile();
   return (D.d_ff + kLogitTile - 1) / kLogitTile * (kLogitTile / 32);
 }
-// 64-bit words of the new_mask_words block: two blocks of entries, {row, run} and {gate value, run}
+// 64-bit words of the new_mask_words block: two blocks of entries, {row, run}, {gate value, run} or z
 inline size_t row_words_at(const lif_layer_desc& D) { return 2 * (size_t)new_mask_entries(D); }
 inline size_t gate_words_at(const lif_layer_desc& D) { return row_words_at(D) + D.d_ff; }
+inline size_t z_words_at(const lif_layer_desc& D) { return gate_words_at(D); }
 inline size_t tagged_words(const lif_layer_desc& D) {
-  return gate_words_at(D) + (D.gate_mode == LIF_GATE_RESIDENT ? D.d_ff : 0);
+  return D.gate_mode == LIF_GATE_RESIDENT ? gate_words_at(D) + D.d_ff
+                                          : z_words_at(D) + (size_t)D.n_streams * D.rank;
 }
 // early: what the kernel may do before its own dependency wait.  kEarlyLists: the lists were
 // final before the kernel ahead of this one passed its wait, so the first bundle's host loads
@@ -187,10 +192,6 @@ enum { kEarlyNone = 0, kEarlyLists = 1, kEarlyMask = 2, kEarlyWatch = 3 };
 cudaError_t launch_fetch_ffn(lif_layer* L, const __half* x, float* partial, cudaStream_t st,
                              int early);
 cudaError_t predict_configure(const lif_layer* L);
-// several input streams (predict_multi.cu)
-cudaError_t predict_multi_configure(const lif_layer* L);
-cudaError_t launch_predict_multi(lif_layer* L, const __half* x, float* logits, int32_t* active_idx,
-                                 int32_t* n_active, cudaStream_t st, cudaEvent_t* ev, int compact);
 // Everything of a decode step behind the predictor, in one launch (step.cu): one input stream, or several
 // as long as their output fits a CTA's registers.
 size_t step_sync_bytes();

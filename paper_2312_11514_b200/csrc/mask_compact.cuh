@@ -28,12 +28,12 @@ __device__ __forceinline__ int block_exclusive_scan_256(int v, int* total, int* 
   return base + inc - v;
 }
 
-// Every CTA calls this after writing its words of `mask_words`.  The CTA that draws the last
+// Every one of `n_ctas` CTAs calls this after writing its words of `mask_words`.  The CTA that draws the last
 // ticket prefix-sums the whole mask (nwords words) into active_idx / n_active and re-arms the
 // ticket; the list order never depends on scheduling.  warp_sums: kThreads / 32 ints and
 // is_last: one int, both in shared memory.
 __device__ __forceinline__ void compact_mask_last_cta(const uint32_t* mask_words, int nwords,
-                                                      int* ticket, int* __restrict__ active_idx,
+                                                      int n_ctas, int* ticket, int* __restrict__ active_idx,
                                                       int* __restrict__ n_active, int* warp_sums,
                                                       int* is_last) {
   const int tid = threadIdx.x;
@@ -41,7 +41,7 @@ __device__ __forceinline__ void compact_mask_last_cta(const uint32_t* mask_words
   if (tid == 0) {     // releases the CTA's words, acquires the others' (one fence, not one per thread)
     int t;
     asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(t) : "l"(ticket) : "memory");
-    *is_last = (t == (int)gridDim.x - 1);
+    *is_last = (t == n_ctas - 1);
   }
   __syncthreads();
   if (!*is_last) return;

@@ -80,6 +80,7 @@ struct StepArgs {
   const int* predictor_run;
   int* next_run;                  // bumped at the end (a predictor without a first stage needs it)
   int32_t* n_act_out;
+  int32_t* row_stamps;            // last_active by row, as long as CNT_ROW_STAMPS names this step
   uint32_t* hit_rows;             // plan: row before the moves | neuron << 16, for the cache CTAs
   const unsigned char* store;
   unsigned char* cache;
@@ -200,6 +201,22 @@ __device__ __forceinline__ bool read_entries(const unsigned long long* const (&e
   }
   return ok != 0;
 }
+// The low half of a word that the predictor run `run` stores beside its entries, once it is there (it is
+// stored with the entry: a poll or two).  checked = false: as it is (see read_entries).
+__device__ __forceinline__ uint32_t word_of_run(const StepArgs& a, const unsigned long long* at, int run,
+                                                bool checked) {
+  unsigned long long v = checked ? 0ull : ld_relaxed64(at);
+  bool there = !checked;
+  for (unsigned i = 0; i < a.spin_limit && !there; ++i) {
+    v = ld_relaxed64(at);
+    there = (int)(v >> 32) == run;
+  }
+  if (!there) {                                            // (row 0, gate value 0)
+    timed_out(a);
+    v = 0;
+  }
+  return (uint32_t)v;
+}
 // Thread 0 waits for the plan; everyone gets it (0 if it did not come: an error is recorded).
 __device__ __forceinline__ unsigned long long wait_plan(const StepArgs& a,
                                                         unsigned long long* shared) {
@@ -225,13 +242,17 @@ __host__ __device__ __forceinline__ size_t x_smem_bytes(int d, int S) {
 }
 
 // ---- window CTA ---------------------------------------------------------------------------------
-// The same plan as the window kernels (window.cu), held in shared memory: slot_of of every neuron
-// and row -> neuron, age of every row are read before the predictor's entries arrive (the window
-// state was last written by this layer's previous step), so between the entries and the flag there
-// are only shared-memory passes and block scans.  What the other CTAs need is written ahead of the
-// flag, the rest of the lists and the state behind it.
+// The same plan as the window kernels (window.cu), held in shared memory: row -> neuron and age of every
+// row are read before the predictor's entries arrive (the window state was last written by this layer's
+// previous step), so between the entries and the flag there are one round trip for the active neurons'
+// rows, shared-memory passes and block scans.  What the other CTAs need is written ahead of the flag,
+// the rest of the lists and the state behind it.
+// The reads ahead of the entries are few and coalesced, because they run beside the predictor: reading slot_of of
+// every neuron (64 KB at 16384) and the stamp of every row by its neuron held back the predictor's CTA on
+// the same SM, and with it the last entry, by 1.5 us (2.2 at 4544 columns).  So the step keeps a copy of the
+// stamps by row, which a window update by another kernel makes out of date (CNT_ROW_STAMPS).
 size_t window_role_smem(int F, int cap) {
-  return 4 * (size_t)F + 8 * (size_t)cap + 4 * (size_t)((F + 31) / 32) + 64;
+  return 4 * (size_t)F + 10 * (size_t)cap + 4 * (size_t)((F + 31) / 32) + 64;
 }
 
 __device__ void window_role(const StepArgs& a, unsigned char* smem) {
@@ -240,43 +261,25 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
   __shared__ int loads;
   const WindowArgs& w = a.w;
   const int tid = threadIdx.x, F = w.F;
-  unsigned short* slot_s = reinterpret_cast<unsigned short*>(smem);   // [F] row or kNoSlot
+  unsigned short* slot_s = reinterpret_cast<unsigned short*>(smem);   // [F] row of each of these, or kNoSlot
   unsigned short* act_s = slot_s + F;                                 // [F] active ids, ascending
-  unsigned short* pid_s = act_s + F;                                  // [cap] row -> neuron
-  unsigned short* age_s = pid_s + w.cap;                              // [cap] steps since active
-  unsigned short* hole_s = age_s + w.cap;                             // [cap] freed rows, ascending
+  int* stamp_s = reinterpret_cast<int*>(act_s + F);                   // [cap] step in which it was active last
+  unsigned short* pid_s = reinterpret_cast<unsigned short*>(stamp_s + w.cap);   // [cap] row -> neuron
+  unsigned short* hole_s = pid_s + w.cap;                             // [cap] freed rows, ascending
   unsigned short* moved_s = hole_s + w.cap;                           // [cap] row - bound -> new row
-  uint32_t* bits = reinterpret_cast<uint32_t*>(moved_s + w.cap);      // [F / 32]
+  uint32_t* bits = reinterpret_cast<uint32_t*>(moved_s + (w.cap + (w.cap & 1)));   // [F / 32]
 
   const int n = w.counts[LIF_CNT_NUM_USED];
   const int t = w.counts[LIF_CNT_STEP];
   const int stale_input = w.counts[LIF_CNT_STATUS] == LIF_ERR_TIMEOUT;   // see window.cu
   const int t_end = t + w.keep - 1;
-  // (-1 becomes kNoSlot by itself)
-  for (int i0 = tid; i0 < F / 4; i0 += 8 * kStepThreads) {
-    int4 s[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (i0 + j * kStepThreads < F / 4) s[j] = reinterpret_cast<const int4*>(w.slot_of)[i0 + j * kStepThreads];
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (i0 + j * kStepThreads < F / 4)
-        reinterpret_cast<ushort4*>(slot_s)[i0 + j * kStepThreads] =
-            make_ushort4((unsigned short)s[j].x, (unsigned short)s[j].y, (unsigned short)s[j].z,
-                         (unsigned short)s[j].w);
-  }
-  for (int s0 = tid; s0 < n; s0 += 4 * kStepThreads) {
-    int id[4], la[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) id[j] = s0 + j * kStepThreads < n ? w.pointers[s0 + j * kStepThreads] : 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) la[j] = s0 + j * kStepThreads < n ? w.last_active[id[j]] : 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (s0 + j * kStepThreads < n) {
-        pid_s[s0 + j * kStepThreads] = (unsigned short)id[j];
-        age_s[s0 + j * kStepThreads] = (unsigned short)min(65535, max(1, t_end - la[j]));
-      }
+  const bool stamps = w.counts[CNT_ROW_STAMPS] == t;
+#pragma unroll 2
+  for (int s = tid; s < n; s += kStepThreads) {
+    const int id = w.pointers[s];
+    const int la = stamps ? a.row_stamps[s] : w.last_active[id];
+    pid_s[s] = (unsigned short)id;
+    stamp_s[s] = la;
   }
   uint32_t act_w[1][kEntriesPerThread];
   read_entries<1>({a.act_entries}, a.n_entries, __ldcg(a.predictor_run), act_w);
@@ -299,6 +302,9 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
         act_s[q++] = (unsigned short)((tid * kEntriesPerThread + i) * 32 + __ffs(m) - 1);
   }
   __syncthreads();
+#pragma unroll 2
+  for (int q = tid; q < na; q += kStepThreads) slot_s[q] = (unsigned short)w.slot_of[act_s[q]];   // (-1: kNoSlot)
+  __syncthreads();
   // each thread owns a run of consecutive rows and of consecutive active neurons
   const int seg = (n + kStepThreads - 1) / kStepThreads;
   const int s0 = min(n, tid * seg), s1 = min(n, s0 + seg);
@@ -306,10 +312,10 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
   const int q0 = min(na, tid * qseg), q1 = min(na, q0 + qseg);
   auto idle_age = [&](int s) {       // 0: active now
     const int id = pid_s[s];
-    return (bits[id >> 5] >> (id & 31)) & 1u ? 0 : (int)age_s[s];
+    return (bits[id >> 5] >> (id & 31)) & 1u ? 0 : max(1, t_end - stamp_s[s]);
   };
   int c_load = 0;
-  for (int q = q0; q < q1; ++q) c_load += slot_s[act_s[q]] == kNoSlot;
+  for (int q = q0; q < q1; ++q) c_load += slot_s[q] == kNoSlot;
   int k_eff = w.k;
   if (w.budget > 0) {                // memory budget: shrink the window for this step if needed
     if (tid <= kMaxBudgetWindow) hist[tid] = 0;
@@ -385,7 +391,7 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
   {
     int p_load = p_load0;
     for (int q = q0; q < q1; ++q) {
-      const int id = act_s[q], s = slot_s[id];
+      const int id = act_s[q], s = slot_s[q];
       if (s == kNoSlot) {
         w.load_slots[p_load] = new_row(p_load);
         ++p_load;
@@ -411,17 +417,22 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
         w.slot_of[id] = -1;
       } else if (s >= bound) {
         const int dst = hole_s[reuse + n_moves - 1 - p_surv++];
+        a.row_stamps[dst] = stamp_s[s];                    // (those of active neurons follow below)
         w.pointers[dst] = id;
         w.slot_of[id] = dst;
         w.bias[dst] = w.bias_up[id];
+      } else if (!stamps) {
+        a.row_stamps[s] = stamp_s[s];
       }
       if (s >= n_kept + n_load) w.pointers[s] = -1;      // tail beyond the rows in use
     }
+    __syncthreads();
     int p_load = p_load0;
     for (int q = q0; q < q1; ++q) {
       const int id = act_s[q];
-      int s = slot_s[id];
-      w.last_active[id] = active_stamp(w, id, t, t_end);
+      int s = slot_s[q];
+      const int stamp = active_stamp(w, id, t, t_end);
+      w.last_active[id] = stamp;
       if (s == kNoSlot) {
         s = new_row(p_load);
         w.load_ids[p_load++] = id;
@@ -432,6 +443,7 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
         if (s >= bound) s = moved_s[s - bound];
         w.hit_slots[q - p_load] = s;
       }
+      a.row_stamps[s] = stamp;
       w.active_slots[q] = s;
       w.active_idx[q] = id;
     }
@@ -447,6 +459,7 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
     w.counts[LIF_CNT_NUM_KEPT] = n_kept;
     w.counts[LIF_CNT_NUM_USED] = n_kept + n_load;
     w.counts[LIF_CNT_STEP] = t + w.keep;
+    w.counts[CNT_ROW_STAMPS] = t + w.keep;
     w.counts[LIF_CNT_K_EFF] = k_eff;
     unsigned long long* totals = reinterpret_cast<unsigned long long*>(w.counts + CNT_TOTALS);
     totals[0] += (unsigned long long)n_load * w.bundle_bytes;
@@ -564,22 +577,6 @@ __device__ __forceinline__ float row_weight(const StepArgs& a, float b, float fi
   if (kGate == LIF_GATE_BUNDLED) return apply_activation(first + b, a.act, a.act_thr) * second;
   if (kGate == LIF_GATE_RESIDENT) return apply_activation(b, a.act, a.act_thr) * first;
   return apply_activation(first + b, a.act, a.act_thr);
-}
-// The low half of a word that the predictor run `run` stores beside its entries, once it is there (it is
-// stored with the entry: a poll or two).  checked = false: as it is (see read_entries).
-__device__ __forceinline__ uint32_t word_of_run(const StepArgs& a, const unsigned long long* at, int run,
-                                                bool checked) {
-  unsigned long long v = checked ? 0ull : ld_relaxed64(at);
-  bool there = !checked;
-  for (unsigned i = 0; i < a.spin_limit && !there; ++i) {
-    v = ld_relaxed64(at);
-    there = (int)(v >> 32) == run;
-  }
-  if (!there) {                                            // (row 0, gate value 0)
-    timed_out(a);
-    v = 0;
-  }
-  return (uint32_t)v;
 }
 // the neuron's bias; resident gate (one stream): its gate value
 template <int kGate>
@@ -1145,7 +1142,9 @@ StepKernel step_kernel_for(const lif_layer_desc& D) {
   return step_kernel<LIF_GATE_NONE, 1>;
 }
 constexpr int kGroupMax = 8, kUngroupedMax = 64, kUngroupedMaxStreams = 16;
-constexpr size_t kCacheRing = 128 * 1024, kFetchRing = 32 * 1024;
+// One step CTA per SM (with less, two fit and are put on one SM where others are not free yet), and beside it one of
+// the next layer's low-rank predictor, 91 KB at 4096 x 128.
+constexpr size_t kCacheRing = 112 * 1024, kCacheRingGate = 128 * 1024, kFetchRing = 32 * 1024;
 
 // CTAs that add up the outputs: 16 pairs of columns or more each, which leaves 16 slices of the partials to
 // a CTA's threads (several streams: 128 pairs).
@@ -1205,7 +1204,7 @@ cudaError_t step_configure(lif_layer* L) {
   L->step_sum_ctas = sum_ctas(D);
   L->step_group = L->step_cache_ctas > hit_partials_max(D) ? kGroupMax : 1;
   const size_t hits = 2 * (((size_t)D.capacity + L->step_cache_ctas - 1) / L->step_cache_ctas);
-  L->step_cache_stages = stages(kCacheRing, x + hits, 1);
+  L->step_cache_stages = stages(D.gate_mode == LIF_GATE_RESIDENT ? kCacheRingGate : kCacheRing, x + hits, 1);
   // (paper's cache order: bundles wait in the ring, see fetch_role; twice the ring keeps the link busy)
   L->step_fetch_stages = stages(D.append_first ? kFetchRing : 2 * kFetchRing, x + ids, 2);
   size_t smem = window_role_smem(D.d_ff, D.capacity);
@@ -1233,6 +1232,7 @@ cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st
   a.predictor_run = L->counts + CNT_PREDICTOR_RUN;
   a.next_run = (int*)(L->counts + CNT_PREDICTOR_RUN);
   a.n_act_out = L->n_tmp;
+  a.row_stamps = L->row_stamps;
   a.hit_rows = L->hit_rows;
   a.store = (const unsigned char*)L->dev_bundles;
   a.cache = (unsigned char*)D.dev_cache;
