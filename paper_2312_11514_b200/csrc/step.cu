@@ -89,6 +89,9 @@ struct StepArgs {
   const __half* b_down;
   float* p_member;                // partial sums of cache CTAs that form groups, [cta][d]
   uint4 *p_hit, *p_new;           // tagged partial sums of cache CTAs (or groups) and fetch CTAs
+  // several streams: each fetch CTA's last row, as tagged words: its down column in pairs of fp16 values
+  // [cta][d / 2], and its weights [cta][8]
+  unsigned long long *last_down, *last_h;
   float* y;
   StepSync* sync;
   int d, n_streams, whole_cache, act;
@@ -535,6 +538,9 @@ __device__ __forceinline__ ulonglong2 load_tagged(const uint4* src) {
   asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(src) : "memory");
   return v;
 }
+__device__ __forceinline__ void store_tagged_word(unsigned long long* dst, uint32_t low, unsigned tag) {
+  store_with_run(dst, low, (int)tag);
+}
 __device__ __forceinline__ bool has_tag(const ulonglong2& v, unsigned tag) {
   return (unsigned)(v.x >> 32) == tag && (unsigned)(v.y >> 32) == tag;
 }
@@ -838,8 +844,51 @@ struct Summer {
     lost = 0;
     t_next = end <= slice ? slice : slice + (end - slice + slices - 1) / slices * slices;
   }
+  // adds the thread's share of the fetch CTAs' last rows to column pair `col`
+  __device__ __forceinline__ void add_last(int n_last, int col) {
+    constexpr int kRows = 16;                              // (all of a thread's: 32 CTAs, 2 slices or more)
+    if (col >= c1) return;
+    const int half_d = a.d >> 1, s = col / half_d;
+    const unsigned long long *down = a.last_down + col % half_d, *h = a.last_h + s;
+    for (int t0 = slice; t0 < n_last; t0 += slices * kRows) {
+      auto ask = [&](unsigned long long (&v)[kRows], const unsigned long long* p, int stride, bool pause) {
+        bool there = false;
+        for (unsigned polls = 0; polls < a.spin_limit && !there; ++polls) {
+          there = true;
+#pragma unroll
+          for (int k = 0; k < kRows; ++k) {
+            const int t = t0 + k * slices;
+            v[k] = t < n_last ? ld_relaxed64(p + (size_t)t * stride) : (unsigned long long)tag << 32;
+          }
+#pragma unroll
+          for (int k = 0; k < kRows; ++k) there = there && (unsigned)(v[k] >> 32) == tag;
+          if (pause && !there) __nanosleep(100);
+        }
+        return there;
+      };
+      // the columns, with pauses while the rows travel; when they are there the weights follow at once
+      unsigned long long v[kRows];
+      uint32_t pair[kRows];
+      bool there = ask(v, down, half_d, true);
+#pragma unroll
+      for (int k = 0; k < kRows; ++k) pair[k] = (uint32_t)v[k];
+      there = there && ask(v, h, 8, false);
+      if (!there) {
+        lost = 1;
+        return;
+      }
+#pragma unroll
+      for (int k = 0; k < kRows; ++k)
+        if (t0 + k * slices < n_last) {
+          const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&pair[k]));
+          const float w = __uint_as_float((uint32_t)v[k]);
+          v_sum.x = fmaf(w, f.x, v_sum.x);
+          v_sum.y = fmaf(w, f.y, v_sum.y);
+        }
+    }
+  }
   // red: kStepThreads values in shared memory
-  __device__ __forceinline__ void finish(float2* red) {
+  __device__ __forceinline__ void finish(float2* red, int n_last) {
     const int tid = threadIdx.x, nvec = a.d >> 3;
     for (int cc = c0; cc < c1; cc += width) {
       const int col = cc + tid % width;
@@ -849,6 +898,10 @@ struct Summer {
         __syncthreads();                                   // red[] is free again
       }
       add(have, col, a.spin_limit);
+      if (kS > 1) {
+        if (lost) timed_out(a);
+        add_last(n_last, col);
+      }
       if (lost) timed_out(a);
       red[tid] = v_sum;
       __syncthreads();
@@ -871,7 +924,10 @@ constexpr size_t kSumSmem = kStepThreads * sizeof(float2);
 
 // ---- sum CTAs ----------------------------------------------------------------------------------------
 // They wait for a word of the fetch CTAs' partials, with pauses, so that they do not load the memory
-// system while the rows travel.  Several streams: for one of each CTA, to read everything at once.  One
+// system while the rows travel.  Several streams: for one of each CTA, to read everything at once, while the
+// CTAs' last rows are still on their way; then for the weights of those, whose terms they add themselves (a
+// partial has as many values as all outputs together, 160 KB for 5 streams at 4096 columns: stored, read and
+// added behind the last bundle that was 9.5 us of a step; a down column and five weights are 5.4).  One
 // stream: for one of the CTA with the fewest rows, adding the cached rows' partials meanwhile if they come
 // first, and then they take what is missing as it comes: a single round trip from the last partial,
 // whichever it is, to y.  With at most two rows per fetch CTA the whole wait is a few microseconds and a
@@ -887,7 +943,9 @@ __device__ void sum_role(const StepArgs& a, int index, unsigned char* smem) {
   const int run = __ldcg(a.predictor_run);
   const unsigned long long plan = wait_plan(a, &plan_s);
   const int n_load = plan_loads(plan);                     // (0: refused)
-  Summer<kS> sum(a, index, a.n_sum_ctas, plan_rows(plan), min(kFetchCtas, n_load));
+  const int n_last = min(kFetchCtas, n_load);              // fetch CTAs with rows; with several of them
+  Summer<kS> sum(a, index, a.n_sum_ctas, plan_rows(plan),
+                 kS == 1 ? n_last : max(0, min(kFetchCtas, n_load - kFetchCtas)));
   const size_t pairs = (size_t)a.n_streams * (a.d >> 1);
   const int n_new = sum.have - sum.have_hit;
   if (kS == 1) {
@@ -905,7 +963,7 @@ __device__ void sum_role(const StepArgs& a, int index, unsigned char* smem) {
     }
   }
   __syncthreads();
-  sum.finish(reinterpret_cast<float2*>(smem));             // kSumSmem bytes
+  sum.finish(reinterpret_cast<float2*>(smem), n_last);     // kSumSmem bytes
   // (by the CTA that started last: every other one has read the number by now)
   if (index == a.n_sum_ctas - 1 && tid == 0) advance_run(a.next_run, run);
 }
@@ -999,8 +1057,16 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   __syncthreads();
   unsigned parity = 0;
   int from = cnt;                                          // first row that was not waited for any longer
+  int given = 0;                                           // several streams: 1 partial, 2 last row handed over
+  unsigned long long* last_down = a.last_down + (size_t)f * (d >> 1);
+  unsigned long long* last_h = a.last_h + f * 8;
   for (int i = 0, st = 0; i < from; ++i) {
     const uint4* row = reinterpret_cast<const uint4*>(ring + (size_t)st * row_bytes);
+    const bool is_last = kS > 1 && i == cnt - 1;
+    if (is_last) {                                         // the partial sum, while the last row travels
+      if (i > 0) store_tagged_partial<kS>(acc, a.p_new + (size_t)f * S * (d >> 1), nvec, S, a.epoch + 1);
+      given = 1;
+    }
     const bool landed = mbar_wait(bars + st, parity, a.wait_polls);
     if (tid == 0 && landed && i + first < cnt) {           // the next one, in the stage of an earlier row?
       const bool reuse = i + first >= stages;
@@ -1021,6 +1087,19 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
     }
     if (tid == 0 && landed && i + 1 < from) store_rows(i + 1);   // (the last one behind the partial sum)
     const float b = row_scalar<kGate>(a, ids[i], run, checked);
+    if (is_last) {
+#pragma unroll
+      for (int k = 0; k < Shape<kS>::kChunks; ++k) {
+        const int v = tid + k * kStepThreads;
+        if (v < nvec) {
+          const uint4 q = row[(kVec - 1) * nvec + v];
+          store_tagged_word(last_down + v, q.x, a.epoch + 1);
+          store_tagged_word(last_down + nvec + v, q.y, a.epoch + 1);
+          store_tagged_word(last_down + 2 * nvec + v, q.z, a.epoch + 1);
+          store_tagged_word(last_down + 3 * nvec + v, q.w, a.epoch + 1);
+        }
+      }
+    }
     float p[kS], p2[kS];
 #pragma unroll
     for (int s = 0; s < kS; ++s) p[s] = p2[s] = 0.f;
@@ -1074,7 +1153,15 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
           v1 += __shfl_xor_sync(0xffffffffu, v1, o);
           v2 += __shfl_xor_sync(0xffffffffu, v2, o);
         }
-        if (lane == 0) h_s[warp] = warp >= S ? 0.f : row_weight<kGate>(a, b, v1, v2);
+        const float h = warp >= S ? 0.f : row_weight<kGate>(a, b, v1, v2);
+        if (lane == 0) {
+          h_s[warp] = h;
+          if (is_last) store_tagged_word(last_h + warp, __float_as_uint(h), a.epoch + 1);
+        }
+      }
+      if (is_last) {
+        given = 2;
+        break;
       }
       __syncthreads();
       axpy_row<kS>(acc, down, h_s, nvec);
@@ -1085,7 +1172,12 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       parity ^= 1u;
     }
   }
-  if (cnt > 0) store_tagged_partial<kS>(acc, a.p_new + (size_t)f * S * (d >> 1), nvec, S, a.epoch + 1);
+  if (kS == 1 ? cnt > 0 : cnt > 1 && given == 0)
+    store_tagged_partial<kS>(acc, a.p_new + (size_t)f * S * (d >> 1), nvec, S, a.epoch + 1);
+  if (kS > 1 && cnt > 0 && given < 2) {                    // given up: nothing comes of the last row
+    for (int v = tid; v < d >> 1; v += kStepThreads) store_tagged_word(last_down + v, 0u, a.epoch + 1);
+    if (tid < 8) store_tagged_word(last_h + tid, 0u, a.epoch + 1);
+  }
   if (tid == 0) {
     if (cnt > 0 && (go < 0 || (go > 0 && !moved))) learn(true);
     store_rows(from);
@@ -1171,7 +1263,9 @@ int hit_partials_max(const lif_layer_desc& D) {
 
 size_t step_sync_bytes() { return sizeof(StepSync); }
 size_t step_tagged_bytes(const lif_layer_desc& D) {
-  return step_kernel_for(D) ? (size_t)(hit_partials_max(D) + kFetchCtas) * D.n_streams * D.d_model * 8 : 0;
+  if (!step_kernel_for(D)) return 0;
+  return (size_t)(hit_partials_max(D) + kFetchCtas) * D.n_streams * D.d_model * 8 +
+         (D.n_streams > 1 ? (size_t)kFetchCtas * (D.d_model * 4 + 8 * 8) : 0);
 }
 
 // Shape of the launch, and whether the single launch applies: streams x width in registers, ids and
@@ -1242,6 +1336,8 @@ cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st
   a.p_member = L->y_partial;
   a.p_hit = (uint4*)L->step_tagged;
   a.p_new = a.p_hit + (size_t)hit_partials_max(D) * D.n_streams * (D.d_model / 2);
+  a.last_down = (unsigned long long*)(a.p_new + (size_t)kFetchCtas * D.n_streams * (D.d_model / 2));
+  a.last_h = a.last_down + (size_t)kFetchCtas * (D.d_model / 2);
   a.y = y;
   a.sync = (StepSync*)L->step_sync;
   a.d = D.d_model;
