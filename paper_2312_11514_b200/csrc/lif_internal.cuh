@@ -72,7 +72,8 @@ struct lif_layer {
   // A second block of as many entries holds the active neurons themselves in the same form.  Behind
   // it a word per neuron, {cache row, run}, written where a neuron is active and cached; with a
   // resident gate another one, {gate value, run}, written where it is active (one stream), else the
-  // predictor's z = x.A, [S][rank] words {value, launch of the predictor}.
+  // predictor's z = x.A, [S][rank] words {value, launch of the predictor},
+  // or its parts' sums, [part][S][rank].
   unsigned long long* new_mask_words;
   int8_t* keep_tok;   // [d_ff] last kept token per neuron (speculative mode)
   float* y_partial;
@@ -172,13 +173,17 @@ inline int new_mask_entries(const lif_layer_desc& D) {
   if (D.gate_mode == LIF_GATE_RESIDENT) return (D.d_ff + gate_predict_tile() - 1) / gate_predict_tile();
   return (D.d_ff + kLogitTile - 1) / kLogitTile * (kLogitTile / 32);
 }
+bool z_by_parts(const lif_layer_desc& D);           // the first predictor stage leaves its parts' sums (predict.cu)
 // 64-bit words of the new_mask_words block: two blocks of entries, {row, run}, {gate value, run} or z
 inline size_t row_words_at(const lif_layer_desc& D) { return 2 * (size_t)new_mask_entries(D); }
 inline size_t gate_words_at(const lif_layer_desc& D) { return row_words_at(D) + D.d_ff; }
 inline size_t z_words_at(const lif_layer_desc& D) { return gate_words_at(D); }
+inline size_t z_words(const lif_layer_desc& D) {
+  return (size_t)D.n_streams * D.rank * (z_by_parts(D) ? z_part_count(D.d_model) : 1);
+}
 inline size_t tagged_words(const lif_layer_desc& D) {
   return D.gate_mode == LIF_GATE_RESIDENT ? gate_words_at(D) + D.d_ff
-                                          : z_words_at(D) + (size_t)D.n_streams * D.rank;
+                                          : z_words_at(D) + z_words(D);
 }
 // early: what the kernel may do before its own dependency wait.  kEarlyLists: the lists were
 // final before the kernel ahead of this one passed its wait, so the first bundle's host loads

@@ -3,8 +3,9 @@
 //
 // One launch for both contractions, fp16 factors with fp32 sums.  Its CTAs take parts in the order in
 // which they start:
-//   z CTAs      (first)  8 (or 4) columns of z = x.A for one, two or four streams, finished: every value
-//                        is stored as one word with the number of this launch
+//   z CTAs      (first)  8 columns of z = x.A for one, two or four streams, finished: every value is
+//                        stored as one word with the number of this launch; or (z_by_parts) the sums of one
+//                        part of A's rows for all columns and streams, which the score CTAs add up
 //   score CTAs  (then)   128 neurons: re-read the words of z until they carry the number, then
 //                        scores = z.B + c, threshold, bit mask; on request the last one to finish turns
 //                        the mask into the sorted list with a block prefix sum
@@ -30,7 +31,7 @@ struct PredictArgs {
   const __half *x, *A, *B;
   const float* c;
   float theta;
-  int d, r, F, keep, compact, first_pass;
+  int d, r, F, keep, compact, first_pass, by_parts;
   // stage 1: runs of rows, `per` rows each; CTAs per column group; streams and columns per CTA
   int parts, rows, lanes, per, groups_of_streams, h, cw, n_z, x_at, red_at;
   // stage 2
@@ -191,6 +192,69 @@ __device__ void z_role(const PredictArgs& a, int S, int part_of_grid, unsigned c
   }
 }
 
+// Where a column group is too long or there are too few of them: a CTA adds one part of A's rows, all columns
+// and streams, and hands over the part's sums.  A's pieces travel into the thread's own slots of shared memory
+// ahead of the wait, whole rows at a time.
+template <int S>
+__device__ void z_part_role(const PredictArgs& a, int part, unsigned char* smem) {
+  const int tid = threadIdx.x, ncg = a.r >> 3, stride = kThreads / ncg;
+  const int cg = tid % ncg, lane = tid / ncg;
+  const int m0 = part * a.rows, m1 = min(a.d, m0 + a.rows);
+  uint4* a_s = reinterpret_cast<uint4*>(smem) + tid;                   // [per][kThreads]
+  __half* x_s = reinterpret_cast<__half*>(smem + a.x_at);              // [S][rows]
+  float* red = reinterpret_cast<float*>(smem + a.red_at);              // [lanes][r]
+  for (int u = 0, m = m0 + lane; lane < stride && m < m1; ++u, m += stride)
+    copy_async16(a_s + u * kThreads, a.A + (size_t)m * a.r + cg * 8);
+#pragma unroll 1
+  for (int pass = a.first_pass; pass < 2; ++pass) {
+    if (pass) {
+      pdl_wait();
+      pdl_trigger();
+    }
+    const int vecs = (m1 - m0) >> 3;
+#pragma unroll 1
+    for (int i = tid; i < S * vecs; i += kThreads) {
+      const int s = i / vecs, v = i - s * vecs;
+      reinterpret_cast<uint4*>(x_s + s * a.rows)[v] = __ldcg(reinterpret_cast<const uint4*>(a.x + (size_t)s * a.d + m0) + v);
+    }
+    if (pass) own_copies_wait();
+    __syncthreads();
+    float2 acc[S][4];
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc[s][k] = make_float2(0.f, 0.f);
+    const uint4* row = a_s;
+#pragma unroll 2
+    for (int m = lane; m < (lane < stride ? m1 - m0 : 0); m += stride, row += kThreads) {
+      float2 f[4];
+      unpack8(*row, f);
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        const float xv = __half2float(x_s[s * a.rows + m]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[s][k] = fma2(make_float2(xv, xv), f[k], acc[s][k]);
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      if (lane < a.lanes) {
+        float2* dst = reinterpret_cast<float2*>(red + lane * a.r + cg * 8);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dst[k] = acc[s][k];
+      }
+      __syncthreads();
+      for (int j = tid; j < a.r; j += kThreads) {
+        float v = 0.f;
+#pragma unroll 8
+        for (int l = 0; l < a.lanes; ++l) v += red[l * a.r + j];
+        if (pass) store_with_run(a.z + ((size_t)part * S + s) * a.r + j, __float_as_uint(v), a.launch);
+      }
+      __syncthreads();
+    }
+  }
+}
+
 // ---- stage 2 -------------------------------------------------------------------------------------------
 // streams side by side in shared memory: 1, 2, 4 or 8
 __host__ __device__ constexpr int padded(int S) { return S <= 2 ? S : (S <= 4 ? 4 : 8); }
@@ -243,7 +307,30 @@ __device__ void score_role(const PredictArgs& a, int tile, unsigned char* smem) 
   const int my_row = my_col < F ? __ldcg(a.slot_of + my_col) : 0;
   {
     unsigned polls = 0;
-    for (int j = tid; j < r; j += kThreads) {
+    for (int i = tid; a.by_parts && i < S * r; i += kThreads) {          // the parts' sums, in order
+      float sum = 0.f;
+      bool all = true;
+      for (int p0 = 0; p0 < a.parts; p0 += 8) {
+        unsigned long long v[8];
+        bool there;
+        do {
+          there = true;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v[k])
+                         : "l"(a.z + (size_t)min(p0 + k, a.parts - 1) * S * r + i) : "memory");
+            there = there && (!a.tickets || (int)(v[k] >> 32) == a.launch);
+          }
+        } while (pass && !there && polls++ < a.spin_limit);
+        all = all && there;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (p0 + k < a.parts) sum += __uint_as_float((unsigned)v[k]);
+      }
+      if (pass && !all) flag_timeout(a.status);
+      zs[S == 1 ? i : (i % r) * SP + i / r] = all ? sum : __int_as_float(0x7fffffff);
+    }
+    for (int j = tid; !a.by_parts && j < r; j += kThreads) {
       unsigned long long v[S];
       bool there;
       do {
@@ -365,6 +452,7 @@ __global__ void __launch_bounds__(kThreads, 2) predict_kernel(PredictArgs a) {
     a.launch = (int)launch_s;
   }
   if (part >= (unsigned)a.n_z) score_role<S>(a, (int)part - a.n_z, smem);
+  else if (a.by_parts) z_part_role<S>(a, (int)part, smem);
   else if (a.cw == 2) z_role<1, 2>(a, S, (int)part, smem);
   else if (a.cw == 4) z_role<1, 4>(a, S, (int)part, smem);
   else if (S == 1 || a.h == 1) z_role<1, 8>(a, S, (int)part, smem);
@@ -422,6 +510,16 @@ PredictSmem predict_shape(const lif_layer_desc& D, PredictArgs& a) {
   a.cw = 8;
   while (a.h == 1 && a.cw > 2 && a.red_at + (runs + a.parts) * a.cw * 4 > kZSmem) a.cw /= 2;
   m.z = a.red_at + (runs + a.parts) * a.h * a.cw * 4;
+  // By parts: few columns (two z CTAs at rank 16 took 11 us longer than 32 at 6128 rows), as long as the parts'
+  // sums that every score CTA reads are few; one stream of many rows.
+  const size_t z_part = (size_t)a.per * kThreads * 16 + S * a.rows * 2 + (size_t)a.lanes * r * 4;
+  a.by_parts = ((r < 64 && S * r <= 256) || (S == 1 && m.z > kSharedSmem)) && z_part <= kSharedSmem;
+  if (a.by_parts) {
+    a.n_z = a.parts;
+    a.x_at = a.per * kThreads * 16;
+    a.red_at = a.x_at + S * a.rows * 2;
+    m.z = z_part;
+  }
   m.scores = (size_t)padded(S) * r * 4 + (size_t)a.staged_b * kThreads * 16 + (size_t)S * 16 * kLogitTile * 4;
   return m;
 }
@@ -457,6 +555,12 @@ cudaError_t launch_stage(const lif_layer* L, PredictArgs a, const PredictSmem& s
 }
 
 }  // namespace
+
+bool z_by_parts(const lif_layer_desc& D) {
+  PredictArgs a = {};
+  if (D.gate_mode != LIF_GATE_RESIDENT) predict_shape(D, a);
+  return a.by_parts != 0;
+}
 
 // Opt-ins of the kernel (once per layer).
 cudaError_t predict_configure(const lif_layer* L) {

@@ -254,8 +254,11 @@ __host__ __device__ __forceinline__ size_t x_smem_bytes(int d, int S) {
 // every neuron (64 KB at 16384) and the stamp of every row by its neuron held back the predictor's CTA on
 // the same SM, and with it the last entry, by 1.5 us (2.2 at 4544 columns).  So the step keeps a copy of the
 // stamps by row, which a window update by another kernel makes out of date (CNT_ROW_STAMPS).
+// (Up to 4096 neurons slot_of is two loads per thread, and a round trip less between the entries and the plan:
+// with the FFN over every cached row, which waits for the plan, 656 x 2664, 2 layers, 37.2 us without it.)
+constexpr int kSlotsAhead = 4096;
 size_t window_role_smem(int F, int cap) {
-  return 4 * (size_t)F + 10 * (size_t)cap + 4 * (size_t)((F + 31) / 32) + 64;
+  return (F <= kSlotsAhead ? 6 : 4) * (size_t)F + 10 * (size_t)cap + 4 * (size_t)((F + 31) / 32) + 64;
 }
 
 __device__ void window_role(const StepArgs& a, unsigned char* smem) {
@@ -271,11 +274,18 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
   unsigned short* hole_s = pid_s + w.cap;                             // [cap] freed rows, ascending
   unsigned short* moved_s = hole_s + w.cap;                           // [cap] row - bound -> new row
   uint32_t* bits = reinterpret_cast<uint32_t*>(moved_s + (w.cap + (w.cap & 1)));   // [F / 32]
+  unsigned short* of_s = reinterpret_cast<unsigned short*>(bits + (F + 31) / 32);  // [F] slot_of, up to kSlotsAhead
 
   const int n = w.counts[LIF_CNT_NUM_USED];
   const int t = w.counts[LIF_CNT_STEP];
   const int stale_input = w.counts[LIF_CNT_STATUS] == LIF_ERR_TIMEOUT;   // see window.cu
   const int t_end = t + w.keep - 1;
+  if (F <= kSlotsAhead)
+    for (int i = tid; i < F / 4; i += kStepThreads) {
+      const int4 v = reinterpret_cast<const int4*>(w.slot_of)[i];        // (-1 becomes kNoSlot by itself)
+      reinterpret_cast<uint32_t*>(of_s)[2 * i] = (uint32_t)(v.x & 0xffff) | ((uint32_t)v.y << 16);
+      reinterpret_cast<uint32_t*>(of_s)[2 * i + 1] = (uint32_t)(v.z & 0xffff) | ((uint32_t)v.w << 16);
+    }
   const bool stamps = w.counts[CNT_ROW_STAMPS] == t;
 #pragma unroll 2
   for (int s = tid; s < n; s += kStepThreads) {
@@ -306,7 +316,8 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
   }
   __syncthreads();
 #pragma unroll 2
-  for (int q = tid; q < na; q += kStepThreads) slot_s[q] = (unsigned short)w.slot_of[act_s[q]];   // (-1: kNoSlot)
+  for (int q = tid; q < na; q += kStepThreads)
+    slot_s[q] = F <= kSlotsAhead ? of_s[act_s[q]] : (unsigned short)w.slot_of[act_s[q]];
   __syncthreads();
   // each thread owns a run of consecutive rows and of consecutive active neurons
   const int seg = (n + kStepThreads - 1) / kStepThreads;

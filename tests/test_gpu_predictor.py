@@ -46,10 +46,13 @@ def _scores_in_order(x, A, Bm, c):
 
 @pytest.mark.parametrize("S,d,F,r", [
     (1, 8, 8, 8),            # one run with a row
-    (1, 8192, 136, 8),       # most runs: half the columns per CTA
+    (1, 8192, 136, 8),       # by parts: one column group, most lanes
+    (1, 6128, 136, 136),     # ... a column group that is too long
+    (5, 2568, 136, 48),      # ... several streams; a last part of 40 rows
+    (8, 4104, 136, 40),      # by columns at a small rank: many runs, few columns at a time
     (1, 4104, 264, 120),     # a last part of 8 rows
     (1, 1000, 520, 248),     # runs of different lengths, rank not a multiple of 16
-    (1, 8192, 128, 1024),    # few long runs: more rows than a thread holds and stages
+    (1, 8192, 128, 1024),    # few long runs
     (2, 264, 136, 136),
     (3, 1544, 392, 72),
     (5, 4096, 136, 128),
