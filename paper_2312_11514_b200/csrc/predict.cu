@@ -476,6 +476,7 @@ PredictKernel predict_kernel_for(int S) {
 
 constexpr int kMaxStaged = 12;         // pieces of B per thread in shared memory: 48 KB
 constexpr size_t kSharedSmem = 100 * 1024;   // ... with which two predictor CTAs still fit an SM
+constexpr size_t kFewColumns = 40 * 1024;   // see predict_shape
 constexpr int kColumnCtas = 128;       // z CTAs at most, as long as a CTA can take more streams
 constexpr size_t kZSmem = 200 * 1024;  // bytes of shared memory that a z CTA takes with more than 2 columns at a time
 
@@ -510,10 +511,11 @@ PredictSmem predict_shape(const lif_layer_desc& D, PredictArgs& a) {
   a.cw = 8;
   while (a.h == 1 && a.cw > 2 && a.red_at + (runs + a.parts) * a.cw * 4 > kZSmem) a.cw /= 2;
   m.z = a.red_at + (runs + a.parts) * a.h * a.cw * 4;
-  // By parts: few columns (two z CTAs at rank 16 took 11 us longer than 32 at 6128 rows), as long as the parts'
-  // sums that every score CTA reads are few; one stream of many rows.
+  // By parts: few columns of many rows (two z CTAs at rank 16 took 11 us longer than 32 at 6128 rows; at 256
+  // rows they are 0.8 us faster), as long as the parts' sums that every score CTA reads are few; one stream of
+  // many rows.
   const size_t z_part = (size_t)a.per * kThreads * 16 + S * a.rows * 2 + (size_t)a.lanes * r * 4;
-  a.by_parts = ((r < 64 && S * r <= 256) || (S == 1 && m.z > kSharedSmem)) && z_part <= kSharedSmem;
+  a.by_parts = ((r < 64 && S * r <= 256 && m.z > kFewColumns) || (S == 1 && m.z > kSharedSmem)) && z_part <= kSharedSmem;
   if (a.by_parts) {
     a.n_z = a.parts;
     a.x_at = a.per * kThreads * 16;

@@ -254,11 +254,11 @@ __host__ __device__ __forceinline__ size_t x_smem_bytes(int d, int S) {
 // every neuron (64 KB at 16384) and the stamp of every row by its neuron held back the predictor's CTA on
 // the same SM, and with it the last entry, by 1.5 us (2.2 at 4544 columns).  So the step keeps a copy of the
 // stamps by row, which a window update by another kernel makes out of date (CNT_ROW_STAMPS).
-// (Up to 4096 neurons slot_of is two loads per thread, and a round trip less between the entries and the plan:
-// with the FFN over every cached row, which waits for the plan, 656 x 2664, 2 layers, 37.2 us without it.)
-constexpr int kSlotsAhead = 4096;
-size_t window_role_smem(int F, int cap) {
-  return (F <= kSlotsAhead ? 6 : 4) * (size_t)F + 10 * (size_t)cap + 4 * (size_t)((F + 31) / 32) + 64;
+// (Up to 4096 neurons slot_of is two loads per thread, and a round trip less between the entries and the plan;
+// up to 8192 with the FFN over every cached row, which waits for the plan: 656 x 2664, 2 layers, 37.2 us without it.)
+__host__ __device__ __forceinline__ bool slots_ahead(int F, int whole_cache) { return F <= (whole_cache ? 8192 : 4096); }
+size_t window_role_smem(int F, int cap, int whole_cache) {
+  return (slots_ahead(F, whole_cache) ? 6 : 4) * (size_t)F + 10 * (size_t)cap + 4 * (size_t)((F + 31) / 32) + 64;
 }
 
 __device__ void window_role(const StepArgs& a, unsigned char* smem) {
@@ -274,13 +274,14 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
   unsigned short* hole_s = pid_s + w.cap;                             // [cap] freed rows, ascending
   unsigned short* moved_s = hole_s + w.cap;                           // [cap] row - bound -> new row
   uint32_t* bits = reinterpret_cast<uint32_t*>(moved_s + (w.cap + (w.cap & 1)));   // [F / 32]
-  unsigned short* of_s = reinterpret_cast<unsigned short*>(bits + (F + 31) / 32);  // [F] slot_of, up to kSlotsAhead
+  unsigned short* of_s = reinterpret_cast<unsigned short*>(bits + (F + 31) / 32);  // [F] slot_of (slots_ahead)
 
   const int n = w.counts[LIF_CNT_NUM_USED];
   const int t = w.counts[LIF_CNT_STEP];
   const int stale_input = w.counts[LIF_CNT_STATUS] == LIF_ERR_TIMEOUT;   // see window.cu
   const int t_end = t + w.keep - 1;
-  if (F <= kSlotsAhead)
+  const bool ahead = slots_ahead(F, a.whole_cache);
+  if (ahead)
     for (int i = tid; i < F / 4; i += kStepThreads) {
       const int4 v = reinterpret_cast<const int4*>(w.slot_of)[i];        // (-1 becomes kNoSlot by itself)
       reinterpret_cast<uint32_t*>(of_s)[2 * i] = (uint32_t)(v.x & 0xffff) | ((uint32_t)v.y << 16);
@@ -317,7 +318,7 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
   __syncthreads();
 #pragma unroll 2
   for (int q = tid; q < na; q += kStepThreads)
-    slot_s[q] = F <= kSlotsAhead ? of_s[act_s[q]] : (unsigned short)w.slot_of[act_s[q]];
+    slot_s[q] = ahead ? of_s[act_s[q]] : (unsigned short)w.slot_of[act_s[q]];
   __syncthreads();
   // each thread owns a run of consecutive rows and of consecutive active neurons
   const int seg = (n + kStepThreads - 1) / kStepThreads;
@@ -638,6 +639,7 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
   int n, n_moves = 0;
   if (a.whole_cache) {
     pdl_wait();                                            // (gate values of every row)
+    load_x(a, xs);
     const unsigned long long plan = wait_plan(a, &plan_s);
     n = plan_rows(plan);
     n_moves = plan_moves(plan);
@@ -703,7 +705,7 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
       b_s[tid] = kGate == LIF_GATE_RESIDENT && a.whole_cache ? a.gate_val[id]
                                                              : row_scalar<kGate>(a, id, run, checked);
     }
-    if (r0 == 0) load_x(a, xs);                            // while the first rows travel
+    if (r0 == 0 && !a.whole_cache) load_x(a, xs);          // while the first rows travel
     if (r0 == 0 && !a.w.append_first) {                    // ... and the moves
       if (!a.whole_cache) n_moves = plan_moves(wait_plan(a, &plan_s));
       move_rows();
@@ -1312,7 +1314,7 @@ cudaError_t step_configure(lif_layer* L) {
   L->step_cache_stages = stages(D.gate_mode == LIF_GATE_RESIDENT ? kCacheRingGate : kCacheRing, x + hits, 1);
   // (paper's cache order: bundles wait in the ring, see fetch_role; twice the ring keeps the link busy)
   L->step_fetch_stages = stages(D.append_first ? kFetchRing : 2 * kFetchRing, x + ids, 2);
-  size_t smem = window_role_smem(D.d_ff, D.capacity);
+  size_t smem = window_role_smem(D.d_ff, D.capacity, D.ffn_mode == 1);
   const size_t need_c = x + L->step_cache_stages * row + hits, need_f = x + L->step_fetch_stages * row + ids;
   if (need_c > smem) smem = need_c;
   if (need_f > smem) smem = need_f;
