@@ -383,6 +383,7 @@ def measure(args, config_name, steps, warmup, rank, world, local, detail):
             pred_bytes = 2 * cfg.rank * (d + cfg.d_ff) + 4 * cfg.d_ff
             pred_us = kernel_us["predict"] if S > 1 else kernel_us["predict_z"] + kernel_us["predict_scores"]
         pred_gbs = pred_bytes / (pred_us * 1e-6) / 1e9
+        # (one stream: the two stages of the one predictor launch, each replayed alone)
         predictor = {"bound": "hbm", "achieved": pred_gbs, "unit": "GB/s", "frac": pred_gbs / peak,
                      "bytes_per_launch": pred_bytes, "us_per_launch": pred_us}
         link = {"bound": "host_link", "peak": link_peak, "unit": "GB/s",
@@ -454,10 +455,10 @@ def measure(args, config_name, steps, warmup, rank, world, local, detail):
             "e2e": {"value": whole_job_tokens_per_s(K, 1 if sharded else world, ms_e2e), "unit": UNIT,
                     "h2d_bytes_per_step": S * d * 2, "d2h_bytes_per_step": L * S * d * 4,
                     "host_link_bytes_per_step": fetched / K},
-            # per layer-step: z, scores (or the gate kernel alone), then one stream: the step kernel;
-            # several: window, moves, fetch, up + down for cached and for new rows, sum
-            "gpu_launches": ((3 if S == 1 else 10) - (1 if gate_mode == B.GATE_RESIDENT else 0)
-                             + (2 if gate_mode == B.GATE_BUNDLED and S > 1 else 0)) * n_launch,
+            # per layer-step, one stream: the predictor (or the gate kernel) and the step kernel; several: the
+            # predictor as two launches (or the gate kernel), window, moves, fetch, up + down for cached and for new rows, sum
+            "gpu_launches": (2 if S == 1 else 10 - (1 if gate_mode == B.GATE_RESIDENT else 0)
+                             + (2 if gate_mode == B.GATE_BUNDLED else 0)) * n_launch,
             "roofline": roofline,
             "host_link": host_link,
             "separate_kernels": separate,
