@@ -57,9 +57,10 @@ struct PredictArgs {
 // other.  Its pieces of A (one row, 8 columns) travel into its own slots of shared memory ahead of the
 // dependency wait.
 //
-// In a decode step (but for a token's first layer, whose input is there at once) everything behind the wait is executed once before it, on whatever the buffers hold, and
-// the results dropped: a kernel's code comes from L2 at its first use, which behind the wait takes as long as
-// the work itself (512 x 2048, from the wait to the entries: 4.2 us, 2.3 with the first pass).
+// In a decode step (but for a token's first layer, whose input is there at once) everything behind the wait is
+// executed once before it, on whatever the buffers hold, and the results dropped: a kernel's code comes from L2
+// at its first use, which behind the wait takes as long as the work itself (512 x 2048, from the wait to the
+// entries: 4.2 us, 2.3 with the first pass).
 template <int H, int CW>
 __device__ void z_role(const PredictArgs& a, int S, int part_of_grid, unsigned char* smem) {
   constexpr int Q = H * CW;
@@ -293,141 +294,141 @@ __device__ void score_role(const PredictArgs& a, int tile, unsigned char* smem) 
   int run = 0;
 #pragma unroll 1
   for (int pass = S > 1; pass < 2; ++pass) {                           // (see stage 1; z takes longer than this)
-  if (pass) {
-    pdl_wait();
-    // What follows (the window kernel or the single-launch step) reads ahead of its own wait only what was
-    // complete before this one passed, and words that carry this run's number.  (A compacting run is
-    // followed by a kernel that can do nothing before its list: it is released when z is there.)
-    if (!a.compact) pdl_trigger();
-  }
-  if (S == 1 && pass && r > 128) first_rows();                    // (the first pass ended with later ones)
-  run = __ldcg(a.predictor_run);
-  // Whether the neuron already has a cache row is read here, so the mask of neurons to bring in
-  // (active and not cached) costs no round trip of its own.
-  const int my_row = my_col < F ? __ldcg(a.slot_of + my_col) : 0;
-  {
-    unsigned polls = 0;
-    for (int i = tid; a.by_parts && i < S * r; i += kThreads) {          // the parts' sums, in order
-      float sum = 0.f;
-      bool all = true;
-      for (int p0 = 0; p0 < a.parts; p0 += 8) {
-        unsigned long long v[8];
+    if (pass) {
+      pdl_wait();
+      // What follows (the window kernel or the single-launch step) reads ahead of its own wait only what was
+      // complete before this one passed, and words that carry this run's number.  (A compacting run is
+      // followed by a kernel that can do nothing before its list: it is released when z is there.)
+      if (!a.compact) pdl_trigger();
+    }
+    if (S == 1 && pass && r > 128) first_rows();                    // (the first pass ended with later ones)
+    run = __ldcg(a.predictor_run);
+    // Whether the neuron already has a cache row is read here, so the mask of neurons to bring in
+    // (active and not cached) costs no round trip of its own.
+    const int my_row = my_col < F ? __ldcg(a.slot_of + my_col) : 0;
+    {
+      unsigned polls = 0;
+      for (int i = tid; a.by_parts && i < S * r; i += kThreads) {          // the parts' sums, in order
+        float sum = 0.f;
+        bool all = true;
+        for (int p0 = 0; p0 < a.parts; p0 += 8) {
+          unsigned long long v[8];
+          bool there;
+          do {
+            there = true;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v[k])
+                           : "l"(a.z + (size_t)min(p0 + k, a.parts - 1) * S * r + i) : "memory");
+              there = there && (!a.tickets || (int)(v[k] >> 32) == a.launch);
+            }
+          } while (pass && !there && polls++ < a.spin_limit);
+          all = all && there;
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (p0 + k < a.parts) sum += __uint_as_float((unsigned)v[k]);
+        }
+        if (pass && !all) flag_timeout(a.status);
+        zs[S == 1 ? i : (i % r) * SP + i / r] = all ? sum : __int_as_float(0x7fffffff);
+      }
+      for (int j = tid; !a.by_parts && j < r; j += kThreads) {
+        unsigned long long v[S];
         bool there;
         do {
           there = true;
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v[k])
-                         : "l"(a.z + (size_t)min(p0 + k, a.parts - 1) * S * r + i) : "memory");
+          for (int k = 0; k < S; ++k) {
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v[k]) : "l"(a.z + (size_t)k * r + j) : "memory");
             there = there && (!a.tickets || (int)(v[k] >> 32) == a.launch);
           }
         } while (pass && !there && polls++ < a.spin_limit);
-        all = all && there;
+        if (pass && !there) flag_timeout(a.status);
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-          if (p0 + k < a.parts) sum += __uint_as_float((unsigned)v[k]);
+        for (int k = 0; k < S; ++k)                                      // not there: no neuron is active
+          zs[j * SP + k] = there ? __uint_as_float((unsigned)v[k]) : __int_as_float(0x7fffffff);
       }
-      if (pass && !all) flag_timeout(a.status);
-      zs[S == 1 ? i : (i % r) * SP + i / r] = all ? sum : __int_as_float(0x7fffffff);
     }
-    for (int j = tid; !a.by_parts && j < r; j += kThreads) {
-      unsigned long long v[S];
-      bool there;
-      do {
-        there = true;
-#pragma unroll
-        for (int k = 0; k < S; ++k) {
-          asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v[k]) : "l"(a.z + (size_t)k * r + j) : "memory");
-          there = there && (!a.tickets || (int)(v[k] >> 32) == a.launch);
-        }
-      } while (pass && !there && polls++ < a.spin_limit);
-      if (pass && !there) flag_timeout(a.status);
-#pragma unroll
-      for (int k = 0; k < S; ++k)                                      // not there: no neuron is active
-        zs[j * SP + k] = there ? __uint_as_float((unsigned)v[k]) : __int_as_float(0x7fffffff);
-    }
-  }
-  if (pass && a.compact) pdl_trigger();
-  if (pass) own_copies_wait();
-  __syncthreads();
+    if (pass && a.compact) pdl_trigger();
+    if (pass) own_copies_wait();
+    __syncthreads();
 
-  float2 acc[S][4];
+    float2 acc[S][4];
 #pragma unroll
-  for (int s = 0; s < S; ++s)
+    for (int s = 0; s < S; ++s)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) acc[s][e] = make_float2(0.f, 0.f);
+      for (int e = 0; e < 4; ++e) acc[s][e] = make_float2(0.f, 0.f);
 #pragma unroll 1
-  for (int j0 = 0; j0 < r; j0 += 128) {
-    if (j0 > 0) {
+    for (int j0 = 0; j0 < r; j0 += 128) {
+      if (j0 > 0) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int j = j0 + rs + 16 * u, at = (j0 >> 4) - 8 + u;
+          bq[u] = make_uint4(0, 0, 0, 0);
+          if (col < F && j < r)
+            bq[u] = at < a.staged_b ? b_s[at * kThreads + tid] : ld_stream16(a.B + (size_t)j * F + col);
+        }
+      }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        const int j = j0 + rs + 16 * u, at = (j0 >> 4) - 8 + u;
-        bq[u] = make_uint4(0, 0, 0, 0);
-        if (col < F && j < r)
-          bq[u] = at < a.staged_b ? b_s[at * kThreads + tid] : ld_stream16(a.B + (size_t)j * F + col);
-      }
-    }
+        const int j = j0 + rs + 16 * u;
+        if (j < r) {
+          float2 bf[4];
+          unpack8(bq[u], bf);
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int j = j0 + rs + 16 * u;
-      if (j < r) {
-        float2 bf[4];
-        unpack8(bq[u], bf);
+          for (int s = 0; s < S; ++s) {
+            const float zz = zs[j * SP + s];
 #pragma unroll
-        for (int s = 0; s < S; ++s) {
-          const float zz = zs[j * SP + s];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) acc[s][e] = fma2(make_float2(zz, zz), bf[e], acc[s][e]);
+            for (int e = 0; e < 4; ++e) acc[s][e] = fma2(make_float2(zz, zz), bf[e], acc[s][e]);
+          }
         }
       }
     }
-  }
-#pragma unroll
-  for (int s = 0; s < S; ++s) {
-    float4* dst = reinterpret_cast<float4*>(red + (s * 16 + rs) * kLogitTile + cg * 8);
-    dst[0] = make_float4(acc[s][0].x, acc[s][0].y, acc[s][1].x, acc[s][1].y);
-    dst[1] = make_float4(acc[s][2].x, acc[s][2].y, acc[s][3].x, acc[s][3].y);
-  }
-  __syncthreads();
-  // two streams at a time: a warp holds 32 neighbouring neurons of one stream
-  unsigned active_w = 0;                                               // one stream: of the thread's warp
-#pragma unroll
-  for (int s0 = 0; s0 < S; s0 += 2) {
-    const int s = s0 + (tid >> 7);
-    if (s < S) {
-      float v = 0.f;
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v += red[(s * 16 + k) * kLogitTile + n];
-      v += my_c;
-      if (pass && a.logits && my_col < F) a.logits[(size_t)s * F + my_col] = v;
-      active_w = __ballot_sync(0xffffffffu, my_col < F && v > a.theta);
-      if (S > 1 && (tid & 31) == 0) act_w[s][n >> 5] = active_w;
-    }
-  }
-  if (S > 1) __syncthreads();
-  if (tid < kLogitTile) {
-    unsigned m = 0;
-    int last_kept = -1;        // speculative mode: last token < keep in which the neuron is active
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      const unsigned w = S == 1 ? active_w : act_w[s][tid >> 5];
-      m |= w;
-      if (s < a.keep && ((w >> (tid & 31)) & 1u)) last_kept = s;
+      float4* dst = reinterpret_cast<float4*>(red + (s * 16 + rs) * kLogitTile + cg * 8);
+      dst[0] = make_float4(acc[s][0].x, acc[s][0].y, acc[s][1].x, acc[s][1].y);
+      dst[1] = make_float4(acc[s][2].x, acc[s][2].y, acc[s][3].x, acc[s][3].y);
     }
-    if (pass && a.keep_tok && my_col < F) a.keep_tok[my_col] = (int8_t)last_kept;
-    const bool active = (m >> (tid & 31)) & 1u;
-    const unsigned mn = __ballot_sync(0xffffffffu, active && my_row < 0);
-    if (pass && (tid & 31) == 0) {
-      const int word = tile * (kLogitTile / 32) + (tid >> 5);
-      a.mask_words[word] = m;
-      // the neurons to bring in together with this run's number, in one store: a kernel that is already
-      // resident re-reads the entry until the number is the run's
-      store_with_run(a.entries + word, mn, run);
-      if (!a.compact) store_with_run(a.entries + n_entries + word, m, run);   // and the active ones themselves
+    __syncthreads();
+    // two streams at a time: a warp holds 32 neighbouring neurons of one stream
+    unsigned active_w = 0;                                               // one stream: of the thread's warp
+#pragma unroll
+    for (int s0 = 0; s0 < S; s0 += 2) {
+      const int s = s0 + (tid >> 7);
+      if (s < S) {
+        float v = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v += red[(s * 16 + k) * kLogitTile + n];
+        v += my_c;
+        if (pass && a.logits && my_col < F) a.logits[(size_t)s * F + my_col] = v;
+        active_w = __ballot_sync(0xffffffffu, my_col < F && v > a.theta);
+        if (S > 1 && (tid & 31) == 0) act_w[s][n >> 5] = active_w;
+      }
     }
-    if (pass && !a.compact && active && my_row >= 0)                           // ... with the row of each that has one
-      store_with_run(a.entries + 2 * n_entries + my_col, (uint32_t)my_row, run);
-  }
+    if (S > 1) __syncthreads();
+    if (tid < kLogitTile) {
+      unsigned m = 0;
+      int last_kept = -1;        // speculative mode: last token < keep in which the neuron is active
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        const unsigned w = S == 1 ? active_w : act_w[s][tid >> 5];
+        m |= w;
+        if (s < a.keep && ((w >> (tid & 31)) & 1u)) last_kept = s;
+      }
+      if (pass && a.keep_tok && my_col < F) a.keep_tok[my_col] = (int8_t)last_kept;
+      const bool active = (m >> (tid & 31)) & 1u;
+      const unsigned mn = __ballot_sync(0xffffffffu, active && my_row < 0);
+      if (pass && (tid & 31) == 0) {
+        const int word = tile * (kLogitTile / 32) + (tid >> 5);
+        a.mask_words[word] = m;
+        // the neurons to bring in together with this run's number, in one store: a kernel that is already
+        // resident re-reads the entry until the number is the run's
+        store_with_run(a.entries + word, mn, run);
+        if (!a.compact) store_with_run(a.entries + n_entries + word, m, run);   // and the active ones themselves
+      }
+      if (pass && !a.compact && active && my_row >= 0)                           // ... with the row of each that has one
+        store_with_run(a.entries + 2 * n_entries + my_col, (uint32_t)my_row, run);
+    }
   }
   if (!a.compact) return;     // the consumer reads the bit mask itself
   compact_mask_last_cta(a.mask_words, n_entries, a.n_scores, a.done, a.active_idx, a.n_active, warp_sums, &is_last);

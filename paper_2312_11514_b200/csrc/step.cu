@@ -96,6 +96,7 @@ struct StepArgs {
   StepSync* sync;
   int d, n_streams, whole_cache, act;
   float act_thr;
+  int hand_over;                  // several streams: see kHandOver
   int n_cache_ctas, n_sum_ctas, group_size, cache_stages, fetch_stages, fetch_rows_max, hits_max;
   unsigned wait_polls;            // of the first wait for a bulk copy
   unsigned spin_limit;            // of a wait for another CTA
@@ -913,7 +914,7 @@ struct Summer {
       add(have, col, a.spin_limit);
       if (kS > 1) {
         if (lost) timed_out(a);
-        add_last(n_last, col);
+        if (a.hand_over) add_last(n_last, col);
       }
       if (lost) timed_out(a);
       red[tid] = v_sum;
@@ -958,7 +959,7 @@ __device__ void sum_role(const StepArgs& a, int index, unsigned char* smem) {
   const int n_load = plan_loads(plan);                     // (0: refused)
   const int n_last = min(kFetchCtas, n_load);              // fetch CTAs with rows; with several of them
   Summer<kS> sum(a, index, a.n_sum_ctas, plan_rows(plan),
-                 kS == 1 ? n_last : max(0, min(kFetchCtas, n_load - kFetchCtas)));
+                 kS == 1 || !a.hand_over ? n_last : max(0, min(kFetchCtas, n_load - kFetchCtas)));
   const size_t pairs = (size_t)a.n_streams * (a.d >> 1);
   const int n_new = sum.have - sum.have_hit;
   if (kS == 1) {
@@ -1075,7 +1076,7 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   unsigned long long* last_h = a.last_h + f * 8;
   for (int i = 0, st = 0; i < from; ++i) {
     const uint4* row = reinterpret_cast<const uint4*>(ring + (size_t)st * row_bytes);
-    const bool is_last = kS > 1 && i == cnt - 1;
+    const bool is_last = kS > 1 && a.hand_over && i == cnt - 1;
     if (is_last) {                                         // the partial sum, while the last row travels
       if (i > 0) store_tagged_partial<kS>(acc, a.p_new + (size_t)f * S * (d >> 1), nvec, S, a.epoch + 1);
       given = 1;
@@ -1185,9 +1186,10 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
       parity ^= 1u;
     }
   }
-  if (kS == 1 ? cnt > 0 : cnt > 1 && given == 0)
+  const bool hand_over = kS > 1 && a.hand_over;
+  if (!hand_over ? cnt > 0 : cnt > 1 && given == 0)
     store_tagged_partial<kS>(acc, a.p_new + (size_t)f * S * (d >> 1), nvec, S, a.epoch + 1);
-  if (kS > 1 && cnt > 0 && given < 2) {                    // given up: nothing comes of the last row
+  if (hand_over && cnt > 0 && given < 2) {                    // given up: nothing comes of the last row
     for (int v = tid; v < d >> 1; v += kStepThreads) store_tagged_word(last_down + v, 0u, a.epoch + 1);
     if (tid < 8) store_tagged_word(last_h + tid, 0u, a.epoch + 1);
   }
@@ -1250,6 +1252,10 @@ constexpr int kGroupMax = 8, kUngroupedMax = 64, kUngroupedMaxStreams = 16;
 // One step CTA per SM (with less, two fit and are put on one SM where others are not free yet), and beside it one of
 // the next layer's low-rank predictor, 91 KB at 4096 x 128.
 constexpr size_t kCacheRing = 112 * 1024, kCacheRingGate = 128 * 1024, kFetchRing = 32 * 1024;
+
+// Streams x columns from which a fetch CTA hands its last row over instead of adding it to its partial: 5 x 4096 260 ->
+// 250 us (2 layers), 3 x 1544 180 -> 183 (4 layers), where a partial is 37 KB and the further words cost more.
+constexpr int kHandOver = 8192;
 
 // CTAs that add up the outputs: 16 pairs of columns or more each, which leaves 16 slices of the partials to
 // a CTA's threads (several streams: 128 pairs).
@@ -1349,6 +1355,7 @@ cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st
   a.p_member = L->y_partial;
   a.p_hit = (uint4*)L->step_tagged;
   a.p_new = a.p_hit + (size_t)hit_partials_max(D) * D.n_streams * (D.d_model / 2);
+  a.hand_over = D.n_streams > 1 && D.n_streams * D.d_model >= kHandOver;
   a.last_down = (unsigned long long*)(a.p_new + (size_t)kFetchCtas * D.n_streams * (D.d_model / 2));
   a.last_h = a.last_down + (size_t)kFetchCtas * (D.d_model / 2);
   a.y = y;
