@@ -896,8 +896,10 @@ struct Summer {
         if (t0 + k * slices < n_last) {
           const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&pair[k]));
           const float w = __uint_as_float((uint32_t)v[k]);
-          v_sum.x = fmaf(w, f.x, v_sum.x);
-          v_sum.y = fmaf(w, f.y, v_sum.y);
+          if (w != 0.f) {                                  // (as everywhere: a row of weight 0 is not read)
+            v_sum.x = fmaf(w, f.x, v_sum.x);
+            v_sum.y = fmaf(w, f.y, v_sum.y);
+          }
         }
     }
   }

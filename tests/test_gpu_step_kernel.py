@@ -135,3 +135,35 @@ def test_other_tokens_after_a_restore_do_not_meet_words_of_runs_of_the_same_numb
     ora.cache = cache
     run(range(6, 9))
     gpu.close()
+
+
+@pytest.mark.parametrize("S,d,fire", [
+    (2, 4096, 0.003),     # every new neuron is its fetch CTA's only one: its row is handed over
+    (2, 4096, 0.04),      # several rows a CTA, the last one handed over
+    (4, 2048, 0.01),
+    (3, 1032, 0.01),      # not handed over
+])
+def test_a_down_column_is_not_read_by_a_stream_in_which_its_neuron_is_off(S, d, fire):
+    # infinities in the down columns of neurons that are off in stream 0: its output stays, bit for bit,
+    # wherever in the load list the neuron is
+    cfg = W.LifConfig("off", 1, d, 2048, 32, 3, S, 2, fire, 1.0, 0.8, 0.6, 78)
+    gpu, ora = P.make_layer_pair(cfg, 0, b_down=True, capacity=cfg.d_ff, append_first=1)
+    X = W.make_inputs(cfg, device=DEV)
+    y = torch.empty(2, S, d, dtype=torch.float32, device=DEV)
+    gpu.keep["bias_up"].zero_()                    # on in about every second stream
+    ora.bias_up[:] = 0
+    torch.cuda.synchronize()
+    B.lif_decode_step(gpu.handle, X[0], y[0])
+    lists = P.check_decode_step(gpu, ora, X[0].cpu().numpy(), y[0])
+    x = X[0].cpu().numpy().astype(np.float64)
+    pre = x @ ora.bundles[lists["load_ids"], :d].astype(np.float64).T
+    off = lists["load_ids"][(pre[0] < -1e-3) & (pre[1:] > 1e-3).any(axis=0)]
+    assert len(off) > 0
+    gpu.keep["host_bundles"][torch.from_numpy(off.astype(np.int64)), d:] = float("inf")
+    B.lif_reset(gpu.handle)
+    torch.cuda.synchronize()
+    B.lif_decode_step(gpu.handle, X[0], y[1])
+    torch.cuda.synchronize()
+    assert torch.equal(y[0, 0], y[1, 0])
+    assert torch.isinf(y[1, 1:]).any()
+    gpu.close()
