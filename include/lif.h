@@ -396,7 +396,8 @@ lif_status lif_read_state(lif_layer* layer, int32_t* host_pointers, int32_t* hos
  * valid for a layer of the same description.  lif_restore checks the buffer on the host
  * before anything reaches the device (counters in range, pointers and slot_of inverse maps of
  * each other over exactly num_used rows, free rows marked -1, stamps older than the step);
- * LIF_ERR_STATE: it does not describe a state of this layer, and the layer is left as it was. */
+ * LIF_ERR_STATE: it does not describe a state of this layer, and the layer is left as it was.  What
+ * the library counts for its own launches beside the public counters is not taken from the buffer. */
 lif_status lif_snapshot_bytes(lif_layer* layer, size_t* out_bytes);
 lif_status lif_snapshot(lif_layer* layer, void* host_buf, size_t bytes);
 lif_status lif_restore(lif_layer* layer, const void* host_buf, size_t bytes);

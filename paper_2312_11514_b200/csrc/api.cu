@@ -1,6 +1,8 @@
 // C ABI of liblif.so: argument checking, workspace carve-up and stream/event orchestration.
 // Every step of the path runs in the kernels of predict.cu / gate.cu / step.cu, or of window.cu /
 // fetch.cu / ffn*.cu where the calls are made one by one or the single launch does not apply.
+#include <string.h>
+
 #include <new>
 
 #include "lif_internal.cuh"
@@ -710,20 +712,26 @@ lif_status lif_restore(lif_layer* L, const void* host_buf, size_t bytes) {
     if (cached != n) return LIF_ERR_STATE;
   }
   if (cudaDeviceSynchronize() != cudaSuccess) return LIF_ERR_CUDA;
+  // The counters of launches in the counts block are not state: taken from a damaged buffer, or one of a layer with
+  // another rank, every later predictor would wait for words of a launch that never comes.  They begin anew,
+  // as after a reset; the words that carry their numbers are cleared below, and the stamps by row are those of
+  // another state.
+  int32_t counts[LIF_CNT_LEN];
+  memcpy(counts, host_buf, sizeof(counts));
+  for (int i = CNT_PRIVATE; i < CNT_TOTALS; ++i) counts[i] = 0;
+  counts[CNT_PREDICTOR_RUN] = 1;
+  counts[CNT_ROW_STAMPS] = -1;
   StatePart p[5];
   const unsigned char* in = (const unsigned char*)host_buf;
   for (int i = 0, n = state_parts(L, p); i < n; ++i) {
-    if (cudaMemcpy(p[i].dev, in, p[i].bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (cudaMemcpy(p[i].dev, i == 0 ? (const void*)counts : in, p[i].bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
       cudaGetLastError();
       return LIF_ERR_CUDA;
     }
     in += p[i].bytes;
   }
-  // entries of predictor runs after the snapshot must not be taken for those of the next run; the stamps by
-  // row are those of another state
-  const int32_t no_step = -1;
-  if (cudaMemcpy(L->counts + CNT_ROW_STAMPS, &no_step, 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemset(L->new_mask_words, 0, tagged_words(L->desc) * 8) != cudaSuccess ||
+  // words of predictor runs before this must not be taken for those of the next run
+  if (cudaMemset(L->new_mask_words, 0, tagged_words(L->desc) * 8) != cudaSuccess ||
       launch_refill(L, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
     cudaGetLastError();
     return LIF_ERR_CUDA;

@@ -10,8 +10,10 @@
 
 namespace lif {
 
-// Private entries of the counts block (public ones: LIF_CNT_* in lif.h).
+// Private entries of the counts block (public ones: LIF_CNT_* in lif.h).  Those up to CNT_TOTALS number and count
+// launches; lif_restore does not take them from a snapshot.
 enum {
+  CNT_PRIVATE = 16,
   CNT_TICKET_PREDICT = 16,  // "last block done" counter of the score kernel
   CNT_PREDICTOR_RUN = 17,   // number of the predictor run whose masks are (being) written; advanced
                             // by the kernel that ends a decode step, or by the run that compacts

@@ -2,6 +2,8 @@
 on the GPU in forms that cannot fault: a bad row index is replaced before it is used as an
 address, a damaged snapshot is refused on the host, and a wait is made to run out by giving it
 no polls at all while the copies it guards still land before the kernel returns."""
+import copy
+
 import numpy as np
 import pytest
 import torch
@@ -155,6 +157,32 @@ def test_restore_refuses_a_damaged_snapshot_on_the_host():
     B.lif_restore(gpu.handle, snap)          # the intact one is still accepted
     B.lif_decode_step(gpu.handle, X[4], y)
     P.check_decode_step(gpu, ora, X[4].cpu().numpy(), y)
+    gpu.close()
+
+
+@pytest.mark.parametrize("S", [1, 3])
+def test_restore_takes_no_launch_counters_from_the_buffer(S):
+    # words 16-31 of a snapshot's counts block number and count launches; with others in their place every call
+    # after the restore goes on as the snapshotted layer would
+    cfg, gpu, ora, X, y = _warm_layer(S)
+    snap, cache = B.lif_snapshot(gpu.handle), copy.deepcopy(ora.cache)
+    words = np.frombuffer(snap, dtype=np.int32, count=B.CNT_LEN).copy()
+    idx, n = torch.empty(cfg.d_ff, dtype=torch.int32, device=DEV), torch.zeros(1, dtype=torch.int32, device=DEV)
+    for value in (1, -1, 0):
+        words[16:32] = value
+        B.lif_restore(gpu.handle, words.tobytes() + bytes(snap[words.nbytes:]))
+        ora.cache = copy.deepcopy(cache)
+        for t in range(4, 7):
+            B.lif_predict(gpu.handle, X[t], None, idx, n)
+            B.lif_decode_step(gpu.handle, X[t], y)
+            lists = P.check_decode_step(gpu, ora, X[t].cpu().numpy(), y)
+            np.testing.assert_array_equal(idx[:int(n)].cpu().numpy(), gpu.lists()["active_idx"])
+            P.compare_cache_rows(gpu, ora)
+            assert len(lists["load_ids"]) > 0
+        bad = torch.tensor([-1], dtype=torch.int32, device=DEV)
+        B.lif_sparse_ffn(gpu.handle, X[0], bad, torch.ones(1, dtype=torch.int32, device=DEV), y)
+        B.lif_clear_status(gpu.handle)
+        assert B.lif_get_stats(gpu.handle).status == B.LIF_OK
     gpu.close()
 
 
