@@ -258,8 +258,9 @@ __host__ __device__ __forceinline__ size_t x_smem_bytes(int d, int S) {
 // (Up to 4096 neurons slot_of is two loads per thread, and a round trip less between the entries and the plan;
 // up to 8192 with the FFN over every cached row, which waits for the plan: 656 x 2664, 2 layers, 37.2 us without it.)
 __host__ __device__ __forceinline__ bool slots_ahead(int F, int whole_cache) { return F <= (whole_cache ? 8192 : 4096); }
+// (It decides which layers are one launch: with ages of 16 bits, every capacity up to 18900 neurons.)
 size_t window_role_smem(int F, int cap, int whole_cache) {
-  return (slots_ahead(F, whole_cache) ? 6 : 4) * (size_t)F + 10 * (size_t)cap + 4 * (size_t)((F + 31) / 32) + 64;
+  return (slots_ahead(F, whole_cache) ? 6 : 4) * (size_t)F + 8 * (size_t)cap + 4 * (size_t)((F + 31) / 32) + 64;
 }
 
 __device__ void window_role(const StepArgs& a, unsigned char* smem) {
@@ -270,11 +271,11 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
   const int tid = threadIdx.x, F = w.F;
   unsigned short* slot_s = reinterpret_cast<unsigned short*>(smem);   // [F] row of each of these, or kNoSlot
   unsigned short* act_s = slot_s + F;                                 // [F] active ids, ascending
-  int* stamp_s = reinterpret_cast<int*>(act_s + F);                   // [cap] step in which it was active last
-  unsigned short* pid_s = reinterpret_cast<unsigned short*>(stamp_s + w.cap);   // [cap] row -> neuron
+  unsigned short* age_s = act_s + F;                                  // [cap] steps since it was active, at most 65535
+  unsigned short* pid_s = age_s + w.cap;                              // [cap] row -> neuron
   unsigned short* hole_s = pid_s + w.cap;                             // [cap] freed rows, ascending
   unsigned short* moved_s = hole_s + w.cap;                           // [cap] row - bound -> new row
-  uint32_t* bits = reinterpret_cast<uint32_t*>(moved_s + (w.cap + (w.cap & 1)));   // [F / 32]
+  uint32_t* bits = reinterpret_cast<uint32_t*>(moved_s + w.cap);      // [F / 32]
   unsigned short* of_s = reinterpret_cast<unsigned short*>(bits + (F + 31) / 32);  // [F] slot_of (slots_ahead)
 
   const int n = w.counts[LIF_CNT_NUM_USED];
@@ -294,7 +295,7 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
     const int id = w.pointers[s];
     const int la = stamps ? a.row_stamps[s] : w.last_active[id];
     pid_s[s] = (unsigned short)id;
-    stamp_s[s] = la;
+    age_s[s] = (unsigned short)min(65535, max(1, t_end - la));
   }
   uint32_t act_w[1][kEntriesPerThread];
   read_entries<1>({a.act_entries}, a.n_entries, __ldcg(a.predictor_run), act_w);
@@ -328,8 +329,10 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
   const int q0 = min(na, tid * qseg), q1 = min(na, q0 + qseg);
   auto idle_age = [&](int s) {       // 0: active now
     const int id = pid_s[s];
-    return (bits[id >> 5] >> (id & 31)) & 1u ? 0 : max(1, t_end - stamp_s[s]);
+    return (bits[id >> 5] >> (id & 31)) & 1u ? 0 : (int)age_s[s];
   };
+  // (of a row that stays: its age is below k_eff <= 32767 and therefore exact)
+  auto stamp_of = [&](int s) { return t_end - (int)age_s[s]; };
   int c_load = 0;
   for (int q = q0; q < q1; ++q) c_load += slot_s[q] == kNoSlot;
   int k_eff = w.k;
@@ -433,12 +436,12 @@ __device__ void window_role(const StepArgs& a, unsigned char* smem) {
         w.slot_of[id] = -1;
       } else if (s >= bound) {
         const int dst = hole_s[reuse + n_moves - 1 - p_surv++];
-        a.row_stamps[dst] = stamp_s[s];                    // (those of active neurons follow below)
+        a.row_stamps[dst] = stamp_of(s);                   // (those of active neurons follow below)
         w.pointers[dst] = id;
         w.slot_of[id] = dst;
         w.bias[dst] = w.bias_up[id];
       } else if (!stamps) {
-        a.row_stamps[s] = stamp_s[s];
+        a.row_stamps[s] = stamp_of(s);
       }
       if (s >= n_kept + n_load) w.pointers[s] = -1;      // tail beyond the rows in use
     }

@@ -167,3 +167,35 @@ def test_a_down_column_is_not_read_by_a_stream_in_which_its_neuron_is_off(S, d, 
     assert torch.equal(y[0, 0], y[1, 0])
     assert torch.isinf(y[1, 1:]).any()
     gpu.close()
+
+
+@pytest.mark.parametrize("F,cap,one", [
+    (16384, 16384, True),     # a row for every neuron
+    (18176, 18176, True),
+    (32768, 11999, True),     # the largest caches: 4 * d_ff + 8 * capacity bytes in a CTA's shared memory
+    (32768, 12100, False),    # beyond them
+])
+def test_layers_with_large_caches_are_one_launch(F, cap, one):
+    # only the single launch has CTAs that wait for one another, so with no polls its steps end in a timeout
+    cfg = W.LifConfig("large", 1, 8, F, 8, 4, 1, 7, 0.05, 1.0, 0.5, 0.8, 79)
+    gpu, ora = P.make_layer_pair(cfg, 0, b_down=True, capacity=cap, append_first=1)
+    X = W.make_inputs(cfg, device=DEV)
+    y = torch.empty(1, cfg.d_model, dtype=torch.float32, device=DEV)
+    for t in range(cfg.steps):
+        none = t == 4
+        if none:
+            B.lif_set_tuning(gpu.handle, B.TUNE_STEP_POLLS, 0)
+        B.lif_decode_step(gpu.handle, X[t], y)
+        if none:
+            B.lif_set_tuning(gpu.handle, B.TUNE_STEP_POLLS, 1 << 20)
+            assert (gpu.lists()["status"] == B.LIF_ERR_TIMEOUT) == one
+        if none and one:
+            lists = ora.cache.window_update(gpu.lists()["active_idx"])
+            ora.cache.insert(lists, ora.bundles, ora.bias_up)
+            B.lif_clear_status(gpu.handle)
+        else:
+            lists = P.check_decode_step(gpu, ora, X[t].cpu().numpy(), y)
+        assert len(lists["load_ids"]) > 0 and (t < 4 or len(lists["evict_ids"]) > 0)
+        torch.cuda.synchronize()
+        P.compare_cache_rows(gpu, ora)
+    gpu.close()
