@@ -275,14 +275,11 @@ __device__ void score_role(const PredictArgs& a, int tile, unsigned char* smem) 
   const int cg = tid & 15, rs = tid >> 4;
   const int col = tile * kLogitTile + cg * 8;
   uint4 bq[8];
-  auto first_rows = [&]() {
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int j = rs + 16 * u;
-      bq[u] = (col < F && j < r) ? ld_stream16(a.B + (size_t)j * F + col) : make_uint4(0, 0, 0, 0);
-    }
-  };
-  first_rows();
+  for (int u = 0; u < 8; ++u) {
+    const int j = rs + 16 * u;
+    bq[u] = (col < F && j < r) ? ld_stream16(a.B + (size_t)j * F + col) : make_uint4(0, 0, 0, 0);
+  }
   for (int u = 0; u < a.staged_b; ++u) {
     const int j = rs + 16 * (8 + u);
     if (col < F && j < r) copy_async16(b_s + u * kThreads + tid, a.B + (size_t)j * F + col);
@@ -301,7 +298,6 @@ __device__ void score_role(const PredictArgs& a, int tile, unsigned char* smem) 
       // followed by a kernel that can do nothing before its list: it is released when z is there.)
       if (!a.compact) pdl_trigger();
     }
-    if (S == 1 && pass && r > 128) first_rows();                    // (the first pass ended with later ones)
     run = __ldcg(a.predictor_run);
     // Whether the neuron already has a cache row is read here, so the mask of neurons to bring in
     // (active and not cached) costs no round trip of its own.
@@ -358,7 +354,7 @@ __device__ void score_role(const PredictArgs& a, int tile, unsigned char* smem) 
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[s][e] = make_float2(0.f, 0.f);
 #pragma unroll 1
-    for (int j0 = 0; j0 < r; j0 += 128) {
+    for (int j0 = 0; j0 < (pass ? r : min(r, 128)); j0 += 128) {       // (the first pass leaves bq as it is)
       if (j0 > 0) {
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
