@@ -39,6 +39,8 @@
 // rows each the last two rows were worked on one after the other behind the link.  Layers of 4544 and
 // 768 columns 79 -> 77.7 and 16.2 -> 15.9 us, three streams at 1544 47.7 -> 46.7; 16 CTAs asked the
 // same way lose 5% to the gap between a landing and the next request, 24 lose 2%.
+#include <type_traits>
+
 #include "lif_internal.cuh"
 #include "mask_compact.cuh"
 #include "window.cuh"
@@ -672,18 +674,19 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
       }
     __syncthreads();
   }
-  auto move_rows = [&]() {
+  auto move_rows = [&](auto pieces) {                      // 16-byte pieces of a thread in flight
+    constexpr int kPieces = decltype(pieces)::value;
     const int row_vec = kVec * nvec;
     for (int j = c; j < n_moves; j += nc) {
       const uint4* src = reinterpret_cast<const uint4*>(a.cache) + (size_t)__ldcg(a.w.move_src + j) * row_vec;
       uint4* dst = reinterpret_cast<uint4*>(a.cache) + (size_t)__ldcg(a.w.move_dst + j) * row_vec;
-      uint4 v[4];
-      for (int v0 = tid; v0 < row_vec; v0 += 4 * kStepThreads) {
+      uint4 v[kPieces];
+      for (int v0 = tid; v0 < row_vec; v0 += kPieces * kStepThreads) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < kPieces; ++u)
           if (v0 + u * kStepThreads < row_vec) v[u] = ld_stream16(src + v0 + u * kStepThreads);
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < kPieces; ++u)
           if (v0 + u * kStepThreads < row_vec) dst[v0 + u * kStepThreads] = v[u];
       }
     }
@@ -712,7 +715,7 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
     if (r0 == 0 && !a.whole_cache) load_x(a, xs);          // while the first rows travel
     if (r0 == 0 && !a.w.append_first) {                    // ... and the moves
       if (!a.whole_cache) n_moves = plan_moves(wait_plan(a, &plan_s));
-      move_rows();
+      move_rows(std::integral_constant<int, kS == 1 ? 2 : 4>{});   // (beside the sums; see step_kernel's bounds)
     }
     __syncthreads();                                       // x and the rows' scalars
     if (rc <= 0) break;
@@ -795,7 +798,7 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
   if (tid == 0 && last) arrive(&a.sync->groups_done);
   if (a.w.append_first) {                                  // (plan_s was not used before)
     n_moves = plan_moves(wait_plan(a, &plan_s));
-    move_rows();
+    move_rows(std::integral_constant<int, 4>{});
   }
 }
 
@@ -1217,10 +1220,15 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
-// (One stream: two CTAs per SM, 64 registers and 0-4 bytes spilled, so that small layers' steps on several
-// streams share the chip.  Rows of 4096 columns leave shared memory for one CTA anyway; with the bound at one,
-// 94-106 registers and no spill, nothing is faster: tiny 28.7 us against 27-28.4, 768 x 3072 61.9 against
-// 61.9-62.8, opt6p7b 8 layers 386.3 against 386.3-387.5.)
+// One stream: two CTAs per SM, 64 registers and no spill, so that small layers' steps on several streams share the
+// chip: eight layers of 768 x 3072 at once 35.2 us for a step of each, 57.9 with the bound at one CTA (107
+// registers); four 18.4 and 30.4.  Layers one after the other are faster with that bound where nothing else is on
+// the SM (768 x 3072, 4 layers 56.5 us against 59.0; three-vector bundles of 4096 columns 416 against 420) and
+// slower where the next layer's predictor then finds no registers beside the step (opt6p7b, 8 layers 379 against
+// 374; falcon7b, 4 layers 319 against 316).
+// What spills at 64 registers is the row moves beside the sums: with four pieces in flight instead of two 64-72 bytes
+// stored and 124-132 loaded per thread, 1424 x 4576 with the FFN over every cached row, 6 layers 100.8 us against 97.4,
+// 768 x 3072 61.4 against 59.5.
 template <int kGate, int kS>
 __global__ void __launch_bounds__(kStepThreads, kS == 1 ? 2 : 1) step_kernel(StepArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
