@@ -437,9 +437,10 @@ lif_status lif_decode_token_host(lif_layer* const* layers, int32_t n_layers, con
     return LIF_ERR_CUDA;
   for (int l = 0; l < n_layers; ++l) {
     layers[l]->input_late = l == 0;
+    layers[l]->behind_step = l > 0;
     lif_status s = lif_decode_step(layers[l], dev_x, dev_y + (size_t)l * per, compute_stream,
                                    fetch_stream);
-    layers[l]->input_late = 0;
+    layers[l]->input_late = layers[l]->behind_step = 0;
     if (s != LIF_OK) return s;
   }
   if (cudaMemcpyAsync(host_y, dev_y, per * 4 * n_layers, cudaMemcpyDeviceToHost, sc) !=
@@ -477,8 +478,9 @@ lif_status lif_graph_capture(lif_layer* const* layers, int32_t n_layers, void* d
   lif_status s = LIF_OK;
   for (int l = 0; l < n_layers && s == LIF_OK; ++l) {
     layers[l]->input_late = l == 0;
+    layers[l]->behind_step = l > 0;
     s = lif_decode_step(layers[l], dev_x, dev_y + (size_t)l * per, compute_stream, fetch_stream);
-    layers[l]->input_late = 0;
+    layers[l]->input_late = layers[l]->behind_step = 0;
   }
   cudaError_t e = cudaStreamEndCapture(sc, &g->graph);   // always end, also after an error
   if (s == LIF_OK && e == cudaSuccess && cudaGraphInstantiate(&g->exec, g->graph, 0) == cudaSuccess) {

@@ -104,6 +104,7 @@ struct lif_layer {
   unsigned wait_polls; // poll limit of the first wait on each bulk copy
   unsigned spin_limit; // poll limit of the waits of a step's CTAs for one another
   int input_late;      // set while the first layer of a token is enqueued: its input comes from a copy
+  int behind_step;     // set while a later one is: the kernel ahead is this library's step of the layer before
   unsigned predictor_polls;   // ... of the predictor's score CTAs for z
   int early_fetch;    // knob: the plain fetch of lif_decode_step starts early behind the window kernel
   int ends_step;      // set by lif_decode_step: the FFN's last kernel advances the run number

@@ -57,10 +57,14 @@ struct PredictArgs {
 // other.  Its pieces of A (one row, 8 columns) travel into its own slots of shared memory ahead of the
 // dependency wait.
 //
-// In a decode step (but for a token's first layer, whose input is there at once) everything behind the wait is
-// executed once before it, on whatever the buffers hold, and the results dropped: a kernel's code comes from L2
-// at its first use, which behind the wait takes as long as the work itself (512 x 2048, from the wait to the
-// entries: 4.2 us, 2.3 with the first pass).
+// Where the kernel ahead is known to be the step of the layer before (a token's later layers in lif_graph_capture and
+// lif_decode_token_host), which lets this one start early, everything behind the wait is executed once before it,
+// on whatever the buffers hold, and the results dropped: a kernel's code comes from L2 at its first use (opt6p7b,
+// 8 layers 373.7 us a token, 375.1 without; tiny 24.75 and 24.9).  Behind anything else, such as another library's
+// kernel that releases nothing early, the wait is over when this kernel starts and that pass would be in the way:
+// two matrix products between the layers of a captured program, 4 layers of 4096 x 16384 330 us with it and
+// 324 without, 2048 x 8192 154.6 and 148, 768 x 3072 90.3 and 85.1 (with steps back to back there is no difference).
+// The score CTAs have such a pass in either case, while z is computed.
 template <int H, int CW>
 __device__ void z_role(const PredictArgs& a, int S, int part_of_grid, unsigned char* smem) {
   constexpr int Q = H * CW;
@@ -600,7 +604,7 @@ cudaError_t launch_predict(lif_layer* L, const __half* x, float* logits, int32_t
   a.compact = compact;
   // The input of these is there at once, so nothing of the predictor is on chip ahead of it.
   const bool late = compact || L->input_late;
-  a.first_pass = late;
+  a.first_pass = compact || !L->behind_step;                           // (see stage 1)
   a.active_idx = (int*)active_idx;
   a.n_active = (int*)n_active;
   cudaError_t e;

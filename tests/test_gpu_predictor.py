@@ -75,6 +75,52 @@ def test_scores_are_those_of_the_stated_order_of_additions(S, d, F, r):
     gpu.close()
 
 
+@pytest.mark.parametrize("S,d,F,r", [
+    (1, 8, 64, 8),
+    (1, 8192, 136, 8),       # by parts
+    (5, 2568, 136, 48),      # ... several streams
+    (8, 4104, 136, 40),      # few columns at a time
+    (1, 1000, 520, 248),
+    (3, 1544, 392, 72),
+    (8, 7168, 264, 256),     # two streams per CTA
+    (7, 520, 136, 1024),     # four
+])
+def test_later_layers_of_a_graph_equal_steps_by_themselves(S, d, F, r):
+    # the first stage of a graph's later layers runs once ahead of its wait, that of a step by itself does not
+    cfg = W.LifConfig("passes", 3, d, F, r, 2, S, 4, 0.10, 1.0, 0.7, 0.7, 77)
+    gpus = [P.make_layer_pair(cfg, l, capacity=F, append_first=1)[0] for l in range(cfg.n_layers)]
+    X = W.make_inputs(cfg, device=DEV)
+    x = torch.empty(S, d, dtype=torch.float16, device=DEV)
+    y = torch.empty(2, cfg.steps, cfg.n_layers, S, d, dtype=torch.float32, device=DEV)
+    out = torch.empty(cfg.n_layers, S, d, dtype=torch.float32, device=DEV)
+    sc, sf = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = B.lif_graph_capture([gpu.handle for gpu in gpus], x, out, sc, sf)
+    with torch.cuda.stream(sc):
+        for t in range(cfg.steps):
+            x.copy_(X[t])
+            B.lif_graph_launch(graph, sc)
+            y[0, t].copy_(out)
+    torch.cuda.synchronize()
+    state = [gpu.lists() for gpu in gpus]
+    for gpu in gpus:
+        B.lif_reset(gpu.handle)
+    torch.cuda.synchronize()
+    for t in range(cfg.steps):
+        for l, gpu in enumerate(gpus):
+            B.lif_decode_step(gpu.handle, X[t], y[1, t, l], sc, sf)
+    torch.cuda.synchronize()
+    assert torch.equal(y[0], y[1])
+    for gpu, one in zip(gpus, state):
+        other = gpu.lists()
+        assert one["status"] == other["status"] == B.LIF_OK and one["step"] == other["step"] == cfg.steps
+        for key in ("pointers", "slot_of", "last_active"):
+            np.testing.assert_array_equal(one[key], other[key])
+    B.lif_graph_destroy(graph)
+    for gpu in gpus:
+        gpu.close()
+
+
 @pytest.mark.parametrize("S", [1, 3])
 def test_a_score_that_lacks_z_is_not_active_and_the_call_says_so(S):
     cfg = W.LifConfig("lost z", 1, 4096, 2048, 128, 3, S, 5, 0.08, 1.0, 0.8, 0.6, 76)
