@@ -57,9 +57,9 @@ def test_decode_step_at_the_edges(S, d, F, r, fire, gate_mode, append_first):
     assert sum(loads) > 0
 
 
-@pytest.mark.parametrize("S", [1, 3])
-def test_a_refused_update_brings_nothing_in_and_the_next_step_follows_the_oracle(S):
-    cfg = W.LifConfig("refused", 1, 1032, 4096, 32, 3, S, 8, 0.04, 1.0, 0.8, 0.6, 72)
+@pytest.mark.parametrize("S,d", [(1, 1032), (3, 1032), (2, 4096)])       # (the last: rows handed over)
+def test_a_refused_update_brings_nothing_in_and_the_next_step_follows_the_oracle(S, d):
+    cfg = W.LifConfig("refused", 1, d, 4096, 32, 3, S, 8, 0.04, 1.0, 0.8, 0.6, 72)
     gpu, ora = P.make_layer_pair(cfg, 0, b_down=True, append_first=1, capacity=1500)
     X = W.make_inputs(cfg, device=DEV)
     y = torch.empty(S, cfg.d_model, dtype=torch.float32, device=DEV)

@@ -112,15 +112,17 @@ def test_staged_bundles_of_a_file_store_whose_copies_are_given_up(tmp_path):
 
 
 @pytest.mark.parametrize("append_first", [0, 1])
-@pytest.mark.parametrize("S,d,gate_mode", [
-    (1, 264, B.GATE_NONE),           # a ring of 16 stages
-    (1, 8192, B.GATE_BUNDLED),       # two stages of 48 KB
-    (1, 1032, B.GATE_RESIDENT),
-    (5, 1032, B.GATE_NONE),
+@pytest.mark.parametrize("S,d,F,gate_mode", [
+    (1, 264, 4096, B.GATE_NONE),     # a ring of 16 stages
+    (1, 8192, 1024, B.GATE_BUNDLED),   # two stages of 48 KB
+    (1, 1032, 4096, B.GATE_RESIDENT),
+    (5, 1032, 4096, B.GATE_NONE),
+    (5, 2056, 4096, B.GATE_NONE),    # last rows handed over, never reached
+    (4, 2056, 128, B.GATE_NONE),     # ... the only row of its fetch CTA
 ])
-def test_the_single_launch_fills_rows_whose_copies_it_gave_up(S, d, gate_mode, append_first):
+def test_the_single_launch_fills_rows_whose_copies_it_gave_up(S, d, F, gate_mode, append_first):
     act, thr = (B.ACT_FATRELU, 0.05) if gate_mode else (B.ACT_RELU, 0.0)
-    gpu, ora, X, y, streams = _layer(S=S, steps=0, d=d, F=1024 if d == 8192 else 4096, gate_mode=gate_mode,
+    gpu, ora, X, y, streams = _layer(S=S, steps=0, d=d, F=F, gate_mode=gate_mode,
                                      activation=act, act_threshold=thr, append_first=append_first)
     for t in range(6):               # cold (more rows than a ring) and warm (rows of others move) in turn
         lost = t % 2 == 0
@@ -155,14 +157,16 @@ def test_cached_rows_whose_copies_were_given_up_leave_the_layer_usable():
     gpu.close()
 
 
-@pytest.mark.parametrize("S,gate_mode,ffn_mode,append_first", [
-    (1, B.GATE_NONE, 0, 0), (1, B.GATE_NONE, 0, 1), (1, B.GATE_NONE, 1, 0), (1, B.GATE_BUNDLED, 0, 0),
-    (1, B.GATE_BUNDLED, 0, 1), (4, B.GATE_NONE, 0, 0), (4, B.GATE_NONE, 0, 1)])
+@pytest.mark.parametrize("S,d,gate_mode,ffn_mode,append_first", [
+    (1, 1032, B.GATE_NONE, 0, 0), (1, 1032, B.GATE_NONE, 0, 1), (1, 1032, B.GATE_NONE, 1, 0),
+    (1, 1032, B.GATE_BUNDLED, 0, 0), (1, 1032, B.GATE_BUNDLED, 0, 1), (4, 1032, B.GATE_NONE, 0, 0),
+    (4, 1032, B.GATE_NONE, 0, 1),
+    (4, 2056, B.GATE_NONE, 0, 0), (4, 2056, B.GATE_NONE, 0, 1)])     # last rows handed over
 def test_rows_named_by_a_step_whose_parts_gave_up_are_read_again_when_the_status_is_cleared(
-        S, gate_mode, ffn_mode, append_first):
+        S, d, gate_mode, ffn_mode, append_first):
     # Every wait of a CTA for another gives up at once: the window CTA commits the plan, no row of it is
     # moved or brought in.  No copy is left behind: those asked for ahead of the plan are waited for.
-    gpu, ora, X, y, streams = _layer(S=S, steps=0 if ffn_mode else 4, gate_mode=gate_mode, ffn_mode=ffn_mode,
+    gpu, ora, X, y, streams = _layer(S=S, steps=0 if ffn_mode else 4, d=d, gate_mode=gate_mode, ffn_mode=ffn_mode,
                                      append_first=append_first)
     for t in range(4 if ffn_mode else 0):
         B.lif_decode_step(gpu.handle, X[t], y, *streams)
