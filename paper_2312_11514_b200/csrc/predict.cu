@@ -479,7 +479,9 @@ constexpr int kMaxStaged = 12;         // pieces of B per thread in shared memor
 constexpr size_t kSharedSmem = 100 * 1024;   // ... with which two predictor CTAs still fit an SM
 constexpr size_t kFewColumns = 40 * 1024;   // see predict_shape
 constexpr int kColumnCtas = 128;       // z CTAs at most, as long as a CTA can take more streams
-constexpr size_t kZSmem = 200 * 1024;  // bytes of shared memory that a z CTA takes with more than 2 columns at a time
+constexpr size_t kZSmem = 200 * 1024;  // bytes of shared memory that a z CTA takes with more than 2 columns at a
+                                       // time, one stream
+constexpr size_t kZSmemStreams = 224 * 1024;   // ... that it takes with more streams (all 8 columns at a time)
 
 // The launch shape of the two stages and their shared memory.
 struct PredictSmem {
@@ -496,14 +498,16 @@ PredictSmem predict_shape(const lif_layer_desc& D, PredictArgs& a) {
   a.per = (a.rows + a.lanes - 1) / a.lanes;
   if (a.lanes > a.rows) a.lanes = a.rows;                    // (runs without rows)
   const size_t runs = (size_t)a.lanes * a.parts;
+  a.x_at = (int)(runs * a.per) * 16;
+  auto sums_at = [&](int h) { return (a.x_at + h * (d + 2 * a.parts) * 2 + 15) / 16 * 16; };
   // Several streams share a CTA where there would be too many CTAs otherwise (A is read again from L2 by
-  // each).
+  // each), as long as their x and sums fit: four do but for the widest layers (8000 columns at rank 264: 230 KB).
   a.h = 1;
-  while (S > a.h && a.h < (d > 8000 ? 2 : 4) && (r / 8) * ((S + a.h - 1) / a.h) > kColumnCtas) a.h *= 2;
+  while (S > a.h && a.h < 4 && (r / 8) * ((S + a.h - 1) / a.h) > kColumnCtas &&
+         sums_at(2 * a.h) + (runs + a.parts) * 2 * a.h * 8 * 4 <= kZSmemStreams) a.h *= 2;
   a.groups_of_streams = (S + a.h - 1) / a.h;
   a.n_z = r / 8 * a.groups_of_streams;
-  a.x_at = (int)(runs * a.per) * 16;
-  a.red_at = (a.x_at + a.h * (d + 2 * a.parts) * 2 + 15) / 16 * 16;
+  a.red_at = sums_at(a.h);
   a.n_scores = (D.d_ff + kLogitTile - 1) / kLogitTile;
   a.staged_b = (r + 15) / 16 - 8;
   a.staged_b = a.staged_b < 0 ? 0 : (a.staged_b > kMaxStaged ? kMaxStaged : a.staged_b);
@@ -572,7 +576,11 @@ cudaError_t predict_configure(const lif_layer* L) {
   cudaFuncAttributes at;
   cudaError_t e = cudaFuncGetAttributes(&at, k);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, L->max_smem - (int)at.sharedSizeBytes);
+  PredictArgs a = {};
+  const PredictSmem m = predict_shape(L->desc, a);
+  const size_t most = L->max_smem - at.sharedSizeBytes;
+  if (m.z > most || m.scores > most) return cudaErrorInvalidConfiguration;   // (no accepted layer: z at most 224 KB)
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
 cudaError_t launch_predict_one(lif_layer* L, int kernel, const __half* x, cudaStream_t st) {

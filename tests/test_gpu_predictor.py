@@ -58,6 +58,8 @@ def _scores_in_order(x, A, Bm, c):
     (5, 4096, 136, 128),
     (8, 7168, 264, 256),     # two streams per CTA
     (7, 520, 136, 1024),     # four, the last CTA three
+    (8, 8000, 136, 264),     # two: four streams' x and sums, 230 KB, would not fit
+    (8, 8192, 136, 520),     # four of the widest
 ])
 def test_scores_are_those_of_the_stated_order_of_additions(S, d, F, r):
     cfg = W.LifConfig("scores", 1, d, F, r, 2, S, 2, 0.10, 1.0, 0.7, 0.7, 75)
