@@ -48,7 +48,8 @@ def _scores_in_order(x, A, Bm, c):
     (1, 8, 8, 8),            # one run with a row
     (1, 8192, 136, 8),       # by parts: one column group, most lanes
     (1, 6128, 136, 136),     # ... a column group that is too long
-    (5, 2568, 136, 48),      # ... several streams; a last part of 40 rows
+    (5, 2568, 136, 48),      # ... several streams; a last part of 72 rows
+    (2, 2568, 136, 56),      # ... two streams, a number of words that 256 threads do not divide
     (8, 4104, 136, 40),      # by columns at a small rank: many runs, few columns at a time
     (1, 4104, 264, 120),     # a last part of 8 rows
     (1, 1000, 520, 248),     # runs of different lengths, rank not a multiple of 16
