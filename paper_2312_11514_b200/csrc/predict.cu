@@ -490,7 +490,7 @@ PredictKernel predict_kernel_for(int S) {
 
 constexpr int kMaxStaged = 12;         // pieces of B per thread in shared memory: 48 KB
 constexpr size_t kSharedSmem = 100 * 1024;   // ... with which two predictor CTAs still fit an SM
-constexpr size_t kFewColumns = 40 * 1024;   // see predict_shape
+constexpr size_t kFewColumns = 40 * 1024, kFewColumnsTwo = 64 * 1024;   // see predict_shape
 constexpr int kColumnCtas = 128;       // z CTAs at most, as long as a CTA can take more streams
 constexpr size_t kZSmem = 200 * 1024;  // bytes of shared memory that a z CTA takes with more than 2 columns at a
                                        // time, one stream
@@ -529,11 +529,23 @@ PredictSmem predict_shape(const lif_layer_desc& D, PredictArgs& a) {
   a.cw = 8;
   while (a.h == 1 && a.cw > 2 && a.red_at + (runs + a.parts) * a.cw * 4 > kZSmem) a.cw /= 2;
   m.z = a.red_at + (runs + a.parts) * a.h * a.cw * 4;
-  // By parts: few columns of many rows (two z CTAs at rank 16 took 11 us longer than 32 at 6128 rows; at 256
-  // rows they are 0.8 us faster), as long as the parts' sums that every score CTA reads are few; one stream of
-  // many rows.
+  // By parts, or by columns: a z CTA of columns has all rows to add, and at small ranks so many runs that their sums
+  // fit only for 4 or 2 columns at a time; of parts' sums every score CTA reads parts * S * rank words.  us a token,
+  // 4 layers (several streams: 3), d_ff = 2 d, columns / parts:
+  //   one stream, ranks to 64: 1024 x 16 50.7 / 50.4, 2048 x 32 67.7 / 62.7, 2048 x 64 64.1 / 62.8, 4096 x 48 120.9 /
+  //     113, 6128 x 16 264.5 / 221.6 (512 x 32 43.7 / 45 when the words came in four rounds); beyond, where the CTA
+  //     would fill an SM: 4096 x 96 123.1 / 119.5, but 2048 x 96 62.3 / 63.4 and 3072 x 96 86.9 / 89.7;
+  //   two, ranks below 64: 1544 x 32 59.9 / 57, 2048 x 16 69.3 / 65.5, 4096 x 32 116.3 / 113.4, but 1024 x 16 47.6 /
+  //     48.1 and 2048 x 64 67.2 / 69.1;
+  //   more: with 2 columns at a time 4 x 6128 x 16 366 / 340, 6 x 5120 x 16 385 / 355, 8 x 5120 x 16 442 / 420; with 4
+  //     columns 3 x 4096 x 16 165 / 156.5, 4 x 4096 x 16 195.5 / 192.2, 5 x 4608 x 16 (2 layers) 198.4 / 191.9,
+  //     8 x 4096 x 16 299 / 316; with 8 columns 3 x 2048 x 32 80.2 / 81.9, 4 x 4096 x 32 180 / 185.6, 8 x 2048 x 16
+  //     131.3 / 140.2.
   const size_t z_part = (size_t)a.per * kThreads * 16 + S * a.rows * 2 + (size_t)a.lanes * r * 4;
-  a.by_parts = ((r < 64 && S * r <= 256 && m.z > kFewColumns) || (S == 1 && m.z > kSharedSmem)) && z_part <= kSharedSmem;
+  const bool parts_pay = S == 1   ? (r <= 64 && m.z > kFewColumns) || m.z > kSharedSmem
+                         : S == 2 ? r < 64 && m.z > kFewColumnsTwo
+                                  : a.h == 1 && (a.cw == 2 || (a.cw == 4 && S <= 5));
+  a.by_parts = parts_pay && z_part <= kSharedSmem;
   if (a.by_parts) {
     a.n_z = a.parts;
     a.x_at = a.per * kThreads * 16;

@@ -48,8 +48,11 @@ def _scores_in_order(x, A, Bm, c):
     (1, 8, 8, 8),            # one run with a row
     (1, 8192, 136, 8),       # by parts: one column group, most lanes
     (1, 6128, 136, 136),     # ... a column group that is too long
-    (5, 2568, 136, 48),      # ... several streams; a last part of 72 rows
-    (2, 2568, 136, 56),      # ... two streams, a number of words that 256 threads do not divide
+    (5, 2568, 136, 48),      # by columns; a last part of 72 rows
+    (2, 2568, 136, 56),      # by parts, two streams; a number of words that 256 threads do not divide
+    (4, 4104, 136, 16),      # ... four, which would be 4 columns at a time
+    (8, 5120, 136, 16),      # ... eight, which would be 2
+    (1, 1024, 136, 64),      # ... the largest small rank
     (8, 4104, 136, 40),      # by columns at a small rank: many runs, few columns at a time
     (1, 4104, 264, 120),     # a last part of 8 rows
     (1, 1000, 520, 248),     # runs of different lengths, rank not a multiple of 16
@@ -81,7 +84,9 @@ def test_scores_are_those_of_the_stated_order_of_additions(S, d, F, r):
 @pytest.mark.parametrize("S,d,F,r", [
     (1, 8, 64, 8),
     (1, 8192, 136, 8),       # by parts
-    (5, 2568, 136, 48),      # ... several streams
+    (5, 2568, 136, 48),
+    (2, 2568, 136, 48),      # by parts, several streams
+    (8, 5120, 136, 16),
     (8, 4104, 136, 40),      # few columns at a time
     (1, 1000, 520, 248),
     (3, 1544, 392, 72),
