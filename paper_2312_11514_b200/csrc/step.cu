@@ -1074,7 +1074,11 @@ __device__ void fetch_role(const StepArgs& a, int f, unsigned char* smem) {
   };
   if (tid == 0) {
     count_s = cnt;
-    if (kS > 1 && cnt > 0) learn(true);                   // (3 streams at 1544 columns: 46.2 us a step, 46.6 without)
+    // Where rows are short the plan is there before the first one, and asking now is cheaper than between rows: 3 streams
+    // at 1544 columns 160 us (4 layers), 160.9 without.  Wide rows' terms go ahead of the plan: 4 streams at 3704
+    // columns, 2 layers, 230 us with the wait, 222.6 without.  Never in the paper's order, where this waits for the
+    // moves and with them for the cached rows' terms: 2 x 1112, 4 layers, 96.4 us and 75.8, 3 x 4096 407 and 336.
+    if (kS > 1 && cnt > 0 && a.w.append_first && !a.hand_over) learn(true);
   }
   __syncthreads();
   unsigned parity = 0;
