@@ -1267,8 +1267,10 @@ StepKernel step_kernel_for(const lif_layer_desc& D) {
 }
 constexpr int kGroupMax = 8, kUngroupedMax = 64, kUngroupedMaxStreams = 16;
 // One step CTA per SM (with less, two fit and are put on one SM where others are not free yet), and beside it one of
-// the next layer's low-rank predictor, 91 KB at 4096 x 128.
-constexpr size_t kCacheRing = 112 * 1024, kCacheRingGate = 128 * 1024, kFetchRing = 32 * 1024;
+// the next layer's low-rank predictor, 91 KB at 4096 x 128.  With several streams, whose cached rows are many and are
+// added by fewer CTAs, what a CTA can have beside x: 6 streams at 3704 columns, 3 layers, 464 us with 112 KB, 441 with 128,
+// 421 with 160, 416 with 192; 8 x 2048 254.6 and 246, 8 x 3704, one layer, 219 and 198.5; even where a CTA has few rows.
+constexpr size_t kCacheRing = 112 * 1024, kCacheRingGate = 128 * 1024, kCacheRingStreams = 192 * 1024, kFetchRing = 32 * 1024;
 
 // Streams x columns from which a fetch CTA hands its last row over instead of adding it to its partial: 5 x 4096 260 ->
 // 250 us (2 layers), 3 x 1544 180 -> 183 (4 layers), where a partial is 37 KB and the further words cost more.
@@ -1334,7 +1336,8 @@ cudaError_t step_configure(lif_layer* L) {
   L->step_sum_ctas = sum_ctas(D);
   L->step_group = L->step_cache_ctas > hit_partials_max(D) ? kGroupMax : 1;
   const size_t hits = 2 * (((size_t)D.capacity + L->step_cache_ctas - 1) / L->step_cache_ctas);
-  L->step_cache_stages = stages(D.gate_mode == LIF_GATE_RESIDENT ? kCacheRingGate : kCacheRing, x + hits, 1);
+  L->step_cache_stages = stages(D.n_streams > 1 ? kCacheRingStreams
+                                : D.gate_mode == LIF_GATE_RESIDENT ? kCacheRingGate : kCacheRing, x + hits, 1);
   // (paper's cache order: bundles wait in the ring, see fetch_role; twice the ring keeps the link busy)
   L->step_fetch_stages = stages(D.append_first ? kFetchRing : 2 * kFetchRing, x + ids, 2);
   size_t smem = window_role_smem(D.d_ff, D.capacity, D.ffn_mode == 1);
