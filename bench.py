@@ -455,8 +455,9 @@ def measure(args, config_name, steps, warmup, rank, world, local, detail):
             "e2e": {"value": whole_job_tokens_per_s(K, 1 if sharded else world, ms_e2e), "unit": UNIT,
                     "h2d_bytes_per_step": S * d * 2, "d2h_bytes_per_step": L * S * d * 4,
                     "host_link_bytes_per_step": fetched / K},
-            # per layer-step, one stream: the predictor (or the gate kernel) and the step kernel; several: the
-            # predictor as two launches (or the gate kernel), window, moves, fetch, up + down for cached and for new rows, sum
+            # per layer-step, one stream: the predictor (or the gate kernel) and the step kernel; several (batched8,
+            # the one such shape here): the predictor as two launches, because a CTA of its first stage needs an SM's
+            # shared memory (or the gate kernel), window, moves, fetch, up + down for cached and for new rows, sum
             "gpu_launches": (2 if S == 1 else 10 - (1 if gate_mode == B.GATE_RESIDENT else 0)
                              + (2 if gate_mode == B.GATE_BUNDLED else 0)) * n_launch,
             "roofline": roofline,

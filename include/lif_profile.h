@@ -60,8 +60,9 @@ lif_status lif_set_tuning(lif_layer* layer, int32_t key, int32_t value);
 
 /* Phases timed by lif_timing_* (one CUDA event pair each, inside lif_decode_step). */
 enum {
-  LIF_PHASE_PREDICT_Z = 0,      /* (nothing: both stages of the predictor are one launch) */
-  LIF_PHASE_PREDICT_SCORES = 1, /* predictor: x.A, scores, threshold, compaction */
+  LIF_PHASE_PREDICT_Z = 0,      /* x.A where the predictor is two launches (several streams whose input is
+                                   there at once, or a first stage that fills an SM); zero otherwise */
+  LIF_PHASE_PREDICT_SCORES = 1, /* predictor: scores, threshold, compaction; x.A too in one launch */
   LIF_PHASE_WINDOW = 2,         /* window bookkeeping kernel */
   LIF_PHASE_MOVES = 3,          /* row moves */
   LIF_PHASE_FETCH = 4,          /* bundle fetch (on the fetch stream) */

@@ -99,7 +99,7 @@ struct StepArgs {
   int d, n_streams, whole_cache, act;
   float act_thr;
   int hand_over;                  // several streams: see kHandOver
-  int n_cache_ctas, n_sum_ctas, group_size, cache_stages, fetch_stages, fetch_rows_max, hits_max;
+  int n_cache_ctas, n_sum_ctas, group_size, cache_stages, fetch_stages, hits_max;
   unsigned wait_polls;            // of the first wait for a bulk copy
   unsigned spin_limit;            // of a wait for another CTA
   unsigned epoch;                 // steps before this one (filled in by the kernel)
@@ -257,8 +257,10 @@ __host__ __device__ __forceinline__ size_t x_smem_bytes(int d, int S) {
 // every neuron (64 KB at 16384) and the stamp of every row by its neuron held back the predictor's CTA on
 // the same SM, and with it the last entry, by 1.5 us (2.2 at 4544 columns).  So the step keeps a copy of the
 // stamps by row, which a window update by another kernel makes out of date (CNT_ROW_STAMPS).
-// (Up to 4096 neurons slot_of is two loads per thread, and a round trip less between the entries and the plan;
-// up to 8192 with the FFN over every cached row, which waits for the plan: 656 x 2664, 2 layers, 37.2 us without it.)
+// slot_of on chip ahead of the entries: a round trip less between them and the plan, which the FFN over every cached row
+// waits for (4 layers, without / with: 512 x 2048 61.9 / 60.9 us, 768 x 3072 63.8 / 62.6, 2048 x 8192 103.2 / 102.6, 2560 x
+// 10240 133.7 / 133.4).  Otherwise nothing is on the chain behind the plan: even, 512 x 2048 to 2048 x 16384, and not
+// done where it is more than two loads per thread.
 __host__ __device__ __forceinline__ bool slots_ahead(int F, int whole_cache) { return F <= (whole_cache ? 8192 : 4096); }
 // (It decides which layers are one launch: with ages of 16 bits, every capacity up to 18900 neurons.)
 size_t window_role_smem(int F, int cap, int whole_cache) {
@@ -796,7 +798,7 @@ __device__ void cache_role(const StepArgs& a, int c, unsigned char* smem) {
   }
   // (only the paper's cache order waits for this: the rows have been read and moved)
   if (tid == 0 && last) arrive(&a.sync->groups_done);
-  if (a.w.append_first) {                                  // (plan_s was not used before)
+  if (a.w.append_first) {            // (plan_s was not used before: the FFN over every cached row excludes this order)
     n_moves = plan_moves(wait_plan(a, &plan_s));
     move_rows(std::integral_constant<int, 4>{});
   }
@@ -1272,8 +1274,10 @@ constexpr int kGroupMax = 8, kUngroupedMax = 64, kUngroupedMaxStreams = 16;
 // 421 with 160, 416 with 192; 8 x 2048 254.6 and 246, 8 x 3704, one layer, 219 and 198.5; even where a CTA has few rows.
 constexpr size_t kCacheRing = 112 * 1024, kCacheRingGate = 128 * 1024, kCacheRingStreams = 192 * 1024, kFetchRing = 32 * 1024;
 
-// Streams x columns from which a fetch CTA hands its last row over instead of adding it to its partial: 5 x 4096 260 ->
-// 250 us (2 layers), 3 x 1544 180 -> 183 (4 layers), where a partial is 37 KB and the further words cost more.
+// Streams x columns from which a fetch CTA hands its last row over instead of adding it to its partial.  us a token of
+// 3 layers, never / always: 2 x 7168 800.6 / 792.4, 4 x 4096 463.6 / 459, 2 x 4096 184.6 / 178.8, 8 x 1024 97.6 / 95.5,
+// 4 x 2048 153.1 / 152.2; 6 x 1032 105.8 / 104.2 and, with a third of the rows, 85.5 / 86.2, 3 x 2056 94.8 / 94.7; 3 x 1544
+// 81 / 82.1, 2 x 2048 81.7 / 82.8, 2 x 1032 53.7 / 57.3: there a partial is short and the further words cost more.
 constexpr int kHandOver = 8192;
 
 // CTAs that add up the outputs: 16 pairs of columns or more each, which leaves 16 slices of the partials to
@@ -1390,7 +1394,6 @@ cudaError_t launch_step(lif_layer* L, const __half* x, float* y, cudaStream_t st
   a.group_size = L->step_group;
   a.cache_stages = L->step_cache_stages;
   a.fetch_stages = L->step_fetch_stages;
-  a.fetch_rows_max = (D.d_ff + kFetchCtas - 1) / kFetchCtas;
   a.hits_max = (D.capacity + a.n_cache_ctas - 1) / a.n_cache_ctas;
   a.wait_polls = L->wait_polls;
   a.spin_limit = L->spin_limit;
